@@ -107,9 +107,10 @@ typedef struct {
     int outer;                    /* DGMG_OUTER_* (default AUTO)                       */
     double delta;                 /* reliable-update factor, 0 < delta < 1 (0.01)      */
     int autotune;                 /* 1: dgmg_create times the candidate tile shapes of */
-                                  /* the DG-level kernels on this mesh and keeps the   */
-                                  /* fastest (cached per mesh shape in the process);   */
-                                  /* 0 (default): fixed heuristic                      */
+                                  /* the FP32 DG-level kernels on this mesh and keeps  */
+                                  /* the fastest (cached per mesh shape in the         */
+                                  /* process; the FP64 kernels have one shape per      */
+                                  /* degree); 0 (default): fixed heuristic             */
     int p_coarsening;             /* 0 (default): DG degree p straight to continuous   */
                                   /* Q1 (Sec. 5.2); 1: gradual, DG p, p-1, ..., 1, then */
                                   /* Q1 (the nested sequence of the outlook of Sec.    */
@@ -141,10 +142,10 @@ typedef struct {
                                   /* p-coarsening)                                     */
     int tiles[6];                 /* cells per CTA of the DG-level kernels in use:     */
                                   /* FP64 projection, smoothing, residual, then FP32   */
-                                  /* (mixed precision only, else 0); a smoothing entry */
-                                  /* of 0 = the one-thread-per-cell kernel where it    */
-                                  /* applies (3D, exact blocks, FP32 q <= 5, FP64      */
-                                  /* q <= 4), else the default pencil tile             */
+                                  /* (mixed precision only, else 0); an FP32 smoothing */
+                                  /* entry of 0 = the one-thread-per-cell kernel where */
+                                  /* it applies (3D, exact blocks, q <= 5), else the   */
+                                  /* default pencil tile                               */
 } dgmg_info_t;
 
 typedef struct {

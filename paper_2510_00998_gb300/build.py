@@ -15,7 +15,8 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libdgmg.so")
-SOURCES = ["dg_fp64.cu", "dg_fp32.cu", "ctx.cu", "solver.cu", "server.cu", "batch.cu", "cg.cu", "blas.cu", "noalloc.cu",
+SOURCES = ["dg_fx_3d_p6.cu", "dg_fx_3d_p5.cu", "dg_fx_3d_p4.cu", "dg_fx_3d_low.cu", "dg_fx_2d.cu", "fx_host.cpp",
+           "dg_fp64.cu", "dg_fp32.cu", "ctx.cu", "solver.cu", "server.cu", "batch.cu", "cg.cu", "blas.cu", "noalloc.cu",
            "volume.cu",
            "factors.cu", "refelem.cpp"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

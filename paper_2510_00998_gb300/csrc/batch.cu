@@ -281,30 +281,21 @@ const T *level_result(const dgmg_batch &B, int i, int l) {
     return L.u[(B.opts.nu_pre + B.opts.nu_post) & 1];
 }
 
-template <typename T>
-bool cells_apply(const dgmg_batch &B, int q) {
-    return B.dim == 3 && q <= (std::is_same<T, float>::value ? 5 : 4) && B.opts.block_inverse == DGMG_BLOCK_EXACT;
-}
-
-// The one-thread-per-cell kernel for stage `stage` of precision T: the smoothing
-// step, and the residual where the level carries the exact blocks' factors (the
-// FP64 level of a mixed batch only applies the operator and has none).
-template <typename T>
+// The one-thread-per-cell FP32 kernel for stage `stage`: the smoothing step and the
+// residual with exact blocks.
 bool cells_stage(const dgmg_batch &B, int q, int stage) {
-    if (!cells_apply<T>(B, q)) return false;
-    if (stage == TILE_SMOOTH) return true;
-    return stage == TILE_RESIDUAL && !(std::is_same<T, double>::value && B.mixed);
+    return B.dim == 3 && q <= 5 && B.opts.block_inverse == DGMG_BLOCK_EXACT && stage != TILE_PROJECT;
 }
 
 template <typename T>
 int build_block_map(dgmg_batch &B, dgmg_batch::Group &grp, int stage) {
     auto &g = grp.prec<T>();
     const int nf = (int)(B.inst[grp.members[0]]->nloc / grp.q);
+    if (std::is_same<T, double>::value) g.tile[stage] = fx_cells_per_cta(B.dim, grp.q);
     int tile = g.tile[stage];
     if (tile <= 0) {
-        // the one-thread-per-cell smoother where it applies, else ~128 threads
-        const bool cells = cells_stage<T>(B, grp.q, stage);
-        if (cells) {
+        // the one-thread-per-cell kernel where it applies, else ~128 threads
+        if (cells_stage(B, grp.q, stage)) {
             tile = BATCH_ALIGN_CELLS;
         } else {
             tile = std::max(1, 128 / nf);
@@ -321,12 +312,12 @@ int build_block_map(dgmg_batch &B, dgmg_batch::Group &grp, int stage) {
     return B.upload(&g.map[stage], m);
 }
 
-// Tile autotuning of a group's DG-level launches (opts.autotune): every
+// Tile autotuning of a group's FP32 DG-level launches (opts.autotune): every
 // candidate cells-per-CTA value (and, for the smoothing step, the
 // one-thread-per-cell kernel) is timed on the batch's own buffers, one warm-up
 // and three timed launches; the fastest is kept.
-template <typename T>
-int tune_group(dgmg_batch &B, dgmg_batch::Group &grp, T *u, T *bv, cudaStream_t s) {
+int tune_group(dgmg_batch &B, dgmg_batch::Group &grp, float *u, float *bv, cudaStream_t s) {
+    using T = float;
     auto &g = grp.prec<T>();
     const int nf = (int)(B.inst[grp.members[0]]->nloc / grp.q);
     const int exact = B.opts.block_inverse == DGMG_BLOCK_EXACT ? 1 : 0;
@@ -340,11 +331,8 @@ int tune_group(dgmg_batch &B, dgmg_batch::Group &grp, T *u, T *bv, cudaStream_t 
     u += grp.dof0;
     bv += grp.dof0;
     for (int st = 0; st < 3; ++st) {
-        // mixed precision: the FP64 level only applies the operator (its problems
-        // carry no FP64 block-inverse factors), so its smoothing step is never run
-        if (std::is_same<T, double>::value && B.mixed && st == TILE_SMOOTH) continue;
         std::vector<int> cs = cand;
-        if (cells_stage<T>(B, grp.q, st)) cs.insert(cs.begin(), 0);
+        if (cells_stage(B, grp.q, st)) cs.insert(cs.begin(), 0);
         int best = cs[0];
         float best_ms = 1e30f;
         for (int c : cs) {
@@ -354,8 +342,8 @@ int tune_group(dgmg_batch &B, dgmg_batch::Group &grp, T *u, T *bv, cudaStream_t 
                 if (st == TILE_PROJECT)
                     return launch_project_batch<T>(B.dim, grp.q, g.D, g.map[st], g.nblocks[st], g.tile[st], u, 0, s);
                 if (st == TILE_SMOOTH)
-                    return launch_smooth_batch<T>(B.dim, grp.q, g.D, g.map[st], g.nblocks[st], g.tile[st], exact, u,
-                                                  bv, 0, s);
+                    return launch_smooth_batch<T>(B.dim, grp.q, g.D, g.map[st], g.nblocks[st], g.tile[st], exact, 0,
+                                                  u, bv, 0, s);
                 return launch_residual_batch<T>(B.dim, grp.q, g.D, g.map[st], g.nblocks[st], g.tile[st],
                                                 RES_HAS_B | RES_CORNERS, u, bv, nullptr, 0, s);
             };
@@ -441,18 +429,23 @@ int batch_cg_cycle(dgmg_batch &B, int l, cudaStream_t s) {
 template <typename T>
 int batch_vcycle(dgmg_batch &B, const T *r, T *z, cudaStream_t s) {
     const int exact = B.opts.block_inverse == DGMG_BLOCK_EXACT ? 1 : 0;
-    LC(cudaMemsetAsync(z, 0, sizeof(T) * B.ndof, s));
-    for (auto &grp : B.groups)
-        LC(launch_zero_traces_batch<T>(B.dim, grp.q, grp.prec<T>().D, (int)grp.members.size(), s));
-    auto smooth = [&](int k) -> int {
+    // FP64: the first step takes the zero iterate as such, nothing reads the
+    // projections of the last one
+    const bool fx = std::is_same<T, double>::value;
+    if constexpr (!std::is_same<T, double>::value) {
+        LC(cudaMemsetAsync(z, 0, sizeof(T) * B.ndof, s));
+        for (auto &grp : B.groups)
+            LC(launch_zero_traces_batch<T>(B.dim, grp.q, grp.prec<T>().D, (int)grp.members.size(), s));
+    }
+    auto smooth = [&](int k, int flags) -> int {
         for (auto &grp : B.groups) {
             auto &g = grp.prec<T>();
             LC(launch_smooth_batch<T>(B.dim, grp.q, g.D, g.map[TILE_SMOOTH], g.nblocks[TILE_SMOOTH],
-                                      g.tile[TILE_SMOOTH], exact, z + grp.dof0, r + grp.dof0, k & 1, s));
+                                      g.tile[TILE_SMOOTH], exact, flags, z + grp.dof0, r + grp.dof0, k & 1, s));
         }
         return DGMG_OK;
     };
-    for (int k = 0; k < B.opts.nu_pre; ++k) RC(smooth(k));
+    for (int k = 0; k < B.opts.nu_pre; ++k) RC(smooth(k, fx && k == 0 ? SM_ZERO : 0));
     for (auto &grp : B.groups) {
         auto &g = grp.prec<T>();
         LC(launch_residual_batch<T>(B.dim, grp.q, g.D, g.map[TILE_RESIDUAL], g.nblocks[TILE_RESIDUAL],
@@ -466,7 +459,7 @@ int batch_vcycle(dgmg_batch &B, const T *r, T *z, cudaStream_t s) {
         LC(launch_project_batch<T>(B.dim, grp.q, g.D, g.map[TILE_PROJECT], g.nblocks[TILE_PROJECT],
                                    g.tile[TILE_PROJECT], z + grp.dof0, 1, s));
     }
-    for (int k = 0; k < B.opts.nu_post; ++k) RC(smooth(k));
+    for (int k = 0; k < B.opts.nu_post; ++k) RC(smooth(k, fx && k == B.opts.nu_post - 1 ? SM_NO_TRACES : 0));
     return DGMG_OK;
 }
 
@@ -592,11 +585,14 @@ std::vector<BatchDG<T>> group_descriptors(const dgmg_batch &B, const dgmg_batch:
         dgmg_ctx *c = B.inst[i];
         const DGDev<T> &dg = dgmg::dg<T>(*c);
         BatchDG<T> d{};
-        d.c = dg.c;
+        if constexpr (std::is_same<T, double>::value)
+            d.c = dg.c.cst;
+        else
+            d.c = dg.c;
         d.off = cells;
         d.kappa = dg.kappa;
         d.fd = dg.fd;
-        d.fdr = dg.fdr;
+        if constexpr (std::is_same<T, float>::value) d.fdr = dg.fdr;
         d.linv = dg.linv;
         d.tr[0] = dg.tr[0];
         d.tr[1] = dg.tr[1];
@@ -802,8 +798,7 @@ int dgmg_batch_create(int count, const dgmg_mesh *meshes, const int *p, const do
     phase("q1 descriptors");
     if (o.autotune) {
         for (auto &g : B->groups) {
-            RC(tune_group<double>(*B, g, B->z, B->r, B->capture_stream));   // mixed: the FP64 apply only
-            if (B->mixed) RC(tune_group<float>(*B, g, B->z32, B->r32, B->capture_stream));
+            if (B->mixed) RC(tune_group(*B, g, B->z32, B->r32, B->capture_stream));
         }
         phase("autotune");
     }

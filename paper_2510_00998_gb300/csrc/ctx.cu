@@ -302,6 +302,12 @@ namespace dgmg {
 
 int exact_block(const dgmg_ctx &C) { return C.opts.block_inverse == DGMG_BLOCK_EXACT ? 1 : 0; }
 
+// FP64 levels (block fixed-point kernels)
+void fill_const(const dgmg_ctx &C, const DGSpace &S, DGConst<double> &c) {
+    fx_tables(S.re, S.penalty_p, c.tab);
+    fx_level(S.re, S.penalty_p, C.dim, C.n, C.ncell, exact_block(C) ? 1.0 - C.opts.omega_dg : 1.0, c.cst);
+}
+
 template <typename T>
 void fill_const(const dgmg_ctx &C, const DGSpace &S, DGConst<T> &c) {
     std::memset(&c, 0, sizeof(c));
@@ -384,12 +390,12 @@ std::vector<T> convert(const std::vector<double> &v) {
     return std::vector<T>(v.begin(), v.end());
 }
 
-// The per-cell factors (and, FP64, the table of inverse eigenvalue sums) of
-// level D from the FP64 kappa of the finest level, on the set-up stream.
-// FP32 factors are the rounded FP64 ones when those exist (fd64).
+// The per-cell factors of level D from the FP64 kappa of the finest level, on the
+// set-up stream. FP32 factors are the rounded FP64 ones when those exist (fd64).
+// FP64 factors are [S | lambda] in FP64 until finish_factors.
 template <typename T>
 int compute_factors(dgmg_ctx &C, const DGSpace &S, DGDev<T> &D, const double *fd64 = nullptr) {
-    // the residual's factors [S^T M | lambda], from the FP64 factors where there are some
+    // FP32: the residual's factors [S^T M | lambda], from the FP64 factors where there are some
     MassTables mt;
     std::memset(&mt, 0, sizeof(mt));
     for (int a = 0; a < C.dim; ++a) {
@@ -408,10 +414,17 @@ int compute_factors(dgmg_ctx &C, const DGSpace &S, DGDev<T> &D, const double *fd
     RC(fd_input(C, S, in));
     const_cast<DGSpace &>(S).fdin = in;
     LC(launch_fd_factors<T>(in, C.d64.kappa, C.ncell, D.fd, C.setup_stream));
-    if (sizeof(T) == sizeof(double))
-        LC(launch_inverse_eigen_sums(C.dim, S.q, C.ncell, reinterpret_cast<const double *>(D.fd),
-                                     C.opts.omega_dg, reinterpret_cast<double *>(D.linv), C.setup_stream));
-    if (D.fdr) LC((launch_residual_factors<T, T>(C.dim, S.q, C.ncell, D.fd, mt, D.fdr, C.setup_stream)));
+    if constexpr (std::is_same<T, float>::value)
+        if (D.fdr) LC((launch_residual_factors<float, float>(C.dim, S.q, C.ncell, D.fd, mt, D.fdr, C.setup_stream)));
+    return DGMG_OK;
+}
+
+// The FP64 level's factors in the form of its kernels, once the FP32 ones have been
+// taken from them: the table of inverse eigenvalue sums, then S as limbs in place.
+int finish_factors(dgmg_ctx &C, const DGSpace &S, DGDev<double> &D, cudaStream_t s) {
+    if (!D.fd) return DGMG_OK;
+    LC(launch_fx_table(C.dim, S.q, C.ncell, D.fd, C.opts.omega_dg, D.linv, s));
+    LC(launch_fx_factors(C.dim, S.q, C.ncell, D.fd, C.opts.omega_dg, s));
     return DGMG_OK;
 }
 
@@ -421,12 +434,18 @@ int compute_factors(dgmg_ctx &C, const DGSpace &S, DGDev<T> &D, const double *fd
 // input as at set-up; the residual's factors stay the set-up ones.
 template <typename T>
 int recompute_factors(dgmg_ctx &C, const DGSpace &S, DGDev<T> &D, cudaStream_t s) {
-    if (!D.fd) return DGMG_OK;
+    if (!D.fd || S.fdin.dim == 0) return DGMG_OK;   // no input kept for this level: the set-up factors stay
     LC(launch_fd_factors<T>(S.fdin, C.d64.kappa, C.ncell, D.fd, s));
-    if (sizeof(T) == sizeof(double) && D.linv)
-        LC(launch_inverse_eigen_sums(C.dim, S.q, C.ncell, reinterpret_cast<const double *>(D.fd),
-                                     C.opts.omega_dg, reinterpret_cast<double *>(D.linv), s));
+    if constexpr (std::is_same<T, double>::value) RC(finish_factors(C, S, D, s));
     return DGMG_OK;
+}
+
+// Scale of the facet coefficients per axis: 1 in FP32; the FP64 kernels take them
+// times the axis's coefficient (the same on every DG level: it depends on the mesh)
+inline const double *facet_scale(const DGDev<double> &D) { return D.c.cst.sa; }
+inline const double *facet_scale(const DGDev<float> &) {
+    static const double one[3] = {1.0, 1.0, 1.0};
+    return one;
 }
 
 // One DG level in precision T: constants, kappa (uploaded, or shared with the
@@ -446,9 +465,12 @@ int setup_dg(dgmg_ctx &C, const DGSpace &S, DGDev<T> &D, const std::vector<doubl
         D.kfac = const_cast<T *>(shared_kfac);
     } else {
         RC(C.alloc(&D.kfac, C.ncell * 2 * C.dim));
-        LC(launch_facet_coefficients<T>(C.dim, C.n, C.ncell, C.d64.kappa, D.kfac, C.setup_stream));
+        LC(launch_facet_coefficients<T>(C.dim, C.n, C.ncell, C.d64.kappa, facet_scale(D), D.kfac, C.setup_stream));
     }
-    D.c.kfac = D.kfac;
+    if constexpr (std::is_same<T, double>::value)
+        D.c.cst.kfac = D.kfac;
+    else
+        D.c.kfac = D.kfac;
     const int64_t trn = C.ncell * 2 * C.dim * trace_face_stride<T>((int)(S.nloc / S.q));
     if (!smoother) {                  // operator only (projection, residual): no block-inverse factors
         RC(C.alloc(&D.tr[0], trn));
@@ -457,7 +479,7 @@ int setup_dg(dgmg_ctx &C, const DGSpace &S, DGDev<T> &D, const std::vector<doubl
         return DGMG_OK;
     }
     RC(C.alloc(&D.fd, (size_t)C.ncell * C.dim * (S.q * S.q + S.q)));
-    RC(C.alloc(&D.fdr, (size_t)C.ncell * C.dim * (S.q * S.q + S.q)));
+    if (sizeof(T) == sizeof(float)) RC(C.alloc(&D.fdr, (size_t)C.ncell * C.dim * (S.q * S.q + S.q)));
     if (sizeof(T) == sizeof(double)) RC(C.alloc(&D.linv, (size_t)S.ndof));
     RC(compute_factors<T>(C, S, D, fd64));
     RC(C.alloc(&D.tr[0], trn));
@@ -508,6 +530,7 @@ int setup_dg_levels(dgmg_ctx &C, const std::vector<double> &kap) {
         };
         RC(level(C.lvl64[l], C.d64.kappa, nullptr, C.d64.kfac));
         if (mixed) RC(level(C.lvl32[l], C.d32.kappa, C.lvl64[l].D.fd, C.d32.kfac));
+        RC(finish_factors(C, S, C.lvl64[l].D, C.setup_stream));
     }
     RC(C.alloc(&C.res64, C.ndof));
     if (mixed) RC(C.alloc(&C.res32, C.ndof));
@@ -776,12 +799,12 @@ DGDev<T> &dg_level(dgmg_ctx &C, int l) {
 }
 
 template <typename T>
-int level_smooth(dgmg_ctx &C, int l, T *z, const T *b, int cur, cudaStream_t s) {
+int level_smooth(dgmg_ctx &C, int l, T *z, const T *b, int cur, int flags, cudaStream_t s) {
     DGDev<T> &D = dg_level<T>(C, l);
     C.prof.begin(ST_SMOOTH, s);
     if (C.opts.recompute_block) RC(recompute_factors<T>(C, C.dgs[l], D, s));
-    LC(launch_smooth<T>(C.dim, C.dgs[l].q, D.c, l == 0 ? C.tile_of<T>(TILE_SMOOTH) : 0, exact_block(C), z, b,
-                        D.kappa, D.fd, D.linv, D.tr[cur], D.tr[cur ^ 1], s));
+    LC(launch_smooth<T>(C.dim, C.dgs[l].q, D.c, l == 0 ? C.tile_of<T>(TILE_SMOOTH) : 0, exact_block(C), flags, z,
+                        b, D.kappa, D.fd, D.linv, D.tr[cur], D.tr[cur ^ 1], s));
     C.prof.end(s);
     return DGMG_OK;
 }
@@ -841,17 +864,22 @@ int level_cycle(dgmg_ctx &C, int l, const T *b, T *z, cudaStream_t s) {
     DGDev<T> &D = dg_level<T>(C, l);
     const DGSpace &S = C.dgs[l];
     const int64_t trn = C.ncell * 2 * C.dim * trace_face_stride<T>((int)(S.nloc / S.q));
-    LC(cudaMemsetAsync(z, 0, sizeof(T) * S.ndof, s));
-    LC(cudaMemsetAsync(D.tr[0], 0, sizeof(T) * trn, s));   // projections of z = 0
+    // FP64: the first step takes the zero iterate as such (no facet terms, nothing
+    // to clear), and nothing reads the projections of the last one
+    const bool fx = std::is_same<T, double>::value;
+    if (!fx || C.opts.nu_pre == 0) {
+        LC(cudaMemsetAsync(z, 0, sizeof(T) * S.ndof, s));
+        LC(cudaMemsetAsync(D.tr[0], 0, sizeof(T) * trn, s));   // projections of z = 0
+    }
     int cur = 0;
     for (int k = 0; k < C.opts.nu_pre; ++k) {
-        RC(level_smooth<T>(C, l, z, b, cur, s));
+        RC(level_smooth<T>(C, l, z, b, cur, fx && k == 0 ? SM_ZERO : 0, s));
         cur ^= 1;
     }
     RC(coarse_correction<T>(C, l, z, b, cur, s));
     cur = 0;
     for (int k = 0; k < C.opts.nu_post; ++k) {
-        RC(level_smooth<T>(C, l, z, b, cur, s));
+        RC(level_smooth<T>(C, l, z, b, cur, fx && k == C.opts.nu_post - 1 ? SM_NO_TRACES : 0, s));
         cur ^= 1;
     }
     return DGMG_OK;
@@ -872,7 +900,7 @@ int mg_cycle64(dgmg_ctx &C, double *x, const double *b, double *r, cudaStream_t 
     DGDev<double> &D = C.d64;
     int cur = 0;
     for (int k = 0; k < C.opts.nu_pre; ++k) {
-        RC(level_smooth<double>(C, 0, x, b, cur, s));
+        RC(level_smooth<double>(C, 0, x, b, cur, 0, s));
         cur ^= 1;
     }
     RC(coarse_correction<double>(C, 0, x, b, cur, s));
@@ -923,8 +951,8 @@ int apply64(dgmg_ctx &C, const double *u, const double *b, double *out, cudaStre
 }
 
 // ------------------------------------------------------------ tile autotuner
-// For each DG-level kernel (projection, smoothing step, residual + restriction)
-// and each precision the ctx runs, time the candidate cells-per-CTA values on
+// For each FP32 DG-level kernel (projection, smoothing step, residual +
+// restriction) of a mixed-precision ctx, time the candidate cells-per-CTA values on
 // the ctx's own buffers (one warm-up and three timed launches each, CUDA events
 // on the set-up stream) and keep the fastest; for the FP32 smoothing step the
 // one-thread-per-cell kernel (tile 0) competes with the pencil tiles. Results
@@ -937,8 +965,8 @@ struct TileKey {
 static std::mutex g_tile_mu;
 static std::map<TileKey, std::array<int, 6>> g_tile_cache;
 
-template <typename T>
-static int tune_tiles(dgmg_ctx &C, T *u, T *b, int *tile, bool trace, bool smooth) {
+static int tune_tiles(dgmg_ctx &C, float *u, float *b, int *tile, bool trace) {
+    using T = float;
     DGDev<T> &D = dg<T>(C);
     cudaStream_t s = C.setup_stream;
     const int nf = (int)(C.nloc / C.q);
@@ -977,7 +1005,6 @@ static int tune_tiles(dgmg_ctx &C, T *u, T *b, int *tile, bool trace, bool smoot
         cudaEventElapsedTime(&ms, e0, e1);
         return ms;
     };
-    const char *tname = sizeof(T) == 8 ? "fp64" : "fp32";
     // the fastest candidate; the one-thread-per-cell kernel (tile 0) is kept
     // unless another tile is more than 3% faster, so that a near tie in the
     // three-launch timing does not flip the choice from run to run
@@ -986,7 +1013,7 @@ static int tune_tiles(dgmg_ctx &C, T *u, T *b, int *tile, bool trace, bool smoot
         float best_ms = INF, ms0 = INF;
         for (int c : cs) {
             const float ms = time_it([&] { return launch_with(c); });
-            if (trace) std::fprintf(stderr, "dgmg autotune %s %-9s tile %2d: %8.4f ms\n", tname, stage, c, ms / 3);
+            if (trace) std::fprintf(stderr, "dgmg autotune %-9s tile %2d: %8.4f ms\n", stage, c, ms / 3);
             if (c == 0) ms0 = ms;
             if (ms < best_ms) {
                 best_ms = ms;
@@ -996,20 +1023,19 @@ static int tune_tiles(dgmg_ctx &C, T *u, T *b, int *tile, bool trace, bool smoot
         return ms0 < INF && ms0 <= 1.03f * best_ms ? 0 : best;
     };
     std::vector<int> cp = cand;
-    if (C.dim == 3 && C.q <= (std::is_same<T, float>::value ? 5 : 4) && C.opts.basis == DGMG_BASIS_GLL)
+    if (C.dim == 3 && C.q <= 5 && C.opts.basis == DGMG_BASIS_GLL)
         cp.insert(cp.begin(), 0);
     tile[TILE_PROJECT] = pick("project", cp, [&](int c) {
         return launch_project<T>(C.dim, C.q, D.c, c, u, nullptr, D.tr[0], s);
     });
     std::vector<int> cs = cand;
-    if (C.dim == 3 && C.q <= (std::is_same<T, float>::value ? 5 : 4) && exact_block(C)) cs.insert(cs.begin(), 0);
-    if (smooth)                     // (the FP64 smoother of a mixed-precision context never runs)
-        tile[TILE_SMOOTH] = pick("smooth", cs, [&](int c) {
-            return launch_smooth<T>(C.dim, C.q, D.c, c, exact_block(C), u, b, D.kappa, D.fd, D.linv, D.tr[0],
-                                    D.tr[1], s);
-        });
+    if (C.dim == 3 && C.q <= 5 && exact_block(C)) cs.insert(cs.begin(), 0);
+    tile[TILE_SMOOTH] = pick("smooth", cs, [&](int c) {
+        return launch_smooth<T>(C.dim, C.q, D.c, c, exact_block(C), 0, u, b, D.kappa, D.fd, D.linv, D.tr[0], D.tr[1],
+                                s);
+    });
     std::vector<int> cr = cand;
-    if (C.dim == 3 && C.q <= (std::is_same<T, float>::value ? 5 : 4) && exact_fd(C, D)) cr.insert(cr.begin(), 0);
+    if (C.dim == 3 && C.q <= 5 && exact_fd(C, D)) cr.insert(cr.begin(), 0);
     tile[TILE_RESIDUAL] = pick("residual", cr, [&](int c) {
         return launch_residual<T>(C.dim, C.q, D.c, c, RES_HAS_B | RES_CORNERS, u, b, D.kappa, D.tr[0], nullptr,
                                   D.corners, exact_fd(C, D), s);
@@ -1021,7 +1047,7 @@ static int tune_tiles(dgmg_ctx &C, T *u, T *b, int *tile, bool trace, bool smoot
 }
 
 static int autotune_tiles(dgmg_ctx &C) {
-    const bool mixed = C.opts.precision == DGMG_MIXED_FP32;
+    if (C.opts.precision != DGMG_MIXED_FP32) return DGMG_OK;   // the FP64 kernels have one shape per degree
     const TileKey key{{C.dim, C.q, C.n[0], C.n[1], C.n[2], C.opts.precision, C.opts.block_inverse, C.opts.basis}};
     {
         std::lock_guard<std::mutex> lk(g_tile_mu);
@@ -1032,8 +1058,7 @@ static int autotune_tiles(dgmg_ctx &C) {
         }
     }
     const bool trace = std::getenv("DGMG_TRACE_SETUP") != nullptr;
-    RC(tune_tiles<double>(C, C.w_z, C.w_r, C.tile[0], trace, !mixed));
-    if (mixed) RC(tune_tiles<float>(C, C.z32, C.r32, C.tile[1], trace, true));
+    RC(tune_tiles(C, C.z32, C.r32, C.tile[1], trace));
     std::array<int, 6> v;
     for (int k = 0; k < 6; ++k) v[k] = C.tile[k / 3][k % 3];
     std::lock_guard<std::mutex> lk(g_tile_mu);
@@ -1160,11 +1185,9 @@ int create_ctx(const dgmg_mesh *mesh, int p, const double *kappa, const dgmg_opt
     C->opts = o;
     const int nf = (int)(C->nloc / C->q);
     C->cpb = std::max(1, 256 / nf);   // per-pencil tile: as many cells as fit 256 threads
-    for (int k = 0; k < 2; ++k)
-        for (int st = 0; st < 3; ++st) C->tile[k][st] = C->cpb;
-    C->tile[0][TILE_SMOOTH] = 0;   // the one-thread-per-cell smoother and residual where they apply
-    C->tile[1][TILE_SMOOTH] = 0;
-    C->tile[0][TILE_RESIDUAL] = 0;
+    for (int st = 0; st < 3; ++st) C->tile[1][st] = C->cpb;
+    for (int st = 0; st < 3; ++st) C->tile[0][st] = fx_cells_per_cta(C->dim, C->q);
+    C->tile[1][TILE_SMOOTH] = 0;   // the one-thread-per-cell smoother and residual where they apply
     C->tile[1][TILE_RESIDUAL] = 0;
 
     std::vector<double> kap(C->ncell, 1.0);
@@ -1209,6 +1232,7 @@ int create_ctx(const dgmg_mesh *mesh, int p, const double *kappa, const dgmg_opt
     trace.mark("cg upload");
     if (o.precision == DGMG_MIXED_FP32) {
         RC(setup_dg<float>(*C, S0, C->d32, kap, true, nullptr, C->d64.fd));
+        RC(finish_factors(*C, S0, C->d64, C->setup_stream));
         RC(setup_cg<float>(*C, C->cg32));
         RC(setup_q1_plan<float>(*C));
         RC(C->alloc(&C->r32, C->ndof));
@@ -1220,6 +1244,7 @@ int create_ctx(const dgmg_mesh *mesh, int p, const double *kappa, const dgmg_opt
             RC(C->alloc(&C->rold32, C->ndof));
         }
     }
+    if (o.precision != DGMG_MIXED_FP32) RC(finish_factors(*C, S0, C->d64, C->setup_stream));
     RC(setup_dg_levels(*C, kap));
     trace.mark("dg levels");
     if (flags & CREATE_NO_SOLVER) {   // a member of a batch: the batch owns the solver's vectors
@@ -1239,8 +1264,7 @@ int create_ctx(const dgmg_mesh *mesh, int p, const double *kappa, const dgmg_opt
         cudaError_t e = cudaMallocHost((void **)&C->host_scal, sizeof(double) * S_HOST);
         if (e != cudaSuccess) return cuda_fail(e, "cudaMallocHost");
         e = wait_timeouts_addr_fp32(&C->tmo_dev[0]);
-        if (e == cudaSuccess) e = wait_timeouts_addr_fp64(&C->tmo_dev[1]);
-        if (e == cudaSuccess) e = q1_barrier_timeouts_addr(&C->tmo_dev[2]);
+        if (e == cudaSuccess) e = q1_barrier_timeouts_addr(&C->tmo_dev[1]);
         if (e != cudaSuccess) return cuda_fail(e, "cudaGetSymbolAddress");
         e = cudaEventCreateWithFlags(&C->ev, cudaEventDisableTiming);
         if (e != cudaSuccess) return cuda_fail(e, "cudaEventCreate");
@@ -1337,8 +1361,9 @@ int dgmg_update_kappa(dgmg_ctx *C, const double *kappa) {
         DG_CUDA(cudaMemcpyAsync(C->d32.kappa, kap32.data(), sizeof(float) * C->ncell, cudaMemcpyHostToDevice, s));
     DG_CUDA(cudaMemcpyAsync(C->coarse_inv, inv.data(), sizeof(double) * inv.size(), cudaMemcpyHostToDevice, s));
     // facet coefficients (the lower DG levels share the finest level's)
-    LC(launch_facet_coefficients<double>(C->dim, C->n, C->ncell, C->d64.kappa, C->d64.kfac, s));
-    if (mixed) LC(launch_facet_coefficients<float>(C->dim, C->n, C->ncell, C->d64.kappa, C->d32.kfac, s));
+    LC(launch_facet_coefficients<double>(C->dim, C->n, C->ncell, C->d64.kappa, facet_scale(C->d64), C->d64.kfac, s));
+    if (mixed)
+        LC(launch_facet_coefficients<float>(C->dim, C->n, C->ncell, C->d64.kappa, facet_scale(C->d32), C->d32.kfac, s));
     std::vector<std::vector<float>> st32(C->lv.size());
     for (size_t l = 0; l < C->lv.size(); ++l) {
         const std::vector<double> &st = C->lv[l].st;
@@ -1358,6 +1383,7 @@ int dgmg_update_kappa(dgmg_ctx *C, const double *kappa) {
             DGDev<float> &D32 = l == 0 ? C->d32 : C->lvl32[l].D;
             if (D32.fd) RC(compute_factors<float>(*C, C->dgs[l], D32, D64.fd));
         }
+        RC(finish_factors(*C, C->dgs[l], D64, s));
     }
     DG_CUDA(cudaStreamSynchronize(s));
     return DGMG_OK;
@@ -1409,8 +1435,9 @@ int dgmg_smooth(dgmg_ctx *C, double *u, const double *b, int nsteps, void *strea
     for (int k = 0; k < nsteps; ++k) {
         C->prof.begin(ST_SMOOTH, s);
         if (C->opts.recompute_block) RC(recompute_factors<double>(*C, C->dgs[0], D, s));
-        LC(launch_smooth<double>(C->dim, C->q, D.c, C->tile[0][TILE_SMOOTH], exact_block(*C), u, b, D.kappa, D.fd, D.linv,
-                                 D.tr[cur], D.tr[cur ^ 1], s));
+        LC(launch_smooth<double>(C->dim, C->q, D.c, C->tile[0][TILE_SMOOTH], exact_block(*C),
+                                 k == nsteps - 1 ? SM_NO_TRACES : 0, u, b, D.kappa, D.fd, D.linv, D.tr[cur],
+                                 D.tr[cur ^ 1], s));
         C->prof.end(s);
         cur ^= 1;
     }
@@ -1539,9 +1566,9 @@ int dgmg_estimate_bytes(const dgmg_mesh *mesh, int p, const dgmg_opts *opts, siz
     const int64_t tr = ncell * 2 * dim * trace_face_stride<double>((int)nf);
     const int64_t tr32 = ncell * 2 * dim * trace_face_stride<float>((int)nf);
     auto sz = [](int64_t count, size_t elem) { return (size_t)std::max<int64_t>(count, 1) * elem; };
-    size_t dg64 = sz(ncell, 8) + 2 * sz(ncell * dim * (q * q + q), 8) + sz(ndof, 8) + 2 * sz(tr, 8) +
-                  sz(ncell << dim, 8) + sz(ncell * 2 * dim, 8);   // kappa, factors and residual factors,
-                                                                  // table, traces, corners, facet coefficients
+    size_t dg64 = sz(ncell, 8) + sz(ncell * dim * (q * q + q), 8) + sz(ndof, 8) + 2 * sz(tr, 8) +
+                  sz(ncell << dim, 8) + sz(ncell * 2 * dim, 8);   // kappa, factors, table,
+                                                                  // traces, corners, facet coefficients
     size_t dg32 = sz(ncell, 4) + 2 * sz(ncell * dim * (q * q + q), 4) + 2 * sz(tr32, 4) + sz(ncell << dim, 4) +
                   sz(ncell * 2 * dim, 4);
     size_t cg64 = 0, cg32 = 0;
@@ -1582,7 +1609,7 @@ int dgmg_estimate_bytes(const dgmg_mesh *mesh, int p, const dgmg_opts *opts, siz
             const int64_t trl = ncell * 2 * dim * trace_face_stride<double>((int)(nl / ql));
             const int64_t trl32 = ncell * 2 * dim * trace_face_stride<float>((int)(nl / ql));
             const int64_t fdl = ncell * dim * (ql * ql + ql);
-            total += 2 * sz(fdl, 8) + sz(nd, 8) + 2 * sz(trl, 8) + sz(ncell << dim, 8) + 3 * sz(nd, 8);
+            total += sz(fdl, 8) + sz(nd, 8) + 2 * sz(trl, 8) + sz(ncell << dim, 8) + 3 * sz(nd, 8);
             if (mixed) total += 2 * sz(fdl, 4) + 2 * sz(trl32, 4) + sz(ncell << dim, 4) + 3 * sz(nd, 4);
         }
         total += sz(ndof, 8) + (mixed ? sz(ndof, 4) : 0);
@@ -1618,13 +1645,12 @@ long long dgmg_kernel_launches(void) { return g_kernel_launches.load(); }
 
 int dgmg_wait_timeouts(unsigned long long *count) {
     if (!count) return fail(DGMG_EINVAL, "dgmg_wait_timeouts: count is NULL");
-    unsigned long long a = 0, b = 0, c = 0, v = 0;
+    unsigned long long a = 0, c = 0, v = 0;
     cudaError_t e = wait_timeouts_fp32(&a);
-    if (e == cudaSuccess) e = wait_timeouts_fp64(&b);
     if (e == cudaSuccess) e = q1_barrier_timeouts(&c);
     if (e == cudaSuccess) e = wait_timeouts_volume(&v);
     if (e != cudaSuccess) return cuda_fail(e, "dgmg_wait_timeouts");
-    *count = a + b + c + v;
+    *count = a + c + v;
     return DGMG_OK;
 }
 

@@ -35,8 +35,8 @@ template <typename T>
 struct DGDev {
     DGConst<T> c;
     T *kappa = nullptr, *fd = nullptr, *tr[2] = {nullptr, nullptr}, *corners = nullptr;
-    T *linv = nullptr;   // per-node omega / (sum of the cell's eigenvalues); FP64 only
-    T *fdr = nullptr;    // the residual's factors [S^T M | lambda] per cell and axis
+    T *linv = nullptr;   // per-node omega / (sum of the cell's eigenvalues); FP64 only (as integers)
+    T *fdr = nullptr;    // FP32: the residual's factors [S^T M | lambda] per cell and axis
     T *kfac = nullptr;   // facet coefficients [cell][face]
 };
 
@@ -170,9 +170,9 @@ struct dgmg_ctx {
     float *vol_esw = nullptr;
     float vol_fac[165] = {};
     double *host_scal = nullptr;                  // pinned: S_NSCAL scalars, then the wait-counter snapshots
-    // device addresses of the bounded-wait counters (FP32 and FP64 DG kernels,
-    // Q1 grid barrier) on the ctx's device
-    unsigned long long *tmo_dev[3] = {nullptr, nullptr, nullptr};
+    // device addresses of the bounded-wait counters (FP32 DG kernels, Q1 grid
+    // barrier) on the ctx's device
+    unsigned long long *tmo_dev[2] = {nullptr, nullptr};
     double *quad_x1 = nullptr, *quad_V = nullptr, *quad_w = nullptr;
     std::vector<void *> allocs;
     size_t bytes = 0;
@@ -255,8 +255,8 @@ struct dgmg_ctx {
 // slots of ctx->scal
 enum { S_RZ = 0, S_PQ = 1, S_BETA = 2, S_RR = 3, S_RZN = 4, S_RZO = 5, S_BB = 6, S_ZZ = 7, S_ZZ0 = 8, S_XX = 9,
        S_NSCAL = 16 };
-// pinned host slots after the scalars: wait-counter snapshots [start 3 | end 3]
-enum { S_TMO = S_NSCAL, S_HOST = S_NSCAL + 6 };
+// pinned host slots after the scalars: wait-counter snapshots [start 2 | end 2]
+enum { S_TMO = S_NSCAL, S_HOST = S_NSCAL + 4 };
 
 
 #define RC(x)                           \

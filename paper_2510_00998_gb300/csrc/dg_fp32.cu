@@ -10,7 +10,7 @@ cudaError_t launch_project<float>(int dim, int q, const DGConst<float> &c, int c
 }
 
 template <>
-cudaError_t launch_smooth<float>(int dim, int q, const DGConst<float> &c, int cpb, int exact, float *u,
+cudaError_t launch_smooth<float>(int dim, int q, const DGConst<float> &c, int cpb, int exact, int, float *u,
                                 const float *b,
                                 const float *kappa, const float *fd, const float *linv, const float *tr_in, float *tr_out,
                                 cudaStream_t s) {
@@ -31,7 +31,7 @@ cudaError_t launch_project_batch<float>(int dim, int q, const BatchDG<float> *D,
 }
 template <>
 cudaError_t launch_smooth_batch<float>(int dim, int q, const BatchDG<float> *D, const BlockMap *map, int nblocks, int cpb,
-                                    int exact, float *u, const float *b, int cur, cudaStream_t s) {
+                                    int exact, int, float *u, const float *b, int cur, cudaStream_t s) {
     return launch_smooth_batch_impl<float>(dim, q, D, map, nblocks, cpb, exact, u, b, cur, s);
 }
 template <>

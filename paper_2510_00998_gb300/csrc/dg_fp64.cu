@@ -1,59 +1,107 @@
-// Instantiation of the DG-level kernels for double arithmetic.
-#include "dg_kernels.cuh"
+// FP64 on the DG levels: the dispatch to the block fixed-point kernels (dg_fx.cuh)
+// and the FP64 transfers of gradual p-hierarchies.
+#include <array>
+#include <mutex>
+
+#include "internal.h"
+
+#include "dg_transfer.cuh"
 
 namespace dgmg {
 
-template <>
-cudaError_t launch_project<double>(int dim, int q, const DGConst<double> &c, int cpb, double *u, const double *e0,
-                                 double *tr, cudaStream_t s) {
-    return launch_project_impl<double>(dim, q, c, cpb, u, e0, tr, s);
+namespace {
+
+// f(FxRun<dim, q>) for the run-time (dim, q)
+template <typename F>
+auto fx_dispatch(int dim, int q, F f) {
+    switch (dim * 16 + q) {
+        case 2 * 16 + 2: return f(FxRun<2, 2>{});
+        case 2 * 16 + 3: return f(FxRun<2, 3>{});
+        case 2 * 16 + 4: return f(FxRun<2, 4>{});
+        case 2 * 16 + 5: return f(FxRun<2, 5>{});
+        case 2 * 16 + 6: return f(FxRun<2, 6>{});
+        case 2 * 16 + 7: return f(FxRun<2, 7>{});
+        case 3 * 16 + 2: return f(FxRun<3, 2>{});
+        case 3 * 16 + 3: return f(FxRun<3, 3>{});
+        case 3 * 16 + 4: return f(FxRun<3, 4>{});
+        case 3 * 16 + 5: return f(FxRun<3, 5>{});
+        case 3 * 16 + 6: return f(FxRun<3, 6>{});
+        default: return f(FxRun<3, 7>{});
+    }
+}
+bool fx_valid(int dim, int q) { return (dim == 2 || dim == 3) && q >= 2 && q <= QMAX; }
+
+// Tables of the batched launches (GLL nodes, the degree's own penalty), formed
+// once per degree.
+const FxTab &batch_tables(int q) {
+    static std::array<FxTab, QMAX + 1> tabs;
+    static std::array<std::once_flag, QMAX + 1> once;
+    std::call_once(once[q], [q] { fx_tables(make_refelem(q - 1), q - 1, tabs[q]); });
+    return tabs[q];
+}
+
+}  // namespace
+
+int fx_cells_per_cta(int dim, int q) {
+    return fx_dispatch(dim, q, [](auto run) { return decltype(run)::cells_per_cta(); });
 }
 
 template <>
-cudaError_t launch_smooth<double>(int dim, int q, const DGConst<double> &c, int cpb, int exact, double *u,
-                                const double *b,
-                                const double *kappa, const double *fd, const double *linv, const double *tr_in, double *tr_out,
-                                cudaStream_t s) {
-    return launch_smooth_impl<double>(dim, q, c, cpb, exact, u, b, kappa, fd, linv, tr_in, tr_out, s);
+cudaError_t launch_project<double>(int dim, int q, const DGConst<double> &c, int, double *u, const double *e0,
+                                   double *tr, cudaStream_t s) {
+    if (!fx_valid(dim, q)) return cudaErrorInvalidValue;
+    return fx_dispatch(dim, q, [&](auto run) { return decltype(run)::project(c, u, e0, tr, s); });
 }
 
 template <>
-cudaError_t launch_residual<double>(int dim, int q, const DGConst<double> &c, int cpb, int mode, const double *u,
-                                  const double *b, const double *kappa, const double *tr, double *r, double *corners,
-                                  const double *fd, cudaStream_t s) {
-    return launch_residual_impl<double>(dim, q, c, cpb, mode, u, b, kappa, tr, r, corners, fd, s);
+cudaError_t launch_smooth<double>(int dim, int q, const DGConst<double> &c, int, int exact, int flags, double *u,
+                                  const double *b, const double *kappa, const double *fd, const double *linv,
+                                  const double *tr_in, double *tr_out, cudaStream_t s) {
+    if (!fx_valid(dim, q)) return cudaErrorInvalidValue;
+    return fx_dispatch(dim, q, [&](auto run) {
+        return decltype(run)::smooth(c, exact != 0, flags, u, b, kappa, fd, linv, tr_in, tr_out, s);
+    });
 }
 
 template <>
-cudaError_t launch_project_batch<double>(int dim, int q, const BatchDG<double> *D, const BlockMap *map, int nblocks, int cpb,
-                                     double *u, int with_e0, cudaStream_t s) {
-    return launch_project_batch_impl<double>(dim, q, D, map, nblocks, cpb, u, with_e0, s);
+cudaError_t launch_residual<double>(int dim, int q, const DGConst<double> &c, int, int mode, const double *u,
+                                    const double *b, const double *kappa, const double *tr, double *r, double *corners,
+                                    const double *, cudaStream_t s) {
+    if (!fx_valid(dim, q)) return cudaErrorInvalidValue;
+    return fx_dispatch(dim, q,
+                       [&](auto run) { return decltype(run)::residual(c, mode, u, b, kappa, tr, r, corners, s); });
+}
+
+template <>
+cudaError_t launch_project_batch<double>(int dim, int q, const BatchDG<double> *D, const BlockMap *map, int nblocks,
+                                         int, double *u, int with_e0, cudaStream_t s) {
+    if (!fx_valid(dim, q)) return cudaErrorInvalidValue;
+    return fx_dispatch(dim, q, [&](auto run) {
+        return decltype(run)::project_batch(batch_tables(q), D, map, nblocks, u, with_e0, s);
+    });
 }
 template <>
-cudaError_t launch_smooth_batch<double>(int dim, int q, const BatchDG<double> *D, const BlockMap *map, int nblocks, int cpb,
-                                    int exact, double *u, const double *b, int cur, cudaStream_t s) {
-    return launch_smooth_batch_impl<double>(dim, q, D, map, nblocks, cpb, exact, u, b, cur, s);
+cudaError_t launch_smooth_batch<double>(int dim, int q, const BatchDG<double> *D, const BlockMap *map, int nblocks, int,
+                                        int exact, int flags, double *u, const double *b, int cur, cudaStream_t s) {
+    if (!fx_valid(dim, q)) return cudaErrorInvalidValue;
+    return fx_dispatch(dim, q, [&](auto run) {
+        return decltype(run)::smooth_batch(batch_tables(q), exact != 0, D, map, nblocks, flags, u, b, cur, s);
+    });
 }
 template <>
 cudaError_t launch_residual_batch<double>(int dim, int q, const BatchDG<double> *D, const BlockMap *map, int nblocks,
-                                      int cpb, int mode, const double *u, const double *b, double *r, int cur,
-                                      cudaStream_t s) {
-    return launch_residual_batch_impl<double>(dim, q, D, map, nblocks, cpb, mode, u, b, r, cur, s);
-}
-template <>
-cudaError_t launch_zero_traces_batch<double>(int dim, int q, const BatchDG<double> *D, int count, cudaStream_t s) {
-    return launch_zero_traces_batch_impl<double>(dim, q, D, count, s);
+                                          int, int mode, const double *u, const double *b, double *r, int cur,
+                                          cudaStream_t s) {
+    if (!fx_valid(dim, q)) return cudaErrorInvalidValue;
+    return fx_dispatch(dim, q, [&](auto run) {
+        return decltype(run)::residual_batch(batch_tables(q), D, map, nblocks, mode, u, b, r, cur, s);
+    });
 }
 
 template <>
 cudaError_t launch_dg_transfer<double>(int dim, int qf, bool prolong, int64_t ncell, const DGInterp<double> &P,
-                                   const double *in, double *out, cudaStream_t s) {
+                                       const double *in, double *out, cudaStream_t s) {
     return launch_dg_transfer_impl<double>(dim, qf, prolong, ncell, P, in, out, s);
-}
-
-cudaError_t wait_timeouts_fp64(unsigned long long *count) { return read_wait_timeouts(count); }
-cudaError_t wait_timeouts_addr_fp64(unsigned long long **ptr) {
-    return cudaGetSymbolAddress((void **)ptr, g_wait_timeouts);
 }
 
 }  // namespace dgmg

@@ -126,10 +126,22 @@ __global__ void __launch_bounds__(128) k_fd_factors(const __grid_constant__ FDIn
     for (int i = 0; i < q; ++i) out[q * q + i] = (T)lam[i];
 }
 
-// linv[cell][node] = omega / (lambda_x[i] + lambda_y[j] (+ lambda_z[k])) from the
-// factors: the inverse eigenvalue sums with the smoother's damping folded in
-__global__ void k_inverse_eigen_sums(int dim, int q, int64_t ncell, const double *__restrict__ fd, double omega,
-                                     double *__restrict__ linv) {
+// Unit of a cell's table of omega / (sum of eigenvalues): its largest entry (the
+// smallest eigenvalue of every axis) stays below 2^62.
+__device__ int table_unit(int dim, int q, const double *f, double omega) {
+    double s = 0.0;
+    for (int a = 0; a < dim; ++a) {
+        double m = f[a * (q * q + q)];
+        for (int i = 1; i < q; ++i) m = fmin(m, f[a * (q * q + q) + i]);
+        s += m;
+    }
+    return ilogb(omega / s) - 61;
+}
+
+// The inverse eigenvalue sums of every cell with the smoother's damping folded in,
+// as 64-bit integers of the cell's unit
+__global__ void k_fx_table(int dim, int q, int64_t ncell, const double *__restrict__ fd, double omega,
+                           long long *__restrict__ linv) {
     const int64_t nloc = dim == 3 ? (int64_t)q * q * q : (int64_t)q * q;
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= ncell * nloc) return;
@@ -138,13 +150,42 @@ __global__ void k_inverse_eigen_sums(int dim, int q, int64_t ncell, const double
     const double *f = fd + cell * dim * fds + q * q;
     double s = f[node % q] + f[fds + (node / q) % q];
     if (dim == 3) s += f[2 * fds + node / (q * q)];
-    linv[idx] = omega / s;
+    linv[idx] = llrint(ldexp(omega / s, -table_unit(dim, q, f, omega)));
 }
 
-// kfac[cell][f]: the harmonic mean of kappa across face f (0 on the boundary)
+// fd in place: S of every axis as limbs of one unit (every row and column sum of
+// the magnitudes below 2^62), the unit in the word after it, and in the word after
+// axis 0's the unit of the table; one thread per cell
+__global__ void k_fx_factors(int dim, int q, int64_t ncell, double *__restrict__ fd, double omega) {
+    const int64_t cell = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (cell >= ncell) return;
+    const int fds = q * q + q;
+    double *f = fd + cell * dim * fds;
+    const int el = table_unit(dim, q, f + q * q, omega);
+    for (int a = 0; a < dim; ++a) {
+        double *S = f + a * fds;
+        Limb *out = reinterpret_cast<Limb *>(S);
+        double top = 0.0;
+        for (int i = 0; i < q; ++i) {
+            double rs = 0.0, cs = 0.0;
+            for (int j = 0; j < q; ++j) {
+                rs += fabs(S[i * q + j]);
+                cs += fabs(S[j * q + i]);
+            }
+            top = fmax(top, fmax(rs, cs));
+        }
+        const int e = ilogb(top) - 61;
+        for (int i = 0; i < q * q; ++i) out[i] = limb_of(llrint(ldexp(S[i], -e)));
+        out[q * q] = Limb{e, 0};
+        if (a == 0) out[q * q + 1] = Limb{el, 0};
+    }
+}
+
+// kfac[cell][f]: the harmonic mean of kappa across face f (0 on the boundary),
+// times the scale of its axis
 template <typename T>
 __global__ void k_facet_coefficients(int dim, int n0, int n1, int n2, int64_t ncell, const double *__restrict__ kappa,
-                                     T *__restrict__ kfac) {
+                                     double sc0, double sc1, double sc2, T *__restrict__ kfac) {
     const int nface = 2 * dim;
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= ncell * nface) return;
@@ -158,7 +199,7 @@ __global__ void k_facet_coefficients(int dim, int n0, int n1, int n2, int64_t nc
     if (cn >= 0 && cn < na) {
         const int64_t st = a == 0 ? 1 : (a == 1 ? s1 : s2);
         const double kK = kappa[cell], kN = kappa[cell + (side ? st : -st)];
-        v = 2.0 * kK * kN / (kK + kN);
+        v = 2.0 * kK * kN / (kK + kN) * (a == 0 ? sc0 : (a == 1 ? sc1 : sc2));
     }
     kfac[idx] = (T)v;
 }
@@ -166,17 +207,20 @@ __global__ void k_facet_coefficients(int dim, int n0, int n1, int n2, int64_t nc
 }  // namespace
 
 template <typename T>
-cudaError_t launch_facet_coefficients(int dim, const int *n, int64_t ncell, const double *kappa, T *kfac,
-                                      cudaStream_t s) {
+cudaError_t launch_facet_coefficients(int dim, const int *n, int64_t ncell, const double *kappa, const double *scale,
+                                      T *kfac, cudaStream_t s) {
     const int64_t m = ncell * 2 * dim;
     if (m == 0) return cudaSuccess;
     count_launches(1);
     k_facet_coefficients<T><<<(unsigned)((m + 255) / 256), 256, 0, s>>>(dim, n[0], n[1], dim == 3 ? n[2] : 1, ncell,
-                                                                        kappa, kfac);
+                                                                        kappa, scale[0], scale[1],
+                                                                        dim == 3 ? scale[2] : 0.0, kfac);
     return cudaGetLastError();
 }
-template cudaError_t launch_facet_coefficients<double>(int, const int *, int64_t, const double *, double *, cudaStream_t);
-template cudaError_t launch_facet_coefficients<float>(int, const int *, int64_t, const double *, float *, cudaStream_t);
+template cudaError_t launch_facet_coefficients<double>(int, const int *, int64_t, const double *, const double *,
+                                                       double *, cudaStream_t);
+template cudaError_t launch_facet_coefficients<float>(int, const int *, int64_t, const double *, const double *,
+                                                      float *, cudaStream_t);
 
 template <typename T>
 cudaError_t launch_fd_factors(const FDInput &in, const double *kappa, int64_t ncell, T *fd, cudaStream_t s) {
@@ -189,12 +233,20 @@ cudaError_t launch_fd_factors(const FDInput &in, const double *kappa, int64_t nc
 template cudaError_t launch_fd_factors<double>(const FDInput &, const double *, int64_t, double *, cudaStream_t);
 template cudaError_t launch_fd_factors<float>(const FDInput &, const double *, int64_t, float *, cudaStream_t);
 
-cudaError_t launch_inverse_eigen_sums(int dim, int q, int64_t ncell, const double *fd, double omega,
-                                      double *linv, cudaStream_t s) {
+cudaError_t launch_fx_table(int dim, int q, int64_t ncell, const double *fd, double omega, double *linv,
+                            cudaStream_t s) {
     const int64_t n = ncell * (dim == 3 ? (int64_t)q * q * q : (int64_t)q * q);
     if (n == 0) return cudaSuccess;
     count_launches(1);
-    k_inverse_eigen_sums<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(dim, q, ncell, fd, omega, linv);
+    k_fx_table<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(dim, q, ncell, fd, omega,
+                                                           reinterpret_cast<long long *>(linv));
+    return cudaGetLastError();
+}
+
+cudaError_t launch_fx_factors(int dim, int q, int64_t ncell, double *fd, double omega, cudaStream_t s) {
+    if (ncell == 0) return cudaSuccess;
+    count_launches(1);
+    k_fx_factors<<<(unsigned)((ncell + 127) / 128), 128, 0, s>>>(dim, q, ncell, fd, omega);
     return cudaGetLastError();
 }
 
@@ -230,8 +282,6 @@ cudaError_t launch_residual_factors(int dim, int q, int64_t ncell, const TI *fd,
     k_residual_factors<TI, TO><<<(unsigned)((n + 127) / 128), 128, 0, s>>>(dim, q, ncell, fd, m, fdr);
     return cudaGetLastError();
 }
-template cudaError_t launch_residual_factors<double, double>(int, int, int64_t, const double *, const MassTables &,
-                                                             double *, cudaStream_t);
 template cudaError_t launch_residual_factors<double, float>(int, int, int64_t, const double *, const MassTables &,
                                                             float *, cudaStream_t);
 template cudaError_t launch_residual_factors<float, float>(int, int, int64_t, const float *, const MassTables &,

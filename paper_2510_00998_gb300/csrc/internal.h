@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "dgmg.h"
+#include "fx.cuh"
 
 namespace dgmg {
 
@@ -38,14 +39,12 @@ __host__ __device__ constexpr int trace_face_stride(int nf) {
 // Process-wide count of kernels launched by the library (dgmg_kernel_launches).
 extern std::atomic<long long> g_kernel_launches;
 inline void count_launches(int k) { g_kernel_launches.fetch_add(k, std::memory_order_relaxed); }
-// Bounded waits that ran out in the kernels of the float / double translation unit.
+// Bounded waits that ran out in the FP32 kernels of the DG levels and of the volume term.
 cudaError_t wait_timeouts_fp32(unsigned long long *count);
-cudaError_t wait_timeouts_fp64(unsigned long long *count);
 cudaError_t wait_timeouts_volume(unsigned long long *count);
 // device addresses of the same counters on the current device (for
 // stream-ordered snapshots)
 cudaError_t wait_timeouts_addr_fp32(unsigned long long **ptr);
-cudaError_t wait_timeouts_addr_fp64(unsigned long long **ptr);
 
 // ------------------------------------------------------- reference element
 // 1D Lagrange element of degree p on [-1,1] with GLL (Sec. 2.2) or GL
@@ -90,16 +89,11 @@ struct MassTables {
 template <typename TI, typename TO>
 cudaError_t launch_residual_factors(int dim, int q, int64_t ncell, const TI *fd, const MassTables &m, TO *fdr,
                                     cudaStream_t s);
-// kfac[cell][2 axis + side] = 2 kappa_K kappa_N / (kappa_K + kappa_N) across each
-// interior face (0 on the boundary), from the FP64 kappa
+// kfac[cell][2 axis + side] = scale[axis] 2 kappa_K kappa_N / (kappa_K + kappa_N)
+// across each interior face (0 on the boundary), from the FP64 kappa
 template <typename T>
-cudaError_t launch_facet_coefficients(int dim, const int *n, int64_t ncell, const double *kappa, T *kfac,
-                                      cudaStream_t s);
-// linv[cell][node] = omega / (sum of the cell's eigenvalues at the node): the
-// smoother's damping folded into the table
-cudaError_t launch_inverse_eigen_sums(int dim, int q, int64_t ncell, const double *fd, double omega,
-                                      double *linv, cudaStream_t s);
-
+cudaError_t launch_facet_coefficients(int dim, const int *n, int64_t ncell, const double *kappa, const double *scale,
+                                      T *kfac, cudaStream_t s);
 // ------------------------------------------------------------ kernels API
 // Constant data of one DG level, passed to kernels by value.
 template <typename T>
@@ -129,6 +123,48 @@ struct DGConst {
     // face (formed once per level, updated with kappa)
     const T *kfac;
 };
+
+// FP64 levels run in block fixed-point arithmetic (fx.cuh, dg_fx.cuh): their
+// constants are the limbs of the reference element's tables and of the level's
+// mesh-dependent vectors.
+struct FxLevel {
+    FxTab tab;
+    FxConst cst;
+};
+template <>
+struct DGConst<double> : FxLevel {};
+// the tables of the element (basis, facet penalty of degree penalty_p)
+void fx_tables(const RefElem1D &re, int penalty_p, FxTab &tab);
+// mesh-dependent vectors; keep = 1 - omega (exact blocks) or 1
+void fx_level(const RefElem1D &re, int penalty_p, int dim, const int *n, int64_t ncell, double keep, FxConst &cst);
+// cells of one work item of the FP64 kernels
+int fx_cells_per_cta(int dim, int q);
+template <typename T>
+struct BatchDG;
+struct BlockMap;
+// the FP64 kernels of one (dimension, nodes per axis) (dg_fx.cuh)
+template <int DIM, int Q>
+struct FxRun {
+    static cudaError_t project(const FxLevel &l, double *u, const double *e0, double *tr, cudaStream_t s);
+    static cudaError_t smooth(const FxLevel &l, bool exact, int flags, double *u, const double *b, const double *kappa,
+                              const double *fd, const double *linv, const double *tri, double *tro, cudaStream_t s);
+    static cudaError_t residual(const FxLevel &l, int mode, const double *u, const double *b, const double *kappa,
+                                const double *tr, double *r, double *corners, cudaStream_t s);
+    static cudaError_t project_batch(const FxTab &tab, const BatchDG<double> *D, const BlockMap *map, int nblocks,
+                                     double *u, int with_e0, cudaStream_t s);
+    static cudaError_t smooth_batch(const FxTab &tab, bool exact, const BatchDG<double> *D, const BlockMap *map,
+                                    int nblocks, int flags, double *u, const double *b, int cur, cudaStream_t s);
+    static cudaError_t residual_batch(const FxTab &tab, const BatchDG<double> *D, const BlockMap *map, int nblocks,
+                                      int mode, const double *u, const double *b, double *r, int cur, cudaStream_t s);
+    static int cells_per_cta();
+};
+// linv[cell][node] = omega / (sum of the cell's eigenvalues) as 64-bit integers of
+// one exponent per cell, from the FP64 factors [S | lambda]; then, in place, the
+// factors as limbs: per axis S, its exponent in the word after it (h of a Limb);
+// the word after axis 0's exponent holds the table's.
+cudaError_t launch_fx_table(int dim, int q, int64_t ncell, const double *fd, double omega, double *linv,
+                            cudaStream_t s);
+cudaError_t launch_fx_factors(int dim, int q, int64_t ncell, double *fd, double omega, cudaStream_t s);
 
 // Q1 level description for the CG kernels.
 template <typename T>
@@ -171,6 +207,15 @@ struct BatchDG {
     T *tr[2];
     T *corners;
     const T *e0;          // the instance's Q1 level-0 correction (p-prolongation source)
+};
+template <>
+struct BatchDG<double> {
+    FxConst c;
+    int64_t off;
+    const double *kappa, *fd, *linv;
+    double *tr[2];
+    double *corners;
+    const double *e0;
 };
 // CTA -> (instance, first cell of the CTA within the instance)
 struct BlockMap {
@@ -242,8 +287,11 @@ unsigned persistent_grid(const void *fn, int threads, size_t smem, int64_t items
 template <typename T>
 cudaError_t launch_project(int dim, int q, const DGConst<T> &c, int cpb, T *u, const T *e0,
                            T *tr, cudaStream_t s);
+// SM_ZERO: the iterate is zero (u and its traces need not be set and are not
+// read); SM_NO_TRACES: the projections of the new iterate are not wanted (FP64)
+enum { SM_ZERO = 1, SM_NO_TRACES = 2 };
 template <typename T>
-cudaError_t launch_smooth(int dim, int q, const DGConst<T> &c, int cpb, int exact, T *u, const T *b,
+cudaError_t launch_smooth(int dim, int q, const DGConst<T> &c, int cpb, int exact, int flags, T *u, const T *b,
                           const T *kappa, const T *fd, const T *linv, const T *tr_in, T *tr_out, cudaStream_t s);
 // mode bits for launch_residual
 // RES_DIRECT (batched FP32 one-thread-per-cell residual): A_KK u in the direct
@@ -263,7 +311,7 @@ cudaError_t launch_project_batch(int dim, int q, const BatchDG<T> *D, const Bloc
 // cpb 0: the one-thread-per-cell smoother (32 cells per CTA)
 template <typename T>
 cudaError_t launch_smooth_batch(int dim, int q, const BatchDG<T> *D, const BlockMap *map, int nblocks, int cpb,
-                                int exact, T *u, const T *b, int cur, cudaStream_t s);
+                                int exact, int flags, T *u, const T *b, int cur, cudaStream_t s);
 template <typename T>
 cudaError_t launch_residual_batch(int dim, int q, const BatchDG<T> *D, const BlockMap *map, int nblocks, int cpb,
                                   int mode, const T *u, const T *b, T *r, int cur, cudaStream_t s);

@@ -48,11 +48,11 @@ int post_scalars(dgmg_ctx *C, cudaStream_t s) {
     return DGMG_OK;
 }
 
-// Stream-ordered snapshot of the bounded-wait counters (FP32 and FP64 DG
-// kernels, Q1 grid barrier) into pinned slot `at` (0 start, 1 end of a run).
+// Stream-ordered snapshot of the bounded-wait counters (FP32 DG kernels, Q1 grid
+// barrier) into pinned slot `at` (0 start, 1 end of a run).
 int snapshot_timeouts(dgmg_ctx *C, int at, cudaStream_t s) {
-    for (int k = 0; k < 3; ++k)
-        LC(cudaMemcpyAsync(C->host_scal + S_TMO + 3 * at + k, C->tmo_dev[k], sizeof(unsigned long long),
+    for (int k = 0; k < 2; ++k)
+        LC(cudaMemcpyAsync(C->host_scal + S_TMO + 2 * at + k, C->tmo_dev[k], sizeof(unsigned long long),
                            cudaMemcpyDeviceToHost, s));
     return DGMG_OK;
 }
@@ -71,9 +71,9 @@ int check_timeouts(dgmg_ctx *C, cudaStream_t s) {
     RC(snapshot_timeouts(C, 1, s));
     LC(cudaStreamSynchronize(s));
     bool grew = false;
-    for (int k = 0; k < 3; ++k) grew = grew || snapshot_value(C, 3 + k) != snapshot_value(C, k);
+    for (int k = 0; k < 2; ++k) grew = grew || snapshot_value(C, 2 + k) != snapshot_value(C, k);
     if (!grew) return DGMG_OK;
-    if (snapshot_value(C, 5) != snapshot_value(C, 2)) g_q1_one_launch_off.store(1);
+    if (snapshot_value(C, 3) != snapshot_value(C, 1)) g_q1_one_launch_off.store(1);
     return fail(DGMG_ETIMEOUT,
                 "a bounded device-side wait ran out during the solve (bulk-copy mbarrier or Q1 grid barrier); "
                 "the result is not to be trusted");

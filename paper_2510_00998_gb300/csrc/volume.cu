@@ -376,8 +376,15 @@ void jacobi_eigen(int n, std::vector<double> &A, std::vector<double> &V) {
 // The ctx's shared data of both forms, built at its first call (kept in the
 // ctx, freed with it): E swizzled on the device, the sum-factorised factors.
 int vol_setup(dgmg_ctx &C, cudaStream_t s) {
-    const DGConst<double> &c = C.d64.c;
     const int q = VQ;
+    std::vector<double> M[3], K[3];               // the h-scaled 1D matrices
+    for (int a = 0; a < 3; ++a) {
+        const double h = 1.0 / C.n[a];
+        for (int i = 0; i < q * q; ++i) {
+            M[a].push_back(C.re.M[i] * h / 2.0);
+            K[a].push_back(C.re.K[i] * 2.0 / h);
+        }
+    }
     // E[n][k] = sum_a (K_a along a, M_b along the others), node i + q j + q^2 k
     std::vector<float> Esw(OPERAND_BYTES / 4, 0.f);
     for (int n = 0; n < VNL; ++n)
@@ -386,7 +393,7 @@ int vol_setup(dgmg_ctx &C, cudaStream_t s) {
             double e = 0.0;
             for (int a = 0; a < 3; ++a) {
                 double t = 1.0;
-                for (int d = 0; d < 3; ++d) t *= (d == a ? c.K[d] : c.M[d])[ni[d] * q + ki[d]];
+                for (int d = 0; d < 3; ++d) t *= (d == a ? K[d] : M[d])[ni[d] * q + ki[d]];
                 e += t;
             }
             // TF32 (round to nearest, ties away: 10 mantissa bits kept)
@@ -400,7 +407,8 @@ int vol_setup(dgmg_ctx &C, cudaStream_t s) {
     RC(C.upload(&C.vol_esw, Esw));
     // generalised eigenvectors per axis: M = L L^T, L^-1 K L^-T = Q Lam Q^T, V = L^-T Q
     for (int a = 0; a < 3; ++a) {
-        std::vector<double> Mm(c.M[a], c.M[a] + q * q), Km(c.K[a], c.K[a] + q * q), Li(q * q);
+        const std::vector<double> &Mm = M[a], &Km = K[a];
+        std::vector<double> Li(q * q);
         if (!cholesky_inverse_lower(q, Mm.data(), Li.data())) return fail(DGMG_EINVAL, "mass not SPD");
         std::vector<double> A(q * q, 0.0), Qv;
         for (int i = 0; i < q; ++i)
