@@ -429,14 +429,8 @@ int batch_cg_cycle(dgmg_batch &B, int l, cudaStream_t s) {
 template <typename T>
 int batch_vcycle(dgmg_batch &B, const T *r, T *z, cudaStream_t s) {
     const int exact = B.opts.block_inverse == DGMG_BLOCK_EXACT ? 1 : 0;
-    // FP64: the first step takes the zero iterate as such, nothing reads the
-    // projections of the last one
-    const bool fx = std::is_same<T, double>::value;
-    if constexpr (!std::is_same<T, double>::value) {
-        LC(cudaMemsetAsync(z, 0, sizeof(T) * B.ndof, s));
-        for (auto &grp : B.groups)
-            LC(launch_zero_traces_batch<T>(B.dim, grp.q, grp.prec<T>().D, (int)grp.members.size(), s));
-    }
+    // the first step takes the zero iterate as such (nu_pre >= 1), nothing reads the
+    // projections of the last one; z between the problems stays zero
     auto smooth = [&](int k, int flags) -> int {
         for (auto &grp : B.groups) {
             auto &g = grp.prec<T>();
@@ -445,7 +439,7 @@ int batch_vcycle(dgmg_batch &B, const T *r, T *z, cudaStream_t s) {
         }
         return DGMG_OK;
     };
-    for (int k = 0; k < B.opts.nu_pre; ++k) RC(smooth(k, fx && k == 0 ? SM_ZERO : 0));
+    for (int k = 0; k < B.opts.nu_pre; ++k) RC(smooth(k, k == 0 ? SM_ZERO : 0));
     for (auto &grp : B.groups) {
         auto &g = grp.prec<T>();
         LC(launch_residual_batch<T>(B.dim, grp.q, g.D, g.map[TILE_RESIDUAL], g.nblocks[TILE_RESIDUAL],
@@ -459,7 +453,7 @@ int batch_vcycle(dgmg_batch &B, const T *r, T *z, cudaStream_t s) {
         LC(launch_project_batch<T>(B.dim, grp.q, g.D, g.map[TILE_PROJECT], g.nblocks[TILE_PROJECT],
                                    g.tile[TILE_PROJECT], z + grp.dof0, 1, s));
     }
-    for (int k = 0; k < B.opts.nu_post; ++k) RC(smooth(k, fx && k == B.opts.nu_post - 1 ? SM_NO_TRACES : 0));
+    for (int k = 0; k < B.opts.nu_post; ++k) RC(smooth(k, k == B.opts.nu_post - 1 ? SM_NO_TRACES : 0));
     return DGMG_OK;
 }
 

@@ -864,22 +864,21 @@ int level_cycle(dgmg_ctx &C, int l, const T *b, T *z, cudaStream_t s) {
     DGDev<T> &D = dg_level<T>(C, l);
     const DGSpace &S = C.dgs[l];
     const int64_t trn = C.ncell * 2 * C.dim * trace_face_stride<T>((int)(S.nloc / S.q));
-    // FP64: the first step takes the zero iterate as such (no facet terms, nothing
-    // to clear), and nothing reads the projections of the last one
-    const bool fx = std::is_same<T, double>::value;
-    if (!fx || C.opts.nu_pre == 0) {
+    // the first step takes the zero iterate as such (no facet terms, nothing to
+    // clear), and nothing reads the projections of the last one
+    if (C.opts.nu_pre == 0) {
         LC(cudaMemsetAsync(z, 0, sizeof(T) * S.ndof, s));
         LC(cudaMemsetAsync(D.tr[0], 0, sizeof(T) * trn, s));   // projections of z = 0
     }
     int cur = 0;
     for (int k = 0; k < C.opts.nu_pre; ++k) {
-        RC(level_smooth<T>(C, l, z, b, cur, fx && k == 0 ? SM_ZERO : 0, s));
+        RC(level_smooth<T>(C, l, z, b, cur, k == 0 ? SM_ZERO : 0, s));
         cur ^= 1;
     }
     RC(coarse_correction<T>(C, l, z, b, cur, s));
     cur = 0;
     for (int k = 0; k < C.opts.nu_post; ++k) {
-        RC(level_smooth<T>(C, l, z, b, cur, fx && k == C.opts.nu_post - 1 ? SM_NO_TRACES : 0, s));
+        RC(level_smooth<T>(C, l, z, b, cur, k == C.opts.nu_post - 1 ? SM_NO_TRACES : 0, s));
         cur ^= 1;
     }
     return DGMG_OK;

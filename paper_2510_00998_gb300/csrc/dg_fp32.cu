@@ -10,11 +10,11 @@ cudaError_t launch_project<float>(int dim, int q, const DGConst<float> &c, int c
 }
 
 template <>
-cudaError_t launch_smooth<float>(int dim, int q, const DGConst<float> &c, int cpb, int exact, int, float *u,
+cudaError_t launch_smooth<float>(int dim, int q, const DGConst<float> &c, int cpb, int exact, int flags, float *u,
                                 const float *b,
                                 const float *kappa, const float *fd, const float *linv, const float *tr_in, float *tr_out,
                                 cudaStream_t s) {
-    return launch_smooth_impl<float>(dim, q, c, cpb, exact, u, b, kappa, fd, linv, tr_in, tr_out, s);
+    return launch_smooth_impl<float>(dim, q, c, cpb, exact, flags, u, b, kappa, fd, linv, tr_in, tr_out, s);
 }
 
 template <>
@@ -31,8 +31,8 @@ cudaError_t launch_project_batch<float>(int dim, int q, const BatchDG<float> *D,
 }
 template <>
 cudaError_t launch_smooth_batch<float>(int dim, int q, const BatchDG<float> *D, const BlockMap *map, int nblocks, int cpb,
-                                    int exact, int, float *u, const float *b, int cur, cudaStream_t s) {
-    return launch_smooth_batch_impl<float>(dim, q, D, map, nblocks, cpb, exact, u, b, cur, s);
+                                    int exact, int flags, float *u, const float *b, int cur, cudaStream_t s) {
+    return launch_smooth_batch_impl<float>(dim, q, D, map, nblocks, cpb, exact, flags, u, b, cur, s);
 }
 template <>
 cudaError_t launch_residual_batch<float>(int dim, int q, const BatchDG<float> *D, const BlockMap *map, int nblocks,
@@ -40,11 +40,6 @@ cudaError_t launch_residual_batch<float>(int dim, int q, const BatchDG<float> *D
                                       cudaStream_t s) {
     return launch_residual_batch_impl<float>(dim, q, D, map, nblocks, cpb, mode, u, b, r, cur, s);
 }
-template <>
-cudaError_t launch_zero_traces_batch<float>(int dim, int q, const BatchDG<float> *D, int count, cudaStream_t s) {
-    return launch_zero_traces_batch_impl<float>(dim, q, D, count, s);
-}
-
 template <>
 cudaError_t launch_dg_transfer<float>(int dim, int qf, bool prolong, int64_t ncell, const DGInterp<float> &P,
                                    const float *in, float *out, cudaStream_t s) {

@@ -511,7 +511,7 @@ __global__ void __launch_bounds__(256) k_project(DGConst<T> c, int cpb, T *__res
 // tr_out (ping-pong: every cell reads projections of the same iterate).
 // ---------------------------------------------------------------------------
 template <int DIM, int Q, typename T>
-__device__ __forceinline__ void k_smooth_body(const DGConst<T> &c, int64_t cell0, int cpb, int exact, T *__restrict__ u, const T *__restrict__ b, const T *__restrict__ kappa, const T *__restrict__ fd, const T *__restrict__ linv, const T *__restrict__ tr_in, T *__restrict__ tr_out) {
+__device__ __forceinline__ void k_smooth_body(const DGConst<T> &c, int64_t cell0, int cpb, int exact, int flags, T *__restrict__ u, const T *__restrict__ b, const T *__restrict__ kappa, const T *__restrict__ fd, const T *__restrict__ linv, const T *__restrict__ tr_in, T *__restrict__ tr_out) {
     using G = Geo<DIM, Q, T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *sFD = reinterpret_cast<T *>(smem_raw);   // [cpb][DIM][FDSP], 16-byte aligned blocks
@@ -533,7 +533,13 @@ __device__ __forceinline__ void k_smooth_body(const DGConst<T> &c, int64_t cell0
     __shared__ T sT[DIM * Q * Q + 2 * DIM * Q];
     stage_mass_rank1<DIM, Q, T>(c, sMw, sMu);
     if (!exact) stage_block_tables<DIM, Q, T>(c, sT);
-    block_copy(sU, u + cell0 * G::NL, (int64_t)ncl * G::NL);
+    // a zero iterate: u = 0, no facet terms (mask 0)
+    const bool zero = (flags & SM_ZERO) != 0;
+    if (zero) {
+        for (int i = threadIdx.x; i < ncl * G::NL; i += blockDim.x) sU[i] = T(0);
+    } else {
+        block_copy(sU, u + cell0 * G::NL, (int64_t)ncl * G::NL);
+    }
     block_copy(sR, b + cell0 * G::NL, (int64_t)ncl * G::NL);
     for (int64_t i = threadIdx.x; i < (int64_t)ncl * DIM * G::FDS; i += blockDim.x)
         sFD[(i / G::FDS) * G::FDSP + i % G::FDS] = fd[cell0 * DIM * G::FDS + i];
@@ -541,17 +547,19 @@ __device__ __forceinline__ void k_smooth_body(const DGConst<T> &c, int64_t cell0
     T *myK = sK + lc * (G::NFACE + 1);
     if (active) {
         cell_coords<DIM>(cell, c.n, ci);
-        load_neighbour_traces<DIM, Q, T>(c, cell, ci, t, tr_in, kappa, myF, myK, myK + G::NFACE);
+        if (!zero) load_neighbour_traces<DIM, Q, T>(c, cell, ci, t, tr_in, kappa, myF, myK, myK + G::NFACE);
     }
     __syncthreads();
     T *myR = sR + lc * G::NL;
     T *myU = sU + lc * G::NL;
-    const int mask = active ? interior_mask<DIM>(ci, c.n) : 0;
-    if (!exact) build_block_1d<DIM, Q, T>(c, sT, active, t, myK, mask, sKT + lc * DIM * Q * Q);
-    lift_coefficients<DIM, Q, T>(c, active, t, myK, mask, sC + lc * G::NLC);   // read after facet_mass's barriers
-    facet_mass<DIM, Q, T>(sMw, sMu, active, t, myF, sDot + lc * G::NDOT, mask);
-    lift_neighbours<DIM, Q, T>(c, active, t, myR, myF, sC + lc * G::NLC, mask);
-    if (!exact)
+    if (!zero) {
+        const int mask = active ? interior_mask<DIM>(ci, c.n) : 0;
+        if (!exact) build_block_1d<DIM, Q, T>(c, sT, active, t, myK, mask, sKT + lc * DIM * Q * Q);
+        lift_coefficients<DIM, Q, T>(c, active, t, myK, mask, sC + lc * G::NLC);   // read after facet_mass's barriers
+        facet_mass<DIM, Q, T>(sMw, sMu, active, t, myF, sDot + lc * G::NDOT, mask);
+        lift_neighbours<DIM, Q, T>(c, active, t, myR, myF, sC + lc * G::NLC, mask);
+    }
+    if (!exact && !zero)
         subtract_block_apply<DIM, Q, T>(c, active, t, myU, myR, sA + lc * G::NL, sB + lc * G::NL,
                                         sKT + lc * DIM * Q * Q, sMw, sMu);
     const T *myS = sFD + lc * DIM * G::FDSP;     // S_a at a*FDSP, lambda_a at a*FDSP + Q*Q
@@ -654,10 +662,10 @@ __device__ __forceinline__ void k_smooth_body(const DGConst<T> &c, int64_t cell0
         }
 #pragma unroll
         for (int i = 0; i < Q; ++i) myU[G::vidx(0, t, i)] = un[i];
-        write_pencil_traces<DIM, Q, T>(c, 0, t, un, trc);
+        if (!(flags & SM_NO_TRACES)) write_pencil_traces<DIM, Q, T>(c, 0, t, un, trc);
     }
     __syncthreads();
-    if (active) {
+    if (active && !(flags & SM_NO_TRACES)) {
 #pragma unroll
         for (int dir = 1; dir < DIM; ++dir) {
             T x[Q];
@@ -670,8 +678,8 @@ __device__ __forceinline__ void k_smooth_body(const DGConst<T> &c, int64_t cell0
 }
 
 template <int DIM, int Q, typename T>
-__global__ void __launch_bounds__(256) k_smooth(DGConst<T> c, int cpb, int exact, T *__restrict__ u, const T *__restrict__ b, const T *__restrict__ kappa, const T *__restrict__ fd, const T *__restrict__ linv, const T *__restrict__ tr_in, T *__restrict__ tr_out) {
-    k_smooth_body<DIM, Q, T>(c, (int64_t)blockIdx.x * cpb, cpb, exact, u, b, kappa, fd, linv, tr_in, tr_out);
+__global__ void __launch_bounds__(256) k_smooth(DGConst<T> c, int cpb, int exact, int flags, T *__restrict__ u, const T *__restrict__ b, const T *__restrict__ kappa, const T *__restrict__ fd, const T *__restrict__ linv, const T *__restrict__ tr_in, T *__restrict__ tr_out) {
+    k_smooth_body<DIM, Q, T>(c, (int64_t)blockIdx.x * cpb, cpb, exact, flags, u, b, kappa, fd, linv, tr_in, tr_out);
 }
 
 // ---------------------------------------------------------------------------
@@ -822,29 +830,29 @@ __global__ void __launch_bounds__(256) k_project_batch(const BatchDG<T> *__restr
 template <int DIM, int Q, typename T>
 __global__ void __launch_bounds__(256) k_smooth_batch(const BatchDG<T> *__restrict__ D,
                                                        const BlockMap *__restrict__ map, int nblocks, int cpb,
-                                                       int exact, T *u, const T *b, int cur) {
+                                                       int exact, int flags, T *u, const T *b, int cur) {
     using G = Geo<DIM, Q, T>;
     __shared__ __align__(16) BatchDG<T> sd;
     for (int k = blockIdx.x; k < nblocks; k += gridDim.x) {
         if (k != (int)blockIdx.x) __syncthreads();
         const BlockMap m = map[k];
         load_batch_desc(D + m.inst, &sd);
-        k_smooth_body<DIM, Q, T>(sd.c, m.cell0, cpb, exact, u + sd.off * G::NL, b + sd.off * G::NL, sd.kappa, sd.fd,
+        k_smooth_body<DIM, Q, T>(sd.c, m.cell0, cpb, exact, flags, u + sd.off * G::NL, b + sd.off * G::NL, sd.kappa, sd.fd,
                                  sd.linv, sd.tr[cur], sd.tr[cur ^ 1]);
     }
 }
 
 template <typename T, int Q>
 __global__ void __launch_bounds__(32) k_smooth_cells_batch(const BatchDG<T> *__restrict__ D,
-                                                            const BlockMap *__restrict__ map, int nblocks, T *u,
-                                                            const T *b, int cur) {
+                                                            const BlockMap *__restrict__ map, int nblocks,
+                                                            int flags, T *u, const T *b, int cur) {
     constexpr int NL = Q * Q * Q;
     __shared__ __align__(16) BatchDG<T> sd;
     for (int k = blockIdx.x; k < nblocks; k += gridDim.x) {
         if (k != (int)blockIdx.x) __syncthreads();
         const BlockMap m = map[k];
         load_batch_desc(D + m.inst, &sd);
-        smooth_cells_body<T, Q>(sd.c, m.cell0, u + sd.off * NL, b + sd.off * NL, sd.kappa, sd.fd, sd.linv,
+        smooth_cells_body<T, Q>(sd.c, m.cell0, flags, u + sd.off * NL, b + sd.off * NL, sd.kappa, sd.fd, sd.linv,
                                 sd.tr[cur], sd.tr[cur ^ 1], k != (int)blockIdx.x);
     }
 }
@@ -892,16 +900,6 @@ __global__ void __launch_bounds__(256) k_residual_batch(const BatchDG<T> *__rest
         k_residual_body<DIM, Q, T>(sd.c, m.cell0, cpb, mode, u + sd.off * G::NL, b ? b + sd.off * G::NL : nullptr,
                                    sd.kappa, sd.tr[cur], r ? r + sd.off * G::NL : nullptr, sd.corners);
     }
-}
-
-// tr[0] of instance blockIdx.x := 0 (projections of a zero iterate)
-template <int DIM, int Q, typename T>
-__global__ void k_zero_traces_batch(const BatchDG<T> *__restrict__ D) {
-    using G = Geo<DIM, Q, T>;
-    const BatchDG<T> &d = D[blockIdx.x];
-    const int64_t n = d.c.ncell * G::TR;
-    T *tr = d.tr[0];
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) tr[i] = T(0);
 }
 
 // Shared-memory bytes per CTA of each kernel.
@@ -964,7 +962,7 @@ struct DGLaunch {
         k_project<DIM, Q, T><<<(unsigned)grid, cpb * G::NF, sm, s>>>(c, cpb, u, e0, tr);
         return cudaGetLastError();
     }
-    static cudaError_t smooth(const DGConst<T> &c, int cpb, int exact, T *u, const T *b, const T *kappa,
+    static cudaError_t smooth(const DGConst<T> &c, int cpb, int exact, int flags, T *u, const T *b, const T *kappa,
                               const T *fd, const T *linv, const T *tri, T *tro, cudaStream_t s) {
         if constexpr (CELLS_OK) if (c.ncell < (int64_t(1) << 31)) {   // 32-bit cell indices
             // bulk copies want 16-byte aligned vectors, factors and table; the face
@@ -973,7 +971,7 @@ struct DGLaunch {
             const bool aligned = ((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(b) |
                                    reinterpret_cast<uintptr_t>(fd) | reinterpret_cast<uintptr_t>(linv)) & 15) == 0 &&
                                  ((reinterpret_cast<uintptr_t>(tri) | reinterpret_cast<uintptr_t>(tro)) & tra) == 0;
-            if (cpb <= 0 && exact && aligned && !c.gl) return smooth_cells(c, u, b, kappa, fd, linv, tri, tro, s);
+            if (cpb <= 0 && exact && aligned && !c.gl) return smooth_cells(c, flags, u, b, kappa, fd, linv, tri, tro, s);
         }
         if (cpb <= 0) cpb = default_cpb();
         const size_t sm = smem_smooth<DIM, Q, T>(cpb, exact != 0);
@@ -985,13 +983,14 @@ struct DGLaunch {
         const int64_t grid = (c.ncell + cpb - 1) / cpb;
         if (grid == 0) return cudaSuccess;
         count_launches(1);
-        k_smooth<DIM, Q, T><<<(unsigned)grid, cpb * G::NF, sm, s>>>(c, cpb, exact, u, b, kappa, fd, linv, tri, tro);
+        k_smooth<DIM, Q, T><<<(unsigned)grid, cpb * G::NF, sm, s>>>(c, cpb, exact, flags, u, b, kappa, fd, linv, tri,
+                                                                    tro);
         return cudaGetLastError();
     }
     // 3D exact-block smoothing step with one thread per cell (k_smooth_cells):
     // FP32 q <= 5, FP64 q <= 4 (the cell must fit in the registers of a thread)
     static constexpr bool CELLS_OK = DIM == 3 && (std::is_same<T, float>::value ? Q <= 5 : Q <= 4);
-    static cudaError_t smooth_cells(const DGConst<T> &c, T *u, const T *b, const T *kappa, const T *fd,
+    static cudaError_t smooth_cells(const DGConst<T> &c, int flags, T *u, const T *b, const T *kappa, const T *fd,
                                     const T *linv, const T *tri, T *tro, cudaStream_t s) {
         if constexpr (CELLS_OK) {
             using CG = CellGeo<T, Q>;
@@ -1004,7 +1003,7 @@ struct DGLaunch {
             const int64_t grid = (c.ncell + CG::W - 1) / CG::W;
             if (grid == 0) return cudaSuccess;
             count_launches(1);
-            k_smooth_cells<T, Q><<<(unsigned)grid, CG::W, CG::BYTES, s>>>(c, u, b, kappa, fd, linv, tri, tro);
+            k_smooth_cells<T, Q><<<(unsigned)grid, CG::W, CG::BYTES, s>>>(c, flags, u, b, kappa, fd, linv, tri, tro);
             return cudaGetLastError();
         } else {
             return cudaErrorInvalidValue;
@@ -1067,8 +1066,8 @@ struct DGLaunch {
                                      cpb * G::NF, smp, s>>>(D, map, nblocks, cpb, u, with_e0);
         return cudaGetLastError();
     }
-    static cudaError_t smooth_batch(const BatchDG<T> *D, const BlockMap *map, int nblocks, int cpb, int exact, T *u,
-                                    const T *b, int cur, cudaStream_t s) {
+    static cudaError_t smooth_batch(const BatchDG<T> *D, const BlockMap *map, int nblocks, int cpb, int exact,
+                                    int flags, T *u, const T *b, int cur, cudaStream_t s) {
         if (nblocks <= 0) return cudaSuccess;
         if constexpr (CELLS_OK) {
             if (cpb <= 0 && exact) {
@@ -1082,7 +1081,7 @@ struct DGLaunch {
                 count_launches(1);
                 k_smooth_cells_batch<T, Q><<<persistent_grid((const void *)k_smooth_cells_batch<T, Q>, CG::W, CG::BYTES,
                                                              nblocks),
-                                             CG::W, CG::BYTES, s>>>(D, map, nblocks, u, b, cur);
+                                             CG::W, CG::BYTES, s>>>(D, map, nblocks, flags, u, b, cur);
                 return cudaGetLastError();
             }
         }
@@ -1095,7 +1094,7 @@ struct DGLaunch {
         count_launches(1);
         const size_t sms = smem_smooth<DIM, Q, T>(cpb, exact != 0);
         k_smooth_batch<DIM, Q, T><<<persistent_grid((const void *)k_smooth_batch<DIM, Q, T>, cpb * G::NF, sms, nblocks),
-                                    cpb * G::NF, sms, s>>>(D, map, nblocks, cpb, exact, u, b, cur);
+                                    cpb * G::NF, sms, s>>>(D, map, nblocks, cpb, exact, flags, u, b, cur);
         return cudaGetLastError();
     }
     static cudaError_t residual_batch(const BatchDG<T> *D, const BlockMap *map, int nblocks, int cpb, int mode,
@@ -1145,12 +1144,6 @@ struct DGLaunch {
         const size_t smr = smem_residual<DIM, Q, T>(cpb);
         k_residual_batch<DIM, Q, T><<<persistent_grid((const void *)k_residual_batch<DIM, Q, T>, cpb * G::NF, smr, nblocks),
                                       cpb * G::NF, smr, s>>>(D, map, nblocks, cpb, mode, u, b, r, cur);
-        return cudaGetLastError();
-    }
-    static cudaError_t zero_traces_batch(const BatchDG<T> *D, int count, cudaStream_t s) {
-        if (count <= 0) return cudaSuccess;
-        count_launches(1);
-        k_zero_traces_batch<DIM, Q, T><<<count, 256, 0, s>>>(D);
         return cudaGetLastError();
     }
     static cudaError_t residual(const DGConst<T> &c, int cpb, int mode, const T *u, const T *b, const T *kappa,
@@ -1207,9 +1200,9 @@ cudaError_t launch_project_impl(int dim, int q, const DGConst<T> &c, int cpb, T 
     DGMG_DISPATCH(dim, q, project(c, cpb, u, e0, tr, s))
 }
 template <typename T>
-cudaError_t launch_smooth_impl(int dim, int q, const DGConst<T> &c, int cpb, int exact, T *u, const T *b,
+cudaError_t launch_smooth_impl(int dim, int q, const DGConst<T> &c, int cpb, int exact, int flags, T *u, const T *b,
                                const T *kappa, const T *fd, const T *linv, const T *tri, T *tro, cudaStream_t s) {
-    DGMG_DISPATCH(dim, q, smooth(c, cpb, exact, u, b, kappa, fd, linv, tri, tro, s))
+    DGMG_DISPATCH(dim, q, smooth(c, cpb, exact, flags, u, b, kappa, fd, linv, tri, tro, s))
 }
 template <typename T>
 cudaError_t launch_residual_impl(int dim, int q, const DGConst<T> &c, int cpb, int mode, const T *u, const T *b,
@@ -1223,17 +1216,13 @@ cudaError_t launch_project_batch_impl(int dim, int q, const BatchDG<T> *D, const
 }
 template <typename T>
 cudaError_t launch_smooth_batch_impl(int dim, int q, const BatchDG<T> *D, const BlockMap *map, int nblocks, int cpb,
-                                     int exact, T *u, const T *b, int cur, cudaStream_t s) {
-    DGMG_DISPATCH(dim, q, smooth_batch(D, map, nblocks, cpb, exact, u, b, cur, s))
+                                     int exact, int flags, T *u, const T *b, int cur, cudaStream_t s) {
+    DGMG_DISPATCH(dim, q, smooth_batch(D, map, nblocks, cpb, exact, flags, u, b, cur, s))
 }
 template <typename T>
 cudaError_t launch_residual_batch_impl(int dim, int q, const BatchDG<T> *D, const BlockMap *map, int nblocks,
                                        int cpb, int mode, const T *u, const T *b, T *r, int cur, cudaStream_t s) {
     DGMG_DISPATCH(dim, q, residual_batch(D, map, nblocks, cpb, mode, u, b, r, cur, s))
-}
-template <typename T>
-cudaError_t launch_zero_traces_batch_impl(int dim, int q, const BatchDG<T> *D, int count, cudaStream_t s) {
-    DGMG_DISPATCH(dim, q, zero_traces_batch(D, count, s))
 }
 
 }  // namespace dgmg

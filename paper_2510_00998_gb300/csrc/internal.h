@@ -288,7 +288,7 @@ template <typename T>
 cudaError_t launch_project(int dim, int q, const DGConst<T> &c, int cpb, T *u, const T *e0,
                            T *tr, cudaStream_t s);
 // SM_ZERO: the iterate is zero (u and its traces need not be set and are not
-// read); SM_NO_TRACES: the projections of the new iterate are not wanted (FP64)
+// read); SM_NO_TRACES: the projections of the new iterate are not wanted
 enum { SM_ZERO = 1, SM_NO_TRACES = 2 };
 template <typename T>
 cudaError_t launch_smooth(int dim, int q, const DGConst<T> &c, int cpb, int exact, int flags, T *u, const T *b,
@@ -315,9 +315,6 @@ cudaError_t launch_smooth_batch(int dim, int q, const BatchDG<T> *D, const Block
 template <typename T>
 cudaError_t launch_residual_batch(int dim, int q, const BatchDG<T> *D, const BlockMap *map, int nblocks, int cpb,
                                   int mode, const T *u, const T *b, T *r, int cur, cudaStream_t s);
-// zero tr[0] of every instance (one CTA per instance)
-template <typename T>
-cudaError_t launch_zero_traces_batch(int dim, int q, const BatchDG<T> *D, int count, cudaStream_t s);
 
 // CG kernels (cg.cu)
 template <typename T>

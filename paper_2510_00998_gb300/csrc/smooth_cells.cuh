@@ -537,7 +537,7 @@ __device__ __forceinline__ void stage_bulk(bool full, int lane, uint64_t *bar, T
 }
 
 template <typename T, int Q>
-__device__ __forceinline__ void smooth_cells_body(const DGConst<T> &c, int64_t cell0, T *__restrict__ u, const T *__restrict__ b, const T *__restrict__ kappa, const T *__restrict__ fd, const T *__restrict__ linv, const T *__restrict__ tr_in, T *__restrict__ tr_out, bool reuse = false) {
+__device__ __forceinline__ void smooth_cells_body(const DGConst<T> &c, int64_t cell0, int flags, T *__restrict__ u, const T *__restrict__ b, const T *__restrict__ kappa, const T *__restrict__ fd, const T *__restrict__ linv, const T *__restrict__ tr_in, T *__restrict__ tr_out, bool reuse = false) {
     using G = CellGeo<T, Q>;
     constexpr int W = G::W, NL = G::NL, FDS = G::FDS, TR = G::TR, FS = G::FS;
     extern __shared__ __align__(128) unsigned char smem_c[];
@@ -573,7 +573,12 @@ __device__ __forceinline__ void smooth_cells_body(const DGConst<T> &c, int64_t c
         mask = interior_mask<3>(ci, c.n);
     }
     const int s1 = c.n[0], s2 = c.n[0] * c.n[1];
-    if (!G::LEAN) stage_face<T, Q>(0, cell_neighbour(0, mask, cell, s1, s2), lane, tr_in, sB, &bars[4]);
+    // from a zero iterate there are no facet terms: the factors at once
+    const bool zero = (flags & SM_ZERO) != 0;
+    if (zero)
+        stage_bulk<T>(full, lane, &bars[2], sB, fd + cell0 * 3 * FDS, W * 3 * FDS, ncl * 3 * FDS);
+    else if (!G::LEAN)
+        stage_face<T, Q>(0, cell_neighbour(0, mask, cell, s1, s2), lane, tr_in, sB, &bars[4]);
 
     // r = b
     if (full)
@@ -588,12 +593,13 @@ __device__ __forceinline__ void smooth_cells_body(const DGConst<T> &c, int64_t c
     // area A is free: FP32 the second neighbour face, FP64 the factors
     if (G::LEAN)
         stage_bulk<T>(full, lane, &bars[1], sA, fd + cell0 * 3 * FDS, W * 3 * FDS, ncl * 3 * FDS);
-    else
+    else if (!zero)
         stage_face<T, Q>(1, cell_neighbour(1, mask, cell, s1, s2), lane, tr_in, sA, &bars[5]);
 
     // r -= N u_nb: the two faces normal to axis p, then rotate the next axis to x
+    // (three rotations are none)
 #pragma unroll 1
-    for (int p = 0; p < 3; ++p) {
+    for (int p = 0; p < 3 && !zero; ++p) {
         T dv[Q];
         const int ta = p == 2 ? 0 : p + 1, tb = p == 0 ? 2 : p - 1;
         const int sa = p == 1 ? Q : 1, sb = p == 1 ? 1 : Q;   // the y faces are stored transposed
@@ -628,7 +634,7 @@ __device__ __forceinline__ void smooth_cells_body(const DGConst<T> &c, int64_t c
     }
     // FP32: the previous u into area A (face slot 1 is free now; u is first
     // needed after the inverse)
-    if (!G::LEAN) {
+    if (!G::LEAN && !zero) {
         fence_proxy_async_smem();
         __syncwarp();
         stage_bulk<T>(full, lane, &bars[1], sA, u + cell0 * NL, W * NL, ncl * NL);
@@ -658,7 +664,7 @@ __device__ __forceinline__ void smooth_cells_body(const DGConst<T> &c, int64_t c
     // u <- (1 - w) u + w y (w already in y when the inverse came from the table),
     // stored through area A (the barrier also ends every lane's reads of the
     // factors before area A (FP64) or B (FP32) is rewritten)
-    if (!G::LEAN && full)
+    if (!G::LEAN && full && !zero)
         ok = warp_wait_copies(&bars[1], lane) && ok;
     else
         __syncwarp();
@@ -666,7 +672,10 @@ __device__ __forceinline__ void smooth_cells_body(const DGConst<T> &c, int64_t c
     if (active) {
         const T om = c.omega, keep = T(1) - om;
         const T *uo = G::LEAN ? u + cell * NL : sA + lane * NL;
-        if (table) {
+        if (zero) {
+#pragma unroll
+            for (int e = 0; e < NL; ++e) R[e] = om * R[e];
+        } else if (table) {
 #pragma unroll
             for (int e = 0; e < NL; ++e) R[e] = keep * uo[e] + R[e];
         } else {
@@ -691,7 +700,7 @@ __device__ __forceinline__ void smooth_cells_body(const DGConst<T> &c, int64_t c
         }
         __syncwarp();
         // traces of the new iterate (FP32: slots in areas B and A)
-        cells_write_traces<T, Q>(c, R, lane, active, cell, sB, sA, tr_out);
+        if (!(flags & SM_NO_TRACES)) cells_write_traces<T, Q>(c, R, lane, active, cell, sB, sA, tr_out);
     }
     bulk_wait_read_all();
 }
@@ -1161,11 +1170,11 @@ __global__ void __launch_bounds__(32) k_residual_cells_direct(const __grid_const
 }
 
 template <typename T, int Q>
-__global__ void __launch_bounds__(32) k_smooth_cells(const __grid_constant__ DGConst<T> c, T *__restrict__ u,
+__global__ void __launch_bounds__(32) k_smooth_cells(const __grid_constant__ DGConst<T> c, int flags, T *__restrict__ u,
                                                      const T *__restrict__ b, const T *__restrict__ kappa,
                                                      const T *__restrict__ fd, const T *__restrict__ linv,
                                                      const T *__restrict__ tr_in, T *__restrict__ tr_out) {
-    smooth_cells_body<T, Q>(c, (int64_t)blockIdx.x * CellGeo<T, Q>::W, u, b, kappa, fd, linv, tr_in, tr_out);
+    smooth_cells_body<T, Q>(c, (int64_t)blockIdx.x * CellGeo<T, Q>::W, flags, u, b, kappa, fd, linv, tr_in, tr_out);
 }
 
 // Host-side read of the timeout counter of this translation unit.
