@@ -423,8 +423,8 @@ int compute_factors(dgmg_ctx &C, const DGSpace &S, DGDev<T> &D, const double *fd
 // taken from them: the table of inverse eigenvalue sums, then S as limbs in place.
 int finish_factors(dgmg_ctx &C, const DGSpace &S, DGDev<double> &D, cudaStream_t s) {
     if (!D.fd) return DGMG_OK;
-    LC(launch_fx_table(C.dim, S.q, C.ncell, D.fd, C.opts.omega_dg, D.linv, s));
-    LC(launch_fx_factors(C.dim, S.q, C.ncell, D.fd, C.opts.omega_dg, s));
+    // (the level's corner sums, written anew by every residual, are the scratch)
+    LC(launch_fx_factors(C.dim, S.q, C.ncell, D.fd, C.opts.omega_dg, D.linv, reinterpret_cast<int *>(D.corners), s));
     return DGMG_OK;
 }
 

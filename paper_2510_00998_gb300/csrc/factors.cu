@@ -126,22 +126,28 @@ __global__ void __launch_bounds__(128) k_fd_factors(const __grid_constant__ FDIn
     for (int i = 0; i < q; ++i) out[q * q + i] = (T)lam[i];
 }
 
-// Unit of a cell's table of omega / (sum of eigenvalues): its largest entry (the
-// smallest eigenvalue of every axis) stays below 2^62.
-__device__ int table_unit(int dim, int q, const double *f, double omega) {
+// Largest biased exponent that an entry omega / (sum of eigenvalues) of a cell's table
+// can have, from the smallest eigenvalue of every axis (positive FP64 numbers are
+// ordered as their bits); one thread per cell
+__global__ void k_fx_table_unit(int dim, int q, int64_t ncell, const double *__restrict__ fd, double omega,
+                                int *__restrict__ unit) {
+    const int64_t cell = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (cell >= ncell) return;
+    const int fds = q * q + q;
     double s = 0.0;
     for (int a = 0; a < dim; ++a) {
-        double m = f[a * (q * q + q)];
-        for (int i = 1; i < q; ++i) m = fmin(m, f[a * (q * q + q) + i]);
-        s += m;
+        const double *f = fd + (cell * dim + a) * fds + q * q;
+        long long m = __double_as_longlong(f[0]);
+        for (int i = 1; i < q; ++i) m = min(m, __double_as_longlong(f[i]));
+        s += __longlong_as_double(m);
     }
-    return ilogb(omega / s) - 61;
+    unit[cell] = ilogb(omega) - ilogb(s) + 1 + 1023;
 }
 
-// The inverse eigenvalue sums of every cell with the smoother's damping folded in,
-// as 64-bit integers of the cell's unit
+// The inverse eigenvalue sums of every cell with the smoother's damping folded in, as
+// 64-bit integers below 2^62 of the cell's unit
 __global__ void k_fx_table(int dim, int q, int64_t ncell, const double *__restrict__ fd, double omega,
-                           long long *__restrict__ linv) {
+                           const int *__restrict__ unit, long long *__restrict__ linv) {
     const int64_t nloc = dim == 3 ? (int64_t)q * q * q : (int64_t)q * q;
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= ncell * nloc) return;
@@ -150,35 +156,30 @@ __global__ void k_fx_table(int dim, int q, int64_t ncell, const double *__restri
     const double *f = fd + cell * dim * fds + q * q;
     double s = f[node % q] + f[fds + (node / q) % q];
     if (dim == 3) s += f[2 * fds + node / (q * q)];
-    linv[idx] = llrint(ldexp(omega / s, -table_unit(dim, q, f, omega)));
+    linv[idx] = fx_from(omega / s, unit[cell]) << 2;
 }
 
 // fd in place: S of every axis as limbs of one unit (every row and column sum of
 // the magnitudes below 2^62), the unit in the word after it, and in the word after
-// axis 0's the unit of the table; one thread per cell
-__global__ void k_fx_factors(int dim, int q, int64_t ncell, double *__restrict__ fd, double omega) {
-    const int64_t cell = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (cell >= ncell) return;
-    const int fds = q * q + q;
-    double *f = fd + cell * dim * fds;
-    const int el = table_unit(dim, q, f + q * q, omega);
-    for (int a = 0; a < dim; ++a) {
-        double *S = f + a * fds;
-        Limb *out = reinterpret_cast<Limb *>(S);
-        double top = 0.0;
-        for (int i = 0; i < q; ++i) {
-            double rs = 0.0, cs = 0.0;
-            for (int j = 0; j < q; ++j) {
-                rs += fabs(S[i * q + j]);
-                cs += fabs(S[j * q + i]);
-            }
-            top = fmax(top, fmax(rs, cs));
+// axis 0's the unit of the table; one thread per cell and axis
+__global__ void k_fx_factors(int dim, int q, int64_t ncell, double *__restrict__ fd, const int *__restrict__ unit) {
+    const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (id >= ncell * dim) return;
+    double *S = fd + id * (q * q + q);
+    Limb *out = reinterpret_cast<Limb *>(S);
+    double top = 0.0;
+    for (int i = 0; i < q; ++i) {
+        double rs = 0.0, cs = 0.0;
+        for (int j = 0; j < q; ++j) {
+            rs += fabs(S[i * q + j]);
+            cs += fabs(S[j * q + i]);
         }
-        const int e = ilogb(top) - 61;
-        for (int i = 0; i < q * q; ++i) out[i] = limb_of(llrint(ldexp(S[i], -e)));
-        out[q * q] = Limb{e, 0};
-        if (a == 0) out[q * q + 1] = Limb{el, 0};
+        top = fmax(top, fmax(rs, cs));
     }
+    const int ev = ilogb(top) + 1023;
+    for (int i = 0; i < q * q; ++i) out[i] = limb_of(fx_from(S[i], ev) << 2);
+    out[q * q] = Limb{fx_unit(ev) - 2, 0};
+    if (id % dim == 0) out[q * q + 1] = Limb{fx_unit(unit[id / dim]) - 2, 0};
 }
 
 // kfac[cell][f]: the harmonic mean of kappa across face f (0 on the boundary),
@@ -233,20 +234,15 @@ cudaError_t launch_fd_factors(const FDInput &in, const double *kappa, int64_t nc
 template cudaError_t launch_fd_factors<double>(const FDInput &, const double *, int64_t, double *, cudaStream_t);
 template cudaError_t launch_fd_factors<float>(const FDInput &, const double *, int64_t, float *, cudaStream_t);
 
-cudaError_t launch_fx_table(int dim, int q, int64_t ncell, const double *fd, double omega, double *linv,
-                            cudaStream_t s) {
-    const int64_t n = ncell * (dim == 3 ? (int64_t)q * q * q : (int64_t)q * q);
-    if (n == 0) return cudaSuccess;
-    count_launches(1);
-    k_fx_table<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(dim, q, ncell, fd, omega,
-                                                           reinterpret_cast<long long *>(linv));
-    return cudaGetLastError();
-}
-
-cudaError_t launch_fx_factors(int dim, int q, int64_t ncell, double *fd, double omega, cudaStream_t s) {
+cudaError_t launch_fx_factors(int dim, int q, int64_t ncell, double *fd, double omega, double *linv, int *unit,
+                              cudaStream_t s) {
+    const int64_t nodes = ncell * (dim == 3 ? (int64_t)q * q * q : (int64_t)q * q);
     if (ncell == 0) return cudaSuccess;
-    count_launches(1);
-    k_fx_factors<<<(unsigned)((ncell + 127) / 128), 128, 0, s>>>(dim, q, ncell, fd, omega);
+    count_launches(3);
+    k_fx_table_unit<<<(unsigned)((ncell + 127) / 128), 128, 0, s>>>(dim, q, ncell, fd, omega, unit);
+    k_fx_table<<<(unsigned)((nodes + 255) / 256), 256, 0, s>>>(dim, q, ncell, fd, omega, unit,
+                                                               reinterpret_cast<long long *>(linv));
+    k_fx_factors<<<(unsigned)((ncell * dim + 127) / 128), 128, 0, s>>>(dim, q, ncell, fd, unit);
     return cudaGetLastError();
 }
 

@@ -161,10 +161,9 @@ struct FxRun {
 // linv[cell][node] = omega / (sum of the cell's eigenvalues) as 64-bit integers of
 // one exponent per cell, from the FP64 factors [S | lambda]; then, in place, the
 // factors as limbs: per axis S, its exponent in the word after it (h of a Limb);
-// the word after axis 0's exponent holds the table's.
-cudaError_t launch_fx_table(int dim, int q, int64_t ncell, const double *fd, double omega, double *linv,
-                            cudaStream_t s);
-cudaError_t launch_fx_factors(int dim, int q, int64_t ncell, double *fd, double omega, cudaStream_t s);
+// the word after axis 0's exponent holds the table's. unit: scratch, one per cell.
+cudaError_t launch_fx_factors(int dim, int q, int64_t ncell, double *fd, double omega, double *linv, int *unit,
+                              cudaStream_t s);
 
 // Q1 level description for the CG kernels.
 template <typename T>
