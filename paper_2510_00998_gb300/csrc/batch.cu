@@ -46,34 +46,86 @@ constexpr int BATCH_ALIGN_CELLS = 32;   // one CTA of the one-thread-per-cell sm
 // Per-problem CG: every problem runs its own conjugate-gradient recurrence
 // (its own alpha and beta); a problem whose residual met its bound is frozen
 // (active = 0) and its x, r and p are left untouched.
-constexpr int SEG_BLOCKS = 16;   // CTAs per problem of the segmented kernels
+// CTAs per problem of the segmented kernels: a batch of three problems still covers
+// the SMs, and the partial sums of 256 fit a few kilobytes
+constexpr int SEG_BLOCKS = 64, SEG_THREADS = 256;
 
-// part[i][blockIdx.x] = partial sum of a*b over problem i = blockIdx.y
+// 16 bytes of a vector at a time. Products and sums are FP64 in both precisions.
 template <typename T>
-__global__ void k_seg_dot_partial(const int64_t *__restrict__ off, const int64_t *__restrict__ len,
-                                  const T *__restrict__ a, const T *__restrict__ b, double *__restrict__ part) {
-    __shared__ double red[256];
-    const int i = blockIdx.y;
-    const int64_t o = off[i], n = len[i];
-    double s = 0.0;
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
-        s += (double)a[o + k] * (double)b[o + k];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) part[(int64_t)i * SEG_BLOCKS + blockIdx.x] = red[0];
+struct SegVec;
+template <>
+struct SegVec<float> {
+    using type = float4;
+    static constexpr int N = 4;
+};
+template <>
+struct SegVec<double> {
+    using type = double2;
+    static constexpr int N = 2;
+};
+template <typename T>
+__device__ __forceinline__ void seg_load(const T *p, T *v) {
+    *reinterpret_cast<typename SegVec<T>::type *>(v) = *reinterpret_cast<const typename SegVec<T>::type *>(p);
+}
+template <typename T>
+__device__ __forceinline__ void seg_store(T *p, const T *v) {
+    *reinterpret_cast<typename SegVec<T>::type *>(p) = *reinterpret_cast<const typename SegVec<T>::type *>(v);
 }
 
-// out[i] = sum of the SEG_BLOCKS partials of problem i (fixed order)
-__global__ void k_seg_dot_final(int count, const double *__restrict__ part, double *__restrict__ out) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= count) return;
+// the CTA's sum of v in thread 0, fixed order
+__device__ __forceinline__ double seg_block_sum(double v) {
+    __shared__ double red[SEG_THREADS / 32];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
     double s = 0.0;
-    for (int k = 0; k < SEG_BLOCKS; ++k) s += part[(int64_t)i * SEG_BLOCKS + k];
-    out[i] = s;
+    if (threadIdx.x == 0)
+        for (int w = 0; w < SEG_THREADS / 32; ++w) s += red[w];
+    return s;
+}
+
+// part[i][blockIdx.x] = partial sum of a.b over problem i = blockIdx.y, and with W = 2
+// part[count + i][...] that of c.b (b read once). The slices start on 16 bytes (a
+// multiple of 32 cells); two independent sums per product hide the FP64 latency.
+template <typename T, int W>
+__global__ void __launch_bounds__(SEG_THREADS) k_seg_dot_partial(const int64_t *__restrict__ off,
+                                                                 const int64_t *__restrict__ len,
+                                                                 const T *__restrict__ a, const T *__restrict__ b,
+                                                                 const T *__restrict__ c, double *__restrict__ part) {
+    constexpr int V = SegVec<T>::N;
+    const int i = blockIdx.y;
+    const int64_t o = off[i], n = len[i], nv = n / V, stride = (int64_t)gridDim.x * blockDim.x;
+    double s[W][2] = {};
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < nv; k += stride) {
+        T x[W][V], y[V];
+        seg_load<T>(b + o + k * V, y);
+        seg_load<T>(a + o + k * V, x[0]);
+        if constexpr (W == 2) seg_load<T>(c + o + k * V, x[1]);
+#pragma unroll
+        for (int w = 0; w < W; ++w)
+#pragma unroll
+            for (int e = 0; e < V; ++e) s[w][e & 1] = fma((double)x[w][e], (double)y[e], s[w][e & 1]);
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        for (int64_t k = nv * V; k < n; ++k) {
+            s[0][0] = fma((double)a[o + k], (double)b[o + k], s[0][0]);
+            if constexpr (W == 2) s[1][0] = fma((double)c[o + k], (double)b[o + k], s[1][0]);
+        }
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+        const double v = seg_block_sum(s[w][0] + s[w][1]);
+        if (threadIdx.x == 0) part[((int64_t)w * gridDim.y + i) * SEG_BLOCKS + blockIdx.x] = v;
+    }
+}
+
+// out[i] = sum of the SEG_BLOCKS partials of row i (fixed order); one warp per row
+__global__ void k_seg_dot_final(int rows, const double *__restrict__ part, double *__restrict__ out) {
+    const int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (i >= rows) return;
+    double s = part[(int64_t)i * SEG_BLOCKS + lane] + part[(int64_t)i * SEG_BLOCKS + 32 + lane];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) out[i] = s;
 }
 
 // active problems: beta = <r,z>_new / <r,z>; <r,z> <- <r,z>_new
@@ -106,49 +158,80 @@ __global__ void k_seg_beta_flex(int count, const int *__restrict__ active, doubl
 
 // active problems: p = z + beta p
 template <typename T>
-__global__ void k_seg_update_p(const int64_t *__restrict__ off, const int64_t *__restrict__ len,
-                               const int *__restrict__ active, const double *__restrict__ beta, T *__restrict__ p,
-                               const T *__restrict__ z) {
+__global__ void __launch_bounds__(SEG_THREADS) k_seg_update_p(const int64_t *__restrict__ off,
+                                                              const int64_t *__restrict__ len,
+                                                              const int *__restrict__ active,
+                                                              const double *__restrict__ beta, T *__restrict__ p,
+                                                              const T *__restrict__ z) {
+    constexpr int V = SegVec<T>::N;
     const int i = blockIdx.y;
     if (!active[i]) return;
-    const int64_t o = off[i], n = len[i];
+    const int64_t o = off[i], n = len[i], nv = n / V;
     const T bt = (T)beta[i];
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
-        p[o + k] = z[o + k] + bt * p[o + k];
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < nv; k += (int64_t)gridDim.x * blockDim.x) {
+        T pv[V], zv[V];
+        seg_load<T>(p + o + k * V, pv);
+        seg_load<T>(z + o + k * V, zv);
+#pragma unroll
+        for (int e = 0; e < V; ++e) pv[e] = zv[e] + bt * pv[e];
+        seg_store<T>(p + o + k * V, pv);
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        for (int64_t k = o + nv * V; k < o + n; ++k) p[k] = z[k] + bt * p[k];
 }
 
-// active problems: alpha = <r,z> / <p,q>; x += alpha p; r -= alpha q
-__global__ void k_seg_update_xr(const int64_t *__restrict__ off, const int64_t *__restrict__ len,
-                                const int *__restrict__ active, const double *__restrict__ rz,
-                                const double *__restrict__ pq, double *__restrict__ x, double *__restrict__ r,
-                                const double *__restrict__ p, const double *__restrict__ q) {
+// Active problems: alpha = <r,z> / <p,q>; x += alpha p; r -= alpha q (and, FP32 with
+// rold, r_old = r); every problem: the partial sums of ||r||^2 of the new r in the
+// same pass.
+template <typename T>
+__global__ void __launch_bounds__(SEG_THREADS) k_seg_update_xr(const int64_t *__restrict__ off,
+                                                               const int64_t *__restrict__ len,
+                                                               const int *__restrict__ active,
+                                                               const double *__restrict__ rz,
+                                                               const double *__restrict__ pq, T *__restrict__ x,
+                                                               T *__restrict__ r, T *__restrict__ rold,
+                                                               const T *__restrict__ p, const T *__restrict__ q,
+                                                               double *__restrict__ part) {
+    constexpr int V = SegVec<T>::N;
     const int i = blockIdx.y;
-    if (!active[i]) return;
-    const int64_t o = off[i], n = len[i];
-    const double alpha = rz[i] / pq[i];
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
-        x[o + k] += alpha * p[o + k];
-        r[o + k] -= alpha * q[o + k];
+    const bool act = active[i] != 0;
+    const int64_t o = off[i], n = len[i], nv = n / V, stride = (int64_t)gridDim.x * blockDim.x;
+    const T alpha = act ? (T)(rz[i] / pq[i]) : T(0);
+    double s[2] = {};
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < nv; k += stride) {
+        const int64_t at = o + k * V;
+        T rv[V];
+        seg_load<T>(r + at, rv);
+        if (act) {
+            T xv[V], pv[V], qv[V];
+            seg_load<T>(x + at, xv);
+            seg_load<T>(p + at, pv);
+            seg_load<T>(q + at, qv);
+            if (rold) seg_store<T>(rold + at, rv);
+#pragma unroll
+            for (int e = 0; e < V; ++e) {
+                xv[e] += alpha * pv[e];
+                rv[e] -= alpha * qv[e];
+            }
+            seg_store<T>(x + at, xv);
+            seg_store<T>(r + at, rv);
+        }
+#pragma unroll
+        for (int e = 0; e < V; ++e) s[e & 1] = fma((double)rv[e], (double)rv[e], s[e & 1]);
     }
-}
-
-// Mixed precision (reliable updates), active problems: alpha = <r,z> / <p,q>;
-// xs += alpha p; r_old = r; r -= alpha q, all FP32
-__global__ void k_seg_update_xr32(const int64_t *__restrict__ off, const int64_t *__restrict__ len,
-                                  const int *__restrict__ active, const double *__restrict__ rz,
-                                  const double *__restrict__ pq, float *__restrict__ xs, float *__restrict__ r,
-                                  float *__restrict__ rold, const float *__restrict__ p,
-                                  const float *__restrict__ q) {
-    const int i = blockIdx.y;
-    if (!active[i]) return;
-    const int64_t o = off[i], n = len[i];
-    const float alpha = (float)(rz[i] / pq[i]);
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
-        const float ri = r[o + k];
-        rold[o + k] = ri;
-        xs[o + k] += alpha * p[o + k];
-        r[o + k] = ri - alpha * q[o + k];
-    }
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        for (int64_t k = o + nv * V; k < o + n; ++k) {
+            T rk = r[k];
+            if (act) {
+                if (rold) rold[k] = rk;
+                x[k] += alpha * p[k];
+                rk -= alpha * q[k];
+                r[k] = rk;
+            }
+            s[0] = fma((double)rk, (double)rk, s[0]);
+        }
+    const double v = seg_block_sum(s[0] + s[1]);
+    if (threadIdx.x == 0) part[(int64_t)i * SEG_BLOCKS + blockIdx.x] = v;
 }
 
 // x += xs (FP64 accumulation of the FP32 correction), xs = 0, whole batch
@@ -459,19 +542,40 @@ int batch_vcycle(dgmg_batch &B, const T *r, T *z, cudaStream_t s) {
 
 unsigned small_grid(int count) { return (unsigned)((count + 127) / 128); }
 
-// out[i] = <a_i, b_i> for every problem (deterministic: fixed partial order; FP64 sums)
-template <typename T>
-int seg_dot(dgmg_batch &B, const T *a, const T *b, double *out, cudaStream_t s) {
-    count_launches(2);
-    k_seg_dot_partial<T><<<dim3(SEG_BLOCKS, B.count), 256, 0, s>>>(B.d_off, B.d_len, a, b, B.part);
-    k_seg_dot_final<<<small_grid(B.count), 128, 0, s>>>(B.count, B.part, out);
+// the rows of partial sums in B.part to out, one warp each
+int seg_final(dgmg_batch &B, int rows, double *out, cudaStream_t s) {
+    count_launches(1);
+    k_seg_dot_final<<<(unsigned)((rows + 3) / 4), 128, 0, s>>>(rows, B.part, out);
     LC(cudaGetLastError());
     return DGMG_OK;
 }
 
-// ||v_i||^2 of every problem to the host (pinned) and the active flags
-int batch_norms(dgmg_batch &B, const double *v, cudaStream_t s) {
-    RC(seg_dot(B, v, v, B.d_norm, s));
+// out[i] = <a_i, b_i> for every problem (deterministic: fixed partial order; FP64
+// sums); with c also out[count + i] = <c_i, b_i>
+template <typename T>
+int seg_dot(dgmg_batch &B, const T *a, const T *b, double *out, cudaStream_t s, const T *c = nullptr) {
+    count_launches(1);
+    const dim3 grid(SEG_BLOCKS, B.count);
+    if (c)
+        k_seg_dot_partial<T, 2><<<grid, SEG_THREADS, 0, s>>>(B.d_off, B.d_len, a, b, c, B.part);
+    else
+        k_seg_dot_partial<T, 1><<<grid, SEG_THREADS, 0, s>>>(B.d_off, B.d_len, a, b, c, B.part);
+    LC(cudaGetLastError());
+    return seg_final(B, (c ? 2 : 1) * B.count, out, s);
+}
+
+// x += alpha p, r -= alpha q of the active problems and ||r_i||^2 of all of them
+template <typename T>
+int seg_update_xr(dgmg_batch &B, T *x, T *r, T *rold, const T *p, const T *q, cudaStream_t s) {
+    count_launches(1);
+    k_seg_update_xr<T><<<dim3(SEG_BLOCKS, B.count), SEG_THREADS, 0, s>>>(B.d_off, B.d_len, B.active, B.rz, B.pq, x, r,
+                                                                          rold, p, q, B.part);
+    LC(cudaGetLastError());
+    return seg_final(B, B.count, B.d_norm, s);
+}
+
+// the norms in B.d_norm to the host (pinned) and the active flags
+int post_norms(dgmg_batch &B, cudaStream_t s) {
     count_launches(1);
     k_seg_flags<<<small_grid(B.count), 128, 0, s>>>(B.count, B.d_norm, B.d_bb, B.opts.rtol * B.opts.rtol, B.active);
     LC(cudaGetLastError());
@@ -479,16 +583,19 @@ int batch_norms(dgmg_batch &B, const double *v, cudaStream_t s) {
     return DGMG_OK;
 }
 
+// ||v_i||^2 of every problem, to the host, and the active flags
+int batch_norms(dgmg_batch &B, const double *v, cudaStream_t s) {
+    RC(seg_dot(B, v, v, B.d_norm, s));
+    return post_norms(B, s);
+}
+
 // FP64: alpha step of every active problem: q = A p, <p,q>, x += alpha p,
 // r -= alpha q, then ||r_i||^2 and the flags
 int alpha_step(dgmg_batch &B, cudaStream_t s) {
     RC(batch_apply(B, B.p, nullptr, B.q, s));
     RC(seg_dot<double>(B, B.p, B.q, B.pq, s));
-    count_launches(1);
-    k_seg_update_xr<<<dim3(SEG_BLOCKS * 4, B.count), 256, 0, s>>>(B.d_off, B.d_len, B.active, B.rz, B.pq, B.x,
-                                                                    B.r, B.p, B.q);
-    LC(cudaGetLastError());
-    return batch_norms(B, B.r, s);
+    RC(seg_update_xr<double>(B, B.x, B.r, nullptr, B.p, B.q, s));
+    return post_norms(B, s);
 }
 
 // One iteration of every active problem. FP64: z = V(r), beta, p = z + beta p,
@@ -502,26 +609,21 @@ int batch_iteration(dgmg_batch &B, cudaStream_t s) {
         RC(seg_dot<double>(B, B.r, B.z, B.rzn, s));
         count_launches(2);
         k_seg_beta<<<small_grid(B.count), 128, 0, s>>>(B.count, B.active, B.rz, B.rzn, B.beta);
-        k_seg_update_p<double><<<dim3(SEG_BLOCKS * 4, B.count), 256, 0, s>>>(B.d_off, B.d_len, B.active, B.beta,
+        k_seg_update_p<double><<<dim3(SEG_BLOCKS, B.count), SEG_THREADS, 0, s>>>(B.d_off, B.d_len, B.active, B.beta,
                                                                               B.p, B.z);
         LC(cudaGetLastError());
         return alpha_step(B, s);
     }
     RC(batch_vcycle<float>(B, B.r32, B.z32, s));
-    RC(seg_dot<float>(B, B.r32, B.z32, B.rzn, s));
-    RC(seg_dot<float>(B, B.rold32, B.z32, B.rzo, s));
+    RC(seg_dot<float>(B, B.r32, B.z32, B.rzn, s, B.rold32));   // and <r_old, z> into rzo, the row after rzn
     count_launches(2);
     k_seg_beta_flex<<<small_grid(B.count), 128, 0, s>>>(B.count, B.active, B.rz, B.rzn, B.rzo, B.beta);
-    k_seg_update_p<float><<<dim3(SEG_BLOCKS * 4, B.count), 256, 0, s>>>(B.d_off, B.d_len, B.active, B.beta, B.p32,
+    k_seg_update_p<float><<<dim3(SEG_BLOCKS, B.count), SEG_THREADS, 0, s>>>(B.d_off, B.d_len, B.active, B.beta, B.p32,
                                                                          B.z32);
     LC(cudaGetLastError());
     RC(batch_apply32(B, B.p32, B.q32, s));
     RC(seg_dot<float>(B, B.p32, B.q32, B.pq, s));
-    count_launches(1);
-    k_seg_update_xr32<<<dim3(SEG_BLOCKS * 4, B.count), 256, 0, s>>>(B.d_off, B.d_len, B.active, B.rz, B.pq,
-                                                                      B.xs32, B.r32, B.rold32, B.p32, B.q32);
-    LC(cudaGetLastError());
-    RC(seg_dot<float>(B, B.r32, B.r32, B.d_norm, s));
+    RC(seg_update_xr<float>(B, B.xs32, B.r32, B.rold32, B.p32, B.q32, s));
     LC(cudaMemcpyAsync(B.h_norm, B.d_norm, sizeof(double) * B.count, cudaMemcpyDeviceToHost, s));
     return DGMG_OK;
 }
@@ -774,15 +876,16 @@ int dgmg_batch_create(int count, const dgmg_mesh *meshes, const int *p, const do
     }
     RC(B->upload(&B->d_off, B->dof_off));
     RC(B->upload(&B->d_len, B->dof_len));
-    for (double **v : {&B->d_norm, &B->d_bb, &B->rz, &B->rzn, &B->pq, &B->beta}) RC(B->alloc(v, count));
-    RC(B->alloc(&B->part, (size_t)count * SEG_BLOCKS));
+    for (double **v : {&B->d_norm, &B->d_bb, &B->rz, &B->pq, &B->beta}) RC(B->alloc(v, count));
+    RC(B->alloc(&B->rzn, 2 * (size_t)count));      // <r, z> of the new residual, <r_old, z>
+    B->rzo = B->rzn + count;
+    RC(B->alloc(&B->part, 2 * (size_t)count * SEG_BLOCKS));
     RC(B->alloc(&B->active, count));
     if (B->mixed) {
         for (float **v : {&B->r32, &B->z32, &B->p32, &B->q32, &B->xs32, &B->rold32}) {
             RC(B->alloc(v, B->ndof));
             LC(cudaMemset(*v, 0, sizeof(float) * B->ndof));
         }
-        RC(B->alloc(&B->rzo, count));
     }
     LC(cudaMallocHost((void **)&B->h_norm, sizeof(double) * count));
     LC(cudaEventCreateWithFlags(&B->ev, cudaEventDisableTiming));
@@ -874,11 +977,7 @@ int dgmg_batch_solve(dgmg_batch *B, const double *const *b, double *const *x, dg
         LC(cudaMemcpyAsync(B->p32, B->z32, sizeof(float) * B->ndof, cudaMemcpyDeviceToDevice, s));
         RC(batch_apply32(*B, B->p32, B->q32, s));
         RC(seg_dot<float>(*B, B->p32, B->q32, B->pq, s));
-        count_launches(1);
-        k_seg_update_xr32<<<dim3(SEG_BLOCKS * 4, n), 256, 0, s>>>(B->d_off, B->d_len, B->active, B->rz, B->pq,
-                                                                    B->xs32, B->r32, B->rold32, B->p32, B->q32);
-        LC(cudaGetLastError());
-        RC(seg_dot<float>(*B, B->r32, B->r32, B->d_norm, s));
+        RC(seg_update_xr<float>(*B, B->xs32, B->r32, B->rold32, B->p32, B->q32, s));
         LC(cudaMemcpyAsync(B->h_norm, B->d_norm, sizeof(double) * n, cudaMemcpyDeviceToHost, s));
         std::vector<int> act(n);
         for (int i = 0; i < n; ++i) act[i] = rel[i] > B->opts.rtol;
