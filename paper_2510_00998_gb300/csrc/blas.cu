@@ -1,10 +1,11 @@
-// FP64 vector kernels of the outer conjugate-gradient loop: deterministic
-// two-stage dot products (fixed grid, fixed reduction order), the CG updates
+// Vector kernels of the outer conjugate-gradient loop, FP64 and FP32: deterministic
+// dot products (grid a function of the length, fixed reduction order), the CG updates
 // with step lengths read from device memory, precision casts, and the
 // right-hand-side quadrature (b_i = (f, phi_i), the right-hand side of
 // Eq. weak_form_IP). The CG loop uses one multigrid cycle as its preconditioner
 // (P^-1 of Sec. 5.1 "Exit criterion").
 #include <algorithm>
+#include <type_traits>
 
 #include "internal.h"
 
@@ -25,89 +26,211 @@ __device__ __forceinline__ double block_sum(double v, double *sh) {
     return v;   // valid in thread 0
 }
 
-__global__ void k_dot_partial(int64_t n, const double *__restrict__ x, const double *__restrict__ y,
-                              double *__restrict__ partials) {
-    __shared__ double sh[32];
-    double s = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        s += x[i] * y[i];
-    s = block_sum(s, sh);
-    if (threadIdx.x == 0) partials[blockIdx.x] = s;
+// One vector load of 16 bytes, or (VEC = false: some vector is not 16-byte aligned)
+// one element.
+template <typename T, bool VEC>
+struct Pack {
+    static constexpr int N = VEC ? 16 / (int)sizeof(T) : 1;
+    alignas(VEC ? 16 : sizeof(T)) T v[N];
+    __device__ __forceinline__ void load(const T *p) {
+        if constexpr (VEC) {
+            using V = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
+            *reinterpret_cast<V *>(v) = *reinterpret_cast<const V *>(p);
+        } else {
+            v[0] = *p;
+        }
+    }
+    __device__ __forceinline__ void store(T *p) const {
+        if constexpr (VEC) {
+            using V = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
+            *reinterpret_cast<V *>(p) = *reinterpret_cast<const V *>(v);
+        } else {
+            *p = v[0];
+        }
+    }
+};
+
+// s += a.b of two packs, accumulated in FP64. FP32: the four products of a pack are
+// summed in FP32 (fused multiply-adds) first; such a group sum carries an error of a
+// few FP32 ulps of its terms, the order of the rounding of the vector entries
+// themselves. Single elements are multiplied in FP64.
+template <typename T, bool VEC>
+__device__ __forceinline__ void pack_dot(double &s, const Pack<T, VEC> &a, const Pack<T, VEC> &b) {
+    if constexpr (VEC && sizeof(T) == 4) {
+        s += (double)fmaf(a.v[3], b.v[3], fmaf(a.v[2], b.v[2], fmaf(a.v[1], b.v[1], a.v[0] * b.v[0])));
+    } else {
+#pragma unroll
+        for (int e = 0; e < Pack<T, VEC>::N; ++e) s = fma((double)a.v[e], (double)b.v[e], s);
+    }
 }
 
-// The same with 16-byte loads, two per vector in flight per thread (x, y
-// 16-byte aligned); the n % 2 tail goes to the last thread of the grid.
-__global__ void __launch_bounds__(DOT_THREADS) k_dot_partial_v(int64_t n, const double *__restrict__ x,
-                                                               const double *__restrict__ y,
-                                                               double *__restrict__ partials) {
+// The end of a dot product: every block stores its W partial sums; the block that
+// arrives last at the ticket (which wraps back to 0) adds them up in their fixed order
+// and writes out[0 .. W). One launch instead of two (a second kernel costs 3.7 us and
+// a launch gap). scal, when given: the CG direction update's beta from <r,z> = out[0]
+// (Fletcher-Reeves; with W = 2 Polak-Ribiere, out[1] = <r_old,z>) and the shift of <r,z>.
+template <int W>
+__device__ __forceinline__ void dot_finish(const double *s, double *partials, double *out0, double *out1, double *scal) {
     __shared__ double sh[32];
-    const double2 *x2 = reinterpret_cast<const double2 *>(x), *y2 = reinterpret_cast<const double2 *>(y);
-    const int64_t n2 = n >> 1, stride = (int64_t)gridDim.x * blockDim.x;
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    double s0 = 0.0, s1 = 0.0;
-    for (; i + stride < n2; i += 2 * stride) {
-        const double2 a = x2[i], b = y2[i], c = x2[i + stride], d = y2[i + stride];
-        s0 = fma(a.x, b.x, s0);
-        s0 = fma(a.y, b.y, s0);
-        s1 = fma(c.x, d.x, s1);
-        s1 = fma(c.y, d.y, s1);
+    __shared__ unsigned last;
+    double v[W];
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+        v[w] = block_sum(s[w], sh);
+        if (threadIdx.x == 0) partials[w * DOT_BLOCKS + blockIdx.x] = v[w];
+        __syncthreads();
     }
-    if (i < n2) {
-        const double2 a = x2[i], b = y2[i];
-        s0 = fma(a.x, b.x, s0);
-        s0 = fma(a.y, b.y, s0);
-    }
-    if ((n & 1) && blockIdx.x == gridDim.x - 1 && threadIdx.x == blockDim.x - 1) s1 = fma(x[n - 1], y[n - 1], s1);
-    const double s = block_sum(s0 + s1, sh);
-    if (threadIdx.x == 0) partials[blockIdx.x] = s;
-}
-
-__global__ void k_dot2_partial(int64_t n, const double *__restrict__ x, const double *__restrict__ y,
-                               const double *__restrict__ z, double *__restrict__ partials) {
-    __shared__ double sh[32];
-    double s = 0.0, t = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const double yi = y[i];
-        s += x[i] * yi;
-        t += z[i] * yi;
-    }
-    s = block_sum(s, sh);
-    __syncthreads();
-    t = block_sum(t, sh);
+    unsigned *ticket = reinterpret_cast<unsigned *>(partials + 2 * DOT_BLOCKS);
     if (threadIdx.x == 0) {
-        partials[blockIdx.x] = s;
-        partials[gridDim.x + blockIdx.x] = t;
+        __threadfence();
+        last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+        double t = 0.0;
+        for (unsigned i = threadIdx.x; i < gridDim.x; i += blockDim.x) t += __ldcg(partials + w * DOT_BLOCKS + i);
+        v[w] = block_sum(t, sh);
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        if (out0) *out0 = v[0];
+        if (W == 2 && out1) *out1 = v[W - 1];
+        if (scal) {
+            scal[2] = W == 2 ? (v[0] - v[W - 1]) / scal[0] : v[0] / scal[0];   // beta
+            scal[0] = v[0];                                                   // <r,z>
+        }
     }
 }
 
-__global__ void k_reduce(int np, const double *__restrict__ partials, double *__restrict__ out) {
-    __shared__ double sh[32];
-    double s = 0.0;
-    for (int i = threadIdx.x; i < np; i += blockDim.x) s += partials[i];
-    s = block_sum(s, sh);
-    if (threadIdx.x == 0) *out = s;
-}
-
-// slots of the scalar array used by the CG kernels
-__global__ void k_update_xr(int64_t n, double *__restrict__ x, double *__restrict__ r, const double *__restrict__ p,
-                            const double *__restrict__ q, const double *__restrict__ scal) {
-    const double alpha = scal[0] / scal[1];   // rz / pq
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        x[i] += alpha * p[i];
-        r[i] -= alpha * q[i];
+// out0 = a.b, and with W = 2 out1 = c.b (b read once). Four loads per vector in flight.
+template <typename T, int W, bool VEC>
+__global__ void __launch_bounds__(DOT_THREADS) k_dot(int64_t n, const T *__restrict__ a, const T *__restrict__ b,
+                                                     const T *__restrict__ c, double *__restrict__ partials, double *out0,
+                                                     double *out1, double *scal) {
+    using P = Pack<T, VEC>;
+    constexpr int U = 4;
+    const int64_t nv = n / P::N, stride = (int64_t)gridDim.x * blockDim.x;
+    double s[W] = {}, t[W] = {};
+    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    for (; i + (U - 1) * stride < nv; i += U * stride) {
+        P x[U], y[U], z[W == 2 ? U : 1];
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+            y[k].load(b + (i + k * stride) * P::N);
+            x[k].load(a + (i + k * stride) * P::N);
+            if constexpr (W == 2) z[k].load(c + (i + k * stride) * P::N);
+        }
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+            pack_dot<T, VEC>(k & 1 ? t[0] : s[0], x[k], y[k]);
+            if constexpr (W == 2) pack_dot<T, VEC>(k & 1 ? t[1] : s[1], z[k], y[k]);
+        }
     }
+    for (; i < nv; i += stride) {
+        P x, y;
+        y.load(b + i * P::N);
+        x.load(a + i * P::N);
+        pack_dot<T, VEC>(s[0], x, y);
+        if constexpr (W == 2) {
+            x.load(c + i * P::N);
+            pack_dot<T, VEC>(s[1], x, y);
+        }
+    }
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == blockDim.x - 1)
+        for (int64_t k = nv * P::N; k < n; ++k) {
+            s[0] = fma((double)a[k], (double)b[k], s[0]);
+            if constexpr (W == 2) s[1] = fma((double)c[k], (double)b[k], s[1]);
+        }
+#pragma unroll
+    for (int w = 0; w < W; ++w) s[w] += t[w];
+    dot_finish<W>(s, partials, out0, out1, scal);
 }
 
-__global__ void k_update_p(int64_t n, double *__restrict__ p, const double *__restrict__ z,
-                           const double *__restrict__ scal) {
-    const double beta = scal[2];
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        p[i] = z[i] + beta * p[i];
+// out0 = ||r||^2, out1 = ||x - y||^2 (the two norms of a stationary iteration)
+template <bool VEC>
+__global__ void __launch_bounds__(DOT_THREADS) k_norms(int64_t n, const double *__restrict__ r, const double *__restrict__ x,
+                                                       const double *__restrict__ y, double *__restrict__ partials,
+                                                       double *out0, double *out1) {
+    using P = Pack<double, VEC>;
+    const int64_t nv = n / P::N, stride = (int64_t)gridDim.x * blockDim.x;
+    double s[2] = {};
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nv; i += stride) {
+        P a, b, c;
+        a.load(r + i * P::N);
+        b.load(x + i * P::N);
+        c.load(y + i * P::N);
+        pack_dot<double, VEC>(s[0], a, a);
+#pragma unroll
+        for (int e = 0; e < P::N; ++e) b.v[e] -= c.v[e];
+        pack_dot<double, VEC>(s[1], b, b);
+    }
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == blockDim.x - 1)
+        for (int64_t k = nv * P::N; k < n; ++k) {
+            const double d = x[k] - y[k];
+            s[0] = fma(r[k], r[k], s[0]);
+            s[1] = fma(d, d, s[1]);
+        }
+    dot_finish<2>(s, partials, out0, out1, nullptr);
 }
 
-__global__ void k_sub(int64_t n, const double *__restrict__ a, const double *__restrict__ b, double *__restrict__ out) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = a[i] - b[i];
+// x += alpha p, r_old = r (when given), r -= alpha q, out = ||r||^2 of the new r in the
+// same pass; alpha = scal[0] / scal[1] = <r,z> / <p,q>
+template <typename T, bool VEC>
+__global__ void __launch_bounds__(DOT_THREADS) k_update_xr(int64_t n, T *__restrict__ x, T *__restrict__ r,
+                                                           T *__restrict__ rold, const T *__restrict__ p,
+                                                           const T *__restrict__ q, const double *__restrict__ scal,
+                                                           double *__restrict__ partials, double *out) {
+    using P = Pack<T, VEC>;
+    const T alpha = (T)(scal[0] / scal[1]);
+    const int64_t nv = n / P::N, stride = (int64_t)gridDim.x * blockDim.x;
+    double s[1] = {};
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nv; i += stride) {
+        P ri, pi, qi, xi;
+        ri.load(r + i * P::N);
+        pi.load(p + i * P::N);
+        qi.load(q + i * P::N);
+        xi.load(x + i * P::N);
+        if (rold) ri.store(rold + i * P::N);
+#pragma unroll
+        for (int e = 0; e < P::N; ++e) {
+            xi.v[e] = fma(alpha, pi.v[e], xi.v[e]);
+            ri.v[e] = fma(-alpha, qi.v[e], ri.v[e]);
+        }
+        xi.store(x + i * P::N);
+        ri.store(r + i * P::N);
+        pack_dot<T, VEC>(s[0], ri, ri);
+    }
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == blockDim.x - 1)
+        for (int64_t k = nv * P::N; k < n; ++k) {
+            const T ri = r[k], rn = fma(-alpha, q[k], ri);
+            if (rold) rold[k] = ri;
+            x[k] = fma(alpha, p[k], x[k]);
+            r[k] = rn;
+            s[0] = fma((double)rn, (double)rn, s[0]);
+        }
+    dot_finish<1>(s, partials, out, nullptr, nullptr);
+}
+
+// p = z + beta p, beta = scal[2]
+template <typename T, bool VEC>
+__global__ void __launch_bounds__(DOT_THREADS) k_update_p(int64_t n, T *__restrict__ p, const T *__restrict__ z,
+                                                          const double *__restrict__ scal) {
+    using P = Pack<T, VEC>;
+    const T beta = (T)scal[2];
+    const int64_t nv = n / P::N, stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nv; i += stride) {
+        P pi, zi;
+        pi.load(p + i * P::N);
+        zi.load(z + i * P::N);
+#pragma unroll
+        for (int e = 0; e < P::N; ++e) pi.v[e] = fma(beta, pi.v[e], zi.v[e]);
+        pi.store(p + i * P::N);
+    }
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == blockDim.x - 1)
+        for (int64_t k = nv * P::N; k < n; ++k) p[k] = fma(beta, p[k], z[k]);
 }
 
 __global__ void k_d2f(int64_t n, const double *__restrict__ x, float *__restrict__ y) {
@@ -118,155 +241,6 @@ __global__ void k_d2f(int64_t n, const double *__restrict__ x, float *__restrict
 __global__ void k_f2d(int64_t n, const float *__restrict__ x, double *__restrict__ y) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         y[i] = (double)x[i];
-}
-
-__global__ void k_copy_scalar(const double *src, double *dst) { *dst = *src; }
-
-// FP32 vectors with FP64 accumulation (the inner loop of the mixed solver)
-//
-// Vectorised form: 16-byte loads, two float4 per vector in flight per thread;
-// the four products of a float4 are summed in FP32 (fused multiply-adds) and
-// each such group sum is accumulated in FP64. A group sum carries an error of
-// a few FP32 ulps of its terms, the order of the FP32 rounding of the vector
-// entries themselves. The n % 4 tail goes to the last thread of the grid.
-__device__ __forceinline__ float dot4(const float4 a, const float4 b) {
-    return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, a.x * b.x)));
-}
-
-// partials[block] = sum x.y; with z: partials[gridDim + block] = sum z.y
-template <bool TWO>
-__global__ void __launch_bounds__(DOT_THREADS) k_dotf_partial_v(int64_t n, const float *__restrict__ x,
-                                                                const float *__restrict__ y,
-                                                                const float *__restrict__ z,
-                                                                double *__restrict__ partials) {
-    __shared__ double sh[32];
-    const float4 *x4 = reinterpret_cast<const float4 *>(x), *y4 = reinterpret_cast<const float4 *>(y);
-    const float4 *z4 = reinterpret_cast<const float4 *>(z);
-    const int64_t n4 = n >> 2, stride = (int64_t)gridDim.x * blockDim.x;
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    double s = 0.0, t = 0.0;
-    for (; i + stride < n4; i += 2 * stride) {
-        const float4 b0 = y4[i], b1 = y4[i + stride];
-        const float4 a0 = x4[i], a1 = x4[i + stride];
-        if (TWO) {
-            const float4 c0 = z4[i], c1 = z4[i + stride];
-            t += (double)dot4(c0, b0) + (double)dot4(c1, b1);
-        }
-        s += (double)dot4(a0, b0) + (double)dot4(a1, b1);
-    }
-    if (i < n4) {
-        const float4 b0 = y4[i];
-        s += (double)dot4(x4[i], b0);
-        if (TWO) t += (double)dot4(z4[i], b0);
-    }
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == blockDim.x - 1)
-        for (int64_t k = n4 << 2; k < n; ++k) {
-            s += (double)x[k] * (double)y[k];
-            if (TWO) t += (double)z[k] * (double)y[k];
-        }
-    s = block_sum(s, sh);
-    if (TWO) {
-        __syncthreads();
-        t = block_sum(t, sh);
-    }
-    if (threadIdx.x == 0) {
-        partials[blockIdx.x] = s;
-        if (TWO) partials[gridDim.x + blockIdx.x] = t;
-    }
-}
-
-// xs += alpha p, r -= alpha q, rold = old r, and partials[block] = sum of the
-// new r squared (the CG update and the residual norm in one pass; 16-byte
-// aligned vectors; group sums as in k_dotf_partial_v)
-__global__ void __launch_bounds__(DOT_THREADS) k_update_xr_dot_f(int64_t n, float *__restrict__ xs,
-                                                                 float *__restrict__ r, float *__restrict__ rold,
-                                                                 const float *__restrict__ p,
-                                                                 const float *__restrict__ q,
-                                                                 const double *__restrict__ scal,
-                                                                 double *__restrict__ partials) {
-    __shared__ double sh[32];
-    const float alpha = (float)(scal[0] / scal[1]);
-    float4 *xs4 = reinterpret_cast<float4 *>(xs), *r4 = reinterpret_cast<float4 *>(r);
-    float4 *ro4 = reinterpret_cast<float4 *>(rold);
-    const float4 *p4 = reinterpret_cast<const float4 *>(p), *q4 = reinterpret_cast<const float4 *>(q);
-    const int64_t n4 = n >> 2, stride = (int64_t)gridDim.x * blockDim.x;
-    double s = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += stride) {
-        const float4 ri = r4[i], pi = p4[i], qi = q4[i];
-        float4 xi = xs4[i];
-        if (rold) ro4[i] = ri;
-        xi.x = fmaf(alpha, pi.x, xi.x);
-        xi.y = fmaf(alpha, pi.y, xi.y);
-        xi.z = fmaf(alpha, pi.z, xi.z);
-        xi.w = fmaf(alpha, pi.w, xi.w);
-        float4 rn;
-        rn.x = fmaf(-alpha, qi.x, ri.x);
-        rn.y = fmaf(-alpha, qi.y, ri.y);
-        rn.z = fmaf(-alpha, qi.z, ri.z);
-        rn.w = fmaf(-alpha, qi.w, ri.w);
-        xs4[i] = xi;
-        r4[i] = rn;
-        s += (double)dot4(rn, rn);
-    }
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == blockDim.x - 1)
-        for (int64_t k = n4 << 2; k < n; ++k) {
-            const float ri = r[k];
-            if (rold) rold[k] = ri;
-            xs[k] = fmaf(alpha, p[k], xs[k]);
-            const float rn = fmaf(-alpha, q[k], ri);
-            r[k] = rn;
-            s += (double)rn * (double)rn;
-        }
-    s = block_sum(s, sh);
-    if (threadIdx.x == 0) partials[blockIdx.x] = s;
-}
-
-__global__ void k_dotf_partial(int64_t n, const float *__restrict__ x, const float *__restrict__ y,
-                               double *__restrict__ partials) {
-    __shared__ double sh[32];
-    double s = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        s += (double)x[i] * (double)y[i];
-    s = block_sum(s, sh);
-    if (threadIdx.x == 0) partials[blockIdx.x] = s;
-}
-
-__global__ void k_dot2f_partial(int64_t n, const float *__restrict__ x, const float *__restrict__ y,
-                                const float *__restrict__ z, double *__restrict__ partials) {
-    __shared__ double sh[32];
-    double s = 0.0, t = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const double yi = y[i];
-        s += (double)x[i] * yi;
-        t += (double)z[i] * yi;
-    }
-    s = block_sum(s, sh);
-    __syncthreads();
-    t = block_sum(t, sh);
-    if (threadIdx.x == 0) {
-        partials[blockIdx.x] = s;
-        partials[gridDim.x + blockIdx.x] = t;
-    }
-}
-
-// xs += alpha p, r -= alpha q, rold = old r (when given), alpha = scal[0] / scal[1]
-__global__ void k_update_xr_f(int64_t n, float *__restrict__ xs, float *__restrict__ r, float *__restrict__ rold,
-                              const float *__restrict__ p, const float *__restrict__ q,
-                              const double *__restrict__ scal) {
-    const float alpha = (float)(scal[0] / scal[1]);
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float ri = r[i];
-        if (rold) rold[i] = ri;
-        xs[i] += alpha * p[i];
-        r[i] = ri - alpha * q[i];
-    }
-}
-
-__global__ void k_update_p_f(int64_t n, float *__restrict__ p, const float *__restrict__ z,
-                             const double *__restrict__ scal) {
-    const float beta = (float)scal[2];
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        p[i] = z[i] + beta * p[i];
 }
 
 // x += xs (FP64 accumulation of the FP32 correction), xs = 0
@@ -367,24 +341,74 @@ inline bool aligned16(const void *a, const void *b, const void *c = nullptr, con
              reinterpret_cast<uintptr_t>(d) | reinterpret_cast<uintptr_t>(e)) & 15) == 0;
 }
 
-cudaError_t launch_dot(int64_t n, const double *x, const double *y, double *partials, double *out, cudaStream_t s) {
-    count_launches(2);
-    if (aligned16(x, y))
-        k_dot_partial_v<<<DOT_BLOCKS, DOT_THREADS, 0, s>>>(n, x, y, partials);
-    else
-        k_dot_partial<<<DOT_BLOCKS, DOT_THREADS, 0, s>>>(n, x, y, partials);
-    k_reduce<<<1, 512, 0, s>>>(DOT_BLOCKS, partials, out);
-    return cudaGetLastError();
+// blocks of a vector kernel: about two rounds of 16-byte loads per thread, at most four
+// blocks per SM; a function of the length alone, so the sums have one order per length
+static unsigned vector_blocks(int64_t n, int item) {
+    const int64_t b = (n * item / 16 + 2 * DOT_THREADS - 1) / (2 * DOT_THREADS);
+    return (unsigned)std::max<int64_t>(1, std::min<int64_t>(b, DOT_BLOCKS));
 }
 
-cudaError_t launch_dot2(int64_t n, const double *x, const double *y, const double *z, double *partials,
-                        double *out_xy, double *out_zy, cudaStream_t s) {
-    count_launches(3);
-    k_dot2_partial<<<DOT_BLOCKS, DOT_THREADS, 0, s>>>(n, x, y, z, partials);
-    k_reduce<<<1, 512, 0, s>>>(DOT_BLOCKS, partials, out_xy);
-    k_reduce<<<1, 512, 0, s>>>(DOT_BLOCKS, partials + DOT_BLOCKS, out_zy);
+template <typename T>
+cudaError_t launch_dot(int64_t n, const T *a, const T *b, double *partials, double *out, cudaStream_t s, double *scal) {
+    count_launches(1);
+    const unsigned g = vector_blocks(n, sizeof(T));
+    if (aligned16(a, b))
+        k_dot<T, 1, true><<<g, DOT_THREADS, 0, s>>>(n, a, b, nullptr, partials, out, nullptr, scal);
+    else
+        k_dot<T, 1, false><<<g, DOT_THREADS, 0, s>>>(n, a, b, nullptr, partials, out, nullptr, scal);
     return cudaGetLastError();
 }
+template <typename T>
+cudaError_t launch_dot2(int64_t n, const T *a, const T *b, const T *c, double *partials, double *out_ab, double *out_cb,
+                        cudaStream_t s, double *scal) {
+    count_launches(1);
+    const unsigned g = vector_blocks(n, sizeof(T));
+    if (aligned16(a, b, c))
+        k_dot<T, 2, true><<<g, DOT_THREADS, 0, s>>>(n, a, b, c, partials, out_ab, out_cb, scal);
+    else
+        k_dot<T, 2, false><<<g, DOT_THREADS, 0, s>>>(n, a, b, c, partials, out_ab, out_cb, scal);
+    return cudaGetLastError();
+}
+cudaError_t launch_norms(int64_t n, const double *r, const double *x, const double *y, double *partials, double *out_rr,
+                         double *out_dd, cudaStream_t s) {
+    count_launches(1);
+    const unsigned g = vector_blocks(n, sizeof(double));
+    if (aligned16(r, x, y))
+        k_norms<true><<<g, DOT_THREADS, 0, s>>>(n, r, x, y, partials, out_rr, out_dd);
+    else
+        k_norms<false><<<g, DOT_THREADS, 0, s>>>(n, r, x, y, partials, out_rr, out_dd);
+    return cudaGetLastError();
+}
+template <typename T>
+cudaError_t launch_update_xr(int64_t n, T *x, T *r, T *rold, const T *p, const T *q, const double *scal,
+                             double *partials, double *out_rr, cudaStream_t s) {
+    count_launches(1);
+    const unsigned g = vector_blocks(n, sizeof(T));
+    if (aligned16(x, r, rold, p, q))
+        k_update_xr<T, true><<<g, DOT_THREADS, 0, s>>>(n, x, r, rold, p, q, scal, partials, out_rr);
+    else
+        k_update_xr<T, false><<<g, DOT_THREADS, 0, s>>>(n, x, r, rold, p, q, scal, partials, out_rr);
+    return cudaGetLastError();
+}
+template <typename T>
+cudaError_t launch_update_p(int64_t n, T *p, const T *z, const double *scal, cudaStream_t s) {
+    count_launches(1);
+    const unsigned g = vector_blocks(n, sizeof(T));
+    if (aligned16(p, z))
+        k_update_p<T, true><<<g, DOT_THREADS, 0, s>>>(n, p, z, scal);
+    else
+        k_update_p<T, false><<<g, DOT_THREADS, 0, s>>>(n, p, z, scal);
+    return cudaGetLastError();
+}
+#define DGMG_BLAS_INST(T)                                                                                             \
+    template cudaError_t launch_dot<T>(int64_t, const T *, const T *, double *, double *, cudaStream_t, double *);     \
+    template cudaError_t launch_dot2<T>(int64_t, const T *, const T *, const T *, double *, double *, double *,        \
+                                        cudaStream_t, double *);                                                      \
+    template cudaError_t launch_update_xr<T>(int64_t, T *, T *, T *, const T *, const T *, const double *, double *,   \
+                                             double *, cudaStream_t);                                                 \
+    template cudaError_t launch_update_p<T>(int64_t, T *, const T *, const double *, cudaStream_t);
+DGMG_BLAS_INST(double)
+DGMG_BLAS_INST(float)
 
 cudaError_t launch_cast_d2f(int64_t n, const double *x, float *y, cudaStream_t s) {
     count_launches(1);
@@ -395,31 +419,6 @@ cudaError_t launch_cast_d2f(int64_t n, const double *x, float *y, cudaStream_t s
 cudaError_t launch_cast_f2d(int64_t n, const float *x, double *y, cudaStream_t s) {
     count_launches(1);
     k_f2d<<<grid_for(n), 256, 0, s>>>(n, x, y);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_pcg_update_xr(int64_t n, double *x, double *r, const double *p, const double *q,
-                                 const double *scal, cudaStream_t s) {
-    count_launches(1);
-    k_update_xr<<<grid_for(n), 256, 0, s>>>(n, x, r, p, q, scal);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_pcg_update_p(int64_t n, double *p, const double *z, const double *scal, cudaStream_t s) {
-    count_launches(1);
-    k_update_p<<<grid_for(n), 256, 0, s>>>(n, p, z, scal);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_sub(int64_t n, const double *a, const double *b, double *out, cudaStream_t s) {
-    count_launches(1);
-    k_sub<<<grid_for(n), 256, 0, s>>>(n, a, b, out);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_copy_scalar(const double *src, double *dst, cudaStream_t s) {
-    count_launches(1);
-    k_copy_scalar<<<1, 1, 0, s>>>(src, dst);
     return cudaGetLastError();
 }
 
@@ -443,54 +442,6 @@ cudaError_t launch_load_vector(int dim, int q, int mq, int64_t ncell, const doub
     if (q > QMAX || mq > LV_MQ || ncell > 0x7fffffff) return cudaErrorInvalidValue;
     count_launches(1);
     k_load_vector<<<(unsigned)ncell, LV_THREADS, 0, s>>>(dim, q, mq, ncell, V, wq, fq, b);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_dotf(int64_t n, const float *x, const float *y, double *partials, double *out, cudaStream_t s) {
-    count_launches(2);
-    if (aligned16(x, y))
-        k_dotf_partial_v<false><<<DOT_BLOCKS, DOT_THREADS, 0, s>>>(n, x, y, nullptr, partials);
-    else
-        k_dotf_partial<<<DOT_BLOCKS, DOT_THREADS, 0, s>>>(n, x, y, partials);
-    k_reduce<<<1, 512, 0, s>>>(DOT_BLOCKS, partials, out);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_dot2f(int64_t n, const float *x, const float *y, const float *z, double *partials,
-                         double *out_xy, double *out_zy, cudaStream_t s) {
-    count_launches(3);
-    if (aligned16(x, y, z))
-        k_dotf_partial_v<true><<<DOT_BLOCKS, DOT_THREADS, 0, s>>>(n, x, y, z, partials);
-    else
-        k_dot2f_partial<<<DOT_BLOCKS, DOT_THREADS, 0, s>>>(n, x, y, z, partials);
-    k_reduce<<<1, 512, 0, s>>>(DOT_BLOCKS, partials, out_xy);
-    k_reduce<<<1, 512, 0, s>>>(DOT_BLOCKS, partials + DOT_BLOCKS, out_zy);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_update_xr_f(int64_t n, float *xs, float *r, float *rold, const float *p, const float *q,
-                               const double *scal, cudaStream_t s) {
-    count_launches(1);
-    k_update_xr_f<<<grid_for(n), 256, 0, s>>>(n, xs, r, rold, p, q, scal);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_update_xr_dot_f(int64_t n, float *xs, float *r, float *rold, const float *p, const float *q,
-                                   const double *scal, double *partials, double *out_rr, cudaStream_t s) {
-    if (!aligned16(xs, r, rold, p, q)) {
-        const cudaError_t e = launch_update_xr_f(n, xs, r, rold, p, q, scal, s);
-        if (e != cudaSuccess) return e;
-        return launch_dotf(n, r, r, partials, out_rr, s);
-    }
-    count_launches(2);
-    k_update_xr_dot_f<<<DOT_BLOCKS, DOT_THREADS, 0, s>>>(n, xs, r, rold, p, q, scal, partials);
-    k_reduce<<<1, 512, 0, s>>>(DOT_BLOCKS, partials, out_rr);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_update_p_f(int64_t n, float *p, const float *z, const double *scal, cudaStream_t s) {
-    count_launches(1);
-    k_update_p_f<<<grid_for(n), 256, 0, s>>>(n, p, z, scal);
     return cudaGetLastError();
 }
 

@@ -1258,7 +1258,8 @@ int create_ctx(const dgmg_mesh *mesh, int p, const double *kappa, const dgmg_opt
     RC(C->alloc(&C->w_q, C->ndof));
     RC(C->alloc(&C->w_rold, C->ndof));
     RC(C->alloc(&C->scal, S_NSCAL));
-    RC(C->alloc(&C->partials, 2 * DOT_BLOCKS));
+    RC(C->alloc(&C->partials, DOT_WORK));
+    DG_CUDA(cudaMemsetAsync(C->partials, 0, sizeof(double) * DOT_WORK, C->setup_stream));
     {
         cudaError_t e = cudaMallocHost((void **)&C->host_scal, sizeof(double) * S_HOST);
         if (e != cudaSuccess) return cuda_fail(e, "cudaMallocHost");
@@ -1593,7 +1594,7 @@ int dgmg_estimate_bytes(const dgmg_mesh *mesh, int p, const dgmg_opts *opts, siz
         cg32 += sz(ints, 4) + sz(dbl, 4);
         for (int a = 0; a < 3; ++a) cur[a] = nxt[a];
     }
-    size_t total = sz(nv * nv, 8) + dg64 + cg64 + 5 * sz(ndof, 8) + sz(S_NSCAL, 8) + sz(2 * DOT_BLOCKS, 8) +
+    size_t total = sz(nv * nv, 8) + dg64 + cg64 + 5 * sz(ndof, 8) + sz(S_NSCAL, 8) + sz(DOT_WORK, 8) +
                    sz(p + 2, 8) + sz((int64_t)q * (p + 2), 8) + sz(3 * (p + 2), 8);
     if (mixed) total += dg32 + cg32 + 2 * sz(ndof, 4) + (reliable ? 4 * sz(ndof, 4) : 0);
     if (q1_blocks_for(dim, mixed) > 0)   // the plans of the cooperative Q1 cycle and their counters

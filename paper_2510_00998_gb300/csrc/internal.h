@@ -350,28 +350,28 @@ template <typename T>
 cudaError_t launch_coarse_solve_batch(const BatchCG<T> *D, const VertMap *map, int nb, cudaStream_t s);
 
 // BLAS-1 and helpers (blas.cu)
-cudaError_t launch_dot(int64_t n, const double *x, const double *y, double *partials,
-                       double *out, cudaStream_t s);
-cudaError_t launch_dot2(int64_t n, const double *x, const double *y, const double *z,
-                        double *partials, double *out_xy, double *out_zy, cudaStream_t s);
+// partials: DOT_WORK doubles, zero before their first use, of one stream at a time.
+// out = a.b; with scal the CG scalars are updated too: beta = scal[2] = out / scal[0],
+// scal[0] = out
+template <typename T>
+cudaError_t launch_dot(int64_t n, const T *a, const T *b, double *partials, double *out, cudaStream_t s,
+                       double *scal = nullptr);
+// a.b and c.b; with scal beta = scal[2] = (a.b - c.b) / scal[0], scal[0] = a.b
+template <typename T>
+cudaError_t launch_dot2(int64_t n, const T *a, const T *b, const T *c, double *partials, double *out_ab, double *out_cb,
+                        cudaStream_t s, double *scal = nullptr);
+// ||r||^2 and ||x - y||^2
+cudaError_t launch_norms(int64_t n, const double *r, const double *x, const double *y, double *partials, double *out_rr,
+                         double *out_dd, cudaStream_t s);
+// x += alpha p, r_old = r (unless null), r -= alpha q, out_rr = ||r||^2; alpha = scal[0] / scal[1]
+template <typename T>
+cudaError_t launch_update_xr(int64_t n, T *x, T *r, T *rold, const T *p, const T *q, const double *scal,
+                             double *partials, double *out_rr, cudaStream_t s);
+// p = z + scal[2] p
+template <typename T>
+cudaError_t launch_update_p(int64_t n, T *p, const T *z, const double *scal, cudaStream_t s);
 cudaError_t launch_cast_d2f(int64_t n, const double *x, float *y, cudaStream_t s);
 cudaError_t launch_cast_f2d(int64_t n, const float *x, double *y, cudaStream_t s);
-cudaError_t launch_pcg_update_xr(int64_t n, double *x, double *r, const double *p,
-                                 const double *q, const double *scal, cudaStream_t s);
-cudaError_t launch_pcg_update_p(int64_t n, double *p, const double *z, const double *scal,
-                                cudaStream_t s);
-cudaError_t launch_sub(int64_t n, const double *a, const double *b, double *out, cudaStream_t s);
-cudaError_t launch_copy_scalar(const double *src, double *dst, cudaStream_t s);
-cudaError_t launch_dotf(int64_t n, const float *x, const float *y, double *partials, double *out,
-                        cudaStream_t s);
-cudaError_t launch_dot2f(int64_t n, const float *x, const float *y, const float *z, double *partials,
-                         double *out_xy, double *out_zy, cudaStream_t s);
-cudaError_t launch_update_xr_f(int64_t n, float *xs, float *r, float *rold, const float *p, const float *q,
-                               const double *scal, cudaStream_t s);
-// launch_update_xr_f and *out_rr = ||r||^2 of the updated r, in one pass over the vectors
-cudaError_t launch_update_xr_dot_f(int64_t n, float *xs, float *r, float *rold, const float *p, const float *q,
-                                   const double *scal, double *partials, double *out_rr, cudaStream_t s);
-cudaError_t launch_update_p_f(int64_t n, float *p, const float *z, const double *scal, cudaStream_t s);
 cudaError_t launch_accumulate_f2d(int64_t n, double *x, float *xs, cudaStream_t s);
 cudaError_t launch_quad_points(int dim, int q, const int *n, int mq, const double *xq1,
                                double *xq, int64_t ncell, cudaStream_t s);
@@ -385,5 +385,6 @@ int residual_restrict_with_scratch(dgmg_ctx *C, const double *u, const double *b
 
 constexpr int DOT_BLOCKS = 608;     // 4 x 152 SMs
 constexpr int DOT_THREADS = 256;
+constexpr int DOT_WORK = 2 * DOT_BLOCKS + 1;   // two rows of partial sums, the ticket of the last block
 
 }  // namespace dgmg

@@ -21,21 +21,6 @@ namespace dgmg {
 
 namespace {
 
-// beta of the CG direction update (Fletcher-Reeves, or Polak-Ribiere for the
-// flexible variant) and the shift of <r,z>, on the device
-__global__ void k_scalar_beta(double *scal, int flexible) {
-    const double rzn = scal[S_RZN];
-    scal[S_BETA] = flexible ? (rzn - scal[S_RZO]) / scal[S_RZ] : rzn / scal[S_RZ];
-    scal[S_RZ] = rzn;
-}
-
-int launch_beta(dgmg_ctx *C, int flexible, cudaStream_t s) {
-    count_launches(1);
-    k_scalar_beta<<<1, 1, 0, s>>>(C->scal, flexible);
-    LC(cudaGetLastError());
-    return DGMG_OK;
-}
-
 // queue the copy of the whole scalar block to pinned host memory + the event
 int copy_scalars(dgmg_ctx *C, cudaStream_t s) {
     LC(cudaMemcpyAsync(C->host_scal, C->scal, sizeof(double) * S_NSCAL, cudaMemcpyDeviceToHost, s));
@@ -215,19 +200,17 @@ int SolveRun::pcg_chunk(bool update_dir, cudaStream_t st) {
         RC(vcycle64(*C, r, z, st));
         C->prof.begin(ST_VECTOR, st);
         if (flexible)
-            LC(launch_dot2(n, r, z, rold, C->partials, C->scal + S_RZN, C->scal + S_RZO, st));
+            LC(launch_dot2(n, r, z, rold, C->partials, C->scal + S_RZN, C->scal + S_RZO, st, C->scal));
         else
-            LC(launch_dot(n, r, z, C->partials, C->scal + S_RZN, st));
-        RC(launch_beta(C, flexible ? 1 : 0, st));
-        LC(launch_pcg_update_p(n, p, z, C->scal, st));
+            LC(launch_dot(n, r, z, C->partials, C->scal + S_RZN, st, C->scal));
+        LC(launch_update_p(n, p, z, C->scal, st));
         C->prof.end(st);
     }
     RC(apply64(*C, p, nullptr, q, st));                         // q = A p
     C->prof.begin(ST_VECTOR, st);
     LC(launch_dot(n, p, q, C->partials, C->scal + S_PQ, st));
-    if (flexible) LC(cudaMemcpyAsync(rold, r, sizeof(double) * n, cudaMemcpyDeviceToDevice, st));
-    LC(launch_pcg_update_xr(n, x, r, p, q, C->scal, st));      // alpha = rz / pq
-    LC(launch_dot(n, r, r, C->partials, C->scal + S_RR, st));
+    // alpha = rz / pq
+    LC(launch_update_xr<double>(n, x, r, flexible ? rold : nullptr, p, q, C->scal, C->partials, C->scal + S_RR, st));
     C->prof.end(st);
     return copy_scalars(C, st);
 }
@@ -241,15 +224,14 @@ int SolveRun::reliable_chunk(bool update_dir, cudaStream_t st) {
     if (update_dir) {
         RC(dg_vcycle<float>(*C, r32, z32, st));
         C->prof.begin(ST_VECTOR, st);
-        LC(launch_dot2f(n, r32, z32, rold32, C->partials, C->scal + S_RZN, C->scal + S_RZO, st));
-        RC(launch_beta(C, 1, st));
-        LC(launch_update_p_f(n, p32, z32, C->scal, st));
+        LC(launch_dot2<float>(n, r32, z32, rold32, C->partials, C->scal + S_RZN, C->scal + S_RZO, st, C->scal));
+        LC(launch_update_p(n, p32, z32, C->scal, st));
         C->prof.end(st);
     }
     RC(apply32(*C, p32, q32, st));
     C->prof.begin(ST_VECTOR, st);
-    LC(launch_dotf(n, p32, q32, C->partials, C->scal + S_PQ, st));
-    LC(launch_update_xr_dot_f(n, xs, r32, rold32, p32, q32, C->scal, C->partials, C->scal + S_RR, st));
+    LC(launch_dot<float>(n, p32, q32, C->partials, C->scal + S_PQ, st));
+    LC(launch_update_xr<float>(n, xs, r32, rold32, p32, q32, C->scal, C->partials, C->scal + S_RR, st));
     C->prof.end(st);
     return copy_scalars(C, st);
 }
@@ -259,15 +241,13 @@ int SolveRun::reliable_chunk(bool update_dir, cudaStream_t st) {
 // caller's b), r = b - A x, ||r||^2 and ||x - x_old||^2, scalars to the host.
 int SolveRun::mg_chunk(cudaStream_t st) {
     const int64_t n = C->ndof;
-    double *xold = C->w_p, *dx = C->w_q, *r = C->w_r, *bc = C->w_rold;
+    double *xold = C->w_p, *r = C->w_r, *bc = C->w_rold;
     C->prof.begin(ST_VECTOR, st);
     LC(cudaMemcpyAsync(xold, x, sizeof(double) * n, cudaMemcpyDeviceToDevice, st));
     C->prof.end(st);
     RC(mg_cycle64(*C, x, bc, r, st));
     C->prof.begin(ST_VECTOR, st);
-    LC(launch_dot(n, r, r, C->partials, C->scal + S_RR, st));
-    LC(launch_sub(n, x, xold, dx, st));
-    LC(launch_dot(n, dx, dx, C->partials, C->scal + S_ZZ, st));
+    LC(launch_norms(n, r, x, xold, C->partials, C->scal + S_RR, C->scal + S_ZZ, st));
     C->prof.end(st);
     return copy_scalars(C, st);
 }
@@ -411,8 +391,8 @@ int SolveRun::advance(bool blocking) {
                 ADV_CUDA(cudaMemsetAsync(xs, 0, sizeof(float) * n, s));
                 ADV(dg_vcycle<float>(*C, r32, z32, s));
                 C->prof.begin(ST_VECTOR, s);
-                ADV_CUDA(launch_dotf(n, r32, z32, C->partials, C->scal + S_RZ, s));
-                ADV_CUDA(launch_dotf(n, z32, z32, C->partials, C->scal + S_ZZ0, s));
+                ADV_CUDA(launch_dot<float>(n, r32, z32, C->partials, C->scal + S_RZ, s));
+                ADV_CUDA(launch_dot<float>(n, z32, z32, C->partials, C->scal + S_ZZ0, s));
                 ADV_CUDA(cudaMemcpyAsync(p32, z32, sizeof(float) * n, cudaMemcpyDeviceToDevice, s));
                 C->prof.end(s);
                 it = 1;
@@ -495,7 +475,7 @@ int SolveRun::advance(bool blocking) {
                     ++nres;
                     ADV_CUDA(launch_dot(n, r, r, C->partials, C->scal + S_RR, s));
                 }
-                if (it > 0) ADV_CUDA(launch_dotf(n, z32, z32, C->partials, C->scal + S_ZZ, s));
+                if (it > 0) ADV_CUDA(launch_dot<float>(n, z32, z32, C->partials, C->scal + S_ZZ, s));
                 ADV(post_scalars(C, s));
                 state = R_WAIT_FIN;
                 break;
