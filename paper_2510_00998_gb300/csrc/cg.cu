@@ -37,11 +37,8 @@ __device__ __forceinline__ void vcoords(int64_t v, const int *m, int *c) {
 // b0[v] = sum over the 2^d cells around interior vertex v of the cell's corner
 // partial sum for that vertex (fixed order: deterministic p-restriction).
 template <int DIM, typename T>
-__device__ __forceinline__ void corner_gather_at(int n0, int n1, int n2, const T *__restrict__ corners,
-                                                 T *__restrict__ b0, int64_t v) {
+__device__ __forceinline__ T corner_sum_at(int n0, int n1, int n2, const T *__restrict__ corners, int64_t v) {
     const int m[3] = {n0 - 1, n1 - 1, n2 - 1};
-    const int64_t nv = DIM == 3 ? (int64_t)m[0] * m[1] * m[2] : (int64_t)m[0] * m[1];
-    if (v >= nv) return;
     int c[3];
     vcoords<DIM>(v, m, c);
     T s = T(0);
@@ -54,7 +51,14 @@ __device__ __forceinline__ void corner_gather_at(int n0, int n1, int n2, const T
         const int corner = (~a) & ((1 << DIM) - 1);
         s += corners[cell * (1 << DIM) + corner];
     }
-    b0[v] = s;
+    return s;
+}
+
+template <int DIM, typename T>
+__device__ __forceinline__ void corner_gather_at(int n0, int n1, int n2, const T *__restrict__ corners,
+                                                 T *__restrict__ b0, int64_t v) {
+    const int64_t nv = DIM == 3 ? (int64_t)(n0 - 1) * (n1 - 1) * (n2 - 1) : (int64_t)(n0 - 1) * (n1 - 1);
+    if (v < nv) b0[v] = corner_sum_at<DIM, T>(n0, n1, n2, corners, v);
 }
 
 template <int DIM, typename T>
@@ -77,10 +81,10 @@ __device__ __forceinline__ T stencil_apply(const CGLevelDev<T> &L, int64_t v, co
         sv[k] = in ? __ldg(L.st + (int64_t)k * L.nv + v) : T(0);
         uv[k] = in ? u[w] : T(0);
     }
-    T s = T(0);
+    T s[3] = {};   // three chains of dependent sums
 #pragma unroll
-    for (int k = 0; k < NS; ++k) s += sv[k] * uv[k];
-    return s;
+    for (int k = 0; k < NS; ++k) s[k / (NS / 3)] += sv[k] * uv[k];
+    return (s[0] + s[1]) + s[2];
 }
 
 template <int DIM, typename T>
@@ -121,51 +125,56 @@ __global__ void k_cg_residual(CGLevelDev<T> L, const T *__restrict__ u, const T 
     cg_residual_at<DIM, T>(L, u, b, r, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
-// rc[V] = sum_i P_h[i][V] rf[i]: per axis, the fine children of coarse vertex V.
+// sum_i P_h[i][V] rf[i]: per axis, the fine children of coarse vertex V, at most
+// 2f - 1 <= 5 (weights padded to 5). Eight lanes share a vertex, each takes every
+// eighth of its rows of children along x: the rows' loads are all in flight and the
+// chain of dependent sums is short (one thread per vertex took 5.4 us a level in FP64,
+// against 3.2 of a Jacobi step). All 32 lanes of a warp call it; V < 0: no vertex.
+// Every lane of a group returns the sum.
+constexpr int RS_LANES = 8;
 template <int DIM, typename T>
-__device__ __forceinline__ void h_restrict_at(const CGLevelDev<T> &L, const T *rf, T *rc,
-                                              int64_t V) {
-    const int64_t ncv = DIM == 3 ? (int64_t)L.mc[0] * L.mc[1] * L.mc[2] : (int64_t)L.mc[0] * L.mc[1];
-    if (V >= ncv) return;
-    int C[3] = {0, 0, 0};
-    vcoords<DIM>(V, L.mc, C);
-    const int sx = __ldg(L.rs_start[0] + C[0]), nx = __ldg(L.rs_cnt[0] + C[0]);
-    const int sy = __ldg(L.rs_start[1] + C[1]), ny = __ldg(L.rs_cnt[1] + C[1]);
-    const int sz = DIM == 3 ? __ldg(L.rs_start[2] + C[2]) : 0, nz = DIM == 3 ? __ldg(L.rs_cnt[2] + C[2]) : 1;
-    // at most 2f - 1 <= 5 children per axis (weights padded to 5): loops unrolled
-    // to 5 with the counts as predicates, so that all loads are in flight together
-    T wx[5], wy[5], wz[5];
-#pragma unroll
-    for (int i = 0; i < 5; ++i) {
-        wx[i] = __ldg(L.rs_w[0] + C[0] * 5 + i);
-        wy[i] = __ldg(L.rs_w[1] + C[1] * 5 + i);
-        wz[i] = DIM == 3 ? __ldg(L.rs_w[2] + C[2] * 5 + i) : T(i == 0 ? 1 : 0);
-    }
+__device__ __forceinline__ T h_restrict_at(const CGLevelDev<T> &L, const T *rf, int64_t V) {
+    constexpr int ROWS = DIM == 3 ? 25 : 5, R = (ROWS + RS_LANES - 1) / RS_LANES;
+    const int lane = threadIdx.x & (RS_LANES - 1);
     T s = T(0);
+    if (V >= 0) {
+        int C[3] = {0, 0, 0};
+        vcoords<DIM>(V, L.mc, C);
+        const int sx = __ldg(L.rs_start[0] + C[0]), nx = __ldg(L.rs_cnt[0] + C[0]);
+        const int sy = __ldg(L.rs_start[1] + C[1]), ny = __ldg(L.rs_cnt[1] + C[1]);
+        const int sz = DIM == 3 ? __ldg(L.rs_start[2] + C[2]) : 0, nz = DIM == 3 ? __ldg(L.rs_cnt[2] + C[2]) : 1;
+        T wx[5], w[R], f[R][5];
 #pragma unroll
-    for (int k = 0; k < (DIM == 3 ? 5 : 1); ++k) {
-        if (k >= nz) break;
-        T f[25];   // the plane's children, loaded before they are summed
+        for (int i = 0; i < 5; ++i) wx[i] = __ldg(L.rs_w[0] + C[0] * 5 + i);
 #pragma unroll
-        for (int j = 0; j < 5; ++j) {
-            const T *row = rf + (int64_t)L.m[0] * ((sy + j) + (int64_t)L.m[1] * (sz + k)) + sx;
+        for (int a = 0; a < R; ++a) {
+            const int row = lane + a * RS_LANES, k = DIM == 3 ? row / 5 : 0, j = DIM == 3 ? row - 5 * k : row;
+            const bool in = row < ROWS && j < ny && k < nz;
+            w[a] = in ? __ldg(L.rs_w[1] + C[1] * 5 + j) : T(0);
+            if (DIM == 3 && in) w[a] *= __ldg(L.rs_w[2] + C[2] * 5 + k);
+            const T *x = rf + (int64_t)L.m[0] * ((sy + j) + (int64_t)L.m[1] * (sz + k)) + sx;
 #pragma unroll
-            for (int i = 0; i < 5; ++i) f[j * 5 + i] = (j < ny && i < nx) ? row[i] : T(0);
+            for (int i = 0; i < 5; ++i) f[a][i] = in && i < nx ? x[i] : T(0);
         }
 #pragma unroll
-        for (int j = 0; j < 5; ++j) {
+        for (int a = 0; a < R; ++a) {
             T sr = T(0);
 #pragma unroll
-            for (int i = 0; i < 5; ++i) sr += wx[i] * f[j * 5 + i];
-            s += wz[k] * wy[j] * sr;
+            for (int i = 0; i < 5; ++i) sr += wx[i] * f[a][i];
+            s += w[a] * sr;
         }
     }
-    rc[V] = s;
+#pragma unroll
+    for (int o = RS_LANES / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
 }
 
 template <int DIM, typename T>
 __global__ void k_h_restrict(CGLevelDev<T> L, const T *__restrict__ rf, T *__restrict__ rc) {
-    h_restrict_at<DIM, T>(L, rf, rc, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, V = t / RS_LANES;
+    const bool in = V < (DIM == 3 ? (int64_t)L.mc[0] * L.mc[1] * L.mc[2] : (int64_t)L.mc[0] * L.mc[1]);
+    const T s = h_restrict_at<DIM, T>(L, rf, in ? V : -1);
+    if (in && t % RS_LANES == 0) rc[V] = s;
 }
 
 // uf[i] += sum_V P_h[i][V] ec[V]: per axis, the (at most two) coarse parents.
@@ -234,13 +243,17 @@ __global__ void k_coarse_solve(int64_t nc, const double *__restrict__ Ainv, cons
     coarse_row<T>(nc, Ainv, r, e, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
-// ---- the whole Q1 h-cycle of one problem in one cooperative launch: every step
-// of the launch-per-step cycle (point Jacobi, residual, restriction, the dense
-// coarsest solve, prolongation) as a loop over the level's vertices split among
-// the blocks, the steps separated by a grid-wide barrier instead of kernel
-// boundaries. The vectors
-// are written and read again inside the one launch, so the per-vertex bodies
-// take them through plain pointers (no __restrict__: no loads through the
+// ---- the whole Q1 h-cycle of one problem in one launch. The cycle is a chain of
+// short steps, so their number and the wait between two of them are what it costs: on
+// the levels [0, dense_from) every step is a loop over the level's vertices split among
+// the blocks of a cooperative grid, separated by a grid-wide barrier; the cycle on
+// level dense_from and everything below it is one product with its matrix, which
+// k_q1_dense_matrix computes at set-up column by column with the very steps it
+// replaces (it is the inverse of the coarsest operator where that level is the last).
+// The gather of the right-hand side is the first step, and whoever writes a level's
+// right-hand side writes the first Jacobi step from the zero iterate with it.
+// The vectors are written and read again inside the one launch, so the per-vertex
+// bodies take them through plain pointers (no __restrict__: no loads through the
 // non-coherent read-only cache); only the stencils and tables use __ldg.
 
 // Waits of the grid barrier that gave up (zero in every healthy run). Once one
@@ -279,7 +292,7 @@ struct GridSync {
             const unsigned long long target = base + (unsigned long long)(k + 1) * gridDim.x;
             if (o + 1 != target) {
                 int it = 0;
-                while ((long long)(ld_acquire_gpu(cnt) - target) < 0 && ++it < (1 << 20)) __nanosleep(32);
+                while ((long long)(ld_acquire_gpu(cnt) - target) < 0 && ++it < (1 << 20)) {}
                 if (it >= (1 << 20)) atomicAdd(&g_q1_barrier_timeouts, 1ull);
             }
         }
@@ -292,14 +305,19 @@ struct BlockSync {
 };
 
 // Work split of one step: on the whole grid every block takes an equal run of
-// consecutive items (a multiple of 32), its threads stride through it, so a
-// level of a few thousand vertices still spreads over all SMs (FP64 FMA
-// throughput per SM is low); in one block the threads stride through all.
+// consecutive warps of items (the runs differ by one warp, so a level of a few
+// thousand vertices spreads over all SMs: FP64 FMA throughput per SM is low); in one
+// block the threads stride through all.
 struct GridEach {
     template <typename F>
     __device__ __forceinline__ void operator()(int64_t n, F &&f) const {
-        const int64_t chunk = ((n + gridDim.x - 1) / gridDim.x + 31) / 32 * 32;
-        const int64_t b = (int64_t)blockIdx.x * chunk, e = b + chunk < n ? b + chunk : n;
+        const int64_t w = (n + 31) / 32, b = w * blockIdx.x / gridDim.x * 32, e = w * (blockIdx.x + 1) / gridDim.x * 32;
+        for (int64_t v = b + threadIdx.x; v < (e < n ? e : n); v += blockDim.x) f(v);
+    }
+    // the same for all lanes of every warp that has an item (f is given v >= n too)
+    template <typename F>
+    __device__ __forceinline__ void warps(int64_t n, F &&f) const {
+        const int64_t w = (n + 31) / 32, b = w * blockIdx.x / gridDim.x * 32, e = w * (blockIdx.x + 1) / gridDim.x * 32;
         for (int64_t v = b + threadIdx.x; v < e; v += blockDim.x) f(v);
     }
 };
@@ -308,70 +326,106 @@ struct BlockEach {
     __device__ __forceinline__ void operator()(int64_t n, F &&f) const {
         for (int64_t v = threadIdx.x; v < n; v += blockDim.x) f(v);
     }
+    template <typename F>
+    __device__ __forceinline__ void warps(int64_t n, F &&f) const {
+        for (int64_t v = threadIdx.x; v < (n + 31) / 32 * 32; v += blockDim.x) f(v);
+    }
 };
 
-// Down the cycle on level l (not the coarsest): nu_pre Jacobi steps from the
-// zero guess, the residual, its restriction into b of level l + 1. The
+// right-hand side s of vertex v on level l, and the level's first iterate: one Jacobi
+// step from zero (u1), or zero (u0) without pre-smoothing
+template <typename T>
+__device__ __forceinline__ void q1_put_rhs(const Q1Plan<T> &p, int l, int64_t v, T s) {
+    p.b[l][v] = s;
+    if (p.nu_pre > 0)
+        p.u1[l][v] = s * p.wd[l][v];
+    else
+        p.u0[l][v] = T(0);
+}
+
+template <int DIM, typename T>
+__device__ __forceinline__ void q1_jacobi_at(const Q1Plan<T> &p, int l, const T *u_in, T *u_out, int64_t v) {
+    const CGLevelDev<T> &L = p.L[l];
+    int c[3] = {0, 0, 0};
+    vcoords<DIM>(v, L.m, c);
+    const T w = __ldg(p.wd[l] + v), bv = p.b[l][v], uv = u_in[v];
+    u_out[v] = uv + w * (bv - stencil_apply<DIM, T>(L, v, c, u_in));
+}
+
+// Down the cycle on level l (not the last) from its right-hand side and first iterate:
+// the other nu_pre - 1 Jacobi steps, the residual, its restriction to level l + 1. The
 // iterate ends in u[nu_pre & 1].
 template <int DIM, typename T, typename Each, typename Sync>
-__device__ __forceinline__ void q1_down(const Q1Plan<T> &p, int l, const Each &each, Sync &sync) {
+__device__ __forceinline__ void q1_down(const Q1Plan<T> &p, int l, bool last, const Each &each, Sync &sync) {
     const CGLevelDev<T> &L = p.L[l];
     T *u[2] = {p.u0[l], p.u1[l]};
     T *b = p.b[l], *r = p.r[l], *bn = p.b[l + 1];
-    const T om = p.omega;
-    int c = 0;
-    for (int k = 0; k < p.nu_pre; ++k) {
+    int c = p.nu_pre > 0 ? 1 : 0;
+    for (int k = 1; k < p.nu_pre; ++k) {
         T *ui = u[c], *uo = u[c ^ 1];
-        const int zero = k == 0;
-        each(L.nv, [&](int64_t v) { cg_jacobi_at<DIM, T>(L, ui, b, uo, om, zero, v); });
+        each(L.nv, [&](int64_t v) { q1_jacobi_at<DIM, T>(p, l, ui, uo, v); });
         c ^= 1;
-        sync();
-    }
-    if (p.nu_pre == 0) {
-        T *u0 = u[0];
-        each(L.nv, [&](int64_t v) { u0[v] = T(0); });
         sync();
     }
     T *uc = u[c];
     each(L.nv, [&](int64_t v) { cg_residual_at<DIM, T>(L, uc, b, r, v); });
     sync();
     const int64_t ncv = DIM == 3 ? (int64_t)L.mc[0] * L.mc[1] * L.mc[2] : (int64_t)L.mc[0] * L.mc[1];
-    each(ncv, [&](int64_t V) { h_restrict_at<DIM, T>(L, r, bn, V); });
+    each.warps(ncv * RS_LANES, [&](int64_t t) {   // whole warps: the lanes of a vertex exchange their sums
+        const int64_t V = t / RS_LANES;
+        const T s = h_restrict_at<DIM, T>(L, r, V < ncv ? V : -1);
+        if (V >= ncv || t % RS_LANES != 0) return;
+        if (last)
+            bn[V] = s;
+        else
+            q1_put_rhs<T>(p, l + 1, V, s);
+    });
     sync();
 }
 
 // Up the cycle on level l: add the prolongated correction ec of level l + 1,
-// nu_post Jacobi steps; returns the level's result, u[(nu_pre + nu_post) & 1].
+// nu_post Jacobi steps; returns the level's result, u[(nu_pre + nu_post) & 1]. No
+// barrier after the last step of level 0: the launch ends there.
 template <int DIM, typename T, typename Each, typename Sync>
 __device__ __forceinline__ const T *q1_up(const Q1Plan<T> &p, int l, const T *ec, const Each &each, Sync &sync) {
     const CGLevelDev<T> &L = p.L[l];
     T *u[2] = {p.u0[l], p.u1[l]};
-    T *b = p.b[l];
-    const T om = p.omega;
     int c = p.nu_pre & 1;
     T *uc = u[c];
     each(L.nv, [&](int64_t v) { h_prolong_at<DIM, T>(L, ec, uc, v); });
-    sync();
+    if (p.nu_post > 0 || l > 0) sync();
     for (int k = 0; k < p.nu_post; ++k) {
         T *ui = u[c], *uo = u[c ^ 1];
-        each(L.nv, [&](int64_t v) { cg_jacobi_at<DIM, T>(L, ui, b, uo, om, 0, v); });
+        each(L.nv, [&](int64_t v) { q1_jacobi_at<DIM, T>(p, l, ui, uo, v); });
         c ^= 1;
-        sync();
+        if (k + 1 < p.nu_post || l > 0) sync();
     }
     return u[c];
 }
 
-// The levels from p.local_from down (small enough for one block: the
-// threshold is lower in FP64, whose FMA throughput per SM is low) and the
-// coarsest solve run in block 0 alone, separated by block barriers; the larger
-// levels use the whole grid.
+// row i of e = E b, one warp: lane-strided (coalesced) products, four sums per lane
+template <typename T>
+__device__ __forceinline__ double q1_dense_row(int n, const double *__restrict__ E, const T *b, int64_t i) {
+    const double *a = E + i * n;
+    double s[4] = {};
+    int j = threadIdx.x & 31;
+    for (; j + 96 < n; j += 128)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) s[k] = fma(__ldg(a + j + 32 * k), (double)b[j + 32 * k], s[k]);
+    for (; j < n; j += 32) s[0] = fma(__ldg(a + j), (double)b[j], s[0]);
+    double t = (s[0] + s[1]) + (s[2] + s[3]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    return t;
+}
+
 template <int DIM, typename T, int TPB>
-__global__ void __launch_bounds__(TPB) k_q1_cycle(const Q1Plan<T> *__restrict__ P, unsigned long long *bar) {
+__global__ void __launch_bounds__(TPB) k_q1_cycle(const __grid_constant__ Q1Plan<T> p,
+                                                  const T *__restrict__ corners, unsigned long long *bar) {
     if (*(volatile unsigned long long *)&g_q1_barrier_timeouts != 0) return;
-    const Q1Plan<T> &p = *P;
-    // the finest level's stencil is first read after the zero-guess Jacobi step:
-    // every block requests its share into L2 now (a hint; 16-byte pieces)
-    if (threadIdx.x == 0 && p.nlev > 0) {
+    // the finest level's stencil is first read after the first barrier: every block
+    // requests its share into L2 now (a hint; 16-byte pieces)
+    if (threadIdx.x == 0) {
         const uint64_t bytes = (uint64_t)(DIM == 3 ? 27 : 9) * p.L[0].nv * sizeof(T);
         const uint64_t chunk = ((bytes + gridDim.x - 1) / gridDim.x + 15) / 16 * 16;
         const uint64_t off = (uint64_t)blockIdx.x * chunk;
@@ -383,35 +437,89 @@ __global__ void __launch_bounds__(TPB) k_q1_cycle(const Q1Plan<T> *__restrict__ 
                              : "memory");
         }
     }
-    const int nl = p.nlev, ls = p.local_from;
+    const int ld = p.dense_from;
     GridSync grid{bar, 0ull, 0u};
     const GridEach on_grid;
-    const int lg = ls < nl - 1 ? ls : nl - 1;   // levels [0, lg) go down on the whole grid
-    for (int l = 0; l < lg; ++l) q1_down<DIM, T>(p, l, on_grid, grid);
-    const T *ec;
-    const T *rc = p.b[nl - 1];
-    T *e = p.u0[nl - 1];
-    const int64_t nc = p.ncoarse;
-    const double *Ainv = p.Ainv;
-    if (ls < nl) {
-        if (blockIdx.x == 0) {
-            BlockSync block;
-            const BlockEach on_block;
-            for (int l = ls; l < nl - 1; ++l) q1_down<DIM, T>(p, l, on_block, block);
-            on_block(nc, [&](int64_t i) { coarse_row<T>(nc, Ainv, rc, e, i); });
-            block();
-            const T *el = e;
-            for (int l = nl - 2; l >= ls; --l) el = q1_up<DIM, T>(p, l, el, on_block, block);
-        }
-        grid();
-        ec = ls == nl - 1 ? e : p.u0[ls];
-        if (ls < nl - 1 && ((p.nu_pre + p.nu_post) & 1)) ec = p.u1[ls];
-    } else {
-        on_grid(nc, [&](int64_t i) { coarse_row<T>(nc, Ainv, rc, e, i); });
-        grid();
-        ec = e;
+    on_grid(p.L[0].nv, [&](int64_t v) {
+        q1_put_rhs<T>(p, 0, v, corner_sum_at<DIM, T>(p.L[0].m[0] + 1, p.L[0].m[1] + 1, p.L[0].m[2] + 1, corners, v));
+    });
+    grid();
+    for (int l = 0; l < ld; ++l) q1_down<DIM, T>(p, l, l + 1 == ld, on_grid, grid);
+    const T *bd = p.b[ld];
+    T *e = p.u0[ld];
+    const int nd = (int)p.ndense, warps = (int)gridDim.x * (TPB / 32);
+    // consecutive warps of rows on different SMs
+    for (int i = (int)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; i < nd; i += warps) {
+        const double t = q1_dense_row<T>(nd, p.E, bd, i);
+        if ((threadIdx.x & 31) == 0) e[i] = (T)t;
     }
-    for (int l = lg - 1; l >= 0; --l) ec = q1_up<DIM, T>(p, l, ec, on_grid, grid);
+    grid();
+    const T *ec = e;
+    for (int l = ld - 1; l >= 0; --l) ec = q1_up<DIM, T>(p, l, ec, on_grid, grid);
+}
+
+// The cycle of a problem whose level 0 is the dense one: every block gathers the
+// right-hand side into shared memory, a warp per row.
+template <int DIM, typename T>
+__global__ void __launch_bounds__(Q1_TPB) k_q1_dense(const __grid_constant__ Q1Plan<T> p,
+                                                     const T *__restrict__ corners) {
+    extern __shared__ __align__(16) unsigned char q1_smem[];
+    T *b = reinterpret_cast<T *>(q1_smem);
+    const int n = (int)p.ndense;
+    for (int v = threadIdx.x; v < n; v += blockDim.x)
+        b[v] = corner_sum_at<DIM, T>(p.L[0].m[0] + 1, p.L[0].m[1] + 1, p.L[0].m[2] + 1, corners, v);
+    __syncthreads();
+    const int i = (int)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    if (i >= n) return;
+    const double t = q1_dense_row<T>(n, p.E, b, i);
+    if ((threadIdx.x & 31) == 0) p.u0[0][i] = (T)t;
+}
+
+// wd = omega / diagonal of a level
+template <typename T>
+__global__ void k_q1_weights(int64_t n, const T *__restrict__ diag, T omega, T *__restrict__ wd) {
+    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (v < n) wd[v] = omega / diag[v];
+}
+
+// E[i][j]: the cycle from level dense_from down applied to the unit vectors e_j, one
+// block per column, with the level vectors in shared memory.
+template <int DIM>
+__global__ void __launch_bounds__(Q1_TPB) k_q1_dense_matrix(const __grid_constant__ Q1Plan<double> plan,
+                                                            const double *__restrict__ Ainv, double *__restrict__ E) {
+    extern __shared__ __align__(16) unsigned char q1_smem[];
+    __shared__ Q1Plan<double> p;
+    const int ld = plan.dense_from, nl = plan.nlev;
+    if (threadIdx.x == 0) {
+        p = plan;
+        double *v = reinterpret_cast<double *>(q1_smem);
+        for (int l = ld; l < nl; ++l) {
+            const int64_t n = p.L[l].nv;
+            p.u0[l] = v;
+            p.u1[l] = v + n;
+            p.b[l] = v + 2 * n;
+            p.r[l] = v + 3 * n;
+            v += 4 * n;
+        }
+    }
+    __syncthreads();
+    const BlockEach each;
+    BlockSync sync;
+    const int64_t nd = p.L[ld].nv, nc = p.L[nl - 1].nv;
+    for (int64_t j = blockIdx.x; j < nd; j += gridDim.x) {
+        each(nd, [&](int64_t v) { q1_put_rhs<double>(p, ld, v, v == j ? 1.0 : 0.0); });
+        sync();
+        for (int l = ld; l < nl - 1; ++l) q1_down<DIM, double>(p, l, l + 1 == nl - 1, each, sync);
+        const double *rc = p.b[nl - 1];
+        double *e = p.u0[nl - 1];
+        each(nc, [&](int64_t i) { coarse_row<double>(nc, Ainv, rc, e, i); });
+        sync();
+        const double *ec = e;
+        for (int l = nl - 2; l >= ld; --l) ec = q1_up<DIM, double>(p, l, ec, each, sync);
+        sync();
+        each(nd, [&](int64_t v) { E[v * nd + j] = ec[v]; });
+        sync();
+    }
 }
 
 // ---- batched forms: work item k covers vertices [v0, v0 + BATCH_VERTS) of
@@ -451,7 +559,12 @@ __global__ void __launch_bounds__(BATCH_VERTS) k_h_restrict_batch(const BatchCG<
     for (int k = blockIdx.x; k < nb; k += gridDim.x) {
         const VertMap m = map[k];
         const BatchCG<T> &d = D[m.desc];
-        h_restrict_at<DIM, T>(d.L, d.r, d.b_next, (int64_t)m.v0 + threadIdx.x);
+        const int64_t ncv = DIM == 3 ? (int64_t)d.L.mc[0] * d.L.mc[1] * d.L.mc[2] : (int64_t)d.L.mc[0] * d.L.mc[1];
+        // the item's BATCH_VERTS vertices, RS_LANES threads each
+        for (int64_t V = m.v0 + (int)threadIdx.x / RS_LANES, e = m.v0 + BATCH_VERTS; V < e; V += BATCH_VERTS / RS_LANES) {
+            const T s = h_restrict_at<DIM, T>(d.L, d.r, V < ncv ? V : -1);
+            if (V < ncv && threadIdx.x % RS_LANES == 0) d.b_next[V] = s;
+        }
     }
 }
 template <int DIM, typename T>
@@ -481,19 +594,19 @@ inline unsigned blocks_for(int64_t n) { return (unsigned)((n + TPB - 1) / TPB); 
 
 // the kernel of precision T, dimension dim, 256 or (wide, FP32) 512 threads
 template <typename T>
-const void *q1_cycle_fn(int dim, bool wide) {
-    if (wide && sizeof(T) == 4)
-        return dim == 3 ? (const void *)k_q1_cycle<3, T, Q1_TPB_WIDE> : (const void *)k_q1_cycle<2, T, Q1_TPB_WIDE>;
-    return dim == 3 ? (const void *)k_q1_cycle<3, T, Q1_TPB> : (const void *)k_q1_cycle<2, T, Q1_TPB>;
+auto q1_cycle_fn(int dim, bool wide) -> void (*)(const Q1Plan<T>, const T *, unsigned long long *) {
+    if constexpr (sizeof(T) == 4) {
+        if (wide) return dim == 3 ? k_q1_cycle<3, T, Q1_TPB_WIDE> : k_q1_cycle<2, T, Q1_TPB_WIDE>;
+    }
+    return dim == 3 ? k_q1_cycle<3, T, Q1_TPB> : k_q1_cycle<2, T, Q1_TPB>;
 }
 
 template <typename T>
-cudaError_t launch_q1_cycle(int dim, const Q1Plan<T> *plan, unsigned long long *bar, int blocks, bool wide,
-                            cudaStream_t s) {
-    const bool w = wide && sizeof(T) == 4;
+cudaError_t launch_q1_cycle(int dim, const Q1Plan<T> &plan, const T *corners, unsigned long long *bar, int blocks,
+                            bool wide, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(blocks);
-    cfg.blockDim = dim3(w ? Q1_TPB_WIDE : Q1_TPB);
+    cfg.blockDim = dim3(wide && sizeof(T) == 4 ? Q1_TPB_WIDE : Q1_TPB);
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;   // all blocks co-resident: the grid barrier cannot wait on an unscheduled block
@@ -501,12 +614,38 @@ cudaError_t launch_q1_cycle(int dim, const Q1Plan<T> *plan, unsigned long long *
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     count_launches(1);
-    if (w) {
-        if (dim == 3) return cudaLaunchKernelEx(&cfg, k_q1_cycle<3, T, Q1_TPB_WIDE>, plan, bar);
-        return cudaLaunchKernelEx(&cfg, k_q1_cycle<2, T, Q1_TPB_WIDE>, plan, bar);
+    return cudaLaunchKernelEx(&cfg, q1_cycle_fn<T>(dim, wide), plan, corners, bar);
+}
+
+template <typename T>
+cudaError_t launch_q1_dense(int dim, const Q1Plan<T> &plan, int64_t n, const T *corners, cudaStream_t s) {
+    count_launches(1);
+    const unsigned grid = (unsigned)((n + Q1_TPB / 32 - 1) / (Q1_TPB / 32));
+    if (dim == 3)
+        k_q1_dense<3, T><<<grid, Q1_TPB, n * sizeof(T), s>>>(plan, corners);
+    else
+        k_q1_dense<2, T><<<grid, Q1_TPB, n * sizeof(T), s>>>(plan, corners);
+    return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_q1_weights(int64_t n, const T *diag, T omega, T *wd, cudaStream_t s) {
+    count_launches(1);
+    k_q1_weights<T><<<blocks_for(n), TPB, 0, s>>>(n, diag, omega, wd);
+    return cudaGetLastError();
+}
+
+// smem: bytes of the level vectors from dense_from down (4 per level)
+cudaError_t launch_q1_dense_matrix(int dim, const Q1Plan<double> &plan, int64_t nd, size_t smem, const double *Ainv,
+                                   double *E, cudaStream_t s) {
+    count_launches(1);
+    const auto fn = dim == 3 ? k_q1_dense_matrix<3> : k_q1_dense_matrix<2>;
+    if (smem > 32 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Q1_DENSE_SMEM);
+        if (e != cudaSuccess) return e;
     }
-    if (dim == 3) return cudaLaunchKernelEx(&cfg, k_q1_cycle<3, T, Q1_TPB>, plan, bar);
-    return cudaLaunchKernelEx(&cfg, k_q1_cycle<2, T, Q1_TPB>, plan, bar);
+    fn<<<(unsigned)nd, Q1_TPB, smem, s>>>(plan, Ainv, E);
+    return cudaGetLastError();
 }
 
 template <typename T>
@@ -575,9 +714,9 @@ cudaError_t launch_h_restrict(int dim, const CGLevelDev<T> &L, const T *rf, T *r
     if (ncv <= 0) return cudaSuccess;
     count_launches(1);
     if (dim == 3)
-        k_h_restrict<3, T><<<blocks_for(ncv), TPB, 0, s>>>(L, rf, rc);
+        k_h_restrict<3, T><<<blocks_for(ncv * RS_LANES), TPB, 0, s>>>(L, rf, rc);
     else
-        k_h_restrict<2, T><<<blocks_for(ncv), TPB, 0, s>>>(L, rf, rc);
+        k_h_restrict<2, T><<<blocks_for(ncv * RS_LANES), TPB, 0, s>>>(L, rf, rc);
     return cudaGetLastError();
 }
 
@@ -697,10 +836,13 @@ cudaError_t launch_coarse_solve_batch(const BatchCG<T> *D, const VertMap *map, i
 DGMG_CG_INST(double)
 DGMG_CG_INST(float)
 
-template cudaError_t launch_q1_cycle<double>(int, const Q1Plan<double> *, unsigned long long *, int, bool,
-                                              cudaStream_t);
-template cudaError_t launch_q1_cycle<float>(int, const Q1Plan<float> *, unsigned long long *, int, bool,
-                                             cudaStream_t);
+#define DGMG_Q1_INST(T)                                                                                               \
+    template cudaError_t launch_q1_cycle<T>(int, const Q1Plan<T> &, const T *, unsigned long long *, int, bool,        \
+                                            cudaStream_t);                                                            \
+    template cudaError_t launch_q1_dense<T>(int, const Q1Plan<T> &, int64_t, const T *, cudaStream_t);                 \
+    template cudaError_t launch_q1_weights<T>(int64_t, const T *, T, T *, cudaStream_t);
+DGMG_Q1_INST(double)
+DGMG_Q1_INST(float)
 template int q1_cycle_max_blocks<double>(int, bool);
 template int q1_cycle_max_blocks<float>(int, bool);
 

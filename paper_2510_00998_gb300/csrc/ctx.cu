@@ -708,17 +708,56 @@ int cg_vcycle(dgmg_ctx &C, int l, cudaStream_t s, T **result) {
     return DGMG_OK;
 }
 
-// The whole Q1 cycle from level 0 (RHS in cg[0].b) as one cooperative launch
-// when the context has its plan; the launch per step otherwise.
+// The whole Q1 cycle from level 0, its right-hand side the gather of the cells' corner
+// sums, as one launch when the context has its plan; the launch per step otherwise.
 template <typename T>
-int q1_cycle(dgmg_ctx &C, cudaStream_t s, T **result) {
+int q1_cycle(dgmg_ctx &C, const T *corners, cudaStream_t s, T **result) {
     auto &lv = cgl<T>(C);
-    Q1Plan<T> *plan = q1plan<T>(C);
-    if (!plan || C.q1_blocks <= 0 || g_q1_one_launch_off.load(std::memory_order_relaxed))
-        return cg_vcycle<T>(C, 0, s, result);
+    const Q1Plan<T> &plan = q1plan<T>(C);
     const int pi = std::is_same<T, float>::value ? 1 : 0;
-    LC(launch_q1_cycle<T>(C.dim, plan, C.q1bar + pi, C.q1_blocks_t[pi], C.q1_wide, s));
-    *result = lv.size() == 1 ? lv[0].u[0] : lv[0].u[(C.opts.nu_pre + C.opts.nu_post) & 1];
+    const bool one = C.q1_ready[pi];
+    if (one && C.q1_dense_from == 0) {
+        LC(launch_q1_dense<T>(C.dim, plan, lv[0].L.nv, corners, s));
+        *result = lv[0].u[0];
+        return DGMG_OK;
+    }
+    if (!one || g_q1_one_launch_off.load(std::memory_order_relaxed)) {
+        LC(launch_corner_gather<T>(C.dim, C.n, corners, lv[0].b, s));
+        return cg_vcycle<T>(C, 0, s, result);
+    }
+    LC(launch_q1_cycle<T>(C.dim, plan, corners, C.q1bar + pi, C.q1_blocks_t[pi], C.q1_wide, s));
+    *result = lv[0].u[(C.opts.nu_pre + C.opts.nu_post) & 1];
+    return DGMG_OK;
+}
+
+// The level from which the Q1 cycle is a dense product: the first of at most
+// Q1_DENSE_MAX vertices whose levels fit the set-up kernel's shared memory, else the
+// coarsest (whose inverse is dense already). smem: bytes of those levels' vectors.
+static int q1_dense_level(const std::vector<int64_t> &nv, size_t *smem = nullptr) {
+    int l = (int)nv.size() - 1;
+    size_t bytes = 4 * sizeof(double) * nv[l];
+    while (l > 0 && nv[l - 1] <= Q1_DENSE_MAX && bytes + 4 * sizeof(double) * nv[l - 1] <= Q1_DENSE_SMEM)
+        bytes += 4 * sizeof(double) * nv[--l];
+    if (smem) *smem = bytes;
+    return l;
+}
+
+// (Re)compute what the one-launch cycle takes from the levels' operators.
+static int q1_refresh(dgmg_ctx &C, cudaStream_t s) {
+    const int nl = (int)C.lv.size();
+    for (int l = 0; l + 1 < nl; ++l) {
+        const int64_t nv = C.lv[l].nv, d = (stencil_size(C.dim) / 2) * nv;
+        if (l < (int)C.q1wd64.size()) LC(launch_q1_weights<double>(nv, C.cg64[l].st + d, C.opts.omega_cg, C.q1wd64[l], s));
+        if (l < (int)C.q1wd32.size())
+            LC(launch_q1_weights<float>(nv, C.cg32[l].st + d, (float)C.opts.omega_cg, C.q1wd32[l], s));
+    }
+    if (C.q1_E) {
+        std::vector<int64_t> nv;
+        for (const CGLevelHost &H : C.lv) nv.push_back(H.nv);
+        size_t smem = 0;
+        const int ld = q1_dense_level(nv, &smem);
+        LC(launch_q1_dense_matrix(C.dim, C.q1plan64, nv[ld], smem, C.coarse_inv, C.q1_E, s));
+    }
     return DGMG_OK;
 }
 
@@ -740,21 +779,24 @@ int setup_q1_plan(dgmg_ctx &C) {
     auto &lv = cgl<T>(C);
     const int nl = (int)lv.size();
     if (nl == 0 || nl > Q1_MAXLEV || C.q1_blocks <= 0) return DGMG_OK;
-    Q1Plan<T> h;
-    std::memset(&h, 0, sizeof(h));
+    Q1Plan<T> &h = q1plan<T>(C);
+    const int pi = std::is_same<T, float>::value ? 1 : 0;
     h.nlev = nl;
     h.nu_pre = C.opts.nu_pre;
     h.nu_post = C.opts.nu_post;
-    h.omega = (T)C.opts.omega_cg;
-    h.ncoarse = lv[nl - 1].L.nv;
-    // the trailing levels small enough for one block: up to 512 vertices in
-    // FP32; in FP64 (about 2 FMA per clock per SM) only a one-vertex coarsest
-    // level (measured on the 32^3, p = 3 hierarchy: a 27-vertex level is
-    // faster on the whole grid, 146 against 159 us per cycle)
-    const int64_t local_max = std::is_same<T, float>::value ? 512 : 1;
-    h.local_from = nl;
-    while (h.local_from > 0 && lv[h.local_from - 1].L.nv <= local_max) --h.local_from;
-    h.Ainv = C.coarse_inv;
+    std::vector<int64_t> nv;
+    for (int l = 0; l < nl; ++l) nv.push_back(lv[l].L.nv);
+    const int ld = q1_dense_level(nv);
+    h.dense_from = C.q1_dense_from = ld;
+    h.ndense = nv[ld];
+    if (ld < nl - 1 && !C.q1_E) RC(C.alloc(&C.q1_E, nv[ld] * nv[ld]));   // by the FP64 plan, which comes first
+    h.E = ld < nl - 1 ? C.q1_E : C.coarse_inv;
+    auto &wd = q1wd<T>(C);
+    wd.assign(nl - 1, nullptr);
+    for (int l = 0; l + 1 < nl; ++l) {
+        RC(C.alloc(&wd[l], nv[l]));
+        h.wd[l] = wd[l];
+    }
     for (int l = 0; l < nl; ++l) {
         h.L[l] = lv[l].L;
         h.u0[l] = lv[l].u[0];
@@ -762,8 +804,10 @@ int setup_q1_plan(dgmg_ctx &C) {
         h.b[l] = lv[l].b;
         h.r[l] = lv[l].r;
     }
-    Q1Plan<T> *d = nullptr;
-    RC(C.upload(&d, std::vector<Q1Plan<T>>{h}));
+    if (ld == 0) {   // a plain launch
+        C.q1_ready[pi] = true;
+        return DGMG_OK;
+    }
     if (!C.q1bar) {
         RC(C.alloc(&C.q1bar, 2));
         DG_CUDA(cudaMemsetAsync(C.q1bar, 0, 2 * sizeof(unsigned long long), C.setup_stream));
@@ -774,9 +818,8 @@ int setup_q1_plan(dgmg_ctx &C) {
         cudaGraphExec_t exec = nullptr;
         bool ok = cudaStreamBeginCapture(C.capture_stream, cudaStreamCaptureModeRelaxed) == cudaSuccess;
         if (ok) {
-            const int pi = std::is_same<T, float>::value ? 1 : 0;
             const cudaError_t el =
-                launch_q1_cycle<T>(C.dim, d, C.q1bar + pi, C.q1_blocks_t[pi], C.q1_wide, C.capture_stream);
+                launch_q1_cycle<T>(C.dim, h, nullptr, C.q1bar + pi, C.q1_blocks_t[pi], C.q1_wide, C.capture_stream);
             g_kernel_launches.fetch_sub(1);   // captured, not launched
             const cudaError_t ee = cudaStreamEndCapture(C.capture_stream, &graph);
             ok = el == cudaSuccess && ee == cudaSuccess && graph &&
@@ -787,7 +830,7 @@ int setup_q1_plan(dgmg_ctx &C) {
         cudaGetLastError();
         capture_ok.store(ok ? 1 : 0);
     }
-    if (capture_ok.load() == 1) q1plan<T>(C) = d;   // else the plan stays unused
+    C.q1_ready[pi] = capture_ok.load() == 1;
     return DGMG_OK;
 }
 
@@ -827,11 +870,9 @@ int coarse_correction(dgmg_ctx &C, int l, T *z, const T *b, int cur, cudaStream_
         LC(launch_residual<T>(C.dim, S.q, D.c, tres, RES_HAS_B | RES_CORNERS, z, b, D.kappa, D.tr[cur], nullptr,
                               D.corners, exact_fd(C, D), s));
         C.prof.end(s);
-        auto &lv = cgl<T>(C);
         C.prof.begin(ST_CG, s);
-        LC(launch_corner_gather<T>(C.dim, C.n, D.corners, lv[0].b, s));
         T *e0 = nullptr;
-        RC(q1_cycle<T>(C, s, &e0));
+        RC(q1_cycle<T>(C, D.corners, s, &e0));
         C.prof.end(s);
         C.prof.begin(ST_PROJECT, s);
         LC(launch_project<T>(C.dim, S.q, D.c, tproj, z, e0, D.tr[0], s));   // z += P e0
@@ -1243,6 +1284,7 @@ int create_ctx(const dgmg_mesh *mesh, int p, const double *kappa, const dgmg_opt
             RC(C->alloc(&C->rold32, C->ndof));
         }
     }
+    RC(q1_refresh(*C, C->setup_stream));
     if (o.precision != DGMG_MIXED_FP32) RC(finish_factors(*C, S0, C->d64, C->setup_stream));
     RC(setup_dg_levels(*C, kap));
     trace.mark("dg levels");
@@ -1385,6 +1427,7 @@ int dgmg_update_kappa(dgmg_ctx *C, const double *kappa) {
         }
         RC(finish_factors(*C, C->dgs[l], D64, s));
     }
+    RC(q1_refresh(*C, s));
     DG_CUDA(cudaStreamSynchronize(s));
     return DGMG_OK;
 }
@@ -1572,12 +1615,14 @@ int dgmg_estimate_bytes(const dgmg_mesh *mesh, int p, const dgmg_opts *opts, siz
     size_t dg32 = sz(ncell, 4) + 2 * sz(ncell * dim * (q * q + q), 4) + 2 * sz(tr32, 4) + sz(ncell << dim, 4) +
                   sz(ncell * 2 * dim, 4);
     size_t cg64 = 0, cg32 = 0;
+    std::vector<int64_t> q1nv;
     int cur[3] = {n[0], n[1], n[2]};
     int64_t nv = 1;
     for (;;) {
         nv = (int64_t)(cur[0] - 1) * (dim >= 2 ? cur[1] - 1 : 1) * (dim == 3 ? cur[2] - 1 : 1);
         cg64 += sz(ns * nv, 8) + 4 * sz(nv, 8);
         cg32 += sz(ns * nv, 4) + 4 * sz(nv, 4);
+        q1nv.push_back(nv);
         bool any = false;
         for (int a = 0; a < dim; ++a) any = any || can_coarsen(cur[a], f);
         if (!any) break;
@@ -1597,8 +1642,12 @@ int dgmg_estimate_bytes(const dgmg_mesh *mesh, int p, const dgmg_opts *opts, siz
     size_t total = sz(nv * nv, 8) + dg64 + cg64 + 5 * sz(ndof, 8) + sz(S_NSCAL, 8) + sz(DOT_WORK, 8) +
                    sz(p + 2, 8) + sz((int64_t)q * (p + 2), 8) + sz(3 * (p + 2), 8);
     if (mixed) total += dg32 + cg32 + 2 * sz(ndof, 4) + (reliable ? 4 * sz(ndof, 4) : 0);
-    if (q1_blocks_for(dim, mixed) > 0)   // the plans of the cooperative Q1 cycle and their counters
-        total += sizeof(Q1Plan<double>) + (mixed ? sizeof(Q1Plan<float>) : 0) + 2 * sizeof(unsigned long long);
+    if (q1_blocks_for(dim, mixed) > 0) {   // the counters, weights and matrix of the one-launch Q1 cycle
+        const int ld = q1_dense_level(q1nv);
+        if (ld > 0) total += 2 * sizeof(unsigned long long);
+        for (size_t l = 0; l + 1 < q1nv.size(); ++l) total += q1nv[l] * (mixed ? 12 : 8);
+        if (ld + 1 < (int)q1nv.size()) total += q1nv[ld] * q1nv[ld] * 8;
+    }
     if (o.p_coarsening == 1 && p >= 2) {
         // lower DG levels p-1 .. 1 (kappa shared with the finest level): factors,
         // traces, corners, iterate, right-hand side and residual; FP64 also the

@@ -141,13 +141,18 @@ struct dgmg_ctx {
     std::vector<CGLevelHost> lv;
     int64_t ncoarse = 0;
     double *coarse_inv = nullptr;
-    // the Q1 cycle as one cooperative launch (q1_blocks > 0): per precision its
-    // plan and two barrier words; q1_blocks = 0 keeps the launch per step
-    Q1Plan<double> *q1plan64 = nullptr;
-    Q1Plan<float> *q1plan32 = nullptr;
+    // the Q1 cycle as one launch (q1_blocks > 0): per precision its plan and a
+    // barrier word; q1_blocks = 0 keeps the launch per step
+    Q1Plan<double> q1plan64 = {};
+    Q1Plan<float> q1plan32 = {};
+    bool q1_ready[2] = {false, false};             // the plan is used [FP64, FP32]
     unsigned long long *q1bar = nullptr;          // arrival counters [FP64, FP32]
     int q1_blocks = 0;
     int q1_blocks_t[2] = {0, 0};                   // blocks of the cycle per precision [FP64, FP32]
+    int q1_dense_from = 0;                         // level from which the cycle is a product with q1_E
+    double *q1_E = nullptr;                        // (null: with the inverse of the coarsest operator)
+    std::vector<double *> q1wd64;                  // omega / diagonal of the levels
+    std::vector<float *> q1wd32;
     bool q1_wide = true;                           // FP32 cycle in 512-thread blocks
     DGDev<double> d64;
     DGDev<float> d32;
@@ -330,7 +335,14 @@ inline const DGDev<T> &dg(const dgmg_ctx &C) {
         return C.d64;
 }
 template <typename T>
-inline Q1Plan<T> *&q1plan(dgmg_ctx &C) {
+inline std::vector<T *> &q1wd(dgmg_ctx &C) {
+    if constexpr (std::is_same<T, float>::value)
+        return C.q1wd32;
+    else
+        return C.q1wd64;
+}
+template <typename T>
+inline Q1Plan<T> &q1plan(dgmg_ctx &C) {
     if constexpr (std::is_same<T, float>::value)
         return C.q1plan32;
     else

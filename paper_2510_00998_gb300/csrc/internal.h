@@ -233,12 +233,14 @@ struct BatchCG {
     int n[3];
     const T *corners;
 };
-// The Q1 h-cycle of one problem as one cooperative launch: every level's
-// operator and transfer tables, its vectors, the coarsest inverse.
+// The Q1 h-cycle of one problem as one launch: every level's operator and transfer
+// tables, its vectors, the matrix of the small levels. A kernel argument: read from
+// device memory it cost every step two round trips to L2 more (a barrier's acquire
+// empties L1).
 constexpr int Q1_MAXLEV = 24;
 // threads per block of the cooperative cycle: 256, or (FP32, wide) 512: one
 // block per SM, more loads of the vertex loops in flight, fewer barrier
-// arrivals, and 512 threads for the levels run in block 0. A 512-thread block
+// arrivals. A 512-thread block
 // holds a whole SM's registers, so its cooperative launch waits for empty SMs
 // where other solves share the GPU (the solve server keeps 256); in FP64 the
 // 512-thread kernel spills.
@@ -246,19 +248,35 @@ constexpr int Q1_TPB = 256, Q1_TPB_WIDE = 512;
 template <typename T>
 struct Q1Plan {
     int nlev, nu_pre, nu_post;
-    int local_from;        // levels >= this one run in one block (nlev: none)
-    T omega;
-    int64_t ncoarse;
-    const double *Ainv;
+    int dense_from;        // the cycle from this level down is the product with E (at most nlev - 1)
+    int64_t ndense;        // vertices of that level
+    const double *E;       // ndense x ndense, row-major
     CGLevelDev<T> L[Q1_MAXLEV];
+    const T *wd[Q1_MAXLEV];   // omega / diagonal of the levels above the coarsest
     T *u0[Q1_MAXLEV], *u1[Q1_MAXLEV], *b[Q1_MAXLEV], *r[Q1_MAXLEV];
 };
-// e on level 0 (u0 or u1 of level 0, by the parity of nu_pre + nu_post) from b
-// on level 0; bar: the plan's own arrival counter (zero before its first
-// launch; every launch on it with the same number of blocks)
+// Levels of at most this many vertices are the dense ones (the first such level of a
+// hierarchy and all below it). The product costs ndense^2 FP64 multiply-adds on the
+// whole chip (3.8 us at 1331 vertices) and one barrier, the steps it replaces 7 barriers
+// (1.3 us) and 7 steps of 1.5 to 5 us a level; the matrix takes 0.65 ms of the set-up at
+// 1331 vertices (growing with their square), and 8 ndense^2 bytes. One cycle, level per
+// level in block-wide or grid-wide steps / with the product: FP64 16^2 p = 2 69 / 6 us,
+// 23^3 p = 2 131 / 42, FP64 V-cycles 109 / 52 and 237 / 149 us.
+constexpr int64_t Q1_DENSE_MAX = 1536;
+constexpr size_t Q1_DENSE_SMEM = 160 * 1024;   // level vectors of the set-up kernel, at most
+// e on level 0 (u0 or u1 of level 0, by the parity of nu_pre + nu_post) from the
+// cells' corner sums; bar: the plan's own arrival counter (zero before its first
+// launch; every launch on it with the same number of blocks); dense_from > 0
 template <typename T>
-cudaError_t launch_q1_cycle(int dim, const Q1Plan<T> *plan, unsigned long long *bar, int blocks, bool wide,
-                            cudaStream_t s);
+cudaError_t launch_q1_cycle(int dim, const Q1Plan<T> &plan, const T *corners, unsigned long long *bar, int blocks,
+                            bool wide, cudaStream_t s);
+// the same of a plan with dense_from = 0 (n = ndense), into u0 of level 0
+template <typename T>
+cudaError_t launch_q1_dense(int dim, const Q1Plan<T> &plan, int64_t n, const T *corners, cudaStream_t s);
+template <typename T>
+cudaError_t launch_q1_weights(int64_t n, const T *diag, T omega, T *wd, cudaStream_t s);
+cudaError_t launch_q1_dense_matrix(int dim, const Q1Plan<double> &plan, int64_t nd, size_t smem, const double *Ainv,
+                                   double *E, cudaStream_t s);
 // the most blocks of the cooperative launch (one per SM), 0 if it cannot run
 template <typename T>
 int q1_cycle_max_blocks(int dim, bool wide);
