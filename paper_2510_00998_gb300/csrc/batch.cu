@@ -688,8 +688,10 @@ std::vector<BatchDG<T>> group_descriptors(const dgmg_batch &B, const dgmg_batch:
         d.off = cells;
         d.kappa = dg.kappa;
         d.fd = dg.fd;
-        if constexpr (std::is_same<T, float>::value) d.fdr = dg.fdr;
-        d.linv = dg.linv;
+        if constexpr (std::is_same<T, float>::value)
+            d.fdr = dg.fdr;
+        else
+            d.linv = dg.linv;
         d.tr[0] = dg.tr[0];
         d.tr[1] = dg.tr[1];
         d.corners = dg.corners;

@@ -29,7 +29,6 @@ struct Geo {
     static constexpr int NF = NL / Q;                          // nodes per face = threads per cell
     static constexpr int NFACE = 2 * DIM;
     static constexpr int FS = trace_face_stride<T>(NF);         // trace values per face (padded)
-    static constexpr int TR = NFACE * FS;                      // trace values per cell
     static constexpr int NC = 1 << DIM;                        // corners per cell
     static constexpr int FDS = Q * Q + Q;                      // fast-diag factors per axis (global)
     static constexpr int VEC = 16 / (int)sizeof(T);            // elements per 16-byte vector
@@ -37,6 +36,15 @@ struct Geo {
     static constexpr int QQV = (Q * Q + VEC - 1) / VEC;        // 16-byte vectors covering S
     static constexpr int NDOT = NFACE * 2 * (DIM == 3 ? Q : 1); // facet-mass dot products per cell
     static constexpr int NLC = NFACE * 2 * Q;                  // lifting coefficients per cell
+    // Traces are stored face by face, [face][cell][FS]: the faces of a run of cells, and
+    // those of their neighbours along an axis, are one piece of memory each.
+    template <typename P>
+    static __device__ __forceinline__ P *face(P *tr, int64_t ncell, int64_t cell, int f) {
+        return tr + (f * ncell + cell) * FS;
+    }
+    // index within a face of the pencil at tangential position t (3D: the tangential
+    // axes in cyclic order after the normal one)
+    static __device__ __forceinline__ int fidx(int dir, int t) { return DIM == 3 && dir == 1 ? t / Q + Q * (t % Q) : t; }
     // volume index of node i of the pencil along `dir` at tangential position t
     static __device__ __forceinline__ int vidx(int dir, int t, int i) {
         if (DIM == 2) return dir == 0 ? i + Q * t : t + Q * i;
@@ -120,9 +128,10 @@ __device__ __forceinline__ void load_neighbour_traces(const DGConst<T> &c, int64
         T g = T(0), h = T(0);
         if (inside) {
             const int64_t nb = cell + (side ? axis_stride<DIM>(c.n, dir) : -axis_stride<DIM>(c.n, dir));
-            const T *src = tr + nb * G::TR + (f ^ 1) * G::FS;
-            g = src[t];
-            h = src[G::NF + t];
+            const T *src = G::face(tr, c.ncell, nb, f ^ 1);
+            const int ft = G::fidx(dir, t);
+            g = src[ft];
+            h = src[G::NF + ft];
         }
         sF[(f * 2 + 0) * G::NF + t] = g;
         sF[(f * 2 + 1) * G::NF + t] = h;
@@ -387,7 +396,7 @@ __device__ __forceinline__ void subtract_block_apply(const DGConst<T> &c, bool a
 // the facet spaces), written to the trace array.
 template <int DIM, int Q, typename T>
 __device__ __forceinline__ void write_pencil_traces(const DGConst<T> &c, int dir, int t, const T *x,
-                                                    T *__restrict__ trc) {
+                                                    T *__restrict__ tr, int64_t cell) {
     using G = Geo<DIM, Q, T>;
     T dlo = T(0), dhi = T(0);
 #pragma unroll
@@ -405,12 +414,13 @@ __device__ __forceinline__ void write_pencil_traces(const DGConst<T> &c, int dir
             vhi += c.vp[i] * x[i];
         }
     }
-    T *lo = trc + (2 * dir) * G::FS;
-    T *hi = trc + (2 * dir + 1) * G::FS;
-    lo[t] = vlo;
-    lo[G::NF + t] = dlo;
-    hi[t] = vhi;
-    hi[G::NF + t] = dhi;
+    T *lo = G::face(tr, c.ncell, cell, 2 * dir);
+    T *hi = G::face(tr, c.ncell, cell, 2 * dir + 1);
+    const int ft = G::fidx(dir, t);
+    lo[ft] = vlo;
+    lo[G::NF + ft] = dlo;
+    hi[ft] = vhi;
+    hi[G::NF + ft] = dhi;
 }
 
 // ---------------------------------------------------------------------------
@@ -445,7 +455,6 @@ __device__ __forceinline__ void k_project_body(const DGConst<T> &c, int64_t cell
         }
     }
     __syncthreads();
-    T *trc = tr + cell * G::TR;
     // pass along x: prolongation and x-face traces
     if (active) {
         T x[Q];
@@ -470,7 +479,7 @@ __device__ __forceinline__ void k_project_body(const DGConst<T> &c, int64_t cell
 #pragma unroll
             for (int i = 0; i < Q; ++i) pu[G::vidx(0, t, i)] = x[i];
         }
-        write_pencil_traces<DIM, Q, T>(c, 0, t, x, trc);
+        write_pencil_traces<DIM, Q, T>(c, 0, t, x, tr, cell);
     }
     if (e0 != nullptr) __syncthreads();
     if (active) {
@@ -480,7 +489,7 @@ __device__ __forceinline__ void k_project_body(const DGConst<T> &c, int64_t cell
             const T *pu = sU + lc * G::NL;
 #pragma unroll
             for (int i = 0; i < Q; ++i) x[i] = pu[G::vidx(dir, t, i)];
-            write_pencil_traces<DIM, Q, T>(c, dir, t, x, trc);
+            write_pencil_traces<DIM, Q, T>(c, dir, t, x, tr, cell);
         }
     }
     if (e0 != nullptr) {
@@ -511,7 +520,7 @@ __global__ void __launch_bounds__(256) k_project(DGConst<T> c, int cpb, T *__res
 // tr_out (ping-pong: every cell reads projections of the same iterate).
 // ---------------------------------------------------------------------------
 template <int DIM, int Q, typename T>
-__device__ __forceinline__ void k_smooth_body(const DGConst<T> &c, int64_t cell0, int cpb, int exact, int flags, T *__restrict__ u, const T *__restrict__ b, const T *__restrict__ kappa, const T *__restrict__ fd, const T *__restrict__ linv, const T *__restrict__ tr_in, T *__restrict__ tr_out) {
+__device__ __forceinline__ void k_smooth_body(const DGConst<T> &c, int64_t cell0, int cpb, int exact, int flags, T *__restrict__ u, const T *__restrict__ b, const T *__restrict__ kappa, const T *__restrict__ fd, const T *__restrict__ tr_in, T *__restrict__ tr_out) {
     using G = Geo<DIM, Q, T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *sFD = reinterpret_cast<T *>(smem_raw);   // [cpb][DIM][FDSP], 16-byte aligned blocks
@@ -600,16 +609,12 @@ __device__ __forceinline__ void k_smooth_body(const DGConst<T> &c, int64_t cell0
             }
 #pragma unroll
             for (int i = 0; i < Q; ++i) x[i] = myR[G::vidx(D, t, i)];
-            // 1 / (lambda_x + lambda_y + lambda_z): from the per-node table when
-            // one is given (saves a division per node; the table holds omega /
-            // the sum, so the damping is then already applied), else divided here
-            const T *li = linv ? linv + cell * G::NL : nullptr;
 #pragma unroll
             for (int i = 0; i < Q; ++i) {
                 T s = T(0);
 #pragma unroll
                 for (int m = 0; m < Q; ++m) s += S[m * Q + i] * x[m];
-                y[i] = li ? s * li[G::vidx(D, t, i)] : s / (lt + lam[i]);
+                y[i] = s / (lt + lam[i]);
             }
 #pragma unroll
             for (int m = 0; m < Q; ++m) {
@@ -644,7 +649,6 @@ __device__ __forceinline__ void k_smooth_body(const DGConst<T> &c, int64_t cell0
         __syncthreads();
     }
     // axis 0: S, damped update, x-face traces
-    T *trc = tr_out + cell * G::TR;
     if (active) {
         T x[Q], un[Q];
         __align__(16) T S[G::QQV * G::VEC];
@@ -658,11 +662,11 @@ __device__ __forceinline__ void k_smooth_body(const DGConst<T> &c, int64_t cell0
             T s = T(0);
 #pragma unroll
             for (int i = 0; i < Q; ++i) s += S[m * Q + i] * x[i];
-            un[m] = linv ? keep * myU[G::vidx(0, t, m)] + s : keep * myU[G::vidx(0, t, m)] + om * s;
+            un[m] = keep * myU[G::vidx(0, t, m)] + om * s;
         }
 #pragma unroll
         for (int i = 0; i < Q; ++i) myU[G::vidx(0, t, i)] = un[i];
-        if (!(flags & SM_NO_TRACES)) write_pencil_traces<DIM, Q, T>(c, 0, t, un, trc);
+        if (!(flags & SM_NO_TRACES)) write_pencil_traces<DIM, Q, T>(c, 0, t, un, tr_out, cell);
     }
     __syncthreads();
     if (active && !(flags & SM_NO_TRACES)) {
@@ -671,15 +675,15 @@ __device__ __forceinline__ void k_smooth_body(const DGConst<T> &c, int64_t cell0
             T x[Q];
 #pragma unroll
             for (int i = 0; i < Q; ++i) x[i] = myU[G::vidx(dir, t, i)];
-            write_pencil_traces<DIM, Q, T>(c, dir, t, x, trc);
+            write_pencil_traces<DIM, Q, T>(c, dir, t, x, tr_out, cell);
         }
     }
     block_copy(u + cell0 * G::NL, sU, (int64_t)ncl * G::NL);
 }
 
 template <int DIM, int Q, typename T>
-__global__ void __launch_bounds__(256) k_smooth(DGConst<T> c, int cpb, int exact, int flags, T *__restrict__ u, const T *__restrict__ b, const T *__restrict__ kappa, const T *__restrict__ fd, const T *__restrict__ linv, const T *__restrict__ tr_in, T *__restrict__ tr_out) {
-    k_smooth_body<DIM, Q, T>(c, (int64_t)blockIdx.x * cpb, cpb, exact, flags, u, b, kappa, fd, linv, tr_in, tr_out);
+__global__ void __launch_bounds__(256) k_smooth(DGConst<T> c, int cpb, int exact, int flags, T *__restrict__ u, const T *__restrict__ b, const T *__restrict__ kappa, const T *__restrict__ fd, const T *__restrict__ tr_in, T *__restrict__ tr_out) {
+    k_smooth_body<DIM, Q, T>(c, (int64_t)blockIdx.x * cpb, cpb, exact, flags, u, b, kappa, fd, tr_in, tr_out);
 }
 
 // ---------------------------------------------------------------------------
@@ -838,7 +842,7 @@ __global__ void __launch_bounds__(256) k_smooth_batch(const BatchDG<T> *__restri
         const BlockMap m = map[k];
         load_batch_desc(D + m.inst, &sd);
         k_smooth_body<DIM, Q, T>(sd.c, m.cell0, cpb, exact, flags, u + sd.off * G::NL, b + sd.off * G::NL, sd.kappa, sd.fd,
-                                 sd.linv, sd.tr[cur], sd.tr[cur ^ 1]);
+                                 sd.tr[cur], sd.tr[cur ^ 1]);
     }
 }
 
@@ -852,7 +856,7 @@ __global__ void __launch_bounds__(32) k_smooth_cells_batch(const BatchDG<T> *__r
         if (k != (int)blockIdx.x) __syncthreads();
         const BlockMap m = map[k];
         load_batch_desc(D + m.inst, &sd);
-        smooth_cells_body<T, Q>(sd.c, m.cell0, flags, u + sd.off * NL, b + sd.off * NL, sd.kappa, sd.fd, sd.linv,
+        smooth_cells_body<T, Q>(sd.c, m.cell0, flags, u + sd.off * NL, b + sd.off * NL, sd.fd,
                                 sd.tr[cur], sd.tr[cur ^ 1], k != (int)blockIdx.x);
     }
 }
@@ -931,10 +935,8 @@ struct DGLaunch {
     static int default_cpb() { return std::max(1, 256 / G::NF); }
     static cudaError_t project(const DGConst<T> &c, int cpb, T *u, const T *e0, T *tr, cudaStream_t s) {
         if constexpr (CELLS_OK) if (c.ncell < (int64_t(1) << 31)) {   // 32-bit cell indices
-            // bulk copies want a 16-byte aligned u; the trace pieces 8- (FP32) or 16-byte (FP64) aligned traces
-            const uintptr_t tra = 15;   // bulk copies of whole (padded) faces
-            if (cpb <= 0 && !c.gl && (reinterpret_cast<uintptr_t>(u) & 15) == 0 &&
-                (reinterpret_cast<uintptr_t>(tr) & tra) == 0) {
+            // bulk copies want 16-byte aligned u and traces
+            if (cpb <= 0 && !c.gl && ((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(tr)) & 15) == 0) {
                 using CG = CellGeo<T, Q>;
                 static bool attr_c = false;
                 if (!attr_c) {
@@ -963,15 +965,13 @@ struct DGLaunch {
         return cudaGetLastError();
     }
     static cudaError_t smooth(const DGConst<T> &c, int cpb, int exact, int flags, T *u, const T *b, const T *kappa,
-                              const T *fd, const T *linv, const T *tri, T *tro, cudaStream_t s) {
+                              const T *fd, const T *tri, T *tro, cudaStream_t s) {
         if constexpr (CELLS_OK) if (c.ncell < (int64_t(1) << 31)) {   // 32-bit cell indices
-            // bulk copies want 16-byte aligned vectors, factors and table; the face
-            // pieces 8- (FP32) or 16-byte (FP64) aligned traces
-            const uintptr_t tra = 15;   // bulk copies of whole (padded) faces
+            // bulk copies want 16-byte aligned vectors, factors and traces
             const bool aligned = ((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(b) |
-                                   reinterpret_cast<uintptr_t>(fd) | reinterpret_cast<uintptr_t>(linv)) & 15) == 0 &&
-                                 ((reinterpret_cast<uintptr_t>(tri) | reinterpret_cast<uintptr_t>(tro)) & tra) == 0;
-            if (cpb <= 0 && exact && aligned && !c.gl) return smooth_cells(c, flags, u, b, kappa, fd, linv, tri, tro, s);
+                                   reinterpret_cast<uintptr_t>(fd) | reinterpret_cast<uintptr_t>(tri) |
+                                   reinterpret_cast<uintptr_t>(tro)) & 15) == 0;
+            if (cpb <= 0 && exact && aligned && !c.gl) return smooth_cells(c, flags, u, b, fd, tri, tro, s);
         }
         if (cpb <= 0) cpb = default_cpb();
         const size_t sm = smem_smooth<DIM, Q, T>(cpb, exact != 0);
@@ -983,15 +983,14 @@ struct DGLaunch {
         const int64_t grid = (c.ncell + cpb - 1) / cpb;
         if (grid == 0) return cudaSuccess;
         count_launches(1);
-        k_smooth<DIM, Q, T><<<(unsigned)grid, cpb * G::NF, sm, s>>>(c, cpb, exact, flags, u, b, kappa, fd, linv, tri,
-                                                                    tro);
+        k_smooth<DIM, Q, T><<<(unsigned)grid, cpb * G::NF, sm, s>>>(c, cpb, exact, flags, u, b, kappa, fd, tri, tro);
         return cudaGetLastError();
     }
-    // 3D exact-block smoothing step with one thread per cell (k_smooth_cells):
-    // FP32 q <= 5, FP64 q <= 4 (the cell must fit in the registers of a thread)
-    static constexpr bool CELLS_OK = DIM == 3 && (std::is_same<T, float>::value ? Q <= 5 : Q <= 4);
-    static cudaError_t smooth_cells(const DGConst<T> &c, int flags, T *u, const T *b, const T *kappa, const T *fd,
-                                    const T *linv, const T *tri, T *tro, cudaStream_t s) {
+    // 3D kernels with one thread per cell: q <= 5 (the cell must fit in the registers
+    // of a thread)
+    static constexpr bool CELLS_OK = DIM == 3 && Q <= 5;
+    static cudaError_t smooth_cells(const DGConst<T> &c, int flags, T *u, const T *b, const T *fd, const T *tri, T *tro,
+                                    cudaStream_t s) {
         if constexpr (CELLS_OK) {
             using CG = CellGeo<T, Q>;
             static bool attr = false;
@@ -1003,7 +1002,7 @@ struct DGLaunch {
             const int64_t grid = (c.ncell + CG::W - 1) / CG::W;
             if (grid == 0) return cudaSuccess;
             count_launches(1);
-            k_smooth_cells<T, Q><<<(unsigned)grid, CG::W, CG::BYTES, s>>>(c, flags, u, b, kappa, fd, linv, tri, tro);
+            k_smooth_cells<T, Q><<<(unsigned)grid, CG::W, CG::BYTES, s>>>(c, flags, u, b, fd, tri, tro);
             return cudaGetLastError();
         } else {
             return cudaErrorInvalidValue;
@@ -1031,7 +1030,7 @@ struct DGLaunch {
     // the direct-form one-thread-per-cell residual (FP32: the CG operator)
     static cudaError_t residual_cells_direct(const DGConst<T> &c, int mode, const T *u, const T *b, const T *kappa,
                                              const T *tr, T *r, T *corners, cudaStream_t s) {
-        if constexpr (CELLS_OK && sizeof(T) == 4) {
+        if constexpr (CELLS_OK) {
             using CG = CellGeo<T, Q>;
             static bool attr = false;
             if (!attr) {
@@ -1101,22 +1100,19 @@ struct DGLaunch {
                                       const T *u, const T *b, T *r, int cur, cudaStream_t s) {
         if (nblocks <= 0) return cudaSuccess;
         if constexpr (CELLS_OK) {
-            if constexpr (sizeof(T) == 4) {
-                if (cpb <= 0 && (mode & RES_DIRECT)) {   // the FP32 CG operator: no b, no corners
-                    using CG = CellGeo<T, Q>;
-                    static bool attr = false;
-                    if (!attr) {
-                        cudaFuncSetAttribute(k_residual_cells_batch_direct<T, Q>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CG::BYTES);
-                        attr = true;
-                    }
-                    count_launches(1);
-                    k_residual_cells_batch_direct<T, Q>
-                        <<<persistent_grid((const void *)k_residual_cells_batch_direct<T, Q>, CG::W, CG::BYTES,
-                                           nblocks),
-                           CG::W, CG::BYTES, s>>>(D, map, nblocks, mode, u, r, cur);
-                    return cudaGetLastError();
+            if (cpb <= 0 && (mode & RES_DIRECT)) {   // the CG operator: no b, no corners
+                using CG = CellGeo<T, Q>;
+                static bool attr = false;
+                if (!attr) {
+                    cudaFuncSetAttribute(k_residual_cells_batch_direct<T, Q>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CG::BYTES);
+                    attr = true;
                 }
+                count_launches(1);
+                k_residual_cells_batch_direct<T, Q>
+                    <<<persistent_grid((const void *)k_residual_cells_batch_direct<T, Q>, CG::W, CG::BYTES, nblocks),
+                       CG::W, CG::BYTES, s>>>(D, map, nblocks, mode, u, r, cur);
+                return cudaGetLastError();
             }
             if (cpb <= 0) {          // the map holds 32-cell blocks; every problem carries its factors
                 using CG = CellGeo<T, Q>;
@@ -1149,17 +1145,15 @@ struct DGLaunch {
     static cudaError_t residual(const DGConst<T> &c, int cpb, int mode, const T *u, const T *b, const T *kappa,
                                 const T *tr, T *r, T *corners, const T *fd, cudaStream_t s) {
         if constexpr (CELLS_OK) if (c.ncell < (int64_t(1) << 31)) {   // 32-bit cell indices
-            // bulk copies of u, b, the factors and r want 16-byte alignment; the
-            // face pieces 8- (FP32) or 16-byte (FP64) aligned traces
-            const uintptr_t tra = 15;   // bulk copies of whole (padded) faces
+            // bulk copies of u, b, the factors, the traces and r want 16-byte alignment
             const uintptr_t vec = reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(fd) |
+                                  reinterpret_cast<uintptr_t>(tr) |
                                   ((mode & RES_HAS_B) ? reinterpret_cast<uintptr_t>(b) : 0) |
                                   ((mode & RES_WRITE_R) ? reinterpret_cast<uintptr_t>(r) : 0);
-            if (cpb <= 0 && fd && !c.gl && (vec & 15) == 0 && (reinterpret_cast<uintptr_t>(tr) & tra) == 0)
+            if (cpb <= 0 && fd && !c.gl && (vec & 15) == 0)
                 return residual_cells(c, mode, u, b, kappa, fd, tr, r, corners, s);
-            // without factors (the FP32 CG operator): A_KK u in the direct form
-            if (sizeof(T) == 4 && cpb <= 0 && !fd && !c.gl && (vec & 15) == 0 &&
-                (reinterpret_cast<uintptr_t>(tr) & tra) == 0)
+            // without factors (the CG operator): A_KK u in the direct form
+            if (cpb <= 0 && !fd && !c.gl && (vec & 15) == 0)
                 return residual_cells_direct(c, mode, u, b, kappa, tr, r, corners, s);
         }
         if (cpb <= 0) cpb = default_cpb();
@@ -1201,8 +1195,8 @@ cudaError_t launch_project_impl(int dim, int q, const DGConst<T> &c, int cpb, T 
 }
 template <typename T>
 cudaError_t launch_smooth_impl(int dim, int q, const DGConst<T> &c, int cpb, int exact, int flags, T *u, const T *b,
-                               const T *kappa, const T *fd, const T *linv, const T *tri, T *tro, cudaStream_t s) {
-    DGMG_DISPATCH(dim, q, smooth(c, cpb, exact, flags, u, b, kappa, fd, linv, tri, tro, s))
+                               const T *kappa, const T *fd, const T *tri, T *tro, cudaStream_t s) {
+    DGMG_DISPATCH(dim, q, smooth(c, cpb, exact, flags, u, b, kappa, fd, tri, tro, s))
 }
 template <typename T>
 cudaError_t launch_residual_impl(int dim, int q, const DGConst<T> &c, int cpb, int mode, const T *u, const T *b,

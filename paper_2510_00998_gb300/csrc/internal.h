@@ -29,11 +29,14 @@ int cuda_fail(cudaError_t e, const char *what);
 
 // Values stored per cell face in a trace buffer: the value and the normal
 // derivative at the q^(d-1) face nodes, padded so that every face of every cell
-// starts on a 16-byte boundary (a bulk copy moves one face). Only FP32 with an
-// odd number of face nodes pads (2 values per face for q = 5 in 3D).
+// starts on a 16-byte boundary (bulk copies). FP32: to an odd number of 16-byte
+// units, so that the lanes of a warp, a face each, read and write shared memory by
+// 16-byte accesses without bank conflicts (52 values for q = 5 in 3D, 36 for q = 4,
+// whose 32 would put all lanes on one bank).
 template <typename T>
 __host__ __device__ constexpr int trace_face_stride(int nf) {
-    return (2 * nf * (int)sizeof(T) + 15) / 16 * 16 / (int)sizeof(T);
+    const int units = (2 * nf * (int)sizeof(T) + 15) / 16;
+    return (sizeof(T) == 4 ? units | 1 : units) * 16 / (int)sizeof(T);
 }
 
 // Process-wide count of kernels launched by the library (dgmg_kernel_launches).
@@ -201,7 +204,7 @@ template <typename T>
 struct BatchDG {
     DGConst<T> c;
     int64_t off;
-    const T *kappa, *fd, *linv;
+    const T *kappa, *fd;
     const T *fdr;         // the residual's factors [S^T M | lambda] (null: operator-only level)
     T *tr[2];
     T *corners;

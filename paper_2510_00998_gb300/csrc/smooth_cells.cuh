@@ -1,5 +1,5 @@
-// Single-touch smoothing step (Algorithm 4, exact diagonal blocks) with one
-// thread per cell, 3D: FP32 for q <= 5, FP64 for q <= 4 nodes per axis.
+// Single-touch smoothing step (Algorithm 4, exact diagonal blocks), residual and
+// projection with one thread per cell, 3D, FP32, q <= 5 nodes per axis.
 //
 // Each thread keeps its whole cell (q^3 values) in registers, so the six
 // tensor passes of the fast-diagonalisation inverse need no transposes through
@@ -7,19 +7,15 @@
 // staged in shared memory in the order they are consumed:
 //   - b and the fast-diagonalisation factors: one bulk (TMA) copy each,
 //     completing on an mbarrier;
-//   - the neighbours' traces, face by face through two slots: every lane
-//     fetches its neighbour's face with one bulk copy (faces are padded to
-//     16 bytes in the trace buffers), the copies of a face completing on one
-//     mbarrier whose byte count lane 0 posts;
-//   - FP32: u of the previous iterate by a bulk copy into the slot area once
-//     the faces are consumed, overlapping the inverse;
-//   - FP64: the per-node table of inverse eigenvalue sums into the slot area
-//     once the faces are consumed (FP64 division is a long sequence on the
-//     FP64 pipe, which bounds the FP64 kernel), then u of the previous iterate
-//     into the same area once the table is used, overlapping the last passes.
+//   - the neighbours' traces, face by face through two slots: traces are stored
+//     [face][cell], so a face of all 32 neighbours is one bulk copy;
+//   - u of the previous iterate by a bulk copy into the slot area once
+//     the faces are consumed, overlapping the inverse.
 // The new u leaves through a bulk store; every lane writes its new traces into
-// its face slots and stores each face with one bulk store. A lane reads its own cell with stride q^3 (odd for odd
-// q, so a warp's 32 loads hit 32 banks).
+// its part of a face slot, and a slot leaves by one bulk store. All of a lane's accesses
+// to shared memory are free of bank conflicts (odd strides, of words or of 16-byte
+// units). Cells with an even number of values (q = 2, 4) are padded in shared memory and
+// come by 16-byte asynchronous copies.
 //
 // The split update of the exact block (u <- (1 - w) u + w A_KK^{-1}(b - N u_nb))
 // needs only the neighbours' traces and b before the inverse, so u itself is
@@ -127,25 +123,22 @@ __device__ __forceinline__ void cell_coords32(int64_t cell, const int *n, int *c
 template <typename T, int Q>
 struct CellGeo {
     static constexpr int NL = Q * Q * Q, NF = Q * Q, FDS = Q * Q + Q;
-    static constexpr int FS = trace_face_stride<T>(NF), TR = 6 * FS;   // trace values per face / cell
-    static constexpr int W = 32;                       // cells per CTA (one per lane)
-    // FP64 (LEAN): the kernel is bound by the FP64 pipe, not by memory, so the
-    // neighbour faces, the table and the previous u are read straight from
-    // global memory by each lane and the traces written the same way; only
-    // area A is staged. That halves the shared memory per CTA, so more CTAs
-    // are resident (a 32^3 mesh fits in one wave).
-    static constexpr bool LEAN = sizeof(T) == 8;
-    // shared memory (values of T), per cell. FP32 smoothing step: area A holds
+    static constexpr int FS = trace_face_stride<T>(NF);   // trace values per face
+    static constexpr int W = 32;                          // cells per CTA (one per lane)
+    // stride of the cells in shared memory: odd (q odd), or an odd number of 16-byte
+    // units accessed as such (q even): a lane's accesses to its own cell have no bank
+    // conflicts (at stride 64, q = 4, all lanes would hit one bank)
+    static constexpr bool PADDED = NL % 2 == 0;
+    static constexpr int CS = PADDED ? (NL / 4 | 1) * 4 : NL;
+    // shared memory (values of T), per cell. Smoothing step: area A holds
     // b, then one neighbour-face slot (FS values) during the facet lifting, then
     // the previous u, then the new u, then one slot of new traces; area B holds
     // the other face slot, then the factors, then the other trace slot (8
-    // one-warp CTAs fit per SM). FP64: area A holds b, then the factors, then the
-    // new u.
-    static constexpr int PA = LEAN ? (NL > 3 * FDS ? NL : 3 * FDS) : NL;
-    static constexpr int PB = LEAN ? 0 : (FS > 3 * FDS ? FS : 3 * FDS);
+    // one-warp CTAs fit per SM).
+    static constexpr int PA = CS > FS ? CS : FS;
+    static constexpr int PB = FS > 3 * FDS ? FS : 3 * FDS;
     static constexpr size_t OFF_B = (size_t)W * PA;
     static constexpr size_t BYTES = (OFF_B + (size_t)W * PB) * sizeof(T);
-    static_assert(LEAN || FS <= NL, "a face slot fits area A");
 };
 
 // Neighbour across face f (= 2 axis + side) of `cell`, -1 where face f is on the
@@ -157,18 +150,58 @@ __device__ __forceinline__ int cell_neighbour(int f, int mask, int64_t cell, int
 }
 
 
-// Stage face f of the lane's neighbour nb (the neighbour's face f^1) into the
-// lane's part of a face slot: one bulk copy per lane that has a neighbour, all
-// completing on `bar`, whose byte count lane 0 posts before any copy is issued.
-// The caller has ended every read of the slot (proxy fence and warp barrier).
+// Stage face f of the lanes' neighbours (their faces f^1) into a face slot. The
+// neighbours of a run of cells along an axis are a run too, so it is one bulk copy of
+// at most 32 faces, completing on `bar` (one small copy per lane kept the copy engine
+// busy: 12 of them per cell and step). Cells outside the mesh are cut off; lanes without
+// a neighbour get some cell's face, which they don't use. Nothing is copied where no
+// lane has a neighbour. The caller has ended every read of the slot (proxy fence and
+// warp barrier).
 template <typename T, int Q>
-__device__ __forceinline__ void stage_face(int f, int nb, int lane, const T *__restrict__ tr, T *slot, uint64_t *bar) {
+__device__ __forceinline__ void stage_face(int f, int mask, int lane, int64_t ncell, int64_t cell0, int ncl, int s1, int s2,
+                                           const T *__restrict__ tr, T *slot, uint64_t *bar) {
     using G = CellGeo<T, Q>;
-    const unsigned with = __ballot_sync(0xffffffffu, nb >= 0);
-    if (lane == 0) mbar_arrive_expect_tx(bar, (unsigned)(__popc(with) * G::FS * (int)sizeof(T)));
+    const unsigned with = __ballot_sync(0xffffffffu, mask & (1 << f));
+    if (lane == 0) {
+        const int st = f < 2 ? 1 : (f < 4 ? s1 : s2);
+        const int64_t first = cell0 + ((f & 1) ? st : -st);
+        const int64_t lo = first < 0 ? 0 : first, hi = first + ncl < ncell ? first + ncl : ncell;
+        const unsigned bytes = with && hi > lo ? (unsigned)((hi - lo) * G::FS * (int)sizeof(T)) : 0u;
+        mbar_arrive_expect_tx(bar, bytes);
+        if (bytes) bulk_load(slot + (lo - first) * G::FS, tr + ((f ^ 1) * ncell + lo) * G::FS, bytes, bar);
+    }
     __syncwarp();
-    if (nb >= 0)
-        bulk_load(slot + lane * G::FS, tr + (int64_t)nb * G::TR + (f ^ 1) * G::FS, (unsigned)(G::FS * sizeof(T)), bar);
+}
+
+// A lane's cell in shared memory (stride CS) to registers, and back
+template <typename T, int Q>
+__device__ __forceinline__ void read_cell(const T *p, T *R) {
+    using G = CellGeo<T, Q>;
+    if constexpr (G::PADDED) {
+#pragma unroll
+        for (int e = 0; e < G::NL / 4; ++e) {
+            const float4 v = reinterpret_cast<const float4 *>(p)[e];
+            R[4 * e] = v.x;
+            R[4 * e + 1] = v.y;
+            R[4 * e + 2] = v.z;
+            R[4 * e + 3] = v.w;
+        }
+    } else {
+#pragma unroll
+        for (int e = 0; e < G::NL; ++e) R[e] = p[e];
+    }
+}
+template <typename T, int Q>
+__device__ __forceinline__ void write_cell(const T *R, T *p) {
+    using G = CellGeo<T, Q>;
+    if constexpr (G::PADDED) {
+#pragma unroll
+        for (int e = 0; e < G::NL / 4; ++e)
+            reinterpret_cast<float4 *>(p)[e] = make_float4(R[4 * e], R[4 * e + 1], R[4 * e + 2], R[4 * e + 3]);
+    } else {
+#pragma unroll
+        for (int e = 0; e < G::NL; ++e) p[e] = R[e];
+    }
 }
 
 // The cell tensor R[x + q y + q^2 z] is kept in registers and only ever worked
@@ -206,29 +239,24 @@ __device__ __forceinline__ void rotate_back(T *R) {
 template <typename T, int Q, bool TRANSPOSE>
 __device__ __forceinline__ void load_matrix(const T *src, T *S) {
     T v[Q * Q];
-    if (sizeof(T) == 4) {                               // 8-byte loads (the matrix is 8-byte aligned)
 #pragma unroll
-        for (int e = 0; e < (Q * Q) / 2; ++e) {
-            const float2 w = reinterpret_cast<const float2 *>(src)[e];
-            v[2 * e] = (T)w.x;
-            v[2 * e + 1] = (T)w.y;
-        }
-        if ((Q * Q) & 1) v[Q * Q - 1] = src[Q * Q - 1];
-    } else {
-#pragma unroll
-        for (int e = 0; e < Q * Q; ++e) v[e] = src[e];
+    for (int e = 0; e < (Q * Q) / 2; ++e) {             // 8-byte loads (the matrix is 8-byte aligned)
+        const float2 w = reinterpret_cast<const float2 *>(src)[e];
+        v[2 * e] = w.x;
+        v[2 * e + 1] = w.y;
     }
+    if ((Q * Q) & 1) v[Q * Q - 1] = src[Q * Q - 1];
 #pragma unroll
     for (int m = 0; m < Q; ++m)
 #pragma unroll
         for (int n = 0; n < Q; ++n) S[m * Q + n] = TRANSPOSE ? v[n * Q + m] : v[m * Q + n];
 }
 
-// Along x with packed pairs of pencils (FP32): outputs of pencils t and t + 1 by
-// one two-lane FMA per term, the matrix entry duplicated in both lanes (the
-// same roundings as the scalar form, half the issue slots).
-template <int Q>
-__device__ __forceinline__ void pass_x2(const float *A, float *R) {
+// Along x: R[., a, b] <- A R[., a, b] for every pencil (A row-major q x q): outputs of
+// pencils t and t + 1 by one two-lane FMA per term, the matrix entry duplicated in both
+// lanes (the same roundings as the scalar form, half the issue slots).
+template <typename T, int Q>
+__device__ __forceinline__ void pass_x(const T *A, T *R) {
 #pragma unroll
     for (int t = 0; t + 1 < Q * Q; t += 2) {
         float2 x[Q];
@@ -258,31 +286,9 @@ __device__ __forceinline__ void pass_x2(const float *A, float *R) {
     }
 }
 
-// Along x: R[., a, b] <- A R[., a, b] for every pencil (A row-major q x q).
-template <typename T, int Q>
-__device__ __forceinline__ void pass_x(const T *A, T *R) {
-    if constexpr (sizeof(T) == 4) {
-        pass_x2<Q>(reinterpret_cast<const float *>(A), reinterpret_cast<float *>(R));
-    } else {
-#pragma unroll
-        for (int t = 0; t < Q * Q; ++t) {
-            T x[Q];
-#pragma unroll
-            for (int n = 0; n < Q; ++n) x[n] = R[n + Q * t];
-#pragma unroll
-            for (int m = 0; m < Q; ++m) {
-                T s = T(0);
-#pragma unroll
-                for (int n = 0; n < Q; ++n) s += A[m * Q + n] * x[n];
-                R[m + Q * t] = s;
-            }
-        }
-    }
-}
-
 // r -= N u_nb for the face normal to the current x axis on side `side`, whose
-// neighbour fields fld = [g | h] (q^2 each) are indexed sa * a + sb * b at the
-// current tangential position (a, b) = (y, z). With G, H the fields after the
+// neighbour fields fld = [g | h] (q^2 each, 16-byte aligned, padded to FS) are indexed
+// a + q b at the current tangential position (a, b) = (y, z). With G, H the fields after the
 // tangential mass M_a (x) M_b (the 1D masses of the original axes now at y and
 // z, applied in their rank-one form M = diag(w) - u u^T: 3q operations per
 // pencil instead of q^2; wa, ua / wb, ub in shared memory):
@@ -291,9 +297,18 @@ __device__ __forceinline__ void pass_x(const T *A, T *R) {
 // The two terms of G share one vector: the pencil at (a, b) takes
 // G(a, b) c with c = sgn kF/2 d + kF gamma e_end, formed once per face.
 template <typename T, int Q>
-__device__ __forceinline__ void lift_x_face(int side, const T *fld, int sa, int sb, const T *wa, const T *ua,
-                                            const T *wb, const T *ub, const T *dv, T gam, T kF, T *R) {
-    constexpr int NF = Q * Q;
+__device__ __forceinline__ void lift_x_face(int side, const T *fld, const T *wa, const T *ua, const T *wb, const T *ub,
+                                            const T *dv, T gam, T kF, T *R) {
+    constexpr int NF = Q * Q, FS = CellGeo<T, Q>::FS;
+    T F[FS];
+#pragma unroll
+    for (int e = 0; e < FS / 4; ++e) {
+        const float4 v = reinterpret_cast<const float4 *>(fld)[e];
+        F[4 * e] = v.x;
+        F[4 * e + 1] = v.y;
+        F[4 * e + 2] = v.z;
+        F[4 * e + 3] = v.w;
+    }
     const T wv = T(0.5) * kF;
     // value field: all layers += G c; derivative field: end layer -= sgn kF/2 H
     T cg[Q];
@@ -305,84 +320,65 @@ __device__ __forceinline__ void lift_x_face(int side, const T *fld, int sa, int 
     }
 #pragma unroll
     for (int comp = 0; comp < 2; ++comp) {
-        const T *f = fld + comp * NF;
+        const T *f = F + comp * NF;
         T t1[NF];                                      // t1[a + q b] = (M_b f(a, .))[b]
-        if constexpr (sizeof(T) == 4) {
-            // rows a and a + 1 together by two-lane FMAs
+        // rows a and a + 1 together by two-lane FMAs
 #pragma unroll
-            for (int a = 0; a + 1 < Q; a += 2) {
-                float2 col[Q];
-                float2 s2 = make_float2(0.f, 0.f);
+        for (int a = 0; a + 1 < Q; a += 2) {
+            float2 col[Q];
+            float2 s2 = make_float2(0.f, 0.f);
 #pragma unroll
-                for (int bb = 0; bb < Q; ++bb) {
-                    col[bb] = make_float2((float)f[sa * a + sb * bb], (float)f[sa * (a + 1) + sb * bb]);
-                    s2 = __ffma2_rn(make_float2((float)ub[bb], (float)ub[bb]), col[bb], s2);
-                }
-#pragma unroll
-                for (int b = 0; b < Q; ++b) {
-                    const float2 t = __ffma2_rn(make_float2(-(float)ub[b], -(float)ub[b]), s2,
-                                                __fmul2_rn(make_float2((float)wb[b], (float)wb[b]), col[b]));
-                    t1[a + Q * b] = (T)t.x;
-                    t1[a + 1 + Q * b] = (T)t.y;
-                }
+            for (int bb = 0; bb < Q; ++bb) {
+                col[bb] = make_float2(f[a + Q * bb], f[a + 1 + Q * bb]);
+                s2 = __ffma2_rn(make_float2(ub[bb], ub[bb]), col[bb], s2);
             }
-            if (Q & 1) {
-                constexpr int a = Q - 1;
-                T col[Q];
-                T s = T(0);
 #pragma unroll
-                for (int bb = 0; bb < Q; ++bb) {
-                    col[bb] = f[sa * a + sb * bb];
-                    s += ub[bb] * col[bb];
-                }
-#pragma unroll
-                for (int b = 0; b < Q; ++b) t1[a + Q * b] = wb[b] * col[b] - ub[b] * s;
-            }
-        } else {
-#pragma unroll
-            for (int a = 0; a < Q; ++a) {
-                T col[Q];
-                T s = T(0);
-#pragma unroll
-                for (int bb = 0; bb < Q; ++bb) {
-                    col[bb] = f[sa * a + sb * bb];
-                    s += ub[bb] * col[bb];
-                }
-#pragma unroll
-                for (int b = 0; b < Q; ++b) t1[a + Q * b] = wb[b] * col[b] - ub[b] * s;
+            for (int b = 0; b < Q; ++b) {
+                const float2 t = __ffma2_rn(make_float2(-ub[b], -ub[b]), s2, __fmul2_rn(make_float2(wb[b], wb[b]), col[b]));
+                t1[a + Q * b] = t.x;
+                t1[a + 1 + Q * b] = t.y;
             }
         }
-        if constexpr (sizeof(T) == 4) {
-            if (comp == 0) {
-                T vv[NF];
+        if (Q & 1) {
+            constexpr int a = Q - 1;
+            T col[Q];
+            T s = T(0);
 #pragma unroll
-                for (int b = 0; b < Q; ++b) {
-                    T s = T(0);
-#pragma unroll
-                    for (int aa = 0; aa < Q; ++aa) s += ua[aa] * t1[aa + Q * b];
-#pragma unroll
-                    for (int a = 0; a < Q; ++a) vv[a + Q * b] = wa[a] * t1[a + Q * b] - ua[a] * s;
-                }
-                // pencils t, t + 1: pen[n] += v c[n] by two-lane FMAs
-                float *Rf = reinterpret_cast<float *>(R);
-#pragma unroll
-                for (int t = 0; t < NF; t += 2) {
-                    if (t + 1 < NF) {
-                        const float2 v2 = make_float2((float)vv[t], (float)vv[t + 1]);
-#pragma unroll
-                        for (int n = 0; n < Q; ++n) {
-                            float2 pp = make_float2(Rf[Q * t + n], Rf[Q * (t + 1) + n]);
-                            pp = __ffma2_rn(v2, make_float2((float)cg[n], (float)cg[n]), pp);
-                            Rf[Q * t + n] = pp.x;
-                            Rf[Q * (t + 1) + n] = pp.y;
-                        }
-                    } else {
-#pragma unroll
-                        for (int n = 0; n < Q; ++n) R[Q * t + n] += vv[t] * cg[n];
-                    }
-                }
-                continue;
+            for (int bb = 0; bb < Q; ++bb) {
+                col[bb] = f[a + Q * bb];
+                s += ub[bb] * col[bb];
             }
+#pragma unroll
+            for (int b = 0; b < Q; ++b) t1[a + Q * b] = wb[b] * col[b] - ub[b] * s;
+        }
+        if (comp == 0) {
+            T vv[NF];
+#pragma unroll
+            for (int b = 0; b < Q; ++b) {
+                T s = T(0);
+#pragma unroll
+                for (int aa = 0; aa < Q; ++aa) s += ua[aa] * t1[aa + Q * b];
+#pragma unroll
+                for (int a = 0; a < Q; ++a) vv[a + Q * b] = wa[a] * t1[a + Q * b] - ua[a] * s;
+            }
+            // pencils t, t + 1: pen[n] += v c[n] by two-lane FMAs
+#pragma unroll
+            for (int t = 0; t < NF; t += 2) {
+                if (t + 1 < NF) {
+                    const float2 v2 = make_float2(vv[t], vv[t + 1]);
+#pragma unroll
+                    for (int n = 0; n < Q; ++n) {
+                        float2 pp = make_float2(R[Q * t + n], R[Q * (t + 1) + n]);
+                        pp = __ffma2_rn(v2, make_float2(cg[n], cg[n]), pp);
+                        R[Q * t + n] = pp.x;
+                        R[Q * (t + 1) + n] = pp.y;
+                    }
+                } else {
+#pragma unroll
+                    for (int n = 0; n < Q; ++n) R[Q * t + n] += vv[t] * cg[n];
+                }
+            }
+            continue;
         }
 #pragma unroll
         for (int b = 0; b < Q; ++b) {
@@ -393,120 +389,91 @@ __device__ __forceinline__ void lift_x_face(int side, const T *fld, int sa, int 
             for (int a = 0; a < Q; ++a) {
                 const T v = wa[a] * t1[a + Q * b] - ua[a] * s;
                 T *pen = R + Q * (a + Q * b);              // the pencil along x at (a, b)
-                if (comp == 0) {
-#pragma unroll
-                    for (int n = 0; n < Q; ++n) pen[n] += v * cg[n];
-                } else {
-                    if (side) pen[Q - 1] += wv * v; else pen[0] -= wv * v;
-                }
+                if (side) pen[Q - 1] += wv * v; else pen[0] -= wv * v;
             }
         }
     }
 }
 
 // Traces of the face normal to the current x axis on side `side` into dst
-// ([value q^2 | derivative q^2], indexed sa * a + sb * b).
+// ([value q^2 | derivative q^2], indexed a + q b, padded to FS, 16-byte aligned).
 template <typename T, int Q>
-__device__ __forceinline__ void x_face_traces(int side, const T *R, const T *dv, int sa, int sb, T *dst) {
-    constexpr int NF = Q * Q;
-    if constexpr (sizeof(T) == 4) {
-        // derivative traces of pencils t and t + 1 by two-lane FMAs
+__device__ __forceinline__ void x_face_traces(int side, const T *R, const T *dv, T *dst) {
+    constexpr int NF = Q * Q, FS = CellGeo<T, Q>::FS;
+    T o[FS];
 #pragma unroll
-        for (int t = 0; t < NF; t += 2) {
-            const int a0 = t % Q, b0 = t / Q;
-            const float *p0 = reinterpret_cast<const float *>(R) + Q * t;
-            if (t + 1 < NF) {
-                const int a1 = (t + 1) % Q, b1 = (t + 1) / Q;
-                const float *p1 = p0 + Q;
-                float2 d = __fmul2_rn(make_float2((float)dv[0], (float)dv[0]), make_float2(p0[0], p1[0]));
+    for (int t = 2 * NF; t < FS; ++t) o[t] = T(0);
+    // derivative traces of pencils t and t + 1 by two-lane FMAs
 #pragma unroll
-                for (int n = 1; n < Q; ++n)
-                    d = __ffma2_rn(make_float2((float)dv[n], (float)dv[n]), make_float2(p0[n], p1[n]), d);
-                dst[sa * a0 + sb * b0] = side ? (T)p0[Q - 1] : (T)p0[0];
-                dst[sa * a1 + sb * b1] = side ? (T)p1[Q - 1] : (T)p1[0];
-                dst[NF + sa * a0 + sb * b0] = (T)d.x;
-                dst[NF + sa * a1 + sb * b1] = (T)d.y;
-            } else {
-                T d = T(0);
+    for (int t = 0; t < NF; t += 2) {
+        const T *p0 = R + Q * t;
+        o[t] = side ? p0[Q - 1] : p0[0];
+        if (t + 1 < NF) {
+            const T *p1 = p0 + Q;
+            float2 d = __fmul2_rn(make_float2(dv[0], dv[0]), make_float2(p0[0], p1[0]));
 #pragma unroll
-                for (int n = 0; n < Q; ++n) d += dv[n] * R[Q * t + n];
-                dst[sa * a0 + sb * b0] = side ? R[Q * t + Q - 1] : R[Q * t];
-                dst[NF + sa * a0 + sb * b0] = d;
-            }
+            for (int n = 1; n < Q; ++n) d = __ffma2_rn(make_float2(dv[n], dv[n]), make_float2(p0[n], p1[n]), d);
+            o[t + 1] = side ? p1[Q - 1] : p1[0];
+            o[NF + t] = d.x;
+            o[NF + t + 1] = d.y;
+        } else {
+            T d = T(0);
+#pragma unroll
+            for (int n = 0; n < Q; ++n) d += dv[n] * p0[n];
+            o[NF + t] = d;
         }
-    } else {
-#pragma unroll
-        for (int b = 0; b < Q; ++b)
-#pragma unroll
-            for (int a = 0; a < Q; ++a) {
-                const T *pen = R + Q * (a + Q * b);
-                T d = T(0);
-#pragma unroll
-                for (int n = 0; n < Q; ++n) d += dv[n] * pen[n];
-                dst[sa * a + sb * b] = side ? pen[Q - 1] : pen[0];
-                dst[NF + sa * a + sb * b] = d;
-            }
     }
+#pragma unroll
+    for (int e = 0; e < FS / 4; ++e)
+        reinterpret_cast<float4 *>(dst)[e] = make_float4(o[4 * e], o[4 * e + 1], o[4 * e + 2], o[4 * e + 3]);
 }
 
-// Traces of the cell tensor R (one per lane) to tr_out[cell][face][FS]: the
-// faces normal to axis p, then rotate. FP32: every lane writes its two faces
-// into its parts of two slots of shared memory (slot0, slot1: W x FS values
-// each, free for the whole call) and stores each with one bulk store (a slot is
-// rewritten once the lane's previous stores have read it); FP64 (LEAN):
-// written per lane. R ends rotated. Only lanes with `write` store.
+// Traces of the cell tensors R (one per lane) to tr_out[face][cell][FS]: the
+// faces normal to axis p, then rotate. Every lane writes its two faces into its parts
+// of two slots of shared memory (slot0, slot1: W x FS values each, free for the whole
+// call); a slot, the same face of all the CTA's cells, leaves by one bulk store (and
+// is rewritten once that has read it). R ends rotated. Only lanes with `write` write.
 template <typename T, int Q>
-__device__ __forceinline__ void cells_write_traces(const DGConst<T> &c, T *R, int lane, bool write, int64_t cell,
+__device__ __forceinline__ void cells_write_traces(const DGConst<T> &c, T *R, int lane, bool write, int64_t cell0, int ncl,
                                                    T *slot0, T *slot1, T *__restrict__ tr_out) {
-    using G = CellGeo<T, Q>;
-    constexpr int FS = G::FS, TR = G::TR;
+    constexpr int FS = CellGeo<T, Q>::FS;
     // unrolled: the two rotations become register renames
 #pragma unroll
     for (int p = 0; p < 3; ++p) {
-        const int sa = p == 1 ? Q : 1, sb = p == 1 ? 1 : Q;
-        if (!G::LEAN && p > 0) bulk_wait_read_all();
+        if (p > 0) {
+            if (lane == 0) bulk_wait_read_all();
+            __syncwarp();
+        }
         if (write) {
 #pragma unroll 1
             for (int side = 0; side < 2; ++side) {
                 T dv[Q];
 #pragma unroll
                 for (int n = 0; n < Q; ++n) dv[n] = side ? c.dp[p][n] : c.d0[p][n];
-                T *dst = G::LEAN ? tr_out + cell * TR + (2 * p + side) * FS : (side ? slot1 : slot0) + lane * FS;
-                x_face_traces<T, Q>(side, R, dv, sa, sb, dst);
+                x_face_traces<T, Q>(side, R, dv, (side ? slot1 : slot0) + lane * FS);
             }
-            if (!G::LEAN) {
-                fence_proxy_async_smem();
+        }
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) {
 #pragma unroll
-                for (int side = 0; side < 2; ++side)
-                    bulk_store(tr_out + cell * TR + (2 * p + side) * FS, (side ? slot1 : slot0) + lane * FS,
-                               (unsigned)(FS * sizeof(T)));
-                bulk_commit();
-            }
+            for (int side = 0; side < 2; ++side)
+                bulk_store(tr_out + ((2 * p + side) * c.ncell + cell0) * FS, side ? slot1 : slot0,
+                           (unsigned)(ncl * FS * sizeof(T)));
+            bulk_commit();
         }
         if (p < 2) rotate<T, Q>(R);
     }
-    if (!G::LEAN) bulk_wait_read_all();
+    if (lane == 0) bulk_wait_read_all();
+    __syncwarp();
 }
-
-template <typename T>
-__device__ __forceinline__ T div_approx(T a, T b);
-template <>
-__device__ __forceinline__ float div_approx<float>(float a, float b) { return __fdividef(a, b); }
-template <>
-__device__ __forceinline__ double div_approx<double>(double a, double b) { return a / b; }
 
 // Divide the transformed cell tensor R[x + q y + q^2 z] by the eigenvalue sums
 // lambda_x + lambda_y + lambda_z of the fast diagonalisation (fd: the cell's
-// factors, axis a at a * (q^2 + q), lambda after S), or multiply it by the
-// precomputed table of their inverses (li, q^3 values) when there is one.
+// factors, axis a at a * (q^2 + q), lambda after S).
 template <typename T, int Q>
-__device__ __forceinline__ void scale_inverse(T *R, const T *fd, const T *li) {
+__device__ __forceinline__ void scale_inverse(T *R, const T *fd) {
     constexpr int FDS = Q * Q + Q;
-    if (li) {
-#pragma unroll
-        for (int e = 0; e < Q * Q * Q; ++e) R[e] *= li[e];
-        return;
-    }
 #pragma unroll
     for (int k = 0; k < Q; ++k) {
         const T lz = fd[2 * FDS + Q * Q + k];
@@ -516,7 +483,7 @@ __device__ __forceinline__ void scale_inverse(T *R, const T *fd, const T *li) {
 #pragma unroll
             for (int i = 0; i < Q; ++i) {
                 const int e = i + Q * (j + Q * k);
-                R[e] = div_approx<T>(R[e], fd[Q * Q + i] + lyz);
+                R[e] = __fdividef(R[e], fd[Q * Q + i] + lyz);
             }
         }
     }
@@ -536,18 +503,75 @@ __device__ __forceinline__ void stage_bulk(bool full, int lane, uint64_t *bar, T
     }
 }
 
+// The cells of the CTA (src: the first one's values) into area dst at stride CS: one
+// bulk copy on `bar`, or 16-byte asynchronous copies where the stride pads. wait_cells
+// ends the wait for either.
 template <typename T, int Q>
-__device__ __forceinline__ void smooth_cells_body(const DGConst<T> &c, int64_t cell0, int flags, T *__restrict__ u, const T *__restrict__ b, const T *__restrict__ kappa, const T *__restrict__ fd, const T *__restrict__ linv, const T *__restrict__ tr_in, T *__restrict__ tr_out, bool reuse = false) {
+__device__ __forceinline__ void stage_cells(bool full, int lane, uint64_t *bar, T *dst, const T *src, int ncl) {
     using G = CellGeo<T, Q>;
-    constexpr int W = G::W, NL = G::NL, FDS = G::FDS, TR = G::TR, FS = G::FS;
+    if constexpr (G::PADDED) {
+        constexpr int V = G::NL / 4;
+#pragma unroll
+        for (int k = 0; k < V; ++k) {
+            const int e = lane + 32 * k;
+            if (e < ncl * V)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(dst + e / V * G::CS + e % V * 4)),
+                             "l"(src + 4 * e)
+                             : "memory");
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    } else {
+        stage_bulk<T>(full, lane, bar, dst, src, (int64_t)G::W * G::NL, ncl * G::NL);
+    }
+}
+template <typename T, int Q>
+__device__ __forceinline__ bool wait_cells(bool full, int lane, uint64_t *bar) {
+    if constexpr (CellGeo<T, Q>::PADDED) {
+        asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    } else {
+        if (full) return warp_wait_copies(bar, lane);
+    }
+    __syncwarp();
+    return true;
+}
+// The cells written by write_cell in area src to global memory; the area is free for
+// the lanes afterwards. (fence_proxy_async_smem and a warp barrier precede.)
+template <typename T, int Q>
+__device__ __forceinline__ void store_cells(bool full, int lane, T *dst, const T *src, int ncl) {
+    using G = CellGeo<T, Q>;
+    if constexpr (G::PADDED) {
+        constexpr int V = G::NL / 4;
+#pragma unroll
+        for (int k = 0; k < V; ++k) {
+            const int e = lane + 32 * k;
+            if (e < ncl * V)
+                reinterpret_cast<float4 *>(dst)[e] = *reinterpret_cast<const float4 *>(src + e / V * G::CS + e % V * 4);
+        }
+    } else if (full) {
+        if (lane == 0) {
+            bulk_store(dst, src, (unsigned)(G::W * G::NL * sizeof(T)));
+            bulk_commit();
+            bulk_wait_read_all();
+        }
+    } else {
+        for (int e = lane; e < ncl * G::NL; e += G::W) dst[e] = src[e];
+    }
+    __syncwarp();
+}
+
+template <typename T, int Q>
+__device__ __forceinline__ void smooth_cells_body(const DGConst<T> &c, int64_t cell0, int flags, T *__restrict__ u,
+                                                  const T *__restrict__ b, const T *__restrict__ fd,
+                                                  const T *__restrict__ tr_in, T *__restrict__ tr_out, bool reuse = false) {
+    using G = CellGeo<T, Q>;
+    constexpr int W = G::W, NL = G::NL, FDS = G::FDS, FS = G::FS, CS = G::CS;
     extern __shared__ __align__(128) unsigned char smem_c[];
-    // area A: b -> face slot 1 (FP32) or the factors (FP64) -> previous u (FP32)
-    //         -> new u -> trace slot 1
-    // area B (FP32): face slot 0 -> factors -> trace slot 0
+    // area A: b -> face slot 1 -> previous u -> new u -> trace slot 1
+    // area B: face slot 0 -> factors -> trace slot 0
     T *sA = reinterpret_cast<T *>(smem_c);
     T *sB = sA + G::OFF_B;
-    // mbarriers: 0 b, 1 previous u (FP32) / factors (FP64), 2 factors (FP32),
-    // 4 face slot 0, 5 face slot 1 (phase k = the slot's k-th face)
+    // mbarriers: 0 b, 1 previous u, 2 factors, 4 face slot 0, 5 face slot 1
+    // (phase k = the slot's k-th face)
     __shared__ __align__(8) uint64_t bars[6];
     __shared__ T sMw[3][Q], sMu[3][Q];
     const int lane = threadIdx.x;
@@ -555,7 +579,6 @@ __device__ __forceinline__ void smooth_cells_body(const DGConst<T> &c, int64_t c
     const bool full = ncl == W;                          // bulk copies of b, u, factors: whole 32-cell blocks
     const bool active = lane < ncl;
     const int64_t cell = cell0 + lane;
-    const bool table = linv != nullptr;
     bool ok = true;                                      // false once a bounded wait ran out
 
     cells_init_bars(bars, 6, lane, reuse);
@@ -563,7 +586,7 @@ __device__ __forceinline__ void smooth_cells_body(const DGConst<T> &c, int64_t c
         sMw[e / Q][e % Q] = c.mw[e / Q][e % Q];
         sMu[e / Q][e % Q] = c.mu[e / Q][e % Q];
     }
-    stage_bulk<T>(full, lane, &bars[0], sA, b + cell0 * NL, W * NL, ncl * NL);
+    stage_cells<T, Q>(full, lane, &bars[0], sA, b + cell0 * NL, ncl);
     // neighbours of this lane's cell (a mask of interior faces and the strides);
     // the first neighbour face is requested at once
     int mask = 0;
@@ -577,24 +600,22 @@ __device__ __forceinline__ void smooth_cells_body(const DGConst<T> &c, int64_t c
     const bool zero = (flags & SM_ZERO) != 0;
     if (zero)
         stage_bulk<T>(full, lane, &bars[2], sB, fd + cell0 * 3 * FDS, W * 3 * FDS, ncl * 3 * FDS);
-    else if (!G::LEAN)
-        stage_face<T, Q>(0, cell_neighbour(0, mask, cell, s1, s2), lane, tr_in, sB, &bars[4]);
+    else
+        stage_face<T, Q>(0, mask, lane, c.ncell, cell0, ncl, s1, s2, tr_in, sB, &bars[4]);
 
     // r = b
-    if (full)
-        ok = warp_wait_copies(&bars[0], lane) && ok;
-    else
-        __syncwarp();
+    ok = wait_cells<T, Q>(full, lane, &bars[0]) && ok;
     T R[NL];
+    if (active) {
+        read_cell<T, Q>(sA + lane * CS, R);
+    } else {
 #pragma unroll
-    for (int e = 0; e < NL; ++e) R[e] = active ? sA[lane * NL + e] : T(0);
+        for (int e = 0; e < NL; ++e) R[e] = T(0);
+    }
     fence_proxy_async_smem();
     __syncwarp();
-    // area A is free: FP32 the second neighbour face, FP64 the factors
-    if (G::LEAN)
-        stage_bulk<T>(full, lane, &bars[1], sA, fd + cell0 * 3 * FDS, W * 3 * FDS, ncl * 3 * FDS);
-    else if (!zero)
-        stage_face<T, Q>(1, cell_neighbour(1, mask, cell, s1, s2), lane, tr_in, sA, &bars[5]);
+    // area A is free: the second neighbour face
+    if (!zero) stage_face<T, Q>(1, mask, lane, c.ncell, cell0, ncl, s1, s2, tr_in, sA, &bars[5]);
 
     // r -= N u_nb: the two faces normal to axis p, then rotate the next axis to x
     // (three rotations are none)
@@ -602,27 +623,24 @@ __device__ __forceinline__ void smooth_cells_body(const DGConst<T> &c, int64_t c
     for (int p = 0; p < 3 && !zero; ++p) {
         T dv[Q];
         const int ta = p == 2 ? 0 : p + 1, tb = p == 0 ? 2 : p - 1;
-        const int sa = p == 1 ? Q : 1, sb = p == 1 ? 1 : Q;   // the y faces are stored transposed
         const T gam = c.gamma[p];
 #pragma unroll
         for (int side = 0; side < 2; ++side) {
             const int f = 2 * p + side;
-            const int nb = cell_neighbour(f, mask, cell, s1, s2);
-            const T kF = nb >= 0 ? c.kfac[cell * 6 + f] : T(0);
+            const bool nb = mask & (1 << f);
+            const T kF = nb ? c.kfac[cell * 6 + f] : T(0);
             T *slot = side ? sA : sB;
-            if (!G::LEAN) ok = warp_wait_phase(&bars[4 + side], (unsigned)(p & 1), lane) && ok;
-            if (active && nb >= 0) {
+            ok = warp_wait_phase(&bars[4 + side], (unsigned)(p & 1), lane) && ok;
+            if (nb) {
 #pragma unroll
                 for (int n = 0; n < Q; ++n) dv[n] = side ? c.dp[p][n] : c.d0[p][n];
-                const T *fld = G::LEAN ? tr_in + (int64_t)nb * TR + (f ^ 1) * FS : slot + lane * FS;
-                lift_x_face<T, Q>(side, fld, sa, sb, sMw[ta], sMu[ta], sMw[tb], sMu[tb], dv, gam, kF, R);
+                lift_x_face<T, Q>(side, slot + lane * FS, sMw[ta], sMu[ta], sMw[tb], sMu[tb], dv, gam, kF, R);
             }
-            if (!G::LEAN && f + 2 < 6) {
+            if (f + 2 < 6) {
                 fence_proxy_async_smem();
                 __syncwarp();
-                stage_face<T, Q>(f + 2, cell_neighbour(f + 2, mask, cell, s1, s2), lane, tr_in, slot,
-                                 &bars[4 + side]);
-            } else if (!G::LEAN && f == 4) {
+                stage_face<T, Q>(f + 2, mask, lane, c.ncell, cell0, ncl, s1, s2, tr_in, slot, &bars[4 + side]);
+            } else if (f == 4) {
                 // area B is free after the last face of slot 0: the factors, whose copy
                 // overlaps the lifting of face 5
                 fence_proxy_async_smem();
@@ -632,26 +650,26 @@ __device__ __forceinline__ void smooth_cells_body(const DGConst<T> &c, int64_t c
         }
         rotate<T, Q>(R);
     }
-    // FP32: the previous u into area A (face slot 1 is free now; u is first
-    // needed after the inverse)
-    if (!G::LEAN && !zero) {
+    // the previous u into area A (face slot 1 is free now; u is first needed after
+    // the inverse)
+    if (!zero) {
         fence_proxy_async_smem();
         __syncwarp();
-        stage_bulk<T>(full, lane, &bars[1], sA, u + cell0 * NL, W * NL, ncl * NL);
+        stage_cells<T, Q>(full, lane, &bars[1], sA, u + cell0 * NL, ncl);
     }
 
     // A_KK^{-1} by fast diagonalisation: S^T along x, y, z; scale by the
     // inverse eigenvalue sums; S along x, y, z
     if (full)
-        ok = warp_wait_copies(&bars[G::LEAN ? 1 : 2], lane) && ok;
+        ok = warp_wait_copies(&bars[2], lane) && ok;
     else
         __syncwarp();
-    const T *myFD = (G::LEAN ? sA : sB) + lane * 3 * FDS;
+    const T *myFD = sB + lane * 3 * FDS;
     // (the tensor-product factors commute, so both halves take the axes in the
     // same order and one loop body serves all six passes)
 #pragma unroll 1
     for (int k = 0; k < 6 && active; ++k) {
-        if (k == 3) scale_inverse<T, Q>(R, myFD, table ? linv + cell * NL : nullptr);
+        if (k == 3) scale_inverse<T, Q>(R, myFD);
         T S[Q * Q];
         if (k < 3)
             load_matrix<T, Q, true>(myFD + k * FDS, S);
@@ -661,48 +679,41 @@ __device__ __forceinline__ void smooth_cells_body(const DGConst<T> &c, int64_t c
         rotate<T, Q>(R);
     }
 
-    // u <- (1 - w) u + w y (w already in y when the inverse came from the table),
-    // stored through area A (the barrier also ends every lane's reads of the
-    // factors before area A (FP64) or B (FP32) is rewritten)
-    if (!G::LEAN && full && !zero)
-        ok = warp_wait_copies(&bars[1], lane) && ok;
-    else
+    // u <- (1 - w) u + w y, stored through area A (the barrier also ends every lane's
+    // reads of the factors before area B is rewritten)
+    if (zero)
         __syncwarp();
-    T *myU = sA + lane * NL;
+    else
+        ok = wait_cells<T, Q>(full, lane, &bars[1]) && ok;
     if (active) {
         const T om = c.omega, keep = T(1) - om;
-        const T *uo = G::LEAN ? u + cell * NL : sA + lane * NL;
+        T *my = sA + lane * CS;
         if (zero) {
 #pragma unroll
             for (int e = 0; e < NL; ++e) R[e] = om * R[e];
-        } else if (table) {
+        } else if constexpr (G::PADDED) {
 #pragma unroll
-            for (int e = 0; e < NL; ++e) R[e] = keep * uo[e] + R[e];
+            for (int e = 0; e < NL / 4; ++e) {
+                const float4 v = reinterpret_cast<const float4 *>(my)[e];
+                R[4 * e] = keep * v.x + om * R[4 * e];
+                R[4 * e + 1] = keep * v.y + om * R[4 * e + 1];
+                R[4 * e + 2] = keep * v.z + om * R[4 * e + 2];
+                R[4 * e + 3] = keep * v.w + om * R[4 * e + 3];
+            }
         } else {
 #pragma unroll
-            for (int e = 0; e < NL; ++e) R[e] = keep * uo[e] + om * R[e];
+            for (int e = 0; e < NL; ++e) R[e] = keep * my[e] + om * R[e];
         }
-#pragma unroll
-        for (int e = 0; e < NL; ++e) myU[e] = R[e];
+        write_cell<T, Q>(R, my);
     }
     fence_proxy_async_smem();
     __syncwarp();
     // a launch whose wait ran out leaves u and the traces of its cells unchanged
     if (ok) {
-        if (full) {
-            if (lane == 0) {
-                bulk_store(u + cell0 * NL, sA, (unsigned)(W * NL * sizeof(T)));
-                bulk_commit();
-                bulk_wait_read_all();                    // area A is read: trace slot 1
-            }
-        } else {
-            for (int e = lane; e < ncl * NL; e += W) u[cell0 * NL + e] = sA[e];
-        }
-        __syncwarp();
-        // traces of the new iterate (FP32: slots in areas B and A)
-        if (!(flags & SM_NO_TRACES)) cells_write_traces<T, Q>(c, R, lane, active, cell, sB, sA, tr_out);
+        store_cells<T, Q>(full, lane, u + cell0 * NL, sA, ncl);
+        // traces of the new iterate (slots in areas B and A)
+        if (!(flags & SM_NO_TRACES)) cells_write_traces<T, Q>(c, R, lane, active, cell0, ncl, sB, sA, tr_out);
     }
-    bulk_wait_read_all();
 }
 
 // Warm-up projection (Alg. 4 preamble) with one thread per cell, 3D, GLL:
@@ -714,10 +725,10 @@ template <typename T, int Q>
 __device__ __forceinline__ void project_cells_body(const DGConst<T> &c, int64_t cell0, T *__restrict__ u,
                                                    const T *__restrict__ e0, T *__restrict__ tr) {
     using G = CellGeo<T, Q>;
-    constexpr int W = G::W, NL = G::NL;
+    constexpr int W = G::W, NL = G::NL, CS = G::CS;
     extern __shared__ __align__(128) unsigned char smem_c[];
-    T *sA = reinterpret_cast<T *>(smem_c);              // u
-    T *sB = sA + G::OFF_B;                               // FP32: trace staging
+    T *sA = reinterpret_cast<T *>(smem_c);              // u, then a trace slot
+    T *sB = sA + G::OFF_B;                               // the other trace slot
     __shared__ __align__(8) uint64_t bars[1];
     const int lane = threadIdx.x;
     const int ncl = (int)min((int64_t)W, c.ncell - cell0);
@@ -729,7 +740,7 @@ __device__ __forceinline__ void project_cells_body(const DGConst<T> &c, int64_t 
         fence_mbar_init();
         fence_proxy_async_smem();
     }
-    stage_bulk<T>(full, lane, &bars[0], sA, u + cell0 * NL, W * NL, ncl * NL);
+    stage_cells<T, Q>(full, lane, &bars[0], sA, u + cell0 * NL, ncl);
     // the corner values of the correction (zero at boundary vertices)
     T ec[8];
     if (e0 != nullptr && active) {
@@ -749,14 +760,14 @@ __device__ __forceinline__ void project_cells_body(const DGConst<T> &c, int64_t 
             ec[k] = interior ? e0[vid] : T(0);
         }
     }
-    if (full) {
-        if (!warp_wait_copies(&bars[0], lane)) return;
-    } else {
-        __syncwarp();
-    }
+    if (!wait_cells<T, Q>(full, lane, &bars[0])) return;
     T R[NL];
+    if (active) {
+        read_cell<T, Q>(sA + lane * CS, R);
+    } else {
 #pragma unroll
-    for (int e = 0; e < NL; ++e) R[e] = active ? sA[lane * NL + e] : T(0);
+        for (int e = 0; e < NL; ++e) R[e] = T(0);
+    }
     if (e0 != nullptr) {
         if (active) {
             // u(i,j,k) += sum over corners of e_c hat_cx(x_i) hat_cy(y_j) hat_cz(z_k), axis by axis
@@ -774,25 +785,15 @@ __device__ __forceinline__ void project_cells_body(const DGConst<T> &c, int64_t 
 #pragma unroll
                     for (int i = 0; i < Q; ++i) R[i + Q * (j + Q * k)] += y0 * c.hat[0][i] + y1 * c.hat[1][i];
                 }
-#pragma unroll
-            for (int e = 0; e < NL; ++e) sA[lane * NL + e] = R[e];
+            write_cell<T, Q>(R, sA + lane * CS);
         }
         fence_proxy_async_smem();
         __syncwarp();
-        if (full) {
-            if (lane == 0) {
-                bulk_store(u + cell0 * NL, sA, (unsigned)(W * NL * sizeof(T)));
-                bulk_commit();
-            }
-        } else {
-            for (int e = lane; e < ncl * NL; e += W) u[cell0 * NL + e] = sA[e];
-        }
+        store_cells<T, Q>(full, lane, u + cell0 * NL, sA, ncl);
     }
-    // area A (u) becomes the second trace slot once its store has read it
-    if (e0 != nullptr && full && lane == 0) bulk_wait_read_all();
+    // area A (u) is the second trace slot
     __syncwarp();
-    cells_write_traces<T, Q>(c, R, lane, active, cell, sB, sA, tr);
-    bulk_wait_read_all();
+    cells_write_traces<T, Q>(c, R, lane, active, cell0, ncl, sB, sA, tr);
 }
 
 template <typename T, int Q>
@@ -927,14 +928,12 @@ __device__ __forceinline__ void direct_volume(const DGConst<T> &c, T kK, const T
 // set-up from the smoother's factors). Then b is added and the neighbour terms are lifted as in the
 // smoothing step. Outputs as for k_residual: r (negated for y = A u) and the
 // cell corner sums of the p-restriction.
-// Staging: u and the factors by bulk copies; FP32: b into u's area once u is
-// in registers, the neighbour faces through the slots once the factors are
-// used; FP64 (LEAN): the factors into u's area, b and the faces read per lane.
-// r leaves through area A by a bulk store.
-// DIRECT (FP32, fd unused): A_KK u in the direct form (direct_volume) instead,
-// for the operator of the FP32 CG recurrences; u stays in area A for the
-// volume passes, the first neighbour face is staged into area B at once, b is
-// read per lane.
+// Staging: u and the factors by bulk copies, b into u's area once u is in registers,
+// the neighbour faces through the slots once the factors are used. r leaves through
+// area A.
+// DIRECT (fd unused): A_KK u in the direct form (direct_volume) instead, for the
+// operator of the CG recurrences; u stays in area A for the volume passes, the first
+// neighbour face is staged into area B at once, b is read per lane.
 template <typename T, int Q, bool DIRECT = false>
 __device__ __forceinline__ void residual_cells_body(const DGConst<T> &c, int64_t cell0, int mode,
                                                     const T *__restrict__ u, const T *__restrict__ b,
@@ -942,12 +941,12 @@ __device__ __forceinline__ void residual_cells_body(const DGConst<T> &c, int64_t
                                                     const T *__restrict__ tr, T *__restrict__ rout,
                                                     T *__restrict__ corners, bool reuse = false) {
     using G = CellGeo<T, Q>;
-    constexpr int W = G::W, NL = G::NL, FDS = G::FDS, TR = G::TR, FS = G::FS;
+    constexpr int W = G::W, NL = G::NL, FDS = G::FDS, FS = G::FS, CS = G::CS;
     extern __shared__ __align__(128) unsigned char smem_c[];
-    T *sA = reinterpret_cast<T *>(smem_c);              // u -> b (FP32) or factors (FP64) -> face slot 1 -> r
-    T *sB = sA + G::OFF_B;                               // FP32: factors -> face slot 0
-    // mbarriers: 0 u, 1 b (FP32) / factors (FP64), 2 factors (FP32), 4 face
-    // slot 0 (area B), 5 face slot 1 (area A) (FP32; phase k = the slot's k-th face)
+    T *sA = reinterpret_cast<T *>(smem_c);              // u -> b -> face slot 1 -> r
+    T *sB = sA + G::OFF_B;                               // factors -> face slot 0
+    // mbarriers: 0 u, 1 b, 2 factors, 4 face slot 0 (area B), 5 face slot 1 (area A)
+    // (phase k = the slot's k-th face)
     __shared__ __align__(8) uint64_t bars[6];
     __shared__ T sMw[3][Q], sMu[3][Q];
     const int lane = threadIdx.x;
@@ -963,10 +962,8 @@ __device__ __forceinline__ void residual_cells_body(const DGConst<T> &c, int64_t
         sMu[e / Q][e % Q] = c.mu[e / Q][e % Q];
     }
     bool ok = true;                                      // false once a bounded wait ran out
-    static_assert(!DIRECT || !G::LEAN, "the direct form is the FP32 operator's");
-    stage_bulk<T>(full, lane, &bars[0], sA, u + cell0 * NL, W * NL, ncl * NL);
-    if (!G::LEAN && !DIRECT)
-        stage_bulk<T>(full, lane, &bars[2], sB, fd + cell0 * 3 * FDS, W * 3 * FDS, ncl * 3 * FDS);
+    stage_cells<T, Q>(full, lane, &bars[0], sA, u + cell0 * NL, ncl);
+    if (!DIRECT) stage_bulk<T>(full, lane, &bars[2], sB, fd + cell0 * 3 * FDS, W * 3 * FDS, ncl * 3 * FDS);
     int mask = 0;
     if (active) {
         int ci[3];
@@ -974,20 +971,17 @@ __device__ __forceinline__ void residual_cells_body(const DGConst<T> &c, int64_t
         mask = interior_mask<3>(ci, c.n);
     }
     const int s1 = c.n[0], s2 = c.n[0] * c.n[1];
-    if (DIRECT) stage_face<T, Q>(0, cell_neighbour(0, mask, cell, s1, s2), lane, tr, sB, &bars[4]);
+    if (DIRECT) stage_face<T, Q>(0, mask, lane, c.ncell, cell0, ncl, s1, s2, tr, sB, &bars[4]);
     const T kK = active ? kappa[cell] : T(1);
 
-    if (full)
-        ok = warp_wait_copies(&bars[0], lane) && ok;
-    else
-        __syncwarp();
+    ok = wait_cells<T, Q>(full, lane, &bars[0]) && ok;
     T R[NL];
     if constexpr (DIRECT) {
         if (active) {
             T kF[6];
 #pragma unroll
             for (int f = 0; f < 6; ++f) kF[f] = c.kfac[cell * 6 + f];
-            direct_volume<T, Q>(c, kK, kF, mask, sA + lane * NL, R);
+            direct_volume<T, Q>(c, kK, kF, mask, sA + lane * CS, R);
             const T *bb = has_b ? b + cell * NL : nullptr;
 #pragma unroll
             for (int e = 0; e < NL; ++e) R[e] = (bb ? bb[e] : T(0)) - R[e];
@@ -997,26 +991,26 @@ __device__ __forceinline__ void residual_cells_body(const DGConst<T> &c, int64_t
         }
         fence_proxy_async_smem();
         __syncwarp();
-        stage_face<T, Q>(1, cell_neighbour(1, mask, cell, s1, s2), lane, tr, sA, &bars[5]);
+        stage_face<T, Q>(1, mask, lane, c.ncell, cell0, ncl, s1, s2, tr, sA, &bars[5]);
     } else {
+        if (active) {
+            read_cell<T, Q>(sA + lane * CS, R);
+        } else {
 #pragma unroll
-        for (int e = 0; e < NL; ++e) R[e] = active ? sA[lane * NL + e] : T(0);
+            for (int e = 0; e < NL; ++e) R[e] = T(0);
+        }
         fence_proxy_async_smem();
         __syncwarp();
-        // area A: the factors (FP64) or b (FP32)
-        if (G::LEAN)
-            stage_bulk<T>(full, lane, &bars[1], sA, fd + cell0 * 3 * FDS, W * 3 * FDS, ncl * 3 * FDS);
-        else if (has_b)
-            stage_bulk<T>(full, lane, &bars[1], sA, b + cell0 * NL, W * NL, ncl * NL);
-        const bool b_staged = !G::LEAN && has_b;
+        // area A: b
+        if (has_b) stage_cells<T, Q>(full, lane, &bars[1], sA, b + cell0 * NL, ncl);
 
         // R = A_KK u: P along x, y, z; times the eigenvalue sums; P^T along x, y, z
         // (the tensor-product factors commute: one loop body for all six passes)
         if (full)
-            ok = warp_wait_copies(&bars[G::LEAN ? 1 : 2], lane) && ok;
+            ok = warp_wait_copies(&bars[2], lane) && ok;
         else
             __syncwarp();
-        const T *myFD = (G::LEAN ? sA : sB) + lane * 3 * FDS;
+        const T *myFD = sB + lane * 3 * FDS;
 #pragma unroll 1
         for (int k = 0; k < 6 && active; ++k) {
             if (k == 3) {
@@ -1041,48 +1035,50 @@ __device__ __forceinline__ void residual_cells_body(const DGConst<T> &c, int64_t
             rotate<T, Q>(R);
         }
         // R = b - A_KK u
-        if (b_staged && full)
-            ok = warp_wait_copies(&bars[1], lane) && ok;
+        if (has_b)
+            ok = wait_cells<T, Q>(full, lane, &bars[1]) && ok;
         else
             __syncwarp();
         if (active) {
-            const T *bb = has_b ? (G::LEAN ? b + cell * NL : sA + lane * NL) : nullptr;
+            if (!has_b) {
 #pragma unroll
-            for (int e = 0; e < NL; ++e) R[e] = (bb ? bb[e] : T(0)) - R[e];
+                for (int e = 0; e < NL; ++e) R[e] = -R[e];
+            } else {
+                T B[NL];
+                read_cell<T, Q>(sA + lane * CS, B);
+#pragma unroll
+                for (int e = 0; e < NL; ++e) R[e] = B[e] - R[e];
+            }
         }
-        // FP32: the neighbour faces into the slots (every lane is done with the
-        // factors in area B and with b in area A)
-        if (!G::LEAN) {
-            fence_proxy_async_smem();
-            __syncwarp();
-            stage_face<T, Q>(0, cell_neighbour(0, mask, cell, s1, s2), lane, tr, sB, &bars[4]);
-            stage_face<T, Q>(1, cell_neighbour(1, mask, cell, s1, s2), lane, tr, sA, &bars[5]);
-        }
+        // the neighbour faces into the slots (every lane is done with the factors in
+        // area B and with b in area A)
+        fence_proxy_async_smem();
+        __syncwarp();
+        stage_face<T, Q>(0, mask, lane, c.ncell, cell0, ncl, s1, s2, tr, sB, &bars[4]);
+        stage_face<T, Q>(1, mask, lane, c.ncell, cell0, ncl, s1, s2, tr, sA, &bars[5]);
     }
     // R -= N u_nb, face pair by face pair as in the smoothing step
 #pragma unroll 1
     for (int p = 0; p < 3; ++p) {
         T dv[Q];
         const int ta = p == 2 ? 0 : p + 1, tb = p == 0 ? 2 : p - 1;
-        const int sa = p == 1 ? Q : 1, sb = p == 1 ? 1 : Q;
         const T gam = c.gamma[p];
 #pragma unroll
         for (int side = 0; side < 2; ++side) {
             const int f = 2 * p + side;
-            const int nb = cell_neighbour(f, mask, cell, s1, s2);
-            const T kF = nb >= 0 ? c.kfac[cell * 6 + f] : T(0);
+            const bool nb = mask & (1 << f);
+            const T kF = nb ? c.kfac[cell * 6 + f] : T(0);
             T *slot = side ? sA : sB;
-            if (!G::LEAN) ok = warp_wait_phase(&bars[4 + side], (unsigned)(p & 1), lane) && ok;
-            if (active && nb >= 0) {
+            ok = warp_wait_phase(&bars[4 + side], (unsigned)(p & 1), lane) && ok;
+            if (nb) {
 #pragma unroll
                 for (int n = 0; n < Q; ++n) dv[n] = side ? c.dp[p][n] : c.d0[p][n];
-                const T *fld = G::LEAN ? tr + (int64_t)nb * TR + (f ^ 1) * FS : slot + lane * FS;
-                lift_x_face<T, Q>(side, fld, sa, sb, sMw[ta], sMu[ta], sMw[tb], sMu[tb], dv, gam, kF, R);
+                lift_x_face<T, Q>(side, slot + lane * FS, sMw[ta], sMu[ta], sMw[tb], sMu[tb], dv, gam, kF, R);
             }
-            if (!G::LEAN && f + 2 < 6) {
+            if (f + 2 < 6) {
                 fence_proxy_async_smem();
                 __syncwarp();
-                stage_face<T, Q>(f + 2, cell_neighbour(f + 2, mask, cell, s1, s2), lane, tr, slot, &bars[4 + side]);
+                stage_face<T, Q>(f + 2, mask, lane, c.ncell, cell0, ncl, s1, s2, tr, slot, &bars[4 + side]);
             }
         }
         rotate<T, Q>(R);
@@ -1093,20 +1089,10 @@ __device__ __forceinline__ void residual_cells_body(const DGConst<T> &c, int64_t
     }
     if ((mode & RES_WRITE_R) && ok) {
         __syncwarp();                                  // every lane is done with area A
-        if (active) {
-#pragma unroll
-            for (int e = 0; e < NL; ++e) sA[lane * NL + e] = R[e];
-        }
+        if (active) write_cell<T, Q>(R, sA + lane * CS);
         fence_proxy_async_smem();
         __syncwarp();
-        if (full) {
-            if (lane == 0) {
-                bulk_store(rout + cell0 * NL, sA, (unsigned)(W * NL * sizeof(T)));
-                bulk_commit();
-            }
-        } else {
-            for (int e = lane; e < ncl * NL; e += W) rout[cell0 * NL + e] = sA[e];
-        }
+        store_cells<T, Q>(full, lane, rout + cell0 * NL, sA, ncl);
     }
     if ((mode & RES_CORNERS) && active && ok) {
         // corner (cx, cy, cz): sum over the nodes of hat_cx(x_i) hat_cy(y_j) hat_cz(z_k) r_ijk
@@ -1146,7 +1132,6 @@ __device__ __forceinline__ void residual_cells_body(const DGConst<T> &c, int64_t
 #pragma unroll
         for (int k = 0; k < 8; ++k) corners[cell * 8 + k] = out[k];
     }
-    bulk_wait_read_all();
 }
 
 template <typename T, int Q>
@@ -1171,10 +1156,9 @@ __global__ void __launch_bounds__(32) k_residual_cells_direct(const __grid_const
 
 template <typename T, int Q>
 __global__ void __launch_bounds__(32) k_smooth_cells(const __grid_constant__ DGConst<T> c, int flags, T *__restrict__ u,
-                                                     const T *__restrict__ b, const T *__restrict__ kappa,
-                                                     const T *__restrict__ fd, const T *__restrict__ linv,
+                                                     const T *__restrict__ b, const T *__restrict__ fd,
                                                      const T *__restrict__ tr_in, T *__restrict__ tr_out) {
-    smooth_cells_body<T, Q>(c, (int64_t)blockIdx.x * CellGeo<T, Q>::W, flags, u, b, kappa, fd, linv, tr_in, tr_out);
+    smooth_cells_body<T, Q>(c, (int64_t)blockIdx.x * CellGeo<T, Q>::W, flags, u, b, fd, tr_in, tr_out);
 }
 
 // Host-side read of the timeout counter of this translation unit.
