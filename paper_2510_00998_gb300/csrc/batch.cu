@@ -87,7 +87,10 @@ __device__ __forceinline__ double seg_block_sum(double v) {
 
 // part[i][blockIdx.x] = partial sum of a.b over problem i = blockIdx.y, and with W = 2
 // part[count + i][...] that of c.b (b read once). The slices start on 16 bytes (a
-// multiple of 32 cells); two independent sums per product hide the FP64 latency.
+// multiple of 32 cells); two independent sums per product hide the FP64 latency, and
+// FP32 values are widened by integer instructions: the FP64 pipe, which bounds this
+// kernel, is left the multiply-adds (18M values, two products: 173 us with its own
+// conversions).
 template <typename T, int W>
 __global__ void __launch_bounds__(SEG_THREADS) k_seg_dot_partial(const int64_t *__restrict__ off,
                                                                  const int64_t *__restrict__ len,
@@ -102,10 +105,13 @@ __global__ void __launch_bounds__(SEG_THREADS) k_seg_dot_partial(const int64_t *
         seg_load<T>(b + o + k * V, y);
         seg_load<T>(a + o + k * V, x[0]);
         if constexpr (W == 2) seg_load<T>(c + o + k * V, x[1]);
+        double yd[V];
+#pragma unroll
+        for (int e = 0; e < V; ++e) yd[e] = widen(y[e]);
 #pragma unroll
         for (int w = 0; w < W; ++w)
 #pragma unroll
-            for (int e = 0; e < V; ++e) s[w][e & 1] = fma((double)x[w][e], (double)y[e], s[w][e & 1]);
+            for (int e = 0; e < V; ++e) s[w][e & 1] = fma(widen(x[w][e]), yd[e], s[w][e & 1]);
     }
     if (blockIdx.x == 0 && threadIdx.x == 0)
         for (int64_t k = nv * V; k < n; ++k) {
@@ -217,7 +223,10 @@ __global__ void __launch_bounds__(SEG_THREADS) k_seg_update_xr(const int64_t *__
             seg_store<T>(r + at, rv);
         }
 #pragma unroll
-        for (int e = 0; e < V; ++e) s[e & 1] = fma((double)rv[e], (double)rv[e], s[e & 1]);
+        for (int e = 0; e < V; ++e) {
+            const double rd = widen(rv[e]);
+            s[e & 1] = fma(rd, rd, s[e & 1]);
+        }
     }
     if (blockIdx.x == 0 && threadIdx.x == 0)
         for (int64_t k = o + nv * V; k < o + n; ++k) {

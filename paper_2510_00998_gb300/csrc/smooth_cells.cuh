@@ -833,88 +833,84 @@ __device__ __forceinline__ void build_kt(const DGConst<T> &c, T kK, const T *kF,
         }
 }
 
+// y = M x for a pair of pencils, the 1D mass in its rank-one form M x = w o x - mu (mu . x)
+template <int Q>
+__device__ __forceinline__ void mass_x2(const float *mw, const float *mu, const float2 *x, float2 *y) {
+    float2 d = __fmul2_rn(make_float2(mu[0], mu[0]), x[0]);
+#pragma unroll
+    for (int n = 1; n < Q; ++n) d = __ffma2_rn(make_float2(mu[n], mu[n]), x[n], d);
+#pragma unroll
+    for (int m = 0; m < Q; ++m)
+        y[m] = __ffma2_rn(make_float2(mw[m], mw[m]), x[m], __fmul2_rn(make_float2(-mu[m], -mu[m]), d));
+}
+
 // R = A_KK u in the direct sum-factorised form A_KK = sum_a Kt_a (x) M (x) M
 // (the rounding of the per-pencil kernels, which the FP32 CG recurrences need),
-// one thread per cell: u in the lane's part Y of shared memory (natural order
-// x + q y + q^2 z), overwritten by the second intermediate. With the 1D masses
-// in their rank-one form M x = w o x - mu (mu . x):
+// one thread per cell: u in Y (natural order x + q y + q^2 z), overwritten by the second
+// intermediate; Y is the lane's part of shared memory (q = 5) or an array (registers):
 //   along z: R = M_z u, Y = Kt_z u;
 //   along y: R <- M_y R, Y <- Kt_y R + M_y Y;
 //   along x: R <- Kt_x R + M_x Y.
 // Each pencil reads and writes only its own positions of Y, and the axes are
-// fixed at compile time (no rotation of R).
+// fixed at compile time (no rotation of R). Pencils are taken in pairs by two-lane
+// FMAs: with 8 warps per SM the chains of dependent instructions bound this kernel
+// (147 us at 64^3 p = 4 with one pencil at a time, 87 by its bytes).
 template <typename T, int Q>
 __device__ __forceinline__ void direct_volume(const DGConst<T> &c, T kK, const T *kF, int mask, T *Y, T *R) {
-    T Kt[Q * Q];
-    build_kt<T, Q, 2>(c, kK, kF, mask, Kt);
+    constexpr int NF = Q * Q;
+    T Kt[NF];
+    // position of node n of pencil t of the pass along axis A
+    auto at = [](int A, int t, int n) {
+        return A == 2 ? t + NF * n : (A == 1 ? t % Q + Q * n + NF * (t / Q) : n + Q * t);
+    };
+    auto pass = [&](auto axis) {
+        constexpr int A = decltype(axis)::value;
+        build_kt<T, Q, A>(c, kK, kF, mask, Kt);
 #pragma unroll
-    for (int j = 0; j < Q; ++j)
+        for (int t = 0; t < NF; t += 2) {
+            constexpr int last = NF - 1;
+            const int t1 = t < last ? t + 1 : t;             // the odd pencil out takes both lanes
+            float2 xa[Q], xb[Q], ma[Q], kt[Q];
 #pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            T x[Q];
+            for (int n = 0; n < Q; ++n) {
+                xb[n] = make_float2(Y[at(A, t, n)], Y[at(A, t1, n)]);
+                xa[n] = A == 2 ? xb[n] : make_float2(R[at(A, t, n)], R[at(A, t1, n)]);
+            }
+            if constexpr (A == 2) {
 #pragma unroll
-            for (int n = 0; n < Q; ++n) x[n] = Y[i + Q * j + Q * Q * n];
-            T d = T(0);
+                for (int m = 0; m < Q; ++m) kt[m] = make_float2(T(0), T(0));
+            } else {
+                mass_x2<Q>(c.mw[A], c.mu[A], xb, kt);
+            }
 #pragma unroll
-            for (int n = 0; n < Q; ++n) d += c.mu[2][n] * x[n];
+            for (int m = 0; m < Q; ++m)
 #pragma unroll
-            for (int m = 0; m < Q; ++m) {
-                T sb = T(0);
+                for (int n = 0; n < Q; ++n)
+                    kt[m] = __ffma2_rn(make_float2(Kt[m * Q + n], Kt[m * Q + n]), xa[n], kt[m]);
+            if constexpr (A != 0) {
+                mass_x2<Q>(c.mw[A], c.mu[A], xa, ma);
 #pragma unroll
-                for (int n = 0; n < Q; ++n) sb += Kt[m * Q + n] * x[n];
-                R[i + Q * j + Q * Q * m] = c.mw[2][m] * x[m] - c.mu[2][m] * d;
-                Y[i + Q * j + Q * Q * m] = sb;
+                for (int m = 0; m < Q; ++m) {
+                    R[at(A, t, m)] = ma[m].x;
+                    Y[at(A, t, m)] = kt[m].x;
+                    if (t1 != t) {
+                        R[at(A, t1, m)] = ma[m].y;
+                        Y[at(A, t1, m)] = kt[m].y;
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int m = 0; m < Q; ++m) {
+                    R[at(A, t, m)] = kt[m].x;
+                    if (t1 != t) R[at(A, t1, m)] = kt[m].y;
+                }
             }
             asm volatile("" ::: "memory");   // keeps later pencils' loads here (no spills)
         }
-    build_kt<T, Q, 1>(c, kK, kF, mask, Kt);
-#pragma unroll
-    for (int k = 0; k < Q; ++k)
-#pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            T xa[Q], xb[Q];
-#pragma unroll
-            for (int n = 0; n < Q; ++n) {
-                xa[n] = R[i + Q * n + Q * Q * k];
-                xb[n] = Y[i + Q * n + Q * Q * k];
-            }
-            T da = T(0), db = T(0);
-#pragma unroll
-            for (int n = 0; n < Q; ++n) {
-                da += c.mu[1][n] * xa[n];
-                db += c.mu[1][n] * xb[n];
-            }
-#pragma unroll
-            for (int m = 0; m < Q; ++m) {
-                T se = c.mw[1][m] * xb[m] - c.mu[1][m] * db;
-#pragma unroll
-                for (int n = 0; n < Q; ++n) se += Kt[m * Q + n] * xa[n];
-                R[i + Q * m + Q * Q * k] = c.mw[1][m] * xa[m] - c.mu[1][m] * da;
-                Y[i + Q * m + Q * Q * k] = se;
-            }
-            asm volatile("" ::: "memory");
-        }
-    build_kt<T, Q, 0>(c, kK, kF, mask, Kt);
-#pragma unroll
-    for (int t = 0; t < Q * Q; ++t) {
-        T xa[Q], xb[Q];
-#pragma unroll
-        for (int n = 0; n < Q; ++n) {
-            xa[n] = R[n + Q * t];
-            xb[n] = Y[n + Q * t];
-        }
-        T db = T(0);
-#pragma unroll
-        for (int n = 0; n < Q; ++n) db += c.mu[0][n] * xb[n];
-#pragma unroll
-        for (int m = 0; m < Q; ++m) {
-            T sy = c.mw[0][m] * xb[m] - c.mu[0][m] * db;
-#pragma unroll
-            for (int n = 0; n < Q; ++n) sy += Kt[m * Q + n] * xa[n];
-            R[m + Q * t] = sy;
-        }
-        asm volatile("" ::: "memory");
-    }
+    };
+    pass(std::integral_constant<int, 2>{});
+    pass(std::integral_constant<int, 1>{});
+    pass(std::integral_constant<int, 0>{});
 }
 
 // Residual r = b - A u with one thread per cell, 3D, exact diagonal blocks
@@ -981,7 +977,13 @@ __device__ __forceinline__ void residual_cells_body(const DGConst<T> &c, int64_t
             T kF[6];
 #pragma unroll
             for (int f = 0; f < 6; ++f) kF[f] = c.kfac[cell * 6 + f];
-            direct_volume<T, Q>(c, kK, kF, mask, sA + lane * CS, R);
+            if constexpr (NL <= 64) {
+                T Y[NL];
+                read_cell<T, Q>(sA + lane * CS, Y);
+                direct_volume<T, Q>(c, kK, kF, mask, Y, R);
+            } else {
+                direct_volume<T, Q>(c, kK, kF, mask, sA + lane * CS, R);
+            }
             const T *bb = has_b ? b + cell * NL : nullptr;
 #pragma unroll
             for (int e = 0; e < NL; ++e) R[e] = (bb ? bb[e] : T(0)) - R[e];
