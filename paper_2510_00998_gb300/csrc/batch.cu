@@ -46,9 +46,15 @@ constexpr int BATCH_ALIGN_CELLS = 32;   // one CTA of the one-thread-per-cell sm
 // Per-problem CG: every problem runs its own conjugate-gradient recurrence
 // (its own alpha and beta); a problem whose residual met its bound is frozen
 // (active = 0) and its x, r and p are left untouched.
-// CTAs per problem of the segmented kernels: a batch of three problems still covers
-// the SMs, and the partial sums of 256 fit a few kilobytes
-constexpr int SEG_BLOCKS = 64, SEG_THREADS = 256;
+// The vector kernels take chunks of equal length, each of one problem, a CTA per chunk:
+// about eight CTAs per SM whatever the sizes of the problems are. (64 CTAs per problem
+// left the largest problem's to run on: two products of 18M values of 24 problems 163
+// us, 33 by their bytes.)
+constexpr int SEG_THREADS = 256, SEG_CHUNK_MIN = 4096, SEG_CHUNK_MAX = 16384, SEG_CTAS = 1216;
+struct SegChunk {
+    int64_t at;          // first value in the batch vectors (a multiple of 4)
+    int n, prob;
+};
 
 // 16 bytes of a vector at a time. Products and sums are FP64 in both precisions.
 template <typename T>
@@ -85,53 +91,69 @@ __device__ __forceinline__ double seg_block_sum(double v) {
     return s;
 }
 
-// part[i][blockIdx.x] = partial sum of a.b over problem i = blockIdx.y, and with W = 2
-// part[count + i][...] that of c.b (b read once). The slices start on 16 bytes (a
-// multiple of 32 cells); two independent sums per product hide the FP64 latency, and
-// FP32 values are widened by integer instructions: the FP64 pipe, which bounds this
-// kernel, is left the multiply-adds (18M values, two products: 173 us with its own
-// conversions).
+constexpr int SEG_UNROLL = 4;   // packs per vector in flight
+
+// part[w][chunk] = partial sum of a.b over the chunk, and with W = 2 that of c.b (b read
+// once). Chunks start on 16 bytes; two independent sums per product hide the FP64
+// latency, and FP32 values are widened by integer instructions: the FP64 pipe is left
+// the multiply-adds.
 template <typename T, int W>
-__global__ void __launch_bounds__(SEG_THREADS) k_seg_dot_partial(const int64_t *__restrict__ off,
-                                                                 const int64_t *__restrict__ len,
-                                                                 const T *__restrict__ a, const T *__restrict__ b,
-                                                                 const T *__restrict__ c, double *__restrict__ part) {
-    constexpr int V = SegVec<T>::N;
-    const int i = blockIdx.y;
-    const int64_t o = off[i], n = len[i], nv = n / V, stride = (int64_t)gridDim.x * blockDim.x;
+__global__ void __launch_bounds__(SEG_THREADS) k_seg_dot_partial(const SegChunk *__restrict__ map, const T *__restrict__ a,
+                                                                 const T *__restrict__ b, const T *__restrict__ c,
+                                                                 double *__restrict__ part) {
+    constexpr int V = SegVec<T>::N, U = SEG_UNROLL;
+    const SegChunk ch = map[blockIdx.x];
+    a += ch.at;
+    b += ch.at;
+    if constexpr (W == 2) c += ch.at;
+    const int nv = ch.n / V;
     double s[W][2] = {};
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < nv; k += stride) {
-        T x[W][V], y[V];
-        seg_load<T>(b + o + k * V, y);
-        seg_load<T>(a + o + k * V, x[0]);
-        if constexpr (W == 2) seg_load<T>(c + o + k * V, x[1]);
-        double yd[V];
+    for (int k0 = threadIdx.x; k0 < nv; k0 += U * SEG_THREADS) {
+        T x[U][W][V], y[U][V];
 #pragma unroll
-        for (int e = 0; e < V; ++e) yd[e] = widen(y[e]);
+        for (int j = 0; j < U; ++j) {
+            const int k = k0 + j * SEG_THREADS;
+            if (k < nv) {
+                seg_load<T>(b + k * V, y[j]);
+                seg_load<T>(a + k * V, x[j][0]);
+                if constexpr (W == 2) seg_load<T>(c + k * V, x[j][1]);
+            }
+        }
 #pragma unroll
-        for (int w = 0; w < W; ++w)
+        for (int j = 0; j < U; ++j) {
+            if (k0 + j * SEG_THREADS < nv) {
 #pragma unroll
-            for (int e = 0; e < V; ++e) s[w][e & 1] = fma(widen(x[w][e]), yd[e], s[w][e & 1]);
+                for (int e = 0; e < V; ++e) {
+                    const double yd = widen(y[j][e]);
+#pragma unroll
+                    for (int w = 0; w < W; ++w) s[w][e & 1] = fma(widen(x[j][w][e]), yd, s[w][e & 1]);
+                }
+            }
+        }
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0)
-        for (int64_t k = nv * V; k < n; ++k) {
-            s[0][0] = fma((double)a[o + k], (double)b[o + k], s[0][0]);
-            if constexpr (W == 2) s[1][0] = fma((double)c[o + k], (double)b[o + k], s[1][0]);
+    if (threadIdx.x == 0)
+        for (int k = nv * V; k < ch.n; ++k) {
+            s[0][0] = fma((double)a[k], (double)b[k], s[0][0]);
+            if constexpr (W == 2) s[1][0] = fma((double)c[k], (double)b[k], s[1][0]);
         }
 #pragma unroll
     for (int w = 0; w < W; ++w) {
         const double v = seg_block_sum(s[w][0] + s[w][1]);
-        if (threadIdx.x == 0) part[((int64_t)w * gridDim.y + i) * SEG_BLOCKS + blockIdx.x] = v;
+        if (threadIdx.x == 0) part[(int64_t)w * gridDim.x + blockIdx.x] = v;
     }
 }
 
-// out[i] = sum of the SEG_BLOCKS partials of row i (fixed order); one warp per row
-__global__ void k_seg_dot_final(int rows, const double *__restrict__ part, double *__restrict__ out) {
-    const int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-    if (i >= rows) return;
-    double s = part[(int64_t)i * SEG_BLOCKS + lane] + part[(int64_t)i * SEG_BLOCKS + 32 + lane];
+// out[w count + i] = sum of the partials of problem i's chunks (fixed order), row w of
+// part; one warp per sum
+__global__ void k_seg_dot_final(int count, int rows, int nchunk, const int *__restrict__ first,
+                                const double *__restrict__ part, double *__restrict__ out) {
+    const int row = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (row >= rows) return;
+    const int w = row / count, i = row - w * count;
+    double s = 0.0;
+    for (int k = first[i] + lane; k < first[i + 1]; k += 32) s += part[(int64_t)w * nchunk + k];
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) out[i] = s;
+    if (lane == 0) out[row] = s;
 }
 
 // active problems: beta = <r,z>_new / <r,z>; <r,z> <- <r,z>_new
@@ -164,34 +186,35 @@ __global__ void k_seg_beta_flex(int count, const int *__restrict__ active, doubl
 
 // active problems: p = z + beta p
 template <typename T>
-__global__ void __launch_bounds__(SEG_THREADS) k_seg_update_p(const int64_t *__restrict__ off,
-                                                              const int64_t *__restrict__ len,
+__global__ void __launch_bounds__(SEG_THREADS) k_seg_update_p(const SegChunk *__restrict__ map,
                                                               const int *__restrict__ active,
                                                               const double *__restrict__ beta, T *__restrict__ p,
                                                               const T *__restrict__ z) {
     constexpr int V = SegVec<T>::N;
-    const int i = blockIdx.y;
-    if (!active[i]) return;
-    const int64_t o = off[i], n = len[i], nv = n / V;
-    const T bt = (T)beta[i];
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < nv; k += (int64_t)gridDim.x * blockDim.x) {
+    const SegChunk ch = map[blockIdx.x];
+    if (!active[ch.prob]) return;
+    p += ch.at;
+    z += ch.at;
+    const int nv = ch.n / V;
+    const T bt = (T)beta[ch.prob];
+#pragma unroll SEG_UNROLL
+    for (int k = threadIdx.x; k < nv; k += SEG_THREADS) {
         T pv[V], zv[V];
-        seg_load<T>(p + o + k * V, pv);
-        seg_load<T>(z + o + k * V, zv);
+        seg_load<T>(p + k * V, pv);
+        seg_load<T>(z + k * V, zv);
 #pragma unroll
         for (int e = 0; e < V; ++e) pv[e] = zv[e] + bt * pv[e];
-        seg_store<T>(p + o + k * V, pv);
+        seg_store<T>(p + k * V, pv);
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0)
-        for (int64_t k = o + nv * V; k < o + n; ++k) p[k] = z[k] + bt * p[k];
+    if (threadIdx.x == 0)
+        for (int k = nv * V; k < ch.n; ++k) p[k] = z[k] + bt * p[k];
 }
 
 // Active problems: alpha = <r,z> / <p,q>; x += alpha p; r -= alpha q (and, FP32 with
 // rold, r_old = r); every problem: the partial sums of ||r||^2 of the new r in the
 // same pass.
 template <typename T>
-__global__ void __launch_bounds__(SEG_THREADS) k_seg_update_xr(const int64_t *__restrict__ off,
-                                                               const int64_t *__restrict__ len,
+__global__ void __launch_bounds__(SEG_THREADS) k_seg_update_xr(const SegChunk *__restrict__ map,
                                                                const int *__restrict__ active,
                                                                const double *__restrict__ rz,
                                                                const double *__restrict__ pq, T *__restrict__ x,
@@ -199,12 +222,13 @@ __global__ void __launch_bounds__(SEG_THREADS) k_seg_update_xr(const int64_t *__
                                                                const T *__restrict__ p, const T *__restrict__ q,
                                                                double *__restrict__ part) {
     constexpr int V = SegVec<T>::N;
-    const int i = blockIdx.y;
-    const bool act = active[i] != 0;
-    const int64_t o = off[i], n = len[i], nv = n / V, stride = (int64_t)gridDim.x * blockDim.x;
-    const T alpha = act ? (T)(rz[i] / pq[i]) : T(0);
+    const SegChunk ch = map[blockIdx.x];
+    const bool act = active[ch.prob] != 0;
+    const int64_t o = ch.at;
+    const int nv = ch.n / V;
+    const T alpha = act ? (T)(rz[ch.prob] / pq[ch.prob]) : T(0);
     double s[2] = {};
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < nv; k += stride) {
+    for (int k = threadIdx.x; k < nv; k += SEG_THREADS) {
         const int64_t at = o + k * V;
         T rv[V];
         seg_load<T>(r + at, rv);
@@ -228,8 +252,8 @@ __global__ void __launch_bounds__(SEG_THREADS) k_seg_update_xr(const int64_t *__
             s[e & 1] = fma(rd, rd, s[e & 1]);
         }
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0)
-        for (int64_t k = o + nv * V; k < o + n; ++k) {
+    if (threadIdx.x == 0)
+        for (int64_t k = o + nv * V; k < o + ch.n; ++k) {
             T rk = r[k];
             if (act) {
                 if (rold) rold[k] = rk;
@@ -240,7 +264,7 @@ __global__ void __launch_bounds__(SEG_THREADS) k_seg_update_xr(const int64_t *__
             s[0] = fma((double)rk, (double)rk, s[0]);
         }
     const double v = seg_block_sum(s[0] + s[1]);
-    if (threadIdx.x == 0) part[(int64_t)i * SEG_BLOCKS + blockIdx.x] = v;
+    if (threadIdx.x == 0) part[blockIdx.x] = v;
 }
 
 // x += xs (FP64 accumulation of the FP32 correction), xs = 0, whole batch
@@ -318,7 +342,8 @@ struct dgmg_batch {
     int64_t ndof = 0;
     double *x = nullptr, *b = nullptr, *r = nullptr, *z = nullptr, *p = nullptr, *q = nullptr;
     std::vector<int64_t> dof_off, dof_len;
-    int64_t *d_off = nullptr, *d_len = nullptr;
+    SegChunk *seg = nullptr;                       // chunks of the vector kernels, problem by problem
+    int *seg_first = nullptr, nseg = 0;            // a problem's first chunk [count + 1]
     double *d_norm = nullptr, *h_norm = nullptr;   // [count] device, pinned host
     double *d_bb = nullptr;                        // ||b_i||^2 (zero b: 1)
     double *rz = nullptr, *rzn = nullptr, *pq = nullptr, *beta = nullptr, *part = nullptr;
@@ -551,10 +576,11 @@ int batch_vcycle(dgmg_batch &B, const T *r, T *z, cudaStream_t s) {
 
 unsigned small_grid(int count) { return (unsigned)((count + 127) / 128); }
 
-// the rows of partial sums in B.part to out, one warp each
+// the rows of partial sums in B.part to out, one warp per sum
 int seg_final(dgmg_batch &B, int rows, double *out, cudaStream_t s) {
     count_launches(1);
-    k_seg_dot_final<<<(unsigned)((rows + 3) / 4), 128, 0, s>>>(rows, B.part, out);
+    const int sums = rows * B.count;
+    k_seg_dot_final<<<(unsigned)((sums + 3) / 4), 128, 0, s>>>(B.count, sums, B.nseg, B.seg_first, B.part, out);
     LC(cudaGetLastError());
     return DGMG_OK;
 }
@@ -564,23 +590,21 @@ int seg_final(dgmg_batch &B, int rows, double *out, cudaStream_t s) {
 template <typename T>
 int seg_dot(dgmg_batch &B, const T *a, const T *b, double *out, cudaStream_t s, const T *c = nullptr) {
     count_launches(1);
-    const dim3 grid(SEG_BLOCKS, B.count);
     if (c)
-        k_seg_dot_partial<T, 2><<<grid, SEG_THREADS, 0, s>>>(B.d_off, B.d_len, a, b, c, B.part);
+        k_seg_dot_partial<T, 2><<<B.nseg, SEG_THREADS, 0, s>>>(B.seg, a, b, c, B.part);
     else
-        k_seg_dot_partial<T, 1><<<grid, SEG_THREADS, 0, s>>>(B.d_off, B.d_len, a, b, c, B.part);
+        k_seg_dot_partial<T, 1><<<B.nseg, SEG_THREADS, 0, s>>>(B.seg, a, b, c, B.part);
     LC(cudaGetLastError());
-    return seg_final(B, (c ? 2 : 1) * B.count, out, s);
+    return seg_final(B, c ? 2 : 1, out, s);
 }
 
 // x += alpha p, r -= alpha q of the active problems and ||r_i||^2 of all of them
 template <typename T>
 int seg_update_xr(dgmg_batch &B, T *x, T *r, T *rold, const T *p, const T *q, cudaStream_t s) {
     count_launches(1);
-    k_seg_update_xr<T><<<dim3(SEG_BLOCKS, B.count), SEG_THREADS, 0, s>>>(B.d_off, B.d_len, B.active, B.rz, B.pq, x, r,
-                                                                          rold, p, q, B.part);
+    k_seg_update_xr<T><<<B.nseg, SEG_THREADS, 0, s>>>(B.seg, B.active, B.rz, B.pq, x, r, rold, p, q, B.part);
     LC(cudaGetLastError());
-    return seg_final(B, B.count, B.d_norm, s);
+    return seg_final(B, 1, B.d_norm, s);
 }
 
 // the norms in B.d_norm to the host (pinned) and the active flags
@@ -618,8 +642,7 @@ int batch_iteration(dgmg_batch &B, cudaStream_t s) {
         RC(seg_dot<double>(B, B.r, B.z, B.rzn, s));
         count_launches(2);
         k_seg_beta<<<small_grid(B.count), 128, 0, s>>>(B.count, B.active, B.rz, B.rzn, B.beta);
-        k_seg_update_p<double><<<dim3(SEG_BLOCKS, B.count), SEG_THREADS, 0, s>>>(B.d_off, B.d_len, B.active, B.beta,
-                                                                              B.p, B.z);
+        k_seg_update_p<double><<<B.nseg, SEG_THREADS, 0, s>>>(B.seg, B.active, B.beta, B.p, B.z);
         LC(cudaGetLastError());
         return alpha_step(B, s);
     }
@@ -627,8 +650,7 @@ int batch_iteration(dgmg_batch &B, cudaStream_t s) {
     RC(seg_dot<float>(B, B.r32, B.z32, B.rzn, s, B.rold32));   // and <r_old, z> into rzo, the row after rzn
     count_launches(2);
     k_seg_beta_flex<<<small_grid(B.count), 128, 0, s>>>(B.count, B.active, B.rz, B.rzn, B.rzo, B.beta);
-    k_seg_update_p<float><<<dim3(SEG_BLOCKS, B.count), SEG_THREADS, 0, s>>>(B.d_off, B.d_len, B.active, B.beta, B.p32,
-                                                                         B.z32);
+    k_seg_update_p<float><<<B.nseg, SEG_THREADS, 0, s>>>(B.seg, B.active, B.beta, B.p32, B.z32);
     LC(cudaGetLastError());
     RC(batch_apply32(B, B.p32, B.q32, s));
     RC(seg_dot<float>(B, B.p32, B.q32, B.pq, s));
@@ -885,12 +907,27 @@ int dgmg_batch_create(int count, const dgmg_mesh *meshes, const int *p, const do
         RC(B->alloc(v, B->ndof));
         LC(cudaMemset(*v, 0, sizeof(double) * B->ndof));
     }
-    RC(B->upload(&B->d_off, B->dof_off));
-    RC(B->upload(&B->d_len, B->dof_len));
+    {
+        int64_t total = 0;
+        for (int i = 0; i < count; ++i) total += B->dof_len[i];
+        const int64_t chunk =
+            std::min<int64_t>(SEG_CHUNK_MAX, std::max<int64_t>(SEG_CHUNK_MIN, (total / SEG_CTAS + 1023) / 1024 * 1024));
+        std::vector<SegChunk> seg;
+        std::vector<int> first;
+        for (int i = 0; i < count; ++i) {
+            first.push_back((int)seg.size());
+            for (int64_t k = 0; k < B->dof_len[i]; k += chunk)
+                seg.push_back(SegChunk{B->dof_off[i] + k, (int)std::min(chunk, B->dof_len[i] - k), i});
+        }
+        first.push_back((int)seg.size());
+        B->nseg = (int)seg.size();
+        RC(B->upload(&B->seg, seg));
+        RC(B->upload(&B->seg_first, first));
+    }
     for (double **v : {&B->d_norm, &B->d_bb, &B->rz, &B->pq, &B->beta}) RC(B->alloc(v, count));
     RC(B->alloc(&B->rzn, 2 * (size_t)count));      // <r, z> of the new residual, <r_old, z>
     B->rzo = B->rzn + count;
-    RC(B->alloc(&B->part, 2 * (size_t)count * SEG_BLOCKS));
+    RC(B->alloc(&B->part, 2 * (size_t)B->nseg));
     RC(B->alloc(&B->active, count));
     if (B->mixed) {
         for (float **v : {&B->r32, &B->z32, &B->p32, &B->q32, &B->xs32, &B->rold32}) {

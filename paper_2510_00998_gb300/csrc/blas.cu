@@ -13,17 +13,24 @@ namespace dgmg {
 
 namespace {
 
-__device__ __forceinline__ double block_sum(double v, double *sh) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0) sh[w] = v;
-    __syncthreads();
-    v = 0.0;
-    if (threadIdx.x < 32) {
-        v = threadIdx.x < (blockDim.x >> 5) ? sh[threadIdx.x] : 0.0;
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+// the block's W sums of s in thread 0, in a fixed order
+template <int W>
+__device__ __forceinline__ void block_sums(const double *s, double *v, double (*sh)[32]) {
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+        double t = s[w];
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+        if ((threadIdx.x & 31) == 0) sh[w][threadIdx.x >> 5] = t;
     }
-    return v;   // valid in thread 0
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+        v[w] = 0.0;
+        if (threadIdx.x < 32) {
+            v[w] = threadIdx.x < (blockDim.x >> 5) ? sh[w][threadIdx.x] : 0.0;
+            for (int o = 16; o > 0; o >>= 1) v[w] += __shfl_down_sync(0xffffffffu, v[w], o);
+        }
+    }
 }
 
 // One vector load of 16 bytes, or (VEC = false: some vector is not 16-byte aligned)
@@ -72,15 +79,13 @@ __device__ __forceinline__ void pack_dot(double &s, const Pack<T, VEC> &a, const
 // (Fletcher-Reeves; with W = 2 Polak-Ribiere, out[1] = <r_old,z>) and the shift of <r,z>.
 template <int W>
 __device__ __forceinline__ void dot_finish(const double *s, double *partials, double *out0, double *out1, double *scal) {
-    __shared__ double sh[32];
+    __shared__ double sh[W][32];
     __shared__ unsigned last;
     double v[W];
+    block_sums<W>(s, v, sh);
+    if (threadIdx.x == 0)
 #pragma unroll
-    for (int w = 0; w < W; ++w) {
-        v[w] = block_sum(s[w], sh);
-        if (threadIdx.x == 0) partials[w * DOT_BLOCKS + blockIdx.x] = v[w];
-        __syncthreads();
-    }
+        for (int w = 0; w < W; ++w) partials[w * DOT_BLOCKS + blockIdx.x] = v[w];
     unsigned *ticket = reinterpret_cast<unsigned *>(partials + 2 * DOT_BLOCKS);
     if (threadIdx.x == 0) {
         __threadfence();
@@ -89,13 +94,13 @@ __device__ __forceinline__ void dot_finish(const double *s, double *partials, do
     __syncthreads();
     if (!last) return;
     __threadfence();
+    double t[W];
 #pragma unroll
     for (int w = 0; w < W; ++w) {
-        double t = 0.0;
-        for (unsigned i = threadIdx.x; i < gridDim.x; i += blockDim.x) t += __ldcg(partials + w * DOT_BLOCKS + i);
-        v[w] = block_sum(t, sh);
-        __syncthreads();
+        t[w] = 0.0;
+        for (unsigned i = threadIdx.x; i < gridDim.x; i += blockDim.x) t[w] += __ldcg(partials + w * DOT_BLOCKS + i);
     }
+    block_sums<W>(t, v, sh);
     if (threadIdx.x == 0) {
         if (out0) *out0 = v[0];
         if (W == 2 && out1) *out1 = v[W - 1];

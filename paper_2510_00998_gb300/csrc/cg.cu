@@ -2,6 +2,8 @@
 // Sec. 5.2): the vertex gather of the p-restriction, damped point Jacobi with
 // the 3^d-point Galerkin stencils, residual, nested h-restriction and
 // h-prolongation, and the dense coarsest solve.
+#include <algorithm>
+
 #include "internal.h"
 
 namespace dgmg {
@@ -475,15 +477,19 @@ __global__ void __launch_bounds__(Q1_TPB) k_q1_dense(const __grid_constant__ Q1P
     if ((threadIdx.x & 31) == 0) p.u0[0][i] = (T)t;
 }
 
-// wd = omega / diagonal of a level
-template <typename T>
-__global__ void k_q1_weights(int64_t n, const T *__restrict__ diag, T omega, T *__restrict__ wd) {
-    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (v < n) wd[v] = omega / diag[v];
+// wd = omega / diagonal of the levels above the coarsest
+template <int DIM, typename T>
+__global__ void k_q1_weights(const __grid_constant__ Q1Plan<T> p, T omega) {
+    for (int l = 0; l < p.nlev - 1; ++l)
+        for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < p.L[l].nv; v += (int64_t)gridDim.x * blockDim.x)
+            p.wd[l][v] = omega / p.L[l].st[(DIM == 3 ? 13 : 4) * p.L[l].nv + v];
 }
 
 // E[i][j]: the cycle from level dense_from down applied to the unit vectors e_j, one
-// block per column, with the level vectors in shared memory.
+// block per column, with the level vectors in shared memory. On level dense_from the
+// iterates before the correction and the residual are zero beyond nu_pre vertices from
+// j: those steps run on that box only (the FP64 pipe bounds the kernel: 1331 vertices
+// 0.64 ms with all vertices in every step).
 template <int DIM>
 __global__ void __launch_bounds__(Q1_TPB) k_q1_dense_matrix(const __grid_constant__ Q1Plan<double> plan,
                                                             const double *__restrict__ Ainv, double *__restrict__ E) {
@@ -505,11 +511,51 @@ __global__ void __launch_bounds__(Q1_TPB) k_q1_dense_matrix(const __grid_constan
     __syncthreads();
     const BlockEach each;
     BlockSync sync;
-    const int64_t nd = p.L[ld].nv, nc = p.L[nl - 1].nv;
+    const CGLevelDev<double> &L = p.L[ld];
+    const int64_t nd = L.nv, nc = p.L[nl - 1].nv, ncv = p.L[ld + 1].nv;
+    const bool last = ld + 1 == nl - 1;
+    double *u[2] = {p.u0[ld], p.u1[ld]}, *b = p.b[ld], *r = p.r[ld], *bn = p.b[ld + 1];
     for (int64_t j = blockIdx.x; j < nd; j += gridDim.x) {
-        each(nd, [&](int64_t v) { q1_put_rhs<double>(p, ld, v, v == j ? 1.0 : 0.0); });
+        each(4 * nd, [&](int64_t v) { u[0][v] = 0.0; });   // u0, u1, b, r of the level
         sync();
-        for (int l = ld; l < nl - 1; ++l) q1_down<DIM, double>(p, l, l + 1 == nl - 1, each, sync);
+        int cj[3] = {0, 0, 0};
+        vcoords<DIM>(j, L.m, cj);
+        // f(v) for the vertices at most `rad` from j
+        auto box = [&](int rad, auto f) {
+            int lo[3] = {0, 0, 0}, n[3] = {1, 1, 1};
+#pragma unroll
+            for (int a = 0; a < DIM; ++a) {
+                lo[a] = max(cj[a] - rad, 0);
+                n[a] = min(cj[a] + rad, L.m[a] - 1) - lo[a] + 1;
+            }
+            for (int k = threadIdx.x; k < n[0] * n[1] * n[2]; k += blockDim.x) {
+                const int q = k / n[0], z = q / n[1];
+                f((int64_t)(lo[0] + k - q * n[0]) + (int64_t)L.m[0] * ((lo[1] + q - z * n[1]) + (int64_t)L.m[1] * (lo[2] + z)));
+            }
+        };
+        if (threadIdx.x == 0) q1_put_rhs<double>(p, ld, j, 1.0);
+        sync();
+        int c = p.nu_pre > 0 ? 1 : 0;
+        for (int k = 1; k < p.nu_pre; ++k) {
+            double *ui = u[c], *uo = u[c ^ 1];
+            box(k, [&](int64_t v) { q1_jacobi_at<DIM, double>(p, ld, ui, uo, v); });
+            c ^= 1;
+            sync();
+        }
+        double *uc = u[c];
+        box(p.nu_pre, [&](int64_t v) { cg_residual_at<DIM, double>(L, uc, b, r, v); });
+        sync();
+        each.warps(ncv * RS_LANES, [&](int64_t t) {
+            const int64_t V = t / RS_LANES;
+            const double s = h_restrict_at<DIM, double>(L, r, V < ncv ? V : -1);
+            if (V >= ncv || t % RS_LANES != 0) return;
+            if (last)
+                bn[V] = s;
+            else
+                q1_put_rhs<double>(p, ld + 1, V, s);
+        });
+        sync();
+        for (int l = ld + 1; l < nl - 1; ++l) q1_down<DIM, double>(p, l, l + 1 == nl - 1, each, sync);
         const double *rc = p.b[nl - 1];
         double *e = p.u0[nl - 1];
         each(nc, [&](int64_t i) { coarse_row<double>(nc, Ainv, rc, e, i); });
@@ -629,9 +675,13 @@ cudaError_t launch_q1_dense(int dim, const Q1Plan<T> &plan, int64_t n, const T *
 }
 
 template <typename T>
-cudaError_t launch_q1_weights(int64_t n, const T *diag, T omega, T *wd, cudaStream_t s) {
+cudaError_t launch_q1_weights(int dim, const Q1Plan<T> &plan, T omega, cudaStream_t s) {
     count_launches(1);
-    k_q1_weights<T><<<blocks_for(n), TPB, 0, s>>>(n, diag, omega, wd);
+    const unsigned grid = std::min(blocks_for(plan.L[0].nv), 1216u);
+    if (dim == 3)
+        k_q1_weights<3, T><<<grid, TPB, 0, s>>>(plan, omega);
+    else
+        k_q1_weights<2, T><<<grid, TPB, 0, s>>>(plan, omega);
     return cudaGetLastError();
 }
 
@@ -840,7 +890,7 @@ DGMG_CG_INST(float)
     template cudaError_t launch_q1_cycle<T>(int, const Q1Plan<T> &, const T *, unsigned long long *, int, bool,        \
                                             cudaStream_t);                                                            \
     template cudaError_t launch_q1_dense<T>(int, const Q1Plan<T> &, int64_t, const T *, cudaStream_t);                 \
-    template cudaError_t launch_q1_weights<T>(int64_t, const T *, T, T *, cudaStream_t);
+    template cudaError_t launch_q1_weights<T>(int, const Q1Plan<T> &, T, cudaStream_t);
 DGMG_Q1_INST(double)
 DGMG_Q1_INST(float)
 template int q1_cycle_max_blocks<double>(int, bool);

@@ -731,31 +731,40 @@ int q1_cycle(dgmg_ctx &C, const T *corners, cudaStream_t s, T **result) {
 }
 
 // The level from which the Q1 cycle is a dense product: the first of at most
-// Q1_DENSE_MAX vertices whose levels fit the set-up kernel's shared memory, else the
-// coarsest (whose inverse is dense already). smem: bytes of those levels' vectors.
-static int q1_dense_level(const std::vector<int64_t> &nv, size_t *smem = nullptr) {
+// Q1_DENSE_MAX vertices (shared: of a server's context, Q1_DENSE_MAX_SHARED) whose
+// levels fit the set-up kernel's shared memory, else the coarsest (whose inverse is
+// dense already). smem: bytes of those levels' vectors.
+static int q1_dense_level(const std::vector<int64_t> &nv, bool shared, size_t *smem = nullptr) {
+    const int64_t most = shared ? Q1_DENSE_MAX_SHARED : Q1_DENSE_MAX;
     int l = (int)nv.size() - 1;
     size_t bytes = 4 * sizeof(double) * nv[l];
-    while (l > 0 && nv[l - 1] <= Q1_DENSE_MAX && bytes + 4 * sizeof(double) * nv[l - 1] <= Q1_DENSE_SMEM)
+    while (l > 0 && nv[l - 1] <= most && bytes + 4 * sizeof(double) * nv[l - 1] <= Q1_DENSE_SMEM)
         bytes += 4 * sizeof(double) * nv[--l];
     if (smem) *smem = bytes;
     return l;
 }
 
+// Bytes of the dense matrix and of the levels' weights (both precisions if mixed).
+static size_t q1_matrix_values(const std::vector<int64_t> &nv, bool shared) {
+    const int ld = q1_dense_level(nv, shared);
+    return ld + 1 < (int)nv.size() ? (size_t)(nv[ld] * nv[ld]) : 0;
+}
+static size_t q1_store_bytes(const std::vector<int64_t> &nv, bool shared, bool mixed) {
+    size_t w = 0;
+    for (size_t l = 0; l + 1 < nv.size(); ++l) w += nv[l];
+    return 8 * (q1_matrix_values(nv, shared) + w) + (mixed ? 4 * w : 0);
+}
+
 // (Re)compute what the one-launch cycle takes from the levels' operators.
 static int q1_refresh(dgmg_ctx &C, cudaStream_t s) {
-    const int nl = (int)C.lv.size();
-    for (int l = 0; l + 1 < nl; ++l) {
-        const int64_t nv = C.lv[l].nv, d = (stencil_size(C.dim) / 2) * nv;
-        if (l < (int)C.q1wd64.size()) LC(launch_q1_weights<double>(nv, C.cg64[l].st + d, C.opts.omega_cg, C.q1wd64[l], s));
-        if (l < (int)C.q1wd32.size())
-            LC(launch_q1_weights<float>(nv, C.cg32[l].st + d, (float)C.opts.omega_cg, C.q1wd32[l], s));
-    }
+    if (!C.q1_store) return DGMG_OK;
+    LC(launch_q1_weights<double>(C.dim, C.q1plan64, C.opts.omega_cg, s));
+    if (C.q1plan32.nlev) LC(launch_q1_weights<float>(C.dim, C.q1plan32, (float)C.opts.omega_cg, s));
     if (C.q1_E) {
         std::vector<int64_t> nv;
         for (const CGLevelHost &H : C.lv) nv.push_back(H.nv);
         size_t smem = 0;
-        const int ld = q1_dense_level(nv, &smem);
+        const int ld = q1_dense_level(nv, !C.q1_wide, &smem);
         LC(launch_q1_dense_matrix(C.dim, C.q1plan64, nv[ld], smem, C.coarse_inv, C.q1_E, s));
     }
     return DGMG_OK;
@@ -786,16 +795,24 @@ int setup_q1_plan(dgmg_ctx &C) {
     h.nu_post = C.opts.nu_post;
     std::vector<int64_t> nv;
     for (int l = 0; l < nl; ++l) nv.push_back(lv[l].L.nv);
-    const int ld = q1_dense_level(nv);
+    const int ld = q1_dense_level(nv, !C.q1_wide);
     h.dense_from = C.q1_dense_from = ld;
     h.ndense = nv[ld];
-    if (ld < nl - 1 && !C.q1_E) RC(C.alloc(&C.q1_E, nv[ld] * nv[ld]));   // by the FP64 plan, which comes first
+    // one buffer: the matrix, the FP64 weights, the FP32 weights (the FP64 plan is made first)
+    if (nl > 1 && !C.q1_store) {
+        RC(C.alloc(reinterpret_cast<unsigned char **>(&C.q1_store),
+                   q1_store_bytes(nv, !C.q1_wide, C.opts.precision == DGMG_MIXED_FP32)));
+        if (ld < nl - 1) C.q1_E = static_cast<double *>(C.q1_store);
+    }
     h.E = ld < nl - 1 ? C.q1_E : C.coarse_inv;
-    auto &wd = q1wd<T>(C);
-    wd.assign(nl - 1, nullptr);
-    for (int l = 0; l + 1 < nl; ++l) {
-        RC(C.alloc(&wd[l], nv[l]));
-        h.wd[l] = wd[l];
+    if (nl > 1) {
+        double *w64 = static_cast<double *>(C.q1_store) + q1_matrix_values(nv, !C.q1_wide);
+        for (int l = 0; pi == 1 && l + 1 < nl; ++l) w64 += nv[l];
+        T *w = reinterpret_cast<T *>(w64);
+        for (int l = 0; l + 1 < nl; ++l) {
+            h.wd[l] = w;
+            w += nv[l];
+        }
     }
     for (int l = 0; l < nl; ++l) {
         h.L[l] = lv[l].L;
@@ -1589,7 +1606,7 @@ int dgmg_load_vector(dgmg_ctx *C, const double *fq, double *b, void *stream) {
     return DGMG_OK;
 }
 
-int dgmg_estimate_bytes(const dgmg_mesh *mesh, int p, const dgmg_opts *opts, size_t *bytes) {
+static int estimate_bytes_of(const dgmg_mesh *mesh, int p, const dgmg_opts *opts, bool shared, size_t *bytes) {
     if (!mesh || !bytes) return fail(DGMG_EINVAL, "mesh and bytes must not be NULL");
     if (mesh->dim != 2 && mesh->dim != 3) return fail(DGMG_EINVAL, "mesh->dim must be 2 or 3");
     if (p < 1 || p > PMAX) return fail(DGMG_EINVAL, "p must be in 1..6");
@@ -1644,10 +1661,9 @@ int dgmg_estimate_bytes(const dgmg_mesh *mesh, int p, const dgmg_opts *opts, siz
                    sz(p + 2, 8) + sz((int64_t)q * (p + 2), 8) + sz(3 * (p + 2), 8);
     if (mixed) total += dg32 + cg32 + 2 * sz(ndof, 4) + (reliable ? 4 * sz(ndof, 4) : 0);
     if (q1_blocks_for(dim, mixed) > 0) {   // the counters, weights and matrix of the one-launch Q1 cycle
-        const int ld = q1_dense_level(q1nv);
+        const int ld = q1_dense_level(q1nv, shared);
         if (ld > 0) total += 2 * sizeof(unsigned long long);
-        for (size_t l = 0; l + 1 < q1nv.size(); ++l) total += q1nv[l] * (mixed ? 12 : 8);
-        if (ld + 1 < (int)q1nv.size()) total += q1nv[ld] * q1nv[ld] * 8;
+        total += q1_store_bytes(q1nv, shared, mixed);
     }
     if (o.p_coarsening == 1 && p >= 2) {
         // lower DG levels p-1 .. 1 (kappa shared with the finest level): factors,
@@ -1666,6 +1682,10 @@ int dgmg_estimate_bytes(const dgmg_mesh *mesh, int p, const dgmg_opts *opts, siz
     }
     *bytes = total;
     return DGMG_OK;
+}
+
+int dgmg_estimate_bytes(const dgmg_mesh *mesh, int p, const dgmg_opts *opts, size_t *bytes) {
+    return estimate_bytes_of(mesh, p, opts, false, bytes);
 }
 
 
@@ -1724,6 +1744,10 @@ int residual_restrict_with_scratch(dgmg_ctx *C, const double *u, const double *b
                                corner_scratch, exact_fd(*C, C->d64), s));
     if (rc) LC(launch_corner_gather<double>(C->dim, C->n, corner_scratch, rc, s));
     return DGMG_OK;
+}
+
+int estimate_bytes_shared(const dgmg_mesh *mesh, int p, const dgmg_opts *opts, size_t *bytes) {
+    return ::estimate_bytes_of(mesh, p, opts, true, bytes);
 }
 
 }  // namespace dgmg

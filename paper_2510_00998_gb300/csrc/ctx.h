@@ -151,8 +151,7 @@ struct dgmg_ctx {
     int q1_blocks_t[2] = {0, 0};                   // blocks of the cycle per precision [FP64, FP32]
     int q1_dense_from = 0;                         // level from which the cycle is a product with q1_E
     double *q1_E = nullptr;                        // (null: with the inverse of the coarsest operator)
-    std::vector<double *> q1wd64;                  // omega / diagonal of the levels
-    std::vector<float *> q1wd32;
+    void *q1_store = nullptr;                      // that matrix and the levels' omega / diagonal
     bool q1_wide = true;                           // FP32 cycle in 512-thread blocks
     DGDev<double> d64;
     DGDev<float> d32;
@@ -335,13 +334,6 @@ inline const DGDev<T> &dg(const dgmg_ctx &C) {
         return C.d64;
 }
 template <typename T>
-inline std::vector<T *> &q1wd(dgmg_ctx &C) {
-    if constexpr (std::is_same<T, float>::value)
-        return C.q1wd32;
-    else
-        return C.q1wd64;
-}
-template <typename T>
 inline Q1Plan<T> &q1plan(dgmg_ctx &C) {
     if constexpr (std::is_same<T, float>::value)
         return C.q1plan32;
@@ -371,6 +363,8 @@ inline const std::vector<CGDev<T>> &cgl(const dgmg_ctx &C) {
 // the kernels of concurrent solves.
 enum { CREATE_NO_SOLVER = 1, CREATE_NO_FP64_SMOOTHER = 2, CREATE_NO_FP64_Q1 = 4, CREATE_SHARED_GPU = 8 };
 int create_ctx(const dgmg_mesh *mesh, int p, const double *kappa, const dgmg_opts *opts, int flags, dgmg_ctx **out);
+// dgmg_estimate_bytes of a context created with CREATE_SHARED_GPU
+int estimate_bytes_shared(const dgmg_mesh *mesh, int p, const dgmg_opts *opts, size_t *bytes);
 
 int mg_cycle64(dgmg_ctx &C, double *x, const double *b, double *r, cudaStream_t s);
 int project64(dgmg_ctx &C, double *x, cudaStream_t s);

@@ -271,17 +271,19 @@ struct Q1Plan {
     int64_t ndense;        // vertices of that level
     const double *E;       // ndense x ndense, row-major
     CGLevelDev<T> L[Q1_MAXLEV];
-    const T *wd[Q1_MAXLEV];   // omega / diagonal of the levels above the coarsest
+    T *wd[Q1_MAXLEV];      // omega / diagonal of the levels above the coarsest
     T *u0[Q1_MAXLEV], *u1[Q1_MAXLEV], *b[Q1_MAXLEV], *r[Q1_MAXLEV];
 };
 // Levels of at most this many vertices are the dense ones (the first such level of a
 // hierarchy and all below it). The product costs ndense^2 FP64 multiply-adds on the
 // whole chip (3.8 us at 1331 vertices) and one barrier, the steps it replaces 7 barriers
-// (1.3 us) and 7 steps of 1.5 to 5 us a level; the matrix takes 0.65 ms of the set-up at
-// 1331 vertices (growing with their square), and 8 ndense^2 bytes. One cycle, level per
-// level in block-wide or grid-wide steps / with the product: FP64 16^2 p = 2 69 / 6 us,
-// 23^3 p = 2 131 / 42, FP64 V-cycles 109 / 52 and 237 / 149 us.
-constexpr int64_t Q1_DENSE_MAX = 1536;
+// (1.3 us) and 7 short steps a level; the matrix takes time at set-up and 8 ndense^2
+// bytes. V-cycle (creation) with the level on the grid / as the dense one: 512
+// vertices 93 / 68 us (0.5 / 0.7 ms), 1089 64 / 50 us (0.55 / 0.8 ms), 1331 93 / 77 us
+// (0.9 / 1.9 ms), 2025 66 / 62 us (0.8 / 1.7 ms), 3025 66 / 76 us: the line lies where
+// the gain pays for the set-up within a solve or two. The server's contexts, admitted by
+// their bytes, stop at half a megabyte.
+constexpr int64_t Q1_DENSE_MAX = 1100, Q1_DENSE_MAX_SHARED = 256;
 constexpr size_t Q1_DENSE_SMEM = 160 * 1024;   // level vectors of the set-up kernel, at most
 // e on level 0 (u0 or u1 of level 0, by the parity of nu_pre + nu_post) from the
 // cells' corner sums; bar: the plan's own arrival counter (zero before its first
@@ -293,7 +295,7 @@ cudaError_t launch_q1_cycle(int dim, const Q1Plan<T> &plan, const T *corners, un
 template <typename T>
 cudaError_t launch_q1_dense(int dim, const Q1Plan<T> &plan, int64_t n, const T *corners, cudaStream_t s);
 template <typename T>
-cudaError_t launch_q1_weights(int64_t n, const T *diag, T omega, T *wd, cudaStream_t s);
+cudaError_t launch_q1_weights(int dim, const Q1Plan<T> &plan, T omega, cudaStream_t s);
 cudaError_t launch_q1_dense_matrix(int dim, const Q1Plan<double> &plan, int64_t nd, size_t smem, const double *Ainv,
                                    double *E, cudaStream_t s);
 // the most blocks of the cooperative launch (one per SM), 0 if it cannot run

@@ -206,6 +206,9 @@ struct dgmg_server {
                 finish(r, DGMG_FAILED, DGMG_EINVAL, dgmg_last_error());
                 continue;
             }
+            // the size of a context of one's own; the server's keeps a smaller Q1 matrix,
+            // and a request is refused only if that does not fit
+            if (est > budget) estimate_bytes_shared(&r->mesh, r->p, &opts, &est);
             if (est > budget) {
                 pending.pop_front();
                 finish(r, DGMG_FAILED, DGMG_EBUDGET,

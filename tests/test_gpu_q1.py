@@ -38,9 +38,8 @@ def _check(ctx, mesh, kap, opts, tol):
 
 @pytest.mark.parametrize("n,p,opts", [
     ((2, 2), 2, {}), ((2, 2, 2), 1, {}), ((16, 16), 2, {}), ((5, 3, 4), 2, {}),
-    ((40, 39), 1, {}),                        # 39 x 38 = 1482 vertices: dense from the finest level
-    ((40, 40), 1, {}), ((41, 40), 1, {}),     # 1521 and 1560: the last dense and the first on the grid
-    ((13, 12, 13), 1, {}), ((13, 13, 13), 1, {}),
+    ((34, 34), 1, {}), ((35, 34), 1, {}),     # 1089 vertices: dense from the finest level; 1122: the first on the grid
+    ((11, 12, 11), 1, {}), ((12, 12, 11), 1, {}),
     ((300, 3), 1, {}), ((2, 70, 3), 1, {}), ((90, 3, 40), 1, {}),
     ((40, 30), 1, {"nu_pre": 0, "nu_post": 1}), ((60, 50), 1, {"nu_pre": 0, "nu_post": 2}),
     ((60, 50), 1, {"nu_pre": 2, "nu_post": 0}), ((22, 21, 20), 1, {"nu_pre": 1, "nu_post": 0}),
