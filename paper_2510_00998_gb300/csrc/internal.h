@@ -53,15 +53,13 @@ cudaError_t wait_timeouts_addr_fp32(unsigned long long **ptr);
 #ifdef __CUDACC__
 // v as FP64 without the FP64 pipe, which converts 1.9 values per SM and clock (and
 // multiplies 1.6): exponent and mantissa are moved to their places by integer
-// instructions; zero, subnormal, infinite and NaN values take the conversion.
+// instructions. Subnormal, infinite and NaN values take the conversion, in a function of
+// its own: a predicated conversion occupies the pipe also where it is not wanted.
+static __device__ __noinline__ double widen_special(float v) { return (double)v; }
 __device__ __forceinline__ double widen(float v) {
-    const unsigned u = __float_as_uint(v);
-    if (((u >> 23) & 0xffu) - 1u >= 254u) {
-        double d;
-        asm volatile("cvt.f64.f32 %0, %1;" : "=d"(d) : "f"(v));   // (volatile: not done ahead for all values)
-        return d;
-    }
-    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + ((1023u - 127u) << 20))), (int)(u << 29));
+    const unsigned u = __float_as_uint(v), m = u & 0x7fffffffu;
+    if (m - 0x00800000u >= 0x7f000000u && m != 0) return widen_special(v);
+    return __hiloint2double((int)((u & 0x80000000u) | (m ? (m >> 3) + ((1023u - 127u) << 20) : 0u)), (int)(u << 29));
 }
 __device__ __forceinline__ double widen(double v) { return v; }
 #endif
