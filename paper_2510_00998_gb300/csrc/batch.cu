@@ -350,6 +350,14 @@ struct dgmg_batch {
     int *active = nullptr;
     cudaEvent_t ev = nullptr;
     cudaStream_t capture_stream = nullptr;
+    // the groups' DG kernels run side by side: group 0 on the caller's stream, the
+    // others on a stream of their own, forked off it and joined again
+    struct Side {
+        cudaStream_t s = nullptr;
+        cudaEvent_t done = nullptr;
+    };
+    std::vector<Side> side;
+    cudaEvent_t fork = nullptr;
     cudaGraphExec_t exec = nullptr;
     long long graph_kernels = 0;
     int graph_uses = 0;
@@ -379,6 +387,11 @@ struct dgmg_batch {
     ~dgmg_batch() {
         if (exec) cudaGraphExecDestroy(exec);
         if (capture_stream) cudaStreamDestroy(capture_stream);
+        for (Side &t : side) {
+            if (t.s) cudaStreamDestroy(t.s);
+            if (t.done) cudaEventDestroy(t.done);
+        }
+        if (fork) cudaEventDestroy(fork);
         if (ev) cudaEventDestroy(ev);
         if (h_norm) cudaFreeHost(h_norm);
         for (void *ptr : allocs) cudaFree(ptr);
@@ -492,31 +505,49 @@ void push_verts(std::vector<VertMap> &m, int desc, int64_t n) {
 }
 
 // ---- batched stages
+// f(group, stream) for every group, side by side: the groups' cells, vectors and traces
+// are their own, and a group's launch alone leaves SMs idle (its last wave; the small
+// groups all the time: 24 problems, p = 1 .. 4, 61.9 ms one group after the other).
+template <typename F>
+int for_groups(dgmg_batch &B, cudaStream_t s, F f) {
+    if (!B.side.empty()) LC(cudaEventRecord(B.fork, s));
+    int rc = DGMG_OK;
+    for (size_t k = 1; k < B.groups.size(); ++k) {
+        auto &t = B.side[k - 1];
+        LC(cudaStreamWaitEvent(t.s, B.fork, 0));
+        if (rc == DGMG_OK) rc = f(B.groups[k], t.s);
+        LC(cudaEventRecord(t.done, t.s));
+    }
+    if (rc == DGMG_OK) rc = f(B.groups[0], s);
+    for (auto &t : B.side) LC(cudaStreamWaitEvent(s, t.done, 0));   // (joined also after a failure)
+    return rc;
+}
+
 int batch_apply(dgmg_batch &B, const double *u, const double *bvec, double *out, cudaStream_t s) {
     const int mode = bvec ? (RES_HAS_B | RES_WRITE_R) : (RES_WRITE_R | RES_NEGATE);
-    for (auto &grp : B.groups) {
+    return for_groups(B, s, [&](dgmg_batch::Group &grp, cudaStream_t t) -> int {
         auto &g = grp.p64;
         LC(launch_project_batch<double>(B.dim, grp.q, g.D, g.map[TILE_PROJECT], g.nblocks[TILE_PROJECT],
-                                        g.tile[TILE_PROJECT], const_cast<double *>(u) + grp.dof0, 0, s));
+                                        g.tile[TILE_PROJECT], const_cast<double *>(u) + grp.dof0, 0, t));
         LC(launch_residual_batch<double>(B.dim, grp.q, g.D, g.map[TILE_RESIDUAL], g.nblocks[TILE_RESIDUAL],
                                          g.tile[TILE_RESIDUAL], mode, u + grp.dof0, bvec ? bvec + grp.dof0 : nullptr,
-                                         out + grp.dof0, 0, s));
-    }
-    return DGMG_OK;
+                                         out + grp.dof0, 0, t));
+        return DGMG_OK;
+    });
 }
 
 // out = A u with the FP32 operator of every problem (projection + residual
 // with b = 0, sign flipped), all groups
 int batch_apply32(dgmg_batch &B, const float *u, float *out, cudaStream_t s) {
-    for (auto &grp : B.groups) {
+    return for_groups(B, s, [&](dgmg_batch::Group &grp, cudaStream_t t) -> int {
         auto &g = grp.p32;
         LC(launch_project_batch<float>(B.dim, grp.q, g.D, g.map[TILE_PROJECT], g.nblocks[TILE_PROJECT],
-                                       g.tile[TILE_PROJECT], const_cast<float *>(u) + grp.dof0, 0, s));
+                                       g.tile[TILE_PROJECT], const_cast<float *>(u) + grp.dof0, 0, t));
         LC(launch_residual_batch<float>(B.dim, grp.q, g.D, g.map[TILE_RESIDUAL], g.nblocks[TILE_RESIDUAL],
                                         g.tile[TILE_RESIDUAL], RES_WRITE_R | RES_NEGATE | RES_DIRECT, u + grp.dof0,
-                                        nullptr, out + grp.dof0, 0, s));
-    }
-    return DGMG_OK;
+                                        nullptr, out + grp.dof0, 0, t));
+        return DGMG_OK;
+    });
 }
 
 template <typename T>
@@ -548,30 +579,29 @@ int batch_vcycle(dgmg_batch &B, const T *r, T *z, cudaStream_t s) {
     const int exact = B.opts.block_inverse == DGMG_BLOCK_EXACT ? 1 : 0;
     // the first step takes the zero iterate as such (nu_pre >= 1), nothing reads the
     // projections of the last one; z between the problems stays zero
-    auto smooth = [&](int k, int flags) -> int {
-        for (auto &grp : B.groups) {
-            auto &g = grp.prec<T>();
-            LC(launch_smooth_batch<T>(B.dim, grp.q, g.D, g.map[TILE_SMOOTH], g.nblocks[TILE_SMOOTH],
-                                      g.tile[TILE_SMOOTH], exact, flags, z + grp.dof0, r + grp.dof0, k & 1, s));
-        }
+    auto smooth = [&](dgmg_batch::Group &grp, int k, int flags, cudaStream_t t) -> int {
+        auto &g = grp.prec<T>();
+        LC(launch_smooth_batch<T>(B.dim, grp.q, g.D, g.map[TILE_SMOOTH], g.nblocks[TILE_SMOOTH], g.tile[TILE_SMOOTH],
+                                  exact, flags, z + grp.dof0, r + grp.dof0, k & 1, t));
         return DGMG_OK;
     };
-    for (int k = 0; k < B.opts.nu_pre; ++k) RC(smooth(k, k == 0 ? SM_ZERO : 0));
-    for (auto &grp : B.groups) {
+    RC(for_groups(B, s, [&](dgmg_batch::Group &grp, cudaStream_t t) -> int {
         auto &g = grp.prec<T>();
+        for (int k = 0; k < B.opts.nu_pre; ++k) RC(smooth(grp, k, k == 0 ? SM_ZERO : 0, t));
         LC(launch_residual_batch<T>(B.dim, grp.q, g.D, g.map[TILE_RESIDUAL], g.nblocks[TILE_RESIDUAL],
                                     g.tile[TILE_RESIDUAL], RES_HAS_B | RES_CORNERS, z + grp.dof0, r + grp.dof0,
-                                    nullptr, B.opts.nu_pre & 1, s));
-    }
+                                    nullptr, B.opts.nu_pre & 1, t));
+        return DGMG_OK;
+    }));
     LC(launch_corner_gather_batch<T>(B.dim, B.cg<T>(), B.gather, B.ngather, s));
     RC(batch_cg_cycle<T>(B, 0, s));
-    for (auto &grp : B.groups) {
+    return for_groups(B, s, [&](dgmg_batch::Group &grp, cudaStream_t t) -> int {
         auto &g = grp.prec<T>();
         LC(launch_project_batch<T>(B.dim, grp.q, g.D, g.map[TILE_PROJECT], g.nblocks[TILE_PROJECT],
-                                   g.tile[TILE_PROJECT], z + grp.dof0, 1, s));
-    }
-    for (int k = 0; k < B.opts.nu_post; ++k) RC(smooth(k, k == B.opts.nu_post - 1 ? SM_NO_TRACES : 0));
-    return DGMG_OK;
+                                   g.tile[TILE_PROJECT], z + grp.dof0, 1, t));
+        for (int k = 0; k < B.opts.nu_post; ++k) RC(smooth(grp, k, k == B.opts.nu_post - 1 ? SM_NO_TRACES : 0, t));
+        return DGMG_OK;
+    });
 }
 
 unsigned small_grid(int count) { return (unsigned)((count + 127) / 128); }
@@ -938,6 +968,12 @@ int dgmg_batch_create(int count, const dgmg_mesh *meshes, const int *p, const do
     LC(cudaMallocHost((void **)&B->h_norm, sizeof(double) * count));
     LC(cudaEventCreateWithFlags(&B->ev, cudaEventDisableTiming));
     LC(cudaStreamCreateWithFlags(&B->capture_stream, cudaStreamNonBlocking));
+    LC(cudaEventCreateWithFlags(&B->fork, cudaEventDisableTiming));
+    B->side.resize(B->groups.size() - 1);
+    for (auto &t : B->side) {
+        LC(cudaStreamCreateWithFlags(&t.s, cudaStreamNonBlocking));
+        LC(cudaEventCreateWithFlags(&t.done, cudaEventDisableTiming));
+    }
     for (dgmg_ctx *c : B->inst) B->bytes += c->bytes;
     LC(cudaDeviceSynchronize());
     phase("q1 descriptors");
