@@ -411,10 +411,10 @@ const T *level_result(const dgmg_batch &B, int i, int l) {
     return L.u[(B.opts.nu_pre + B.opts.nu_post) & 1];
 }
 
-// The one-thread-per-cell FP32 kernel for stage `stage`: the smoothing step and the
-// residual with exact blocks.
+// The one-thread-per-cell FP32 kernel for stage `stage`: the projection, and with exact
+// blocks the smoothing step and the residual.
 bool cells_stage(const dgmg_batch &B, int q, int stage) {
-    return B.dim == 3 && q <= 5 && B.opts.block_inverse == DGMG_BLOCK_EXACT && stage != TILE_PROJECT;
+    return B.dim == 3 && q <= 5 && (B.opts.block_inverse == DGMG_BLOCK_EXACT || stage == TILE_PROJECT);
 }
 
 template <typename T>

@@ -847,6 +847,21 @@ __global__ void __launch_bounds__(256) k_smooth_batch(const BatchDG<T> *__restri
 }
 
 template <typename T, int Q>
+__global__ void __launch_bounds__(32) k_project_cells_batch(const BatchDG<T> *__restrict__ D,
+                                                             const BlockMap *__restrict__ map, int nblocks, T *u,
+                                                             int with_e0) {
+    constexpr int NL = Q * Q * Q;
+    __shared__ __align__(16) BatchDG<T> sd;
+    for (int k = blockIdx.x; k < nblocks; k += gridDim.x) {
+        if (k != (int)blockIdx.x) __syncthreads();
+        const BlockMap m = map[k];
+        load_batch_desc(D + m.inst, &sd);
+        project_cells_body<T, Q>(sd.c, m.cell0, u + sd.off * NL, with_e0 ? sd.e0 : nullptr, sd.tr[0],
+                                 k != (int)blockIdx.x);
+    }
+}
+
+template <typename T, int Q>
 __global__ void __launch_bounds__(32) k_smooth_cells_batch(const BatchDG<T> *__restrict__ D,
                                                             const BlockMap *__restrict__ map, int nblocks,
                                                             int flags, T *u, const T *b, int cur) {
@@ -1053,7 +1068,23 @@ struct DGLaunch {
     static cudaError_t project_batch(const BatchDG<T> *D, const BlockMap *map, int nblocks, int cpb, T *u,
                                      int with_e0, cudaStream_t s) {
         if (nblocks <= 0) return cudaSuccess;
-        if (cpb <= 0) cpb = default_cpb();
+        if constexpr (CELLS_OK) {
+            if (cpb <= 0) {          // the map holds 32-cell blocks
+                using CG = CellGeo<T, Q>;
+                static bool attr_c = false;
+                if (!attr_c) {
+                    cudaFuncSetAttribute(k_project_cells_batch<T, Q>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)CG::BYTES);
+                    attr_c = true;
+                }
+                count_launches(1);
+                k_project_cells_batch<T, Q><<<persistent_grid((const void *)k_project_cells_batch<T, Q>, CG::W, CG::BYTES,
+                                                              nblocks),
+                                              CG::W, CG::BYTES, s>>>(D, map, nblocks, u, with_e0);
+                return cudaGetLastError();
+            }
+        }
+        if (cpb <= 0) return cudaErrorInvalidValue;   // the map was built for 32-cell blocks
         static bool attr = false;
         if (!attr) {
             cudaFuncSetAttribute(k_project_batch<DIM, Q, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);

@@ -723,7 +723,7 @@ __device__ __forceinline__ void smooth_cells_body(const DGConst<T> &c, int64_t c
 // leaves by a bulk store, the traces as in the smoothing step.
 template <typename T, int Q>
 __device__ __forceinline__ void project_cells_body(const DGConst<T> &c, int64_t cell0, T *__restrict__ u,
-                                                   const T *__restrict__ e0, T *__restrict__ tr) {
+                                                   const T *__restrict__ e0, T *__restrict__ tr, bool reuse = false) {
     using G = CellGeo<T, Q>;
     constexpr int W = G::W, NL = G::NL, CS = G::CS;
     extern __shared__ __align__(128) unsigned char smem_c[];
@@ -735,11 +735,7 @@ __device__ __forceinline__ void project_cells_body(const DGConst<T> &c, int64_t 
     const bool full = ncl == W;
     const bool active = lane < ncl;
     const int64_t cell = cell0 + lane;
-    if (full && lane == 0) {
-        mbar_init(&bars[0], 1);
-        fence_mbar_init();
-        fence_proxy_async_smem();
-    }
+    cells_init_bars(bars, 1, lane, reuse);
     stage_cells<T, Q>(full, lane, &bars[0], sA, u + cell0 * NL, ncl);
     // the corner values of the correction (zero at boundary vertices)
     T ec[8];
