@@ -24,12 +24,12 @@
 // d q multiply-adds per node for M instead of two tangential masses per face and
 // field, and no mass at all in the first step from a zero iterate.
 //
-// What bounds it: the integer multiply-add pipe (57% busy at q = 4, 308 of its
-// instructions per node of a smoothing step, 36 of them per matrix pass over the three
-// axes) with the ALU at 38% and 12 to 16 warps per SM to cover the latencies. Measured
+// What bounds it: the integer multiply-add pipe (59% busy at q = 4 with a last wave of
+// CTAs that fills 68% of the chip; about 290 of its instructions per node of a smoothing
+// step) with the ALU at 39% and 12 to 16 warps per SM to cover the latencies. Measured
 // per launch, FP64 pipe kernels before / these: smoothing step 33 x 31 x 32 cells
-// p = 3 0.247 / 0.098 ms, 729^2 cells p = 4 1.11 / 0.51 ms; operator 64 x 60 x 57 cells
-// p = 4 3.04 / 1.0 ms; projection 32^3 cells p = 3 0.042 / 0.022 ms.
+// p = 3 0.247 / 0.096 ms, 729^2 cells p = 4 1.11 / 0.50 ms; operator 64 x 60 x 57 cells
+// p = 4 3.04 / 0.96 ms; projection 32^3 cells p = 3 0.042 / 0.022 ms.
 #pragma once
 
 #include <algorithm>
@@ -224,6 +224,81 @@ __device__ __forceinline__ FxBlock fx_pass(long long *xc, FxBlock b, int a, cons
         }
     }
     return fx_block<Q>(mag, b.e - b.n + ea + 64, L);
+}
+
+// t <- M t along axis a, M the 1D mass, which is symmetric about its centre: with
+// e = x_j + x_j', o = x_j - x_j' (j' = q - 1 - j) the outputs i and i' are
+// (E e)_i +- (O o)_i, E = (M_ij + M_ij') / 2, O = (M_ij - M_ij') / 2: half the
+// multiply-adds (q = 4: 8 of 16 a pencil), for 2 q additions. GL: the mass is diagonal.
+// T: E and O, row-major, or M (GL). |e|, |o| < 2^61 and the h of a row of E and O sum to
+// half of M's, so the sums keep the bounds of Acc. With full matrices: residual 243^2
+// cells p = 6 GL 120 us (now 110), operator 64^3 p = 4 1192 (1141), smoothing 32^3 p = 3
+// 100 (98) a step.
+template <int DIM, int Q>
+__device__ __forceinline__ FxBlock fx_mass(long long *xc, FxBlock b, int a, const Limb *T, int eM, bool gl, FxLane &L) {
+    using G = FxGeo<DIM, Q>;
+    constexpr int H = Q / 2, HE = Q - H;                  // sizes of O and E
+    const FxAxis ax = fx_axis<DIM, Q>(a, L.k);
+    FxMag mag;
+    long long *t = xc + ax.first;
+    if (gl) {
+#pragma unroll 1
+        for (int p = 0; p < G::NP; ++p, t += ax.next)
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                Acc s;
+                acc_zero(s);
+                mac(s, T[i * Q + i], fx_read(t[i * ax.step], b.n));
+                const long long v = acc_value(s);
+                if (G::ALL || L.live) t[i * ax.step] = v;
+                mag.add(v);
+            }
+        return fx_block<Q>(mag, b.e - b.n + eM + 64, L);
+    }
+    Limb E[HE * HE], O[H * H];
+#pragma unroll
+    for (int i = 0; i < HE * HE; ++i) E[i] = T[i];
+#pragma unroll
+    for (int i = 0; i < H * H; ++i) O[i] = T[HE * HE + i];
+#pragma unroll 1
+    for (int p = 0; p < G::NP; ++p, t += ax.next) {
+        Acc se[HE], so[H];
+#pragma unroll
+        for (int i = 0; i < HE; ++i) acc_zero(se[i]);
+#pragma unroll
+        for (int i = 0; i < H; ++i) acc_zero(so[i]);
+#pragma unroll
+        for (int j = 0; j < H; ++j) {
+            const long long x = t[j * ax.step] << b.n, y = t[(Q - 1 - j) * ax.step] << b.n;
+            const Limb e = limb_of(x + y), o = limb_of(x - y);
+#pragma unroll
+            for (int i = 0; i < HE; ++i) mac(se[i], E[i * HE + j], e);
+#pragma unroll
+            for (int i = 0; i < H; ++i) mac(so[i], O[i * H + j], o);
+        }
+        if constexpr (Q % 2 != 0) {
+            const Limb x = fx_read(t[H * ax.step], b.n);
+#pragma unroll
+            for (int i = 0; i < HE; ++i) mac(se[i], E[i * HE + H], x);
+        }
+#pragma unroll
+        for (int i = 0; i < HE; ++i) {
+            const long long ve = acc_value(se[i]);
+            if (i < H) {
+                const long long vo = acc_value(so[i < H ? i : 0]), v = ve + vo, w = ve - vo;
+                if (G::ALL || L.live) {
+                    t[i * ax.step] = v;
+                    t[(Q - 1 - i) * ax.step] = w;
+                }
+                mag.add(v);
+                mag.add(w);
+            } else {
+                if (G::ALL || L.live) t[i * ax.step] = ve;
+                mag.add(ve);
+            }
+        }
+    }
+    return fx_block<Q>(mag, b.e - b.n + eM + 64, L);
 }
 
 // Largest biased exponent of the lane's slab of FP64 values.
@@ -584,9 +659,13 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
             if (!zero) fx_stage_in<DIM, Q>(Y, u + cell0 * NL, ncl * NL, L.lane);
         }
         const int a = k < DIM ? DIM - 1 - k : (k < 2 * DIM ? k - DIM : 3 * DIM - 1 - k);
-        const bool mass = k < DIM, trans = !mass && k < 2 * DIM;
-        const Limb *src = mass ? sTab : myF + a * G::FDS;
-        t = fx_pass<DIM, Q>(xc, t, a, src, trans ? 1 : Q, trans ? Q : 1, mass ? tab.eM : src[Q * Q].h, L);
+        if (k < DIM) {
+            t = fx_mass<DIM, Q>(xc, t, a, sTab, tab.eM, tab.gl != 0, L);
+        } else if constexpr (SMOOTH) {
+            const bool trans = k < 2 * DIM;
+            const Limb *src = myF + a * G::FDS;
+            t = fx_pass<DIM, Q>(xc, t, a, src, trans ? 1 : Q, trans ? Q : 1, src[Q * Q].h, L);
+        }
     }
     if (!SMOOTH && has_b) subtract_from_b();
     if constexpr (SMOOTH) {
@@ -685,8 +764,19 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
 template <int DIM, int Q, int MODE>
 __device__ __forceinline__ const Limb *fx_stage_tables(const FxTab &tab, long long *smem) {
     Limb *s = reinterpret_cast<Limb *>(smem);
+    constexpr int H = Q / 2, HE = Q - H;
     for (int i = threadIdx.x; i < Q * Q; i += blockDim.x) {
-        s[i] = tab.M[i];
+        // the mass as fx_mass reads it: E, then O (GL: M)
+        auto whole = [&](int r, int c) { return ((long long)tab.M[r * Q + c].h << 32) + tab.M[r * Q + c].l; };
+        if (tab.gl) {
+            s[i] = tab.M[i];
+        } else if (i < HE * HE) {
+            const int r = i / HE, c = i - r * HE;
+            s[i] = limb_of((whole(r, c) + whole(r, Q - 1 - c)) >> 1);
+        } else if (i < HE * HE + H * H) {
+            const int r = (i - HE * HE) / H, c = i - HE * HE - r * H;
+            s[i] = limb_of((whole(r, c) - whole(r, Q - 1 - c)) >> 1);
+        }
         if (MODE != FXM_SMOOTH) {
             s[Q * Q + i] = tab.K[i];
             s[2 * Q * Q + i] = tab.L[0][i];
