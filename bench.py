@@ -39,9 +39,12 @@ FP64_NOMINAL_TFLOPS = 1.25       # nominal GB300 dense FP64, context beside the 
 # DRAM bytes (read + write) of one launch of the FP64 smoothing kernel on this
 # workload from one ncu capture, valid only for the kernel sources it was taken
 # on (SHA-256 of the files below); once they change, `traffic` reads null
-SMOOTH_TRAFFIC = {"kernel": "k_smooth_cells<double,4>", "bytes": 116_628_736 + 10_494_464,
-                  "sources_sha256": "7b1b09b1125962089f573f3432c4a423ffed4cdec4c1dcacfab6e84818cc62ad",
-                  "files": ("smooth_cells.cuh", "dg_kernels.cuh", "dg_fp64.cu")}
+SMOOTH_TRAFFIC = {"kernel": "k_fx_cells<3,4,0>", "bytes": None,
+                  "sources_sha256": "0" * 64,
+                  "files": ("fx.cuh", "dg_fx.cuh", "dg_fp64.cu")}
+# 32 x 32 + 64 bit integer multiply-adds per SM and clock (a loop of independent
+# products); the FP64 kernels of the DG levels take three per multiply-add
+INT_MAD_PER_SM_CLK = 30
 
 
 def parse():
@@ -106,8 +109,10 @@ def smooth_traffic(kernel):
 
 # ---------------------------------------------------------------- flop model
 def smooth_flops(n, q):
-    """Floating-point operations of one launch of the FP64 fused smoothing kernel
-    as implemented (an FMA counts 2, a multiplication 1): facet mass on the two
+    """Floating-point operations of one FP64 fused smoothing step in its
+    sum-factorised form (an FMA counts 2, a multiplication 1), the fixed count the
+    rates are quoted on (the kernel's own products are integer multiply-adds, with the
+    tangential masses taken once per node instead of per face): facet mass on the two
     neighbour fields of every interior face side (each 1D mass in its rank-one
     form diag(w) - u u^T: per pencil of q values a dot product, q multiplications
     and q FMAs, 5q operations); lifting (per face node q FMAs for the value
@@ -533,8 +538,9 @@ def run_gb300(args):
     units_local = float(ndof) * smooth_steps_total
     t_max, units = reduce_max_sum((total_ms, units_local), world, dev)
     value = units / (t_max * 1e-3) / 1e9
-    # roofline of the dominant kernel (the fused smoothing step): FP64-pipe
-    # bound, against the FP64 FMA-loop peak measured here, in this run
+    # roofline of the dominant kernel (the fused smoothing step): bound by the integer
+    # multiply-add pipe, which computes its fixed-point products; the FP64 FMA-loop
+    # peak measured here, in this run, beside it
     sm_ms, sm_n = prof["smooth"]
     avg_ms = sm_ms / max(sm_n, 1)
     flops = smooth_flops(N_CELLS, q)
@@ -578,9 +584,9 @@ def run_gb300(args):
     if rank == 0 and not args.no_mixed:
         mixed = mixed_section(flush, stream)
 
-    # the smoothing kernel the tuned context runs (tile 0 = one thread per cell)
-    cells_kernel = ctx.info.tiles[1] == 0 and d == 3 and q <= 4
-    smooth_kernel = f"k_smooth_cells<double,{q}>" if cells_kernel else f"k_smooth<{d},{q},double>"
+    smooth_kernel = f"k_fx_cells<{d},{q},0>"
+    props = torch.cuda.get_device_properties(local)
+    int_peak = 2 * INT_MAD_PER_SM_CLK / 3 * props.multi_processor_count * (clk.get("sm_mhz") or 2070) * 1e-6
     traffic, traffic_note = smooth_traffic(smooth_kernel)
     if rank == 0:
         cpu = None
@@ -596,15 +602,17 @@ def run_gb300(args):
                        "outer": "FP64 PCG", "step": "one full solve from x=0",
                        "l2": "flushed (256 MB write) before every timed step, outside the step's events",
                        "parallelism": f"replicas x{world}"},
-            "roofline": {"bound": "alu", "achieved": achieved, "peak": fp64_peak, "unit": "TFLOP/s",
-                         "frac": achieved / fp64_peak,
+            "roofline": {"bound": "alu", "achieved": achieved, "peak": int_peak, "unit": "TFLOP/s",
+                         "frac": achieved / int_peak, "times_fp64_fma_peak": achieved / fp64_peak,
                          "traffic": traffic, "traffic_note": traffic_note,
                          "kernel": smooth_kernel, "avg_launch_ms": avg_ms,
                          "flops_per_launch": flops,
-                         "frac_at_10dq_flop_per_dof": survey_flops / (avg_ms * 1e-3) / 1e12 / fp64_peak,
+                         "frac_at_10dq_flop_per_dof": survey_flops / (avg_ms * 1e-3) / 1e12 / int_peak,
                          "hbm_bytes_per_launch": smooth_bytes_per_cell(d, q) * ctx.info.ncell,
-                         "peak_note": ("FP64 FMA-loop peak measured in this run (dgmg_fma_peak), of measured; "
-                                       f"nominal {FP64_NOMINAL_TFLOPS}"),
+                         "peak_note": ("64-bit fixed-point multiply-adds: a third of the measured integer "
+                                       f"multiply-add rate ({INT_MAD_PER_SM_CLK} per SM and clock) at the run's SM "
+                                       "clock; the FP64 pipe's FMA-loop peak (dgmg_fma_peak, this run) is under "
+                                       f"measured_peaks_tflops, its nominal {FP64_NOMINAL_TFLOPS}"),
                          "measured_peaks_tflops": {"fp64_fma": fp64_peak, "fp32_fma": fp32_peak,
                                                    "fp32x2_fma": fp32x2_peak, "clocks": peak_clk}},
             "cpu_baseline": cpu,
