@@ -471,7 +471,7 @@ int setup_dg(dgmg_ctx &C, const DGSpace &S, DGDev<T> &D, const std::vector<doubl
         D.c.cst.kfac = D.kfac;
     else
         D.c.kfac = D.kfac;
-    const int64_t trn = C.ncell * 2 * C.dim * trace_face_stride<T>((int)(S.nloc / S.q));
+    const int64_t trn = trace_count<T>(C.ncell, C.dim, (int)(S.nloc / S.q));
     if (!smoother) {                  // operator only (projection, residual): no block-inverse factors
         RC(C.alloc(&D.tr[0], trn));
         RC(C.alloc(&D.tr[1], trn));
@@ -921,12 +921,14 @@ template <typename T>
 int level_cycle(dgmg_ctx &C, int l, const T *b, T *z, cudaStream_t s) {
     DGDev<T> &D = dg_level<T>(C, l);
     const DGSpace &S = C.dgs[l];
-    const int64_t trn = C.ncell * 2 * C.dim * trace_face_stride<T>((int)(S.nloc / S.q));
+    const int64_t trv = trace_values<T>(C.ncell, C.dim, (int)(S.nloc / S.q)),
+                  tre = trace_count<T>(C.ncell, C.dim, (int)(S.nloc / S.q)) - trv;
     // the first step takes the zero iterate as such (no facet terms, nothing to
     // clear), and nothing reads the projections of the last one
     if (C.opts.nu_pre == 0) {
         LC(cudaMemsetAsync(z, 0, sizeof(T) * S.ndof, s));
-        LC(cudaMemsetAsync(D.tr[0], 0, sizeof(T) * trn, s));   // projections of z = 0
+        LC(cudaMemsetAsync(D.tr[0], 0, sizeof(T) * trv, s));   // projections of z = 0
+        if (tre) LC(cudaMemsetAsync(D.tr[0] + trv, TRACE_NO_EXPONENT, sizeof(T) * tre, s));
     }
     int cur = 0;
     for (int k = 0; k < C.opts.nu_pre; ++k) {
@@ -1027,7 +1029,7 @@ static int tune_tiles(dgmg_ctx &C, float *u, float *b, int *tile, bool trace) {
     DGDev<T> &D = dg<T>(C);
     cudaStream_t s = C.setup_stream;
     const int nf = (int)(C.nloc / C.q);
-    const int64_t trn = C.ncell * 2 * C.dim * trace_face_stride<T>(nf);
+    const int64_t trn = trace_count<T>(C.ncell, C.dim, nf);
     std::vector<int> cand;
     for (int c = 1; c <= 64; c *= 2)
         if (c * nf >= 32 && c * nf <= 256) cand.push_back(c);
@@ -1517,7 +1519,7 @@ int dgmg_project(dgmg_ctx *C, double *u, const double *e, double *traces, void *
     RC(check_ctx(C));
     NEED(u);
     NEED(traces);
-    LC(launch_project<double>(C->dim, C->q, C->d64.c, C->tile[0][TILE_PROJECT], u, e, traces, (cudaStream_t)stream));
+    LC(launch_project_user(C->dim, C->q, C->d64.c, u, e, traces, (cudaStream_t)stream));
     return DGMG_OK;
 }
 
@@ -1531,8 +1533,7 @@ int dgmg_residual_restrict(dgmg_ctx *C, const double *u, const double *b, const 
     int mode = RES_HAS_B;
     if (r) mode |= RES_WRITE_R;
     if (rc) mode |= RES_CORNERS;
-    LC(launch_residual<double>(C->dim, C->q, C->d64.c, C->tile[0][TILE_RESIDUAL], mode, u, b, C->d64.kappa, traces, r,
-                               C->d64.corners, exact_fd(*C, C->d64), s));
+    LC(launch_residual_user(C->dim, C->q, C->d64.c, mode, u, b, C->d64.kappa, traces, r, C->d64.corners, s));
     if (rc) LC(launch_corner_gather<double>(C->dim, C->n, C->d64.corners, rc, s));
     return DGMG_OK;
 }
@@ -1624,8 +1625,7 @@ static int estimate_bytes_of(const dgmg_mesh *mesh, int p, const dgmg_opts *opts
     const int64_t ncell = (int64_t)n[0] * n[1] * n[2];
     const int64_t nloc = dim == 3 ? (int64_t)q * q * q : (int64_t)q * q, ndof = ncell * nloc;
     const int64_t nf = nloc / q, ns = dim == 3 ? 27 : 9;
-    const int64_t tr = ncell * 2 * dim * trace_face_stride<double>((int)nf);
-    const int64_t tr32 = ncell * 2 * dim * trace_face_stride<float>((int)nf);
+    const int64_t tr = trace_count<double>(ncell, dim, (int)nf), tr32 = trace_count<float>(ncell, dim, (int)nf);
     auto sz = [](int64_t count, size_t elem) { return (size_t)std::max<int64_t>(count, 1) * elem; };
     size_t dg64 = sz(ncell, 8) + sz(ncell * dim * (q * q + q), 8) + sz(ndof, 8) + 2 * sz(tr, 8) +
                   sz(ncell << dim, 8) + sz(ncell * 2 * dim, 8);   // kappa, factors, table,
@@ -1672,8 +1672,8 @@ static int estimate_bytes_of(const dgmg_mesh *mesh, int p, const dgmg_opts *opts
         for (int pc = p - 1; pc >= 1; --pc) {
             const int ql = pc + 1;
             const int64_t nl = dim == 3 ? (int64_t)ql * ql * ql : (int64_t)ql * ql, nd = ncell * nl;
-            const int64_t trl = ncell * 2 * dim * trace_face_stride<double>((int)(nl / ql));
-            const int64_t trl32 = ncell * 2 * dim * trace_face_stride<float>((int)(nl / ql));
+            const int64_t trl = trace_count<double>(ncell, dim, (int)(nl / ql)),
+                          trl32 = trace_count<float>(ncell, dim, (int)(nl / ql));
             const int64_t fdl = ncell * dim * (ql * ql + ql);
             total += sz(fdl, 8) + sz(nd, 8) + 2 * sz(trl, 8) + sz(ncell << dim, 8) + 3 * sz(nd, 8);
             if (mixed) total += 2 * sz(fdl, 4) + 2 * sz(trl32, 4) + sz(ncell << dim, 4) + 3 * sz(nd, 4);
@@ -1740,8 +1740,7 @@ int residual_restrict_with_scratch(dgmg_ctx *C, const double *u, const double *b
     int mode = RES_HAS_B;
     if (r) mode |= RES_WRITE_R;
     if (rc) mode |= RES_CORNERS;
-    LC(launch_residual<double>(C->dim, C->q, C->d64.c, C->tile[0][TILE_RESIDUAL], mode, u, b, C->d64.kappa, traces, r,
-                               corner_scratch, exact_fd(*C, C->d64), s));
+    LC(launch_residual_user(C->dim, C->q, C->d64.c, mode, u, b, C->d64.kappa, traces, r, corner_scratch, s));
     if (rc) LC(launch_corner_gather<double>(C->dim, C->n, corner_scratch, rc, s));
     return DGMG_OK;
 }

@@ -50,7 +50,12 @@ template <>
 cudaError_t launch_project<double>(int dim, int q, const DGConst<double> &c, int, double *u, const double *e0,
                                    double *tr, cudaStream_t s) {
     if (!fx_valid(dim, q)) return cudaErrorInvalidValue;
-    return fx_dispatch(dim, q, [&](auto run) { return decltype(run)::project(c, u, e0, tr, s); });
+    return fx_dispatch(dim, q, [&](auto run) { return decltype(run)::project(c, false, u, e0, tr, s); });
+}
+cudaError_t launch_project_user(int dim, int q, const DGConst<double> &c, double *u, const double *e0, double *tr,
+                                cudaStream_t s) {
+    if (!fx_valid(dim, q)) return cudaErrorInvalidValue;
+    return fx_dispatch(dim, q, [&](auto run) { return decltype(run)::project(c, true, u, e0, tr, s); });
 }
 
 template <>
@@ -68,8 +73,14 @@ cudaError_t launch_residual<double>(int dim, int q, const DGConst<double> &c, in
                                     const double *b, const double *kappa, const double *tr, double *r, double *corners,
                                     const double *, cudaStream_t s) {
     if (!fx_valid(dim, q)) return cudaErrorInvalidValue;
-    return fx_dispatch(dim, q,
-                       [&](auto run) { return decltype(run)::residual(c, mode, u, b, kappa, tr, r, corners, s); });
+    return fx_dispatch(
+        dim, q, [&](auto run) { return decltype(run)::residual(c, false, mode, u, b, kappa, tr, r, corners, s); });
+}
+cudaError_t launch_residual_user(int dim, int q, const DGConst<double> &c, int mode, const double *u, const double *b,
+                                 const double *kappa, const double *tr, double *r, double *corners, cudaStream_t s) {
+    if (!fx_valid(dim, q)) return cudaErrorInvalidValue;
+    return fx_dispatch(
+        dim, q, [&](auto run) { return decltype(run)::residual(c, true, mode, u, b, kappa, tr, r, corners, s); });
 }
 
 template <>

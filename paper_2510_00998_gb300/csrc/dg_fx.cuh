@@ -28,7 +28,7 @@
 // CTAs that fills 68% of the chip; about 290 of its instructions per node of a smoothing
 // step) with the ALU at 39% and 12 to 16 warps per SM to cover the latencies. Measured
 // per launch, FP64 pipe kernels before / these: smoothing step 33 x 31 x 32 cells
-// p = 3 0.247 / 0.096 ms, 729^2 cells p = 4 1.11 / 0.50 ms; operator 64 x 60 x 57 cells
+// p = 3 0.247 / 0.093 ms, 729^2 cells p = 4 1.11 / 0.50 ms; operator 64 x 60 x 57 cells
 // p = 4 3.04 / 0.96 ms; projection 32^3 cells p = 3 0.042 / 0.022 ms.
 #pragma once
 
@@ -41,7 +41,14 @@
 namespace dgmg {
 
 
-enum { FXM_SMOOTH = 0, FXM_SMOOTH_FULL = 1, FXM_RESIDUAL = 2 };
+// FXM_RESIDUAL_USER: the residual from traces in FP64 (those a caller holds). All other
+// kernels exchange traces as they compute them: integers of one exponent per cell, with
+// the unused leading bits of each face beside it, so that a reader's sums use all their
+// bits (from the exponent alone the errors were three times larger). A face value then
+// costs a shift or two on its way in and next to nothing on its way out; converted to FP64
+// and back it cost some 40 instructions, a sixth of the smoothing step's: 32^3 cells p = 3
+// 98 -> 93 us a step, 23^3 p = 2 V-cycle 149 -> 141 us, 729^2 p = 4 508 -> 501 us.
+enum { FXM_SMOOTH = 0, FXM_SMOOTH_FULL = 1, FXM_RESIDUAL = 2, FXM_RESIDUAL_USER = 3 };
 
 template <int DIM, int Q>
 struct FxGeo {
@@ -64,7 +71,7 @@ struct FxGeo {
     // per cell: first the lifting coefficients (and the blocks D_a), then the factors
     __host__ __device__ static constexpr int small_words(int mode) {
         return ((mode == FXM_SMOOTH ? (LW > DIM * FDS ? LW : DIM * FDS)
-                                    : (LW + DW > DIM * FDS || mode == FXM_RESIDUAL ? LW + DW : DIM * FDS)) |
+                                    : (LW + DW > DIM * FDS || mode >= FXM_RESIDUAL ? LW + DW : DIM * FDS)) |
                 1);
     }
     // per CTA: M, and for the blocks D_a also K, L, R
@@ -146,6 +153,19 @@ __device__ __forceinline__ int fx_cell_max(int v, FxLane &L) {
     int m = row[L.c * Q];
 #pragma unroll
     for (int s = 1; s < Q; ++s) m = imax(m, row[L.c * Q + s]);
+    return m;
+}
+
+// The same with the smallest of each of four bytes.
+template <int Q>
+__device__ __forceinline__ unsigned fx_cell_min4(unsigned v, FxLane &L) {
+    int *row = L.ex + L.row;
+    L.row ^= 32;
+    if (L.live) row[L.lane] = (int)v;
+    __syncwarp();
+    unsigned m = (unsigned)row[L.c * Q];
+#pragma unroll
+    for (int s = 1; s < Q; ++s) m = __vminu4(m, (unsigned)row[L.c * Q + s]);
     return m;
 }
 
@@ -310,15 +330,26 @@ __device__ __forceinline__ int fx_slab_top(const double *y) {
     return mx >> 20;
 }
 
+// Per cell after the traces {e, h[axis]}: values count 2^e (GL: 2^(e + eV + 64)),
+// derivatives along axis a 2^(e + eT[a] + 64); h packs the unused leading bits (of 60) of
+// the axis' traces, byte 2 side + (0 value, 1 derivative).
+template <int DIM, int Q, typename P>
+__device__ __forceinline__ auto fx_trace_units(P *tr, int64_t ncell) {
+    using I = typename std::conditional<std::is_const<P>::value, const int4, int4>::type;
+    return reinterpret_cast<I *>(tr + ncell * FxGeo<DIM, Q>::TR);
+}
+constexpr int FX_NO_TRACE = FX_NONE / 2;     // exponents below: all values are 0
+
 // Traces of the cell from its block in shared memory: per axis and side, value and
 // +axis derivative; derivatives by dot products, values the end nodes (GLL) or dot
-// products (GL).
-template <int DIM, int Q>
+// products (GL). USER: as FP64.
+template <int DIM, int Q, bool USER = false>
 __device__ __forceinline__ void fx_all_traces(const FxTab &tab, const FxConst &cst, const long long *xc, FxBlock b,
-                                              const FxLane &L, bool write, double *__restrict__ cell_tr) {
+                                              FxLane &L, bool write, int64_t cell, double *__restrict__ tr) {
     using G = FxGeo<DIM, Q>;
-    if (!write) return;
     const int e = b.e - b.n;
+    double *cell_tr = tr + cell * G::TR;
+    unsigned room[3] = {0, 0, 0};
 #pragma unroll 1
     for (int a = 0; a < DIM; ++a) {
         const FxAxis ax = fx_axis<DIM, Q>(a, L.k);
@@ -330,8 +361,18 @@ __device__ __forceinline__ void fx_all_traces(const FxTab &tab, const FxConst &c
         const int ed = e + cst.eT[a] + 64;
         double *out = cell_tr + 2 * a * G::FS + L.k * G::NP;
         const long long *t = xc + ax.first;
+        FxMag mag[2][2];
+        auto put = [&](int s, int c, int p, long long w, int ew) {
+            double *to = out + s * G::FS + c * G::NF + p;
+            if (!USER) mag[s][c].add(w);
+            if (!write) return;
+            if (USER)
+                *to = fx_to(w, ew);
+            else
+                *reinterpret_cast<long long *>(to) = w;
+        };
 #pragma unroll 1
-        for (int p = 0; p < G::NP; ++p, t += ax.next, ++out) {
+        for (int p = 0; p < G::NP; ++p, t += ax.next) {
             Limb x[Q];
 #pragma unroll
             for (int i = 0; i < Q; ++i) x[i] = fx_read(t[i * ax.step], b.n);
@@ -341,18 +382,31 @@ __device__ __forceinline__ void fx_all_traces(const FxTab &tab, const FxConst &c
                 acc_zero(v);
 #pragma unroll
                 for (int i = 0; i < Q; ++i) mac(v, d[s][i], x[i]);
-                out[s * G::FS + G::NF] = fx_to(acc_value(v), ed);
+                put(s, 1, p, acc_value(v), ed);
                 if (tab.gl) {
                     acc_zero(v);
 #pragma unroll
                     for (int i = 0; i < Q; ++i) mac(v, tab.v[s][i], x[i]);
-                    out[s * G::FS] = fx_to(acc_value(v), e + tab.eV + 64);
+                    put(s, 0, p, acc_value(v), e + tab.eV + 64);
                 } else {
-                    out[s * G::FS] = fx_to(t[(s ? Q - 1 : 0) * ax.step], b.e);
+                    put(s, 0, p, t[(s ? Q - 1 : 0) * ax.step] << b.n, e);
                 }
             }
         }
+        if (!USER) {
+            unsigned w = 0;
+#pragma unroll
+            for (int s = 0; s < 2; ++s)
+#pragma unroll
+                for (int c = 0; c < 2; ++c) w |= (unsigned)imax(fx_headroom(mag[s][c].top()), 0) << (16 * s + 8 * c);
+            w = fx_cell_min4<Q>(w, L);
+            room[0] = a == 0 ? w : room[0];
+            room[1] = a == 1 ? w : room[1];
+            room[2] = a == 2 ? w : room[2];
+        }
     }
+    if (!USER && write && L.k == 0)
+        fx_trace_units<DIM, Q>(tr, cst.ncell)[cell] = make_int4(e, (int)room[0], (int)room[1], (int)room[2]);
 }
 
 __device__ __forceinline__ void load_batch_desc(const BatchDG<double> *__restrict__ src, BatchDG<double> *dst) {
@@ -398,7 +452,7 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
                                               double *__restrict__ r, double *__restrict__ corners) {
     using G = FxGeo<DIM, Q>;
     constexpr int N = G::N, NP = G::NP, NL = G::NL, NFACE = G::NFACE, SW = G::small_words(MODE);
-    constexpr bool SMOOTH = MODE != FXM_RESIDUAL, FULL = MODE != FXM_SMOOTH;
+    constexpr bool SMOOTH = MODE < FXM_RESIDUAL, FULL = MODE != FXM_SMOOTH, USER = MODE == FXM_RESIDUAL_USER;
     long long *X = smem;                                  // the block the passes work on
     long long *Y = X + G::CW * G::C;                      // u or b on their way in, the result on its way out
     Limb *small = reinterpret_cast<Limb *>(Y + G::CW * G::C);   // coefficients and D_a, later the factors
@@ -448,16 +502,32 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
         // lifting coefficients: facet coefficient x vector, node k of every vector by
         // lane k; the unit of the facet terms from the largest product of a
         // coefficient's and a trace's exponent
-        // (every face's high words are requested at once)
-        int mg[NFACE], mh[NFACE];
+        // units of the neighbour's value and derivative traces (USER: from the high words
+        // of the lane's values, requested at once for every face)
+        int ug[NFACE], uh[NFACE], rg[NFACE], rh[NFACE];   // units, and unused leading bits
 #pragma unroll
         for (int f = 0; f < NFACE; ++f) {
-            const double *nb = face(f >> 1, f & 1, ((mask >> f) & 1) != 0);
-            mg[f] = mh[f] = 0;
+            const int a = f >> 1;
+            if constexpr (USER) {
+                const double *nb = face(a, f & 1, ((mask >> f) & 1) != 0);
+                int mg = 0, mh = 0;
 #pragma unroll
-            for (int p = 0; p < NP; ++p) {
-                mg[f] = imax(mg[f], __ldg(reinterpret_cast<const int *>(nb + p) + 1) & 0x7fffffff);
-                mh[f] = imax(mh[f], __ldg(reinterpret_cast<const int *>(nb + G::NF + p) + 1) & 0x7fffffff);
+                for (int p = 0; p < NP; ++p) {
+                    mg = imax(mg, __ldg(reinterpret_cast<const int *>(nb + p) + 1) & 0x7fffffff);
+                    mh = imax(mh, __ldg(reinterpret_cast<const int *>(nb + G::NF + p) + 1) & 0x7fffffff);
+                }
+                ug[f] = fx_unit(mg >> 20);
+                uh[f] = fx_unit(mh >> 20);
+                rg[f] = rh[f] = 0;
+            } else {
+                const int64_t st = a == 0 ? 1 : (a == 1 ? s1 : s2);
+                const int64_t nb = (mask >> f) & 1 ? cell + (f & 1 ? st : -st) : cell;
+                const int4 en = __ldg(fx_trace_units<DIM, Q>(tr_in, cst.ncell) + nb);
+                const unsigned w = (unsigned)(a == 0 ? en.y : (a == 1 ? en.z : en.w)) >> (f & 1 ? 0 : 16);
+                ug[f] = en.x + (tab.gl ? tab.eV + 64 : 0);
+                uh[f] = en.x + cst.eT[a] + 64;
+                rg[f] = (int)(w & 255u);
+                rh[f] = (int)(w >> 8 & 255u);
             }
         }
         int top = FX_NONE;
@@ -478,14 +548,13 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
             if (L.live) {
                 mine[(f * 2 + 0) * Q + L.k] = limb_of(acc_value(g) << 4);
                 mine[(f * 2 + 1) * Q + L.k] = limb_of(acc_value(h) << 4);
-                if (L.k == 0) {
-                    sLE[(L.c * NFACE + f) * 2 + 0] = lg;
-                    sLE[(L.c * NFACE + f) * 2 + 1] = lh;
+                if (L.k == 0) {                          // the unit of a product, or (USER) of the coefficients
+                    sLE[(L.c * NFACE + f) * 2 + 0] = USER ? lg : lg + ug[f];
+                    sLE[(L.c * NFACE + f) * 2 + 1] = USER ? lh : lh + uh[f];
                 }
             }
-            const int ug = fx_unit(mg[f] >> 20), uh = fx_unit(mh[f] >> 20);
-            if (in && ug > FX_NONE) top = imax(top, ug + lg + 64);
-            if (in && uh > FX_NONE) top = imax(top, uh + lh + 64);
+            if (in && ug[f] > FX_NO_TRACE) top = imax(top, ug[f] - rg[f] + lg + 64);
+            if (in && uh[f] > FX_NO_TRACE) top = imax(top, uh[f] - rh[f] + lh + 64);
         }
         int ed = FX_NONE;
         if constexpr (FULL) {
@@ -553,7 +622,9 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
             for (int s = 0; s < 2; ++s)
 #pragma unroll
                 for (int c = 0; c < 2; ++c) {
-                    ev[s][c] = E - 64 - sLE[(L.c * NFACE + 2 * a + s) * 2 + c] + FX_UNIT;
+                    // the exponent the trace is converted with, or the places it is shifted to the right
+                    ev[s][c] = E - 64 - sLE[(L.c * NFACE + 2 * a + s) * 2 + c];
+                    ev[s][c] = USER ? ev[s][c] + FX_UNIT : imin(imax(ev[s][c], -60), 63);
 #pragma unroll
                     for (int i = 0; i < Q; ++i) cf[s][c][i] = mine[((2 * a + s) * 2 + c) * Q + i];
                 }
@@ -568,7 +639,9 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
                 for (int s = 0; s < 2; ++s)
 #pragma unroll
                     for (int c = 0; c < 2; ++c) {
-                        const long long v = fx_from(__ldg(nb[s] + c * G::NF + p), ev[s][c]);
+                        const double w = __ldg(nb[s] + c * G::NF + p);
+                        const long long v = USER ? fx_from(w, ev[s][c])
+                                                 : (__double_as_longlong(w) << imax(-ev[s][c], 0)) >> imax(ev[s][c], 0);
                         g[s][c] = limb_of(in[s] ? v : 0ll);
                     }
                 Acc v[Q];
@@ -701,7 +774,7 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
         fx_store_out<DIM, Q>((SMOOTH ? u : r) + cell0 * NL, reinterpret_cast<const double *>(Y), ncl * NL, L.lane);
     }
     if constexpr (SMOOTH) {
-        if (!(flags & SM_NO_TRACES)) fx_all_traces<DIM, Q>(tab, cst, xc, t, L, active, tr_out + cell * G::TR);
+        if (!(flags & SM_NO_TRACES)) fx_all_traces<DIM, Q>(tab, cst, xc, t, L, active, cell, tr_out);
     } else if (mode & RES_CORNERS) {
         // corner sums of b - A u: hat values along the slab's axes, then over the slabs
         constexpr int NS = DIM == 3 ? 4 : 2;             // sums per slab
@@ -834,7 +907,7 @@ __global__ void __launch_bounds__(FxGeo<DIM, Q>::NW * 32, FxGeo<DIM, Q>::MINB)
 
 // Warm-up projection of the warp's cells: optionally u += P e (the multilinear hats
 // of the cell's corner values), then the traces.
-template <int DIM, int Q>
+template <int DIM, int Q, bool USER = false>
 __device__ __forceinline__ void fx_project_body(const FxTab &tab, const FxConst &cst, long long *smem, int64_t cell0,
                                                 double *u, const double *__restrict__ e0, double *__restrict__ tr) {
     using G = FxGeo<DIM, Q>;
@@ -930,10 +1003,10 @@ __device__ __forceinline__ void fx_project_body(const FxTab &tab, const FxConst 
         }
         __syncwarp();
     }
-    fx_all_traces<DIM, Q>(tab, cst, xc, t, L, active, tr + cell * G::TR);
+    fx_all_traces<DIM, Q, USER>(tab, cst, xc, t, L, active, cell, tr);
 }
 
-template <int DIM, int Q>
+template <int DIM, int Q, bool USER>
 __global__ void __launch_bounds__(FxGeo<DIM, Q>::NW * 32)
     k_fx_project(const __grid_constant__ FxTab tab, const __grid_constant__ FxConst cst, double *u,
                  const double *__restrict__ e0, double *__restrict__ tr) {
@@ -942,7 +1015,7 @@ __global__ void __launch_bounds__(FxGeo<DIM, Q>::NW * 32)
     const int warp = threadIdx.x >> 5;
     const int64_t cell0 = (int64_t)blockIdx.x * G::CPB + warp * G::CW;
     if (cell0 >= cst.ncell) return;
-    fx_project_body<DIM, Q>(tab, cst, smem_fx + warp * G::warp_words_project(), cell0, u, e0, tr);
+    fx_project_body<DIM, Q, USER>(tab, cst, smem_fx + warp * G::warp_words_project(), cell0, u, e0, tr);
 }
 
 template <int DIM, int Q>
@@ -998,13 +1071,13 @@ cudaError_t fx_run_cells_batch(const FxTab &tab, const BatchDG<double> *D, const
 }
 
 template <int DIM, int Q>
-cudaError_t FxRun<DIM, Q>::project(const FxLevel &l, double *u, const double *e0, double *tr, cudaStream_t s) {
+cudaError_t FxRun<DIM, Q>::project(const FxLevel &l, bool user, double *u, const double *e0, double *tr, cudaStream_t s) {
     using G = FxGeo<DIM, Q>;
     if (l.cst.ncell <= 0) return cudaSuccess;
-    fx_allow_smem(k_fx_project<DIM, Q>, G::bytes_project());
+    const auto fn = user ? k_fx_project<DIM, Q, true> : k_fx_project<DIM, Q, false>;
+    fx_allow_smem(fn, G::bytes_project());
     count_launches(1);
-    k_fx_project<DIM, Q><<<(unsigned)((l.cst.ncell + G::CPB - 1) / G::CPB), G::NW * 32, G::bytes_project(), s>>>(
-        l.tab, l.cst, u, e0, tr);
+    fn<<<(unsigned)((l.cst.ncell + G::CPB - 1) / G::CPB), G::NW * 32, G::bytes_project(), s>>>(l.tab, l.cst, u, e0, tr);
     return cudaGetLastError();
 }
 template <int DIM, int Q>
@@ -1016,8 +1089,11 @@ cudaError_t FxRun<DIM, Q>::smooth(const FxLevel &l, bool exact, int flags, doubl
     return fx_run_cells<DIM, Q, FXM_SMOOTH_FULL>(l, flags, 0, u, b, kappa, fd, linv, tri, tro, nullptr, nullptr, s);
 }
 template <int DIM, int Q>
-cudaError_t FxRun<DIM, Q>::residual(const FxLevel &l, int mode, const double *u, const double *b, const double *kappa,
-                                    const double *tr, double *r, double *corners, cudaStream_t s) {
+cudaError_t FxRun<DIM, Q>::residual(const FxLevel &l, bool user, int mode, const double *u, const double *b,
+                                    const double *kappa, const double *tr, double *r, double *corners, cudaStream_t s) {
+    if (user)
+        return fx_run_cells<DIM, Q, FXM_RESIDUAL_USER>(l, 0, mode, const_cast<double *>(u), b, kappa, nullptr, nullptr,
+                                                       tr, nullptr, r, corners, s);
     return fx_run_cells<DIM, Q, FXM_RESIDUAL>(l, 0, mode, const_cast<double *>(u), b, kappa, nullptr, nullptr, tr,
                                               nullptr, r, corners, s);
 }

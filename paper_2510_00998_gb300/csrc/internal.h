@@ -39,6 +39,19 @@ __host__ __device__ constexpr int trace_face_stride(int nf) {
     return (sizeof(T) == 4 ? units | 1 : units) * 16 / (int)sizeof(T);
 }
 
+// Elements of a level's trace buffer: the faces of every cell, and in FP64 four words per
+// cell after them (the exponent, the unused leading bits of each face's values). Zero
+// traces: the faces zeroed, the bytes of those words TRACE_NO_EXPONENT.
+template <typename T>
+constexpr int64_t trace_values(int64_t ncell, int dim, int nf) {
+    return ncell * 2 * dim * trace_face_stride<T>(nf);
+}
+template <typename T>
+constexpr int64_t trace_count(int64_t ncell, int dim, int nf) {
+    return trace_values<T>(ncell, dim, nf) + (sizeof(T) == 8 ? 2 * ncell : 0);
+}
+constexpr int TRACE_NO_EXPONENT = 0xc0;
+
 // Process-wide count of kernels launched by the library (dgmg_kernel_launches).
 extern std::atomic<long long> g_kernel_launches;
 inline void count_launches(int k) { g_kernel_launches.fetch_add(k, std::memory_order_relaxed); }
@@ -162,11 +175,12 @@ struct BlockMap;
 // the FP64 kernels of one (dimension, nodes per axis) (dg_fx.cuh)
 template <int DIM, int Q>
 struct FxRun {
-    static cudaError_t project(const FxLevel &l, double *u, const double *e0, double *tr, cudaStream_t s);
+    // user: traces in FP64 instead of the kernels' own form
+    static cudaError_t project(const FxLevel &l, bool user, double *u, const double *e0, double *tr, cudaStream_t s);
     static cudaError_t smooth(const FxLevel &l, bool exact, int flags, double *u, const double *b, const double *kappa,
                               const double *fd, const double *linv, const double *tri, double *tro, cudaStream_t s);
-    static cudaError_t residual(const FxLevel &l, int mode, const double *u, const double *b, const double *kappa,
-                                const double *tr, double *r, double *corners, cudaStream_t s);
+    static cudaError_t residual(const FxLevel &l, bool user, int mode, const double *u, const double *b,
+                                const double *kappa, const double *tr, double *r, double *corners, cudaStream_t s);
     static cudaError_t project_batch(const FxTab &tab, const BatchDG<double> *D, const BlockMap *map, int nblocks,
                                      double *u, int with_e0, cudaStream_t s);
     static cudaError_t smooth_batch(const FxTab &tab, bool exact, const BatchDG<double> *D, const BlockMap *map,
@@ -340,6 +354,12 @@ template <typename T>
 cudaError_t launch_residual(int dim, int q, const DGConst<T> &c, int cpb, int mode, const T *u,
                             const T *b, const T *kappa, const T *tr, T *r, T *corners, const T *fd,
                             cudaStream_t s);
+// the FP64 projection and residual with traces in FP64, as callers of the library hold them
+cudaError_t launch_project_user(int dim, int q, const DGConst<double> &c, double *u, const double *e0, double *tr,
+                                cudaStream_t s);
+cudaError_t launch_residual_user(int dim, int q, const DGConst<double> &c, int mode, const double *u, const double *b,
+                                 const double *kappa, const double *tr, double *r, double *corners, cudaStream_t s);
+
 
 template <typename T>
 cudaError_t launch_project_batch(int dim, int q, const BatchDG<T> *D, const BlockMap *map, int nblocks, int cpb,
