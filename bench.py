@@ -39,8 +39,8 @@ FP64_NOMINAL_TFLOPS = 1.25       # nominal GB300 dense FP64, context beside the 
 # DRAM bytes (read + write) of one launch of the FP64 smoothing kernel on this
 # workload from one ncu capture, valid only for the kernel sources it was taken
 # on (SHA-256 of the files below); once they change, `traffic` reads null
-SMOOTH_TRAFFIC = {"kernel": "k_fx_cells<3,4,0>", "bytes": 116_977_664 + 3_158_016,
-                  "sources_sha256": "9ff65c8881b7a374ecbfe1581b6578f2a571c9e308d1d0ba5d870aae3d7765ea",
+SMOOTH_TRAFFIC = {"kernel": "k_fx_cells<3,4,0>", "bytes": 116_969_216 + 2_981_632,
+                  "sources_sha256": "fd894e1a3c43d8ad0ea3091e6a435c491da2f28dd828c7e830ee1822eec5361d",
                   "files": ("fx.cuh", "dg_fx.cuh", "dg_fp64.cu")}
 # 32 x 32 + 64 bit integer multiply-adds per SM and clock (a loop of independent
 # products); the FP64 kernels of the DG levels take three per multiply-add

@@ -2,7 +2,8 @@
 // projection, smoothing step, residual. 2D and 3D, every degree, both bases, exact
 // and interior-only blocks.
 //
-// Work decomposition. q lanes of a warp serve one cell (32 / q cells per warp); the
+// Work decomposition. q lanes of a warp serve one cell (32 / q cells per warp; small 3D
+// meshes of q >= 5: SP lanes per slab, fx_split); the
 // cell tensor stays in shared memory as 64-bit integers of one exponent per cell. A
 // pass along an axis takes the cell's q^(d-1) pencils, q^(d-2) per lane: load q
 // values, apply a q x q matrix held in registers, store. Lane k's pencils along the
@@ -50,14 +51,14 @@ namespace dgmg {
 // 98 -> 93 us a step, 23^3 p = 2 V-cycle 149 -> 141 us, 729^2 p = 4 508 -> 501 us.
 enum { FXM_SMOOTH = 0, FXM_SMOOTH_FULL = 1, FXM_RESIDUAL = 2, FXM_RESIDUAL_USER = 3 };
 
-template <int DIM, int Q>
+template <int DIM, int Q, int SP = 1>
 struct FxGeo {
     static constexpr int N = DIM == 3 ? Q * Q : Q;        // nodes of a slab
     static constexpr int NP = N / Q;                      // pencils per lane, face values per lane
     static constexpr int NL = N * Q, NF = N;              // nodes of a cell, of a face
     static constexpr int NFACE = 2 * DIM, FS = 2 * NF, TR = NFACE * FS, NC = 1 << DIM;
-    static constexpr int CW = 32 / Q;                     // cells per warp
-    static constexpr bool ALL = CW * Q == 32;             // every lane serves a cell
+    static constexpr int CW = 32 / (Q * SP);              // cells per warp
+    static constexpr bool ALL = CW * Q * SP == 32;        // every lane serves a cell
     static constexpr int NW = 4;                          // warps per CTA
     static constexpr int CPB = CW * NW;                   // cells per CTA
     static constexpr int MINB = (Q <= 4 ? 16 : (Q == 5 ? 12 : 8)) / NW;   // CTAs per SM the registers are cut for
@@ -92,51 +93,53 @@ __device__ __forceinline__ void fx_cp_wait() { asm volatile("cp.async.wait_all;\
 
 // The cell tensors of the warp's cells between global memory (contiguous) and the
 // slab rows of shared memory (contiguous too for odd q).
-template <int DIM, int Q>
+template <int DIM, int Q, int SP>
 __device__ __forceinline__ int fx_row_place(int g) {
-    using G = FxGeo<DIM, Q>;
+    using G = FxGeo<DIM, Q, SP>;
     if (G::C == G::NL) return g;
     const int c = g / G::NL, r = g - c * G::NL, row = r / G::N;
     return c * G::C + row * G::S + (r - row * G::N);
 }
-template <int DIM, int Q>
+template <int DIM, int Q, int SP>
 __device__ __forceinline__ void fx_stage_in(void *dst, const double *__restrict__ src, int count, int lane) {
-    using G = FxGeo<DIM, Q>;
+    using G = FxGeo<DIM, Q, SP>;
     constexpr int ROUNDS = (G::CW * G::NL + 31) / 32;
     if (ROUNDS <= 32 && count == G::CW * G::NL) {
 #pragma unroll
         for (int j = 0; j < ROUNDS; ++j) {
             const int g = lane + 32 * j;
             if (G::CW * G::NL % 32 == 0 || j < ROUNDS - 1 || g < G::CW * G::NL)
-                fx_cp8(reinterpret_cast<double *>(dst) + fx_row_place<DIM, Q>(g), src + g);
+                fx_cp8(reinterpret_cast<double *>(dst) + fx_row_place<DIM, Q, SP>(g), src + g);
         }
     } else {
 #pragma unroll 4
-        for (int g = lane; g < count; g += 32) fx_cp8(reinterpret_cast<double *>(dst) + fx_row_place<DIM, Q>(g), src + g);
+        for (int g = lane; g < count; g += 32) fx_cp8(reinterpret_cast<double *>(dst) + fx_row_place<DIM, Q, SP>(g), src + g);
     }
 }
-template <int DIM, int Q>
+template <int DIM, int Q, int SP>
 __device__ __forceinline__ void fx_store_out(double *__restrict__ dst, const double *src, int count, int lane) {
 #pragma unroll 8
-    for (int g = lane; g < count; g += 32) dst[g] = src[fx_row_place<DIM, Q>(g)];
+    for (int g = lane; g < count; g += 32) dst[g] = src[fx_row_place<DIM, Q, SP>(g)];
 }
 
 // The lane's place: cell slot c of the warp, slab k. Lanes beyond CW * q follow slot
 // 0 without writing (live = false).
 struct FxLane {
     int lane, c, k;
+    int sub;                             // which of the SP lanes of its slab
     bool live;
     int *ex;                             // the warp's two rows of lane exponents [2][32]
     int row;                             // the row of the next exchange of them
 };
-template <int DIM, int Q>
+template <int DIM, int Q, int SP>
 __device__ __forceinline__ FxLane fx_lane(int *ex) {
     FxLane L;
     L.lane = threadIdx.x & 31;
-    L.c = L.lane / Q;
-    L.k = L.lane - L.c * Q;
-    L.live = L.c < FxGeo<DIM, Q>::CW;
-    if (!L.live) L.c = L.k = 0;
+    L.c = L.lane / (Q * SP);
+    L.sub = SP == 1 ? 0 : (L.lane - L.c * (Q * SP)) / Q;
+    L.k = L.lane - (L.c * SP + L.sub) * Q;
+    L.live = L.c < FxGeo<DIM, Q, SP>::CW;
+    if (!L.live) L.c = L.k = L.sub = 0;
     L.ex = ex;
     L.row = 0;
     return L;
@@ -173,9 +176,9 @@ __device__ __forceinline__ unsigned fx_cell_min4(unsigned v, FxLane &L) {
 struct FxAxis {
     int first, next, step;
 };
-template <int DIM, int Q>
+template <int DIM, int Q, int SP>
 __device__ __forceinline__ FxAxis fx_axis(int a, int k) {
-    using G = FxGeo<DIM, Q>;
+    using G = FxGeo<DIM, Q, SP>;
     FxAxis x;
     const bool last = a == DIM - 1;
     x.first = last ? (DIM == 3 ? Q * k : k) : G::S * k;
@@ -213,20 +216,20 @@ __device__ __forceinline__ FxBlock fx_block(const FxMag &mag, int e, FxLane &L) 
 
 // t <- A t along axis a. A[i][m] = src[i * si + m * sm] (limbs of unit ea). Axis and
 // matrix are run-time values, so that one copy of the code serves every pass.
-template <int DIM, int Q>
+template <int DIM, int Q, int SP>
 __device__ __forceinline__ FxBlock fx_pass(long long *xc, FxBlock b, int a, const Limb *src, int si, int sm, int ea,
                                            FxLane &L) {
-    using G = FxGeo<DIM, Q>;
-    const FxAxis ax = fx_axis<DIM, Q>(a, L.k);
+    using G = FxGeo<DIM, Q, SP>;
+    const FxAxis ax = fx_axis<DIM, Q, SP>(a, L.k);
     Limb A[Q * Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i)
 #pragma unroll
         for (int m = 0; m < Q; ++m) A[i * Q + m] = src[i * si + m * sm];
     FxMag mag;
-    long long *t = xc + ax.first;
 #pragma unroll 1
-    for (int p = 0; p < G::NP; ++p, t += ax.next) {
+    for (int p = L.sub; p < G::NP; p += SP) {
+        long long *t = xc + ax.first + p * ax.next;
         Acc s[Q];
 #pragma unroll
         for (int i = 0; i < Q; ++i) acc_zero(s[i]);
@@ -243,7 +246,7 @@ __device__ __forceinline__ FxBlock fx_pass(long long *xc, FxBlock b, int a, cons
             mag.add(v);
         }
     }
-    return fx_block<Q>(mag, b.e - b.n + ea + 64, L);
+    return fx_block<Q * SP>(mag, b.e - b.n + ea + 64, L);
 }
 
 // t <- M t along axis a, M the 1D mass, which is symmetric about its centre: with
@@ -254,16 +257,16 @@ __device__ __forceinline__ FxBlock fx_pass(long long *xc, FxBlock b, int a, cons
 // half of M's, so the sums keep the bounds of Acc. With full matrices: residual 243^2
 // cells p = 6 GL 120 us (now 110), operator 64^3 p = 4 1192 (1141), smoothing 32^3 p = 3
 // 100 (98) a step.
-template <int DIM, int Q>
+template <int DIM, int Q, int SP>
 __device__ __forceinline__ FxBlock fx_mass(long long *xc, FxBlock b, int a, const Limb *T, int eM, bool gl, FxLane &L) {
-    using G = FxGeo<DIM, Q>;
+    using G = FxGeo<DIM, Q, SP>;
     constexpr int H = Q / 2, HE = Q - H;                  // sizes of O and E
-    const FxAxis ax = fx_axis<DIM, Q>(a, L.k);
+    const FxAxis ax = fx_axis<DIM, Q, SP>(a, L.k);
     FxMag mag;
-    long long *t = xc + ax.first;
     if (gl) {
 #pragma unroll 1
-        for (int p = 0; p < G::NP; ++p, t += ax.next)
+        for (int p = L.sub; p < G::NP; p += SP) {
+            long long *t = xc + ax.first + p * ax.next;
 #pragma unroll
             for (int i = 0; i < Q; ++i) {
                 Acc s;
@@ -273,7 +276,8 @@ __device__ __forceinline__ FxBlock fx_mass(long long *xc, FxBlock b, int a, cons
                 if (G::ALL || L.live) t[i * ax.step] = v;
                 mag.add(v);
             }
-        return fx_block<Q>(mag, b.e - b.n + eM + 64, L);
+        }
+        return fx_block<Q * SP>(mag, b.e - b.n + eM + 64, L);
     }
     Limb E[HE * HE], O[H * H];
 #pragma unroll
@@ -281,7 +285,8 @@ __device__ __forceinline__ FxBlock fx_mass(long long *xc, FxBlock b, int a, cons
 #pragma unroll
     for (int i = 0; i < H * H; ++i) O[i] = T[HE * HE + i];
 #pragma unroll 1
-    for (int p = 0; p < G::NP; ++p, t += ax.next) {
+    for (int p = L.sub; p < G::NP; p += SP) {
+        long long *t = xc + ax.first + p * ax.next;
         Acc se[HE], so[H];
 #pragma unroll
         for (int i = 0; i < HE; ++i) acc_zero(se[i]);
@@ -318,41 +323,41 @@ __device__ __forceinline__ FxBlock fx_mass(long long *xc, FxBlock b, int a, cons
             }
         }
     }
-    return fx_block<Q>(mag, b.e - b.n + eM + 64, L);
+    return fx_block<Q * SP>(mag, b.e - b.n + eM + 64, L);
 }
 
 // Largest biased exponent of the lane's slab of FP64 values.
-template <int DIM, int Q>
-__device__ __forceinline__ int fx_slab_top(const double *y) {
+template <int DIM, int Q, int SP>
+__device__ __forceinline__ int fx_slab_top(const double *y, int sub) {
     int mx = 0;
 #pragma unroll 4
-    for (int i = 0; i < FxGeo<DIM, Q>::N; ++i) mx = imax(mx, fx_abs_hi(y[i]));
+    for (int i = sub; i < FxGeo<DIM, Q, SP>::N; i += SP) mx = imax(mx, fx_abs_hi(y[i]));
     return mx >> 20;
 }
 
 // Per cell after the traces {e, h[axis]}: values count 2^e (GL: 2^(e + eV + 64)),
 // derivatives along axis a 2^(e + eT[a] + 64); h packs the unused leading bits (of 60) of
 // the axis' traces, byte 2 side + (0 value, 1 derivative).
-template <int DIM, int Q, typename P>
+template <int DIM, int Q, int SP, typename P>
 __device__ __forceinline__ auto fx_trace_units(P *tr, int64_t ncell) {
     using I = typename std::conditional<std::is_const<P>::value, const int4, int4>::type;
-    return reinterpret_cast<I *>(tr + ncell * FxGeo<DIM, Q>::TR);
+    return reinterpret_cast<I *>(tr + ncell * FxGeo<DIM, Q, SP>::TR);
 }
 constexpr int FX_NO_TRACE = FX_NONE / 2;     // exponents below: all values are 0
 
 // Traces of the cell from its block in shared memory: per axis and side, value and
 // +axis derivative; derivatives by dot products, values the end nodes (GLL) or dot
 // products (GL). USER: as FP64.
-template <int DIM, int Q, bool USER = false>
+template <int DIM, int Q, int SP, bool USER = false>
 __device__ __forceinline__ void fx_all_traces(const FxTab &tab, const FxConst &cst, const long long *xc, FxBlock b,
                                               FxLane &L, bool write, int64_t cell, double *__restrict__ tr) {
-    using G = FxGeo<DIM, Q>;
+    using G = FxGeo<DIM, Q, SP>;
     const int e = b.e - b.n;
     double *cell_tr = tr + cell * G::TR;
     unsigned room[3] = {0, 0, 0};
 #pragma unroll 1
     for (int a = 0; a < DIM; ++a) {
-        const FxAxis ax = fx_axis<DIM, Q>(a, L.k);
+        const FxAxis ax = fx_axis<DIM, Q, SP>(a, L.k);
         Limb d[2][Q];
 #pragma unroll
         for (int s = 0; s < 2; ++s)
@@ -360,9 +365,8 @@ __device__ __forceinline__ void fx_all_traces(const FxTab &tab, const FxConst &c
             for (int i = 0; i < Q; ++i) d[s][i] = cst.dt[a][s][i];
         const int ed = e + cst.eT[a] + 64;
         double *out = cell_tr + 2 * a * G::FS + L.k * G::NP;
-        const long long *t = xc + ax.first;
         FxMag mag[2][2];
-        auto put = [&](int s, int c, int p, long long w, int ew) {
+        auto put_at = [&](int s, int c, int p, long long w, int ew) {
             double *to = out + s * G::FS + c * G::NF + p;
             if (!USER) mag[s][c].add(w);
             if (!write) return;
@@ -372,7 +376,9 @@ __device__ __forceinline__ void fx_all_traces(const FxTab &tab, const FxConst &c
                 *reinterpret_cast<long long *>(to) = w;
         };
 #pragma unroll 1
-        for (int p = 0; p < G::NP; ++p, t += ax.next) {
+        for (int p = L.sub; p < G::NP; p += SP) {
+            const long long *t = xc + ax.first + p * ax.next;
+            auto put = [&](int s, int c, long long w, int ew) { put_at(s, c, p, w, ew); };
             Limb x[Q];
 #pragma unroll
             for (int i = 0; i < Q; ++i) x[i] = fx_read(t[i * ax.step], b.n);
@@ -382,14 +388,14 @@ __device__ __forceinline__ void fx_all_traces(const FxTab &tab, const FxConst &c
                 acc_zero(v);
 #pragma unroll
                 for (int i = 0; i < Q; ++i) mac(v, d[s][i], x[i]);
-                put(s, 1, p, acc_value(v), ed);
+                put(s, 1, acc_value(v), ed);
                 if (tab.gl) {
                     acc_zero(v);
 #pragma unroll
                     for (int i = 0; i < Q; ++i) mac(v, tab.v[s][i], x[i]);
-                    put(s, 0, p, acc_value(v), e + tab.eV + 64);
+                    put(s, 0, acc_value(v), e + tab.eV + 64);
                 } else {
-                    put(s, 0, p, t[(s ? Q - 1 : 0) * ax.step] << b.n, e);
+                    put(s, 0, t[(s ? Q - 1 : 0) * ax.step] << b.n, e);
                 }
             }
         }
@@ -399,14 +405,14 @@ __device__ __forceinline__ void fx_all_traces(const FxTab &tab, const FxConst &c
             for (int s = 0; s < 2; ++s)
 #pragma unroll
                 for (int c = 0; c < 2; ++c) w |= (unsigned)imax(fx_headroom(mag[s][c].top()), 0) << (16 * s + 8 * c);
-            w = fx_cell_min4<Q>(w, L);
+            w = fx_cell_min4<Q * SP>(w, L);
             room[0] = a == 0 ? w : room[0];
             room[1] = a == 1 ? w : room[1];
             room[2] = a == 2 ? w : room[2];
         }
     }
     if (!USER && write && L.k == 0)
-        fx_trace_units<DIM, Q>(tr, cst.ncell)[cell] = make_int4(e, (int)room[0], (int)room[1], (int)room[2]);
+        fx_trace_units<DIM, Q, SP>(tr, cst.ncell)[cell] = make_int4(e, (int)room[0], (int)room[1], (int)room[2]);
 }
 
 __device__ __forceinline__ void load_batch_desc(const BatchDG<double> *__restrict__ src, BatchDG<double> *dst) {
@@ -443,21 +449,21 @@ __device__ __forceinline__ void fx_cell_coords(int64_t cell, const int *n, int *
 // the table's); linv: the table as integers.
 // flags: SM_ZERO: the iterate is 0 (u and its traces are not read); SM_NO_TRACES:
 // the new traces are not written. mode (residual): RES_*.
-template <int DIM, int Q, int MODE>
+template <int DIM, int Q, int SP, int MODE>
 __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &cst, const Limb *sTab, long long *smem,
                                               int64_t cell0, int flags, int mode, double *__restrict__ u,
                                               const double *__restrict__ b, const double *__restrict__ kappa,
                                               const double *__restrict__ fd, const double *__restrict__ linv,
                                               const double *__restrict__ tr_in, double *__restrict__ tr_out,
                                               double *__restrict__ r, double *__restrict__ corners) {
-    using G = FxGeo<DIM, Q>;
+    using G = FxGeo<DIM, Q, SP>;
     constexpr int N = G::N, NP = G::NP, NL = G::NL, NFACE = G::NFACE, SW = G::small_words(MODE);
     constexpr bool SMOOTH = MODE < FXM_RESIDUAL, FULL = MODE != FXM_SMOOTH, USER = MODE == FXM_RESIDUAL_USER;
     long long *X = smem;                                  // the block the passes work on
     long long *Y = X + G::CW * G::C;                      // u or b on their way in, the result on its way out
     Limb *small = reinterpret_cast<Limb *>(Y + G::CW * G::C);   // coefficients and D_a, later the factors
     int *sLE = reinterpret_cast<int *>(small + G::CW * SW);     // coefficient exponents [cell][face][field]
-    FxLane L = fx_lane<DIM, Q>(sLE + G::CW * NFACE * 2);
+    FxLane L = fx_lane<DIM, Q, SP>(sLE + G::CW * NFACE * 2);
     const int ncl = (int)(cst.ncell - cell0 < G::CW ? cst.ncell - cell0 : G::CW);
     const bool active = L.live && L.c < ncl;
     const int64_t cell = cell0 + (L.c < ncl ? L.c : 0);
@@ -469,7 +475,7 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
     Limb *mine = small + L.c * SW;
 
     // in flight from the start: u where the residual of the iterate needs it, else b
-    fx_stage_in<DIM, Q>(Y, (FULL && !zero ? u : b) + cell0 * NL, FULL && !zero ? ncl * NL : (has_b ? ncl * NL : 0),
+    fx_stage_in<DIM, Q, SP>(Y, (FULL && !zero ? u : b) + cell0 * NL, FULL && !zero ? ncl * NL : (has_b ? ncl * NL : 0),
                         L.lane);
     auto stage_factors = [&]() {
         if constexpr (SMOOTH) {
@@ -522,7 +528,7 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
             } else {
                 const int64_t st = a == 0 ? 1 : (a == 1 ? s1 : s2);
                 const int64_t nb = (mask >> f) & 1 ? cell + (f & 1 ? st : -st) : cell;
-                const int4 en = __ldg(fx_trace_units<DIM, Q>(tr_in, cst.ncell) + nb);
+                const int4 en = __ldg(fx_trace_units<DIM, Q, SP>(tr_in, cst.ncell) + nb);
                 const unsigned w = (unsigned)(a == 0 ? en.y : (a == 1 ? en.z : en.w)) >> (f & 1 ? 0 : 16);
                 ug[f] = en.x + (tab.gl ? tab.eV + 64 : 0);
                 uh[f] = en.x + cst.eT[a] + 64;
@@ -593,14 +599,14 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
         }
         // one unit E for the whole sum: |D u| < 2^58 and the facet terms < 2^59 per axis,
         // so the sum over the axes stays below 2^62
-        int E = fx_cell_max<Q>(top, L);
+        int E = fx_cell_max<Q * SP>(top, L);
         if constexpr (FULL) {
-            const int ev = fx_cell_max<Q>(fx_slab_top<DIM, Q>(ys), L);
+            const int ev = fx_cell_max<Q * SP>(fx_slab_top<DIM, Q, SP>(ys, L.sub), L);
             E = imax(E, fx_unit(ev) + ed + 64);
             // u as integers of the unit that makes D u come out in E
             const int eu = E - ed - 64 + FX_UNIT;
 #pragma unroll 4
-            for (int i = 0; i < N; ++i) {
+            for (int i = L.sub; i < N; i += SP) {
                 const long long v = fx_from(ys[i], eu);
                 if (L.live) reinterpret_cast<long long *>(ys)[i] = v;
             }
@@ -609,8 +615,8 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
         FxMag mag;
 #pragma unroll 1
         for (int a = 0; a < DIM; ++a) {
-            const FxAxis ax = fx_axis<DIM, Q>(a, L.k);
-            if (a == DIM - 1) __syncwarp();              // this axis crosses the slabs
+            const FxAxis ax = fx_axis<DIM, Q, SP>(a, L.k);
+            if (a == DIM - 1 || (SP > 1 && a > 0)) __syncwarp();   // this axis crosses the lanes' parts
             mag = FxMag();
             Limb B[FULL ? Q * Q : 1], cf[2][2][Q];
             if constexpr (FULL) {
@@ -630,10 +636,10 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
                 }
             const bool in[2] = {((mask >> (2 * a)) & 1) != 0, ((mask >> (2 * a + 1)) & 1) != 0};
             const double *nb[2] = {face(a, 0, in[0]), face(a, 1, in[1])};
-            long long *o = xc + ax.first;
-            const long long *y = Y + L.c * G::C + ax.first;
 #pragma unroll 1
-            for (int p = 0; p < NP; ++p, o += ax.next, y += ax.next) {
+            for (int p = L.sub; p < NP; p += SP) {
+                long long *o = xc + ax.first + p * ax.next;
+                const long long *y = Y + L.c * G::C + ax.first + p * ax.next;
                 Limb g[2][2];
 #pragma unroll
                 for (int s = 0; s < 2; ++s)
@@ -675,12 +681,12 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
                 }
             }
         }
-        t = fx_block<Q>(mag, E, L);
+        t = fx_block<Q * SP>(mag, E, L);
         // more than 60 bits somewhere (the bound on the sum is 2^62): shift those cells
         if (__any_sync(0xffffffffu, t.n < 0)) {
             const int d = imax(-t.n, 0);
 #pragma unroll 4
-            for (int i = 0; i < N; ++i)
+            for (int i = L.sub; i < N; i += SP)
                 if (G::ALL || L.live) xs[i] >>= d;
             t.e += d;
             t.n = imax(t.n, 0);
@@ -688,30 +694,30 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
         }
         // the coefficients are used: the factors (or b) while M is applied
         stage_factors();
-        if (FULL && has_b) fx_stage_in<DIM, Q>(Y, b + cell0 * NL, ncl * NL, L.lane);
+        if (FULL && has_b) fx_stage_in<DIM, Q, SP>(Y, b + cell0 * NL, ncl * NL, L.lane);
     }
     // M along every axis; t <- b - t; S^T along every axis; the table; S along every axis
     const Limb *myF = mine;
     auto subtract_from_b = [&]() {                        // t = A u (or its neighbours' part); in the lane's slab
         fx_cp_wait();
         __syncwarp();
-        const int te = t.e - t.n, E = imax(fx_unit(fx_cell_max<Q>(fx_slab_top<DIM, Q>(ys), L)), te) + 1;
+        const int te = t.e - t.n, E = imax(fx_unit(fx_cell_max<Q * SP>(fx_slab_top<DIM, Q, SP>(ys, L.sub), L)), te) + 1;
         const int ev = E + FX_UNIT;
         FxMag mag;
 #pragma unroll 4
-        for (int i = 0; i < N; ++i) {
+        for (int i = L.sub; i < N; i += SP) {
             const long long v = fx_from(ys[i], ev) - (zero ? 0 : fx_shr(xs[i] << t.n, E - te));
             if (G::ALL || L.live) xs[i] = v;
             mag.add(v);
         }
-        t = fx_block<Q>(mag, E, L);
+        t = fx_block<Q * SP>(mag, E, L);
     };
 #pragma unroll 1
     for (int k = zero ? DIM : 0; k < (SMOOTH ? 3 * DIM : DIM); ++k) {
         if (SMOOTH && k == DIM) {
             subtract_from_b();
             // the table into Y (every lane has read b)
-            fx_stage_in<DIM, Q>(Y, linv + cell0 * NL, ncl * NL, L.lane);
+            fx_stage_in<DIM, Q, SP>(Y, linv + cell0 * NL, ncl * NL, L.lane);
         }
         if (SMOOTH && k == 2 * DIM) {
             fx_cp_wait();
@@ -719,7 +725,7 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
             const long long *li = reinterpret_cast<const long long *>(ys);
             FxMag mag;
 #pragma unroll 4
-            for (int i = 0; i < N; ++i) {
+            for (int i = L.sub; i < N; i += SP) {
                 Acc s;
                 acc_zero(s);
                 mac(s, limb_of(li[i]), fx_read(xs[i], t.n));
@@ -727,17 +733,17 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
                 if (G::ALL || L.live) xs[i] = v;
                 mag.add(v);
             }
-            t = fx_block<Q>(mag, t.e - t.n + myF[Q * Q + 1].h + 64, L);
+            t = fx_block<Q * SP>(mag, t.e - t.n + myF[Q * Q + 1].h + 64, L);
             // the previous iterate into Y (every lane has read the table)
-            if (!zero) fx_stage_in<DIM, Q>(Y, u + cell0 * NL, ncl * NL, L.lane);
+            if (!zero) fx_stage_in<DIM, Q, SP>(Y, u + cell0 * NL, ncl * NL, L.lane);
         }
         const int a = k < DIM ? DIM - 1 - k : (k < 2 * DIM ? k - DIM : 3 * DIM - 1 - k);
         if (k < DIM) {
-            t = fx_mass<DIM, Q>(xc, t, a, sTab, tab.eM, tab.gl != 0, L);
+            t = fx_mass<DIM, Q, SP>(xc, t, a, sTab, tab.eM, tab.gl != 0, L);
         } else if constexpr (SMOOTH) {
             const bool trans = k < 2 * DIM;
             const Limb *src = myF + a * G::FDS;
-            t = fx_pass<DIM, Q>(xc, t, a, src, trans ? 1 : Q, trans ? Q : 1, src[Q * Q].h, L);
+            t = fx_pass<DIM, Q, SP>(xc, t, a, src, trans ? 1 : Q, trans ? Q : 1, src[Q * Q].h, L);
         }
     }
     if (!SMOOTH && has_b) subtract_from_b();
@@ -746,11 +752,11 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
         if (!zero) {                                     // u <- keep u + t
             fx_cp_wait();
             __syncwarp();
-            const int ev = fx_cell_max<Q>(fx_slab_top<DIM, Q>(ys), L);
+            const int ev = fx_cell_max<Q * SP>(fx_slab_top<DIM, Q, SP>(ys, L.sub), L);
             const int eu = fx_unit(ev) + cst.eKeep + 64, te = t.e - t.n, E = imax(eu, te) + 1;
             FxMag mag;
 #pragma unroll 4
-            for (int i = 0; i < N; ++i) {
+            for (int i = L.sub; i < N; i += SP) {
                 Acc s;
                 acc_zero(s);
                 mac(s, cst.keep, limb_of(fx_from(ys[i], ev)));
@@ -758,7 +764,7 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
                 if (G::ALL || L.live) xs[i] = v;
                 mag.add(v);
             }
-            t = fx_block<Q>(mag, E, L);
+            t = fx_block<Q * SP>(mag, E, L);
         }
     }
     // the result leaves through Y
@@ -766,15 +772,15 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
         // without b the block is A u: the residual b - A u is its negative
         const bool neg = !SMOOTH && has_b == ((mode & RES_NEGATE) != 0);
 #pragma unroll 4
-        for (int i = 0; i < N; ++i) {
+        for (int i = L.sub; i < N; i += SP) {
             const double v = fx_to(neg ? -xs[i] : xs[i], t.e);
             if (L.live) ys[i] = v;
         }
         __syncwarp();
-        fx_store_out<DIM, Q>((SMOOTH ? u : r) + cell0 * NL, reinterpret_cast<const double *>(Y), ncl * NL, L.lane);
+        fx_store_out<DIM, Q, SP>((SMOOTH ? u : r) + cell0 * NL, reinterpret_cast<const double *>(Y), ncl * NL, L.lane);
     }
     if constexpr (SMOOTH) {
-        if (!(flags & SM_NO_TRACES)) fx_all_traces<DIM, Q>(tab, cst, xc, t, L, active, cell, tr_out);
+        if (!(flags & SM_NO_TRACES)) fx_all_traces<DIM, Q, SP>(tab, cst, xc, t, L, active, cell, tr_out);
     } else if (mode & RES_CORNERS) {
         // corner sums of b - A u: hat values along the slab's axes, then over the slabs
         constexpr int NS = DIM == 3 ? 4 : 2;             // sums per slab
@@ -795,7 +801,7 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
                 mag.add(s0[c][j]);
             }
         }
-        int e = t.e - t.n + tab.eHat + 64, n = fx_headroom(fx_cell_max<Q>(mag.top(), L));
+        int e = t.e - t.n + tab.eHat + 64, n = fx_headroom(fx_cell_max<Q * SP>(mag.top(), L));
         if constexpr (DIM == 3) {
             mag = FxMag();
 #pragma unroll
@@ -808,7 +814,7 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
                 mag.add(y[c]);
             }
             e += tab.eHat + 64 - n;
-            n = fx_headroom(fx_cell_max<Q>(mag.top(), L));
+            n = fx_headroom(fx_cell_max<Q * SP>(mag.top(), L));
         } else {
             y[0] = s0[0][0];
             y[1] = s0[1][0];
@@ -834,7 +840,7 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
     }
 }
 
-template <int DIM, int Q, int MODE>
+template <int DIM, int Q, int SP, int MODE>
 __device__ __forceinline__ const Limb *fx_stage_tables(const FxTab &tab, long long *smem) {
     Limb *s = reinterpret_cast<Limb *>(smem);
     constexpr int H = Q / 2, HE = Q - H;
@@ -862,34 +868,34 @@ __device__ __forceinline__ const Limb *fx_stage_tables(const FxTab &tab, long lo
     return s;
 }
 
-template <int DIM, int Q, int MODE>
-__global__ void __launch_bounds__(FxGeo<DIM, Q>::NW * 32, FxGeo<DIM, Q>::MINB)
+template <int DIM, int Q, int SP, int MODE>
+__global__ void __launch_bounds__(FxGeo<DIM, Q, SP>::NW * 32, FxGeo<DIM, Q, SP>::MINB)
     k_fx_cells(const __grid_constant__ FxTab tab, const __grid_constant__ FxConst cst, int flags, int mode, double *u,
                const double *b, const double *__restrict__ kappa, const double *__restrict__ fd,
                const double *__restrict__ linv, const double *__restrict__ tr_in, double *__restrict__ tr_out, double *r,
                double *__restrict__ corners) {
-    using G = FxGeo<DIM, Q>;
+    using G = FxGeo<DIM, Q, SP>;
     extern __shared__ __align__(16) long long smem_fx[];
-    const Limb *sTab = fx_stage_tables<DIM, Q, MODE>(tab, smem_fx);
+    const Limb *sTab = fx_stage_tables<DIM, Q, SP, MODE>(tab, smem_fx);
     const int warp = threadIdx.x >> 5;
     const int64_t cell0 = (int64_t)blockIdx.x * G::CPB + warp * G::CW;
     if (cell0 >= cst.ncell) return;
-    fx_cells_body<DIM, Q, MODE>(tab, cst, sTab, smem_fx + G::tab_words(MODE) + warp * G::warp_words(MODE), cell0, flags, mode, u, b,
+    fx_cells_body<DIM, Q, SP, MODE>(tab, cst, sTab, smem_fx + G::tab_words(MODE) + warp * G::warp_words(MODE), cell0, flags, mode, u, b,
                                 kappa, fd, linv, tr_in, tr_out, r, corners);
 }
 
 // Batched form: work item k serves the CPB cells from map[k].cell0 of instance
 // map[k].inst. Persistent CTAs stride through the items; the barriers end every
 // warp's use of the descriptor and of its staging memory.
-template <int DIM, int Q, int MODE>
-__global__ void __launch_bounds__(FxGeo<DIM, Q>::NW * 32, FxGeo<DIM, Q>::MINB)
+template <int DIM, int Q, int SP, int MODE>
+__global__ void __launch_bounds__(FxGeo<DIM, Q, SP>::NW * 32, FxGeo<DIM, Q, SP>::MINB)
     k_fx_cells_batch(const __grid_constant__ FxTab tab, const BatchDG<double> *__restrict__ D,
                      const BlockMap *__restrict__ map, int nblocks, int flags, int mode, double *u, const double *b,
                      double *r, int cur) {
-    using G = FxGeo<DIM, Q>;
+    using G = FxGeo<DIM, Q, SP>;
     extern __shared__ __align__(16) long long smem_fx[];
     __shared__ __align__(16) BatchDG<double> sd;
-    const Limb *sTab = fx_stage_tables<DIM, Q, MODE>(tab, smem_fx);
+    const Limb *sTab = fx_stage_tables<DIM, Q, SP, MODE>(tab, smem_fx);
     const int warp = threadIdx.x >> 5;
     long long *mine = smem_fx + G::tab_words(MODE) + warp * G::warp_words(MODE);
     for (int k = blockIdx.x; k < nblocks; k += gridDim.x) {
@@ -899,7 +905,7 @@ __global__ void __launch_bounds__(FxGeo<DIM, Q>::NW * 32, FxGeo<DIM, Q>::MINB)
         const int64_t cell0 = (int64_t)m.cell0 + warp * G::CW;
         if (cell0 < sd.c.ncell) {
             const int64_t o = sd.off * G::NL;
-            fx_cells_body<DIM, Q, MODE>(tab, sd.c, sTab, mine, cell0, flags, mode, u + o, b ? b + o : nullptr, sd.kappa,
+            fx_cells_body<DIM, Q, SP, MODE>(tab, sd.c, sTab, mine, cell0, flags, mode, u + o, b ? b + o : nullptr, sd.kappa,
                                         sd.fd, sd.linv, sd.tr[cur], sd.tr[cur ^ 1], r ? r + o : nullptr, sd.corners);
         }
     }
@@ -907,19 +913,19 @@ __global__ void __launch_bounds__(FxGeo<DIM, Q>::NW * 32, FxGeo<DIM, Q>::MINB)
 
 // Warm-up projection of the warp's cells: optionally u += P e (the multilinear hats
 // of the cell's corner values), then the traces.
-template <int DIM, int Q, bool USER = false>
+template <int DIM, int Q, int SP, bool USER = false>
 __device__ __forceinline__ void fx_project_body(const FxTab &tab, const FxConst &cst, long long *smem, int64_t cell0,
                                                 double *u, const double *__restrict__ e0, double *__restrict__ tr) {
-    using G = FxGeo<DIM, Q>;
+    using G = FxGeo<DIM, Q, SP>;
     constexpr int N = G::N, NP = G::NP, NL = G::NL;
     long long *X = smem, *Y = X + G::CW * G::C;
-    FxLane L = fx_lane<DIM, Q>(reinterpret_cast<int *>(Y + G::CW * G::C));
+    FxLane L = fx_lane<DIM, Q, SP>(reinterpret_cast<int *>(Y + G::CW * G::C));
     const int ncl = (int)(cst.ncell - cell0 < G::CW ? cst.ncell - cell0 : G::CW);
     const bool active = L.live && L.c < ncl;
     const int64_t cell = cell0 + (L.c < ncl ? L.c : 0);
     long long *xc = X + L.c * G::C, *xs = xc + L.k * G::S;
     double *ys = reinterpret_cast<double *>(Y + L.c * G::C) + L.k * G::S;
-    fx_stage_in<DIM, Q>(Y, u + cell0 * NL, ncl * NL, L.lane);
+    fx_stage_in<DIM, Q, SP>(Y, u + cell0 * NL, ncl * NL, L.lane);
     double ec[G::NC];
     if (e0) {
         int ci[3];
@@ -940,7 +946,7 @@ __device__ __forceinline__ void fx_project_body(const FxTab &tab, const FxConst 
     }
     fx_cp_wait();
     __syncwarp();
-    const int eu = fx_unit(fx_cell_max<Q>(fx_slab_top<DIM, Q>(ys), L));
+    const int eu = fx_unit(fx_cell_max<Q * SP>(fx_slab_top<DIM, Q, SP>(ys, L.sub), L));
     FxBlock t{eu, 0};
     if (e0) {
         int mx = 0;
@@ -960,12 +966,12 @@ __device__ __forceinline__ void fx_project_body(const FxTab &tab, const FxConst 
             z[c] = acc_value(s);
             mag.add(z[c]);
         }
-        const int n = fx_headroom(fx_cell_max<Q>(mag.top(), L));
+        const int n = fx_headroom(fx_cell_max<Q * SP>(mag.top(), L));
         ee += tab.eHat + 64 - n;
         const int ew = ee + (DIM - 1) * (tab.eHat + 64), E = imax(eu, ew) + 1;
         mag = FxMag();
 #pragma unroll 1
-        for (int p = 0; p < NP; ++p) {
+        for (int p = L.sub; p < NP; p += SP) {
             Limb y[2];
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
@@ -993,36 +999,36 @@ __device__ __forceinline__ void fx_project_body(const FxTab &tab, const FxConst 
                 mag.add(v);
             }
         }
-        t = fx_block<Q>(mag, E, L);
-        fx_store_out<DIM, Q>(u + cell0 * NL, reinterpret_cast<const double *>(Y), ncl * NL, L.lane);
+        t = fx_block<Q * SP>(mag, E, L);
+        fx_store_out<DIM, Q, SP>(u + cell0 * NL, reinterpret_cast<const double *>(Y), ncl * NL, L.lane);
     } else {
 #pragma unroll 4
-        for (int i = 0; i < N; ++i) {
+        for (int i = L.sub; i < N; i += SP) {
             const long long v = fx_from(ys[i], eu + FX_UNIT);
             if (L.live) xs[i] = v;
         }
         __syncwarp();
     }
-    fx_all_traces<DIM, Q, USER>(tab, cst, xc, t, L, active, cell, tr);
+    fx_all_traces<DIM, Q, SP, USER>(tab, cst, xc, t, L, active, cell, tr);
 }
 
-template <int DIM, int Q, bool USER>
-__global__ void __launch_bounds__(FxGeo<DIM, Q>::NW * 32)
+template <int DIM, int Q, int SP, bool USER>
+__global__ void __launch_bounds__(FxGeo<DIM, Q, SP>::NW * 32)
     k_fx_project(const __grid_constant__ FxTab tab, const __grid_constant__ FxConst cst, double *u,
                  const double *__restrict__ e0, double *__restrict__ tr) {
-    using G = FxGeo<DIM, Q>;
+    using G = FxGeo<DIM, Q, SP>;
     extern __shared__ __align__(16) long long smem_fx[];
     const int warp = threadIdx.x >> 5;
     const int64_t cell0 = (int64_t)blockIdx.x * G::CPB + warp * G::CW;
     if (cell0 >= cst.ncell) return;
-    fx_project_body<DIM, Q, USER>(tab, cst, smem_fx + warp * G::warp_words_project(), cell0, u, e0, tr);
+    fx_project_body<DIM, Q, SP, USER>(tab, cst, smem_fx + warp * G::warp_words_project(), cell0, u, e0, tr);
 }
 
-template <int DIM, int Q>
-__global__ void __launch_bounds__(FxGeo<DIM, Q>::NW * 32)
+template <int DIM, int Q, int SP>
+__global__ void __launch_bounds__(FxGeo<DIM, Q, SP>::NW * 32)
     k_fx_project_batch(const __grid_constant__ FxTab tab, const BatchDG<double> *__restrict__ D,
                        const BlockMap *__restrict__ map, int nblocks, double *u, int with_e0) {
-    using G = FxGeo<DIM, Q>;
+    using G = FxGeo<DIM, Q, SP>;
     extern __shared__ __align__(16) long long smem_fx[];
     __shared__ __align__(16) BatchDG<double> sd;
     const int warp = threadIdx.x >> 5;
@@ -1032,7 +1038,7 @@ __global__ void __launch_bounds__(FxGeo<DIM, Q>::NW * 32)
         load_batch_desc(D + m.inst, &sd);
         const int64_t cell0 = (int64_t)m.cell0 + warp * G::CW;
         if (cell0 < sd.c.ncell)
-            fx_project_body<DIM, Q>(tab, sd.c, smem_fx + warp * G::warp_words_project(), cell0, u + sd.off * G::NL,
+            fx_project_body<DIM, Q, SP>(tab, sd.c, smem_fx + warp * G::warp_words_project(), cell0, u + sd.off * G::NL,
                                     with_e0 ? sd.e0 : nullptr, sd.tr[0]);
     }
 }
@@ -1042,18 +1048,44 @@ inline void fx_allow_smem(K *kernel, size_t bytes) {      // beside the static d
     if (bytes > 32 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
+// Lanes per slab. On a small mesh a sub-core has at most one warp and that warp's own
+// rate bounds the launch (q = 6: the same 49 us for 576 and 2744 cells), so the pencils
+// of a slab go over SP lanes and a warp takes fewer cells (3D, q >= 5). Residual and four
+// steps, one lane / split: q = 5, 576 cells 37 and 154 / 20 and 70 us, 2197 cells 37 and
+// 154 / 35 and 109, 3375 cells 37 and 154 / 41 and 154; q = 6 576 cells 49 and 197 / 27 and
+// 103, 2744 cells 50 and 204 / 70 and 239 (its second round of pencils is nearly empty);
+// q = 7 512 cells 58 and 263 / 29 and 113, 2197 cells 62 and 271 / 58 and 251.
+template <int DIM, int Q>
+constexpr int fx_split() {
+    return DIM == 3 && Q >= 5 ? (Q == 5 ? 5 : 32 / Q) : 1;
+}
+template <int DIM, int Q>
+inline bool fx_small(int64_t ncell) {
+    return fx_split<DIM, Q>() > 1 && ncell <= (Q == 6 ? 1520 : 2432);
+}
+
+template <int DIM, int Q, int SP, int MODE>
+cudaError_t fx_run_cells_of(const FxLevel &l, int flags, int mode, double *u, const double *b, const double *kappa,
+                         const double *fd, const double *linv, const double *tri, double *tro, double *r,
+                         double *corners, cudaStream_t s) {
+    using G = FxGeo<DIM, Q, SP>;
+    if (l.cst.ncell <= 0) return cudaSuccess;
+    const size_t sm = G::bytes(MODE);
+    fx_allow_smem(k_fx_cells<DIM, Q, SP, MODE>, sm);
+    count_launches(1);
+    k_fx_cells<DIM, Q, SP, MODE><<<(unsigned)((l.cst.ncell + G::CPB - 1) / G::CPB), G::NW * 32, sm, s>>>(
+        l.tab, l.cst, flags, mode, u, b, kappa, fd, linv, tri, tro, r, corners);
+    return cudaGetLastError();
+}
+
 template <int DIM, int Q, int MODE>
 cudaError_t fx_run_cells(const FxLevel &l, int flags, int mode, double *u, const double *b, const double *kappa,
                          const double *fd, const double *linv, const double *tri, double *tro, double *r,
                          double *corners, cudaStream_t s) {
-    using G = FxGeo<DIM, Q>;
-    if (l.cst.ncell <= 0) return cudaSuccess;
-    const size_t sm = G::bytes(MODE);
-    fx_allow_smem(k_fx_cells<DIM, Q, MODE>, sm);
-    count_launches(1);
-    k_fx_cells<DIM, Q, MODE><<<(unsigned)((l.cst.ncell + G::CPB - 1) / G::CPB), G::NW * 32, sm, s>>>(
-        l.tab, l.cst, flags, mode, u, b, kappa, fd, linv, tri, tro, r, corners);
-    return cudaGetLastError();
+    if (fx_small<DIM, Q>(l.cst.ncell))
+        return fx_run_cells_of<DIM, Q, fx_split<DIM, Q>(), MODE>(l, flags, mode, u, b, kappa, fd, linv, tri, tro, r,
+                                                                 corners, s);
+    return fx_run_cells_of<DIM, Q, 1, MODE>(l, flags, mode, u, b, kappa, fd, linv, tri, tro, r, corners, s);
 }
 
 template <int DIM, int Q, int MODE>
@@ -1062,23 +1094,29 @@ cudaError_t fx_run_cells_batch(const FxTab &tab, const BatchDG<double> *D, const
     using G = FxGeo<DIM, Q>;
     if (nblocks <= 0) return cudaSuccess;
     const size_t sm = G::bytes(MODE);
-    fx_allow_smem(k_fx_cells_batch<DIM, Q, MODE>, sm);
+    fx_allow_smem(k_fx_cells_batch<DIM, Q, 1, MODE>, sm);
     count_launches(1);
-    k_fx_cells_batch<DIM, Q, MODE>
-        <<<persistent_grid((const void *)k_fx_cells_batch<DIM, Q, MODE>, G::NW * 32, sm, nblocks), G::NW * 32, sm, s>>>(
+    k_fx_cells_batch<DIM, Q, 1, MODE>
+        <<<persistent_grid((const void *)k_fx_cells_batch<DIM, Q, 1, MODE>, G::NW * 32, sm, nblocks), G::NW * 32, sm, s>>>(
             tab, D, map, nblocks, flags, mode, u, b, r, cur);
     return cudaGetLastError();
 }
 
 template <int DIM, int Q>
 cudaError_t FxRun<DIM, Q>::project(const FxLevel &l, bool user, double *u, const double *e0, double *tr, cudaStream_t s) {
-    using G = FxGeo<DIM, Q>;
     if (l.cst.ncell <= 0) return cudaSuccess;
-    const auto fn = user ? k_fx_project<DIM, Q, true> : k_fx_project<DIM, Q, false>;
-    fx_allow_smem(fn, G::bytes_project());
-    count_launches(1);
-    fn<<<(unsigned)((l.cst.ncell + G::CPB - 1) / G::CPB), G::NW * 32, G::bytes_project(), s>>>(l.tab, l.cst, u, e0, tr);
-    return cudaGetLastError();
+    auto run = [&](auto split) -> cudaError_t {
+        constexpr int SP = decltype(split)::value;
+        using G = FxGeo<DIM, Q, SP>;
+        const auto fn = user ? k_fx_project<DIM, Q, SP, true> : k_fx_project<DIM, Q, SP, false>;
+        fx_allow_smem(fn, G::bytes_project());
+        count_launches(1);
+        fn<<<(unsigned)((l.cst.ncell + G::CPB - 1) / G::CPB), G::NW * 32, G::bytes_project(), s>>>(l.tab, l.cst, u, e0,
+                                                                                                    tr);
+        return cudaGetLastError();
+    };
+    if (fx_small<DIM, Q>(l.cst.ncell)) return run(std::integral_constant<int, fx_split<DIM, Q>()>{});
+    return run(std::integral_constant<int, 1>{});
 }
 template <int DIM, int Q>
 cudaError_t FxRun<DIM, Q>::smooth(const FxLevel &l, bool exact, int flags, double *u, const double *b,
@@ -1103,10 +1141,10 @@ cudaError_t FxRun<DIM, Q>::project_batch(const FxTab &tab, const BatchDG<double>
     using G = FxGeo<DIM, Q>;
     if (nblocks <= 0) return cudaSuccess;
     const size_t sm = G::bytes_project();
-    fx_allow_smem(k_fx_project_batch<DIM, Q>, sm);
+    fx_allow_smem(k_fx_project_batch<DIM, Q, 1>, sm);
     count_launches(1);
-    k_fx_project_batch<DIM, Q>
-        <<<persistent_grid((const void *)k_fx_project_batch<DIM, Q>, G::NW * 32, sm, nblocks), G::NW * 32, sm, s>>>(
+    k_fx_project_batch<DIM, Q, 1>
+        <<<persistent_grid((const void *)k_fx_project_batch<DIM, Q, 1>, G::NW * 32, sm, nblocks), G::NW * 32, sm, s>>>(
             tab, D, map, nblocks, u, with_e0);
     return cudaGetLastError();
 }

@@ -100,3 +100,18 @@ def test_callers_traces_and_own_traces_agree(dgmg, n, p, basis):
     ctx.project(u, None, tr)
     ctx.residual_restrict(u, b, tr, user, None)
     assert _rel(user.cpu().numpy(), own.cpu().numpy()) <= 1e-13
+
+
+@pytest.mark.parametrize("n,p", [((13, 13, 14), 4), ((14, 14, 13), 4), ((12, 12, 10), 5), ((12, 12, 11), 5),
+                                 ((13, 13, 14), 6), ((14, 14, 13), 6)])
+def test_residual_on_both_sides_of_the_split(dgmg, n, p):
+    """3D, p >= 4: meshes just below and just above the size from which a slab has one
+    lane instead of several."""
+    rng = np.random.default_rng(p)
+    kap = np.exp(rng.normal(size=int(np.prod(n))))
+    mesh = sipg.Mesh(n, p)
+    ctx = dgmg.Context(n, p, kap)
+    u, b = rng.normal(size=mesh.ndof), rng.normal(size=mesh.ndof)
+    r = torch.empty(mesh.ndof, dtype=torch.float64, device=DEV)
+    ctx.residual(_t(u), _t(b), r)
+    assert _rel(r.cpu().numpy(), sipg.residual(mesh, u, b, kap)) <= 1e-12
