@@ -56,11 +56,12 @@ FX_HD void acc_zero(Acc &s) {
 }
 // c + a b. On the device as a carry pair, which becomes the one wide multiply-add it
 // is; mad.wide lets the assembler rebalance a sum of products into separate 64-bit
-// adds (12 more instructions per four products, by the opcode counters).
+// adds (12 more instructions per four products, by the opcode counters). The low word
+// is written before the factors are read again: it shares no register with them.
 FX_HD long long mad_wide(int a, int b, long long c) {
 #ifdef __CUDA_ARCH__
     unsigned lo = (unsigned)c, hi = (unsigned)((unsigned long long)c >> 32);
-    asm("mad.lo.cc.s32 %0, %2, %3, %0;\n\tmadc.hi.s32 %1, %2, %3, %1;" : "+r"(lo), "+r"(hi) : "r"(a), "r"(b));
+    asm("mad.lo.cc.s32 %0, %2, %3, %0;\n\tmadc.hi.s32 %1, %2, %3, %1;" : "+&r"(lo), "+r"(hi) : "r"(a), "r"(b));
     return (long long)((unsigned long long)hi << 32 | lo);
 #else
     return c + (long long)a * b;
