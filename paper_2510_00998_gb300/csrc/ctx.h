@@ -35,7 +35,7 @@ template <typename T>
 struct DGDev {
     DGConst<T> c;
     T *kappa = nullptr, *fd = nullptr, *tr[2] = {nullptr, nullptr}, *corners = nullptr;
-    T *linv = nullptr;   // per-node omega / (sum of the cell's eigenvalues); FP64 only (as integers)
+    T *linv = nullptr;   // per-node omega / (sum of the cell's eigenvalues); FP64 only (fx_table_word)
     T *fdr = nullptr;    // FP32: the residual's factors [S^T M | lambda] per cell and axis
     T *kfac = nullptr;   // facet coefficients [cell][face]
 };

@@ -446,7 +446,7 @@ __device__ __forceinline__ void fx_cell_coords(int64_t cell, const int *n, int *
 // A_KK^-1 by fast diagonalisation (Kt_a S_a = M_a S_a Lambda_a): S^T along every
 // axis, times the table omega / (sum of eigenvalues), S along every axis. fd: the
 // cell's limbs of S per axis, their exponents in the words after them (axis 0 also
-// the table's); linv: the table as integers.
+// the table's); linv: the table.
 // flags: SM_ZERO: the iterate is 0 (u and its traces are not read); SM_NO_TRACES:
 // the new traces are not written. mode (residual): RES_*.
 template <int DIM, int Q, int SP, int MODE>
@@ -723,17 +723,17 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
             fx_cp_wait();
             __syncwarp();
             const long long *li = reinterpret_cast<const long long *>(ys);
-            FxMag mag;
+            int least = FX_SCALED_MOST;
+#pragma unroll 4
+            for (int i = L.sub; i < N; i += SP) least = imin(least, fx_scaled_below(xs[i], li[i]));
+            least = FX_SCALED_MOST - fx_cell_max<Q * SP>(FX_SCALED_MOST - least, L);
 #pragma unroll 4
             for (int i = L.sub; i < N; i += SP) {
-                Acc s;
-                acc_zero(s);
-                mac(s, limb_of(li[i]), fx_read(xs[i], t.n));
-                const long long v = acc_value(s);
+                const long long v = fx_scaled(xs[i], li[i], least);
                 if (G::ALL || L.live) xs[i] = v;
-                mag.add(v);
             }
-            t = fx_block<Q * SP>(mag, t.e - t.n + myF[Q * Q + 1].h + 64, L);
+            t = FxBlock{t.e + myF[Q * Q + 1].h - least, 2};   // (the largest is between 2^56 and 2^58)
+            __syncwarp();
             // the previous iterate into Y (every lane has read the table)
             if (!zero) fx_stage_in<DIM, Q, SP>(Y, u + cell0 * NL, ncl * NL, L.lane);
         }

@@ -126,26 +126,34 @@ __global__ void __launch_bounds__(128) k_fd_factors(const __grid_constant__ FDIn
     for (int i = 0; i < q; ++i) out[q * q + i] = (T)lam[i];
 }
 
-// Largest biased exponent that an entry omega / (sum of eigenvalues) of a cell's table
-// can have, from the smallest eigenvalue of every axis (positive FP64 numbers are
-// ordered as their bits); one thread per cell
+// Largest exponent of an entry omega / (sum of eigenvalues) of a cell's table, from the
+// smallest eigenvalue of every axis (rounding can leave one that is not positive where kappa
+// jumps by 1e16: then from every sum); one thread per cell
 __global__ void k_fx_table_unit(int dim, int q, int64_t ncell, const double *__restrict__ fd, double omega,
                                 int *__restrict__ unit) {
     const int64_t cell = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (cell >= ncell) return;
     const int fds = q * q + q;
+    const double *f = fd + cell * dim * fds + q * q;
     double s = 0.0;
+    bool positive = true;
     for (int a = 0; a < dim; ++a) {
-        const double *f = fd + (cell * dim + a) * fds + q * q;
-        long long m = __double_as_longlong(f[0]);
-        for (int i = 1; i < q; ++i) m = min(m, __double_as_longlong(f[i]));
-        s += __longlong_as_double(m);
+        double m = f[a * fds];
+        for (int i = 1; i < q; ++i) m = fmin(m, f[a * fds + i]);
+        positive = positive && m > 0.0;
+        s += m;
     }
-    unit[cell] = ilogb(omega) - ilogb(s) + 1 + 1023;
+    if (!positive)
+        for (int i = 0; i < (dim == 3 ? q * q * q : q * q); ++i) {
+            double t = f[i % q] + f[fds + (i / q) % q];
+            if (dim == 3) t += f[2 * fds + i / (q * q)];
+            s = i == 0 || fabs(t) < fabs(s) ? t : s;
+        }
+    const double top = omega / fabs(s);
+    unit[cell] = isfinite(top) && top > 0.0 ? ilogb(top) : 0;
 }
 
-// The inverse eigenvalue sums of every cell with the smoother's damping folded in, as
-// 64-bit integers below 2^62 of the cell's unit
+// The inverse eigenvalue sums of every cell with the smoother's damping folded in
 __global__ void k_fx_table(int dim, int q, int64_t ncell, const double *__restrict__ fd, double omega,
                            const int *__restrict__ unit, long long *__restrict__ linv) {
     const int64_t nloc = dim == 3 ? (int64_t)q * q * q : (int64_t)q * q;
@@ -156,12 +164,12 @@ __global__ void k_fx_table(int dim, int q, int64_t ncell, const double *__restri
     const double *f = fd + cell * dim * fds + q * q;
     double s = f[node % q] + f[fds + (node / q) % q];
     if (dim == 3) s += f[2 * fds + node / (q * q)];
-    linv[idx] = fx_from(omega / s, unit[cell]) << 2;
+    linv[idx] = fx_table_word(omega / s, unit[cell]);
 }
 
 // fd in place: S of every axis as limbs of one unit (every row and column sum of
 // the magnitudes below 2^62), the unit in the word after it, and in the word after
-// axis 0's the unit of the table; one thread per cell and axis
+// axis 0's the exponent of the table; one thread per cell and axis
 __global__ void k_fx_factors(int dim, int q, int64_t ncell, double *__restrict__ fd, const int *__restrict__ unit) {
     const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (id >= ncell * dim) return;
@@ -179,7 +187,7 @@ __global__ void k_fx_factors(int dim, int q, int64_t ncell, double *__restrict__
     const int ev = ilogb(top) + 1023;
     for (int i = 0; i < q * q; ++i) out[i] = limb_of(fx_from(S[i], ev) << 2);
     out[q * q] = Limb{fx_unit(ev) - 2, 0};
-    if (id % dim == 0) out[q * q + 1] = Limb{fx_unit(unit[id / dim]) - 2, 0};
+    if (id % dim == 0) out[q * q + 1] = Limb{unit[id / dim] + FX_SCALED, 0};
 }
 
 // kfac[cell][f]: the harmonic mean of kappa across face f (0 on the boundary),

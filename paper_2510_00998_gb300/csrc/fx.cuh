@@ -22,6 +22,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 namespace dgmg {
@@ -147,6 +148,43 @@ FX_HD double fx_to(long long t, int e) {
 
 // Arithmetic right shift by d >= 0 of any size.
 FX_HD long long fx_shr(long long t, int d) { return t >> imin(d, 63); }
+
+// Block values times numbers of any spread, as a block again. Where the largest value
+// meets the smallest number (the modes of a cell and the inverses of their eigenvalues)
+// the products are far below the product of the two largest, and one unit for the numbers
+// and one for the bound on the products would cost the ratio's bits: a smoothing step from
+// b = A u had two to six times the FP64 pipe's error. So every number has its exponent and
+// all of its 53 bits, a product is formed from both factors at full length, and the
+// block's unit follows the largest product: fx_scaled_below per value, the least of them
+// to fx_scaled. (A running maximum of the negated sums came out wrong from CUDA 13.0's
+// assembler wherever it was not unrolled in full: the sums are kept positive.)
+//
+// A number of the table as a word: the limbs of its significand (top bit 61, the low 9
+// zero), in those 9 bits of the low limb the exponent below the table's.
+constexpr int FX_BELOW = 511;
+FX_HD long long fx_table_word(double w, int base) {          // |w| < 2^(base + 1)
+    int e = 0;
+    const double f = frexp(w, &e);
+    const int below = base - (e - 1);
+    if (!(f != 0.0) || below > FX_BELOW) return FX_BELOW;    // (and what is not finite: the table is marked)
+    const Limb x = limb_of((long long)ldexp(f, 62));
+    return (long long)((unsigned long long)(unsigned)x.h << 32 | ((unsigned)x.l | (unsigned)below));
+}
+FX_HD int fx_lead(long long t) {                             // the sign's leading copies (at most 32)
+    const int h = (int)(t >> 32);
+    return clz32(h ^ (h >> 31));
+}
+FX_HD int fx_scaled_below(long long t, long long w) { return ((int)w & FX_BELOW) + fx_lead(t); }
+constexpr int FX_SCALED_MOST = FX_BELOW + 32;
+// |t| < 2^60; the result below 2^58, in units of 2^(e + base + FX_SCALED - least) for a t of unit 2^e
+constexpr int FX_SCALED = 64 - 61 + 4;
+FX_HD long long fx_scaled(long long t, long long w, int least) {
+    const int lead = fx_lead(t), below = (int)w & FX_BELOW;
+    Acc s;
+    acc_zero(s);
+    mac(s, Limb{(int)(w >> 32), (int)w & ~FX_BELOW}, limb_of(t << ((lead - 4) & 63)));
+    return acc_value(s) >> imin(below + lead - least, 63);
+}
 
 constexpr int FXQ = 7;                  // most nodes per axis
 

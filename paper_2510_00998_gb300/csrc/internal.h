@@ -189,10 +189,10 @@ struct FxRun {
                                       int mode, const double *u, const double *b, double *r, int cur, cudaStream_t s);
     static int cells_per_cta();
 };
-// linv[cell][node] = omega / (sum of the cell's eigenvalues) as 64-bit integers of
-// one exponent per cell, from the FP64 factors [S | lambda]; then, in place, the
-// factors as limbs: per axis S, its exponent in the word after it (h of a Limb);
-// the word after axis 0's exponent holds the table's. unit: scratch, one per cell.
+// linv[cell][node] = omega / (sum of the cell's eigenvalues) as words of a table (fx.cuh),
+// from the FP64 factors [S | lambda]; then, in place, the factors as limbs: per axis S, its
+// exponent in the word after it (h of a Limb); the word after axis 0's exponent holds the
+// table's. unit: scratch, one per cell.
 cudaError_t launch_fx_factors(int dim, int q, int64_t ncell, double *fd, double omega, double *linv, int *unit,
                               cudaStream_t s);
 

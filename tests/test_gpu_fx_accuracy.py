@@ -1,0 +1,53 @@
+"""How exact the FP64 kernels in block fixed-point arithmetic are, cell by cell, against
+extended precision: coefficients that jump, stretched meshes, values of a wide range
+inside a cell. A cell's error is taken of that cell's largest value."""
+import numpy as np
+import pytest
+
+from ref_long import L, Reference
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+DEV = "cuda:0"
+EPS = 2.0 ** -53
+
+
+@pytest.fixture(scope="module")
+def dgmg():
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2510_00998_gb300 import dgmg as m
+    return m
+
+
+def _t(x):
+    return torch.tensor(np.asarray(x, dtype=np.float64), device=DEV)
+
+
+def _kappa(kind, n, rng):
+    nc = int(np.prod(n))
+    return 10.0 ** rng.uniform(-kind / 2, kind / 2, size=nc) if kind else np.exp(rng.normal(size=nc))
+
+
+def _cell_error(got, ref):
+    e = np.abs(got.cpu().numpy().astype(L).reshape(ref.shape) - ref).max(1)
+    return float((e / np.abs(ref).max(1)).max())
+
+
+@pytest.mark.parametrize("n,p,jumps", [((5, 4, 3), 3, 0), ((5, 4, 3), 3, 6), ((5, 4, 3), 3, 12), ((4, 3, 3), 5, 0),
+                                       ((4, 3, 3), 5, 6), ((9, 8), 4, 0), ((2, 2, 60), 4, 0)])
+@pytest.mark.parametrize("near", [0, 1])
+def test_smoothing_step_per_cell(dgmg, n, p, jumps, near):
+    """One step from a random right-hand side, and (near) from b = A u, where the step
+    has to give u back. The step is 3 d passes of q products, each as good as a sum in FP64
+    with a rounding per product, from eigenvectors and eigenvalues that carry as much."""
+    rng = np.random.default_rng(5)
+    kap = _kappa(jumps, n, rng)
+    ref, ctx = Reference(n, p, kap), dgmg.Context(n, p, kap)
+    u, b = rng.normal(size=(2, ctx.ndof))
+    if near:
+        b = ref.apply(u).reshape(-1).astype(np.float64)
+    v = _t(u)
+    ctx.smooth(v, _t(b), 1)
+    assert _cell_error(v, ref.step(u, b, 0.8)) <= 2 * 3 * len(n) * (p + 1) * EPS
