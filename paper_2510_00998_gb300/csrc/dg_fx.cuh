@@ -851,7 +851,8 @@ __device__ __forceinline__ const Limb *fx_stage_tables(const FxTab &tab, long lo
             s[i] = tab.M[i];
         } else if (i < HE * HE) {
             const int r = i / HE, c = i - r * HE;
-            s[i] = limb_of((whole(r, c) + whole(r, Q - 1 - c)) >> 1);
+            const long long a = whole(r, c), b = whole(r, Q - 1 - c);
+            s[i] = limb_of((a & b) + ((a ^ b) >> 1));    // their mean (the middle one twice: its double has 65 bits)
         } else if (i < HE * HE + H * H) {
             const int r = (i - HE * HE) / H, c = i - HE * HE - r * H;
             s[i] = limb_of((whole(r, c) - whole(r, Q - 1 - c)) >> 1);

@@ -168,7 +168,7 @@ __global__ void k_fx_table(int dim, int q, int64_t ncell, const double *__restri
 }
 
 // fd in place: S of every axis as limbs of one unit (every row and column sum of
-// the magnitudes below 2^62), the unit in the word after it, and in the word after
+// the magnitudes below 2^63, an h below 2^31), the unit in the word after it, and in the word after
 // axis 0's the exponent of the table; one thread per cell and axis
 __global__ void k_fx_factors(int dim, int q, int64_t ncell, double *__restrict__ fd, const int *__restrict__ unit) {
     const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -184,9 +184,9 @@ __global__ void k_fx_factors(int dim, int q, int64_t ncell, double *__restrict__
         }
         top = fmax(top, fmax(rs, cs));
     }
-    const int ev = ilogb(top) + 1023;
-    for (int i = 0; i < q * q; ++i) out[i] = limb_of(fx_from(S[i], ev) << 2);
-    out[q * q] = Limb{fx_unit(ev) - 2, 0};
+    const int ev = ilogb(top * (1.0 + 0x1p-30)) + 1023;
+    for (int i = 0; i < q * q; ++i) out[i] = limb_of(fx_from(S[i], ev) << 3);
+    out[q * q] = Limb{fx_unit(ev) - 3, 0};
     if (id % dim == 0) out[q * q + 1] = Limb{unit[id / dim] + FX_SCALED, 0};
 }
 

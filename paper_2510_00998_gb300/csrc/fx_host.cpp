@@ -86,8 +86,13 @@ std::vector<R> times(int q, const std::vector<R> &A, const std::vector<double> &
 }
 
 // The magnitudes the kernels count on (fx.cuh, mac): the h of a row of a matrix
-// sum to at most 2^31, those of a single factor are at most 2^30.
-constexpr int ROW_BITS = 62, ONE_BITS = 61;
+// sum to at most 2^31, those of a single factor are at most 2^30. The mass, and the
+// eigenvectors (k_fx_factors), whose passes follow one another in the smoothing step, use
+// all of it (pass_unit): with a bit less a step on 40 x 2 x 2 cells, p = 3, was off by up to
+// 1.2e-14 of a cell's largest value (FP64 pipe 4.6e-15, now 5.6e-15), and by up to 1.7e-14
+// from b = A u (7.4e-15, 1.0e-14).
+constexpr int ROW_BITS = 62, ONE_BITS = 61, PASS_BITS = 63;
+int pass_unit(R bound) { return unit_for(bound * (1 + 0x1p-30L), PASS_BITS); }   // (an h stays below 2^31)
 
 // What a level takes from its element: the tables, and M^-1 of the end values.
 struct Element {
@@ -117,7 +122,7 @@ Element make_element(const RefElem1D &re, int penalty_p) {
                 Rt[w][i * q + j] = -wt * (mp[i] * re.dp[j] + dp[i] * re.ep[j]) + pen * mp[i] * re.ep[j];
             }
     }
-    tab.eM = unit_for(row_sum(q, {&M}), ROW_BITS);
+    tab.eM = pass_unit(row_sum(q, {&M}));
     R rows = 0;
     for (int w = 0; w < 4; ++w) rows = std::max(rows, row_sum(q, {&K, &L[w & 1], &Rt[w >> 1]}));
     tab.eD = unit_for(rows, ROW_BITS);

@@ -51,3 +51,16 @@ def test_smoothing_step_per_cell(dgmg, n, p, jumps, near):
     v = _t(u)
     ctx.smooth(v, _t(b), 1)
     assert _cell_error(v, ref.step(u, b, 0.8)) <= 2 * 3 * len(n) * (p + 1) * EPS
+
+
+@pytest.mark.parametrize("seed", [0, 3])
+def test_smoothing_step_on_stretched_cells(dgmg, seed):
+    """The same where one axis' terms are hundreds of times the others'."""
+    n, p = (40, 2, 2), 3
+    rng = np.random.default_rng(seed)
+    kap = _kappa(0, n, rng)
+    ref, ctx = Reference(n, p, kap), dgmg.Context(n, p, kap)
+    u, b = rng.normal(size=(2, ctx.ndof))
+    v = _t(u)
+    ctx.smooth(v, _t(b), 1)
+    assert _cell_error(v, ref.step(u, b, 0.8)) <= 2 * 3 * len(n) * (p + 1) * EPS
