@@ -698,6 +698,13 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
     }
     // M along every axis; t <- b - t; S^T along every axis; the table; S along every axis
     const Limb *myF = mine;
+    // The residual on its way out keeps the bits of b: a subtraction in FP64 per node. (As
+    // a block it has those of the cell's largest value, so that u = 0 did not give b back.)
+    const bool write_r = !SMOOTH && has_b && (mode & RES_WRITE_R) != 0;
+    auto difference = [&](double bi, long long ti) {
+        const double w = fx_to(ti, t.e);
+        return mode & RES_NEGATE ? w - bi : bi - w;
+    };
     auto subtract_from_b = [&]() {                        // t = A u (or its neighbours' part); in the lane's slab
         fx_cp_wait();
         __syncwarp();
@@ -706,8 +713,12 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
         FxMag mag;
 #pragma unroll 4
         for (int i = L.sub; i < N; i += SP) {
-            const long long v = fx_from(ys[i], ev) - (zero ? 0 : fx_shr(xs[i] << t.n, E - te));
-            if (G::ALL || L.live) xs[i] = v;
+            const double bi = ys[i];
+            const long long ti = xs[i], v = fx_from(bi, ev) - (zero ? 0 : fx_shr(ti << t.n, E - te));
+            if (G::ALL || L.live) {
+                xs[i] = v;
+                if (write_r) ys[i] = difference(bi, ti);
+            }
             mag.add(v);
         }
         t = fx_block<Q * SP>(mag, E, L);
@@ -746,7 +757,19 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
             t = fx_pass<DIM, Q, SP>(xc, t, a, src, trans ? 1 : Q, trans ? Q : 1, src[Q * Q].h, L);
         }
     }
-    if (!SMOOTH && has_b) subtract_from_b();
+    if (!SMOOTH && has_b) {
+        if (mode & RES_CORNERS) {
+            subtract_from_b();
+        } else {
+            fx_cp_wait();
+            __syncwarp();
+#pragma unroll 4
+            for (int i = L.sub; i < N; i += SP) {
+                const double v = difference(ys[i], xs[i]);
+                if (L.live) ys[i] = v;
+            }
+        }
+    }
     if constexpr (SMOOTH) {
         // the last pass ran along axis 0, in the lane's own slab
         if (!zero) {                                     // u <- keep u + t
@@ -770,11 +793,13 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
     // the result leaves through Y
     if (SMOOTH || (mode & RES_WRITE_R)) {
         // without b the block is A u: the residual b - A u is its negative
-        const bool neg = !SMOOTH && has_b == ((mode & RES_NEGATE) != 0);
+        const bool neg = !SMOOTH && !(mode & RES_NEGATE);
+        if (!write_r) {
 #pragma unroll 4
-        for (int i = L.sub; i < N; i += SP) {
-            const double v = fx_to(neg ? -xs[i] : xs[i], t.e);
-            if (L.live) ys[i] = v;
+            for (int i = L.sub; i < N; i += SP) {
+                const double v = fx_to(neg ? -xs[i] : xs[i], t.e);
+                if (L.live) ys[i] = v;
+            }
         }
         __syncwarp();
         fx_store_out<DIM, Q, SP>((SMOOTH ? u : r) + cell0 * NL, reinterpret_cast<const double *>(Y), ncl * NL, L.lane);

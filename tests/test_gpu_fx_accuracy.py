@@ -64,3 +64,32 @@ def test_smoothing_step_on_stretched_cells(dgmg, seed):
     v = _t(u)
     ctx.smooth(v, _t(b), 1)
     assert _cell_error(v, ref.step(u, b, 0.8)) <= 2 * 3 * len(n) * (p + 1) * EPS
+
+
+def _wide(rng, n):
+    """Values over 60 binary orders in every cell."""
+    return rng.normal(size=n) * 2.0 ** -rng.uniform(0, 60, size=n)
+
+
+MESHES = [((5, 4), 3, 0), ((5, 4, 3), 2, 0), ((5, 4, 3), 2, 1), ((4, 3, 3), 5, 0), ((3, 4), 6, 1)]
+
+
+@pytest.mark.parametrize("n,p,basis", MESHES)
+def test_residual_keeps_the_bits_of_b(dgmg, n, p, basis):
+    """r = b - A u node by node: where A u is zero, r is b."""
+    rng = np.random.default_rng(p)
+    ctx = dgmg.Context(n, p, _kappa(0, n, rng), basis=basis)
+    b, nl = _t(_wide(rng, ctx.ndof)), (p + 1) ** len(n)
+    u, r = torch.zeros_like(b), torch.empty_like(b)
+    ctx.residual(u, b, r)
+    assert torch.equal(r, b)
+    tr, rc = torch.zeros(ctx.trace_size(), dtype=torch.float64, device=DEV), _t(np.empty(int(ctx.info.nvert0)))
+    for corners in (None, rc):
+        r.zero_()
+        ctx.residual_restrict(u, b, tr, r, corners)
+        assert torch.equal(r, b)
+    u[:nl] = 1.0                                     # the first cell: its neighbours see it, the rest does not
+    ctx.residual(u, b, r)
+    far = torch.ones(ctx.ndof // nl, dtype=torch.bool, device=DEV)
+    far[[0, 1, n[0]] + ([n[0] * n[1]] if len(n) == 3 else [])] = False
+    assert torch.equal(r.view(-1, nl)[far], b.view(-1, nl)[far])
