@@ -347,10 +347,11 @@ constexpr int FX_NO_TRACE = FX_NONE / 2;     // exponents below: all values are 
 
 // Traces of the cell from its block in shared memory: per axis and side, value and
 // +axis derivative; derivatives by dot products, values the end nodes (GLL) or dot
-// products (GL). USER: as FP64.
+// products (GL). USER: as FP64, the end nodes' values from the cell's FP64 values yc.
 template <int DIM, int Q, int SP, bool USER = false>
 __device__ __forceinline__ void fx_all_traces(const FxTab &tab, const FxConst &cst, const long long *xc, FxBlock b,
-                                              FxLane &L, bool write, int64_t cell, double *__restrict__ tr) {
+                                              FxLane &L, bool write, int64_t cell, double *__restrict__ tr,
+                                              const double *yc = nullptr) {
     using G = FxGeo<DIM, Q, SP>;
     const int e = b.e - b.n;
     double *cell_tr = tr + cell * G::TR;
@@ -394,6 +395,8 @@ __device__ __forceinline__ void fx_all_traces(const FxTab &tab, const FxConst &c
 #pragma unroll
                     for (int i = 0; i < Q; ++i) mac(v, tab.v[s][i], x[i]);
                     put(s, 0, acc_value(v), e + tab.eV + 64);
+                } else if (USER) {
+                    if (write) out[s * G::FS + p] = yc[(t - xc) + (s ? Q - 1 : 0) * ax.step];
                 } else {
                     put(s, 0, t[(s ? Q - 1 : 0) * ax.step] << b.n, e);
                 }
@@ -972,8 +975,7 @@ __device__ __forceinline__ void fx_project_body(const FxTab &tab, const FxConst 
     }
     fx_cp_wait();
     __syncwarp();
-    const int eu = fx_unit(fx_cell_max<Q * SP>(fx_slab_top<DIM, Q, SP>(ys, L.sub), L));
-    FxBlock t{eu, 0};
+    int top = 0;                                          // of the new u, by its high words
     if (e0) {
         int mx = 0;
 #pragma unroll
@@ -994,8 +996,7 @@ __device__ __forceinline__ void fx_project_body(const FxTab &tab, const FxConst 
         }
         const int n = fx_headroom(fx_cell_max<Q * SP>(mag.top(), L));
         ee += tab.eHat + 64 - n;
-        const int ew = ee + (DIM - 1) * (tab.eHat + 64), E = imax(eu, ew) + 1;
-        mag = FxMag();
+        const int ew = ee + (DIM - 1) * (tab.eHat + 64);
 #pragma unroll 1
         for (int p = L.sub; p < NP; p += SP) {
             Limb y[2];
@@ -1017,25 +1018,28 @@ __device__ __forceinline__ void fx_project_body(const FxTab &tab, const FxConst 
                 acc_zero(s);
                 mac(s, tab.hat[0][i], y[0]);
                 mac(s, tab.hat[1][i], y[1]);
-                const long long v = fx_shr(acc_value(s), E - ew) + fx_from(ys[i + Q * p], E + FX_UNIT);
-                if (L.live) {
-                    xs[i + Q * p] = v;
-                    ys[i + Q * p] = fx_to(v, E);
-                }
-                mag.add(v);
+                // node by node in FP64: u keeps its bits, whatever its cell's largest value is
+                const double v = ys[i + Q * p] + fx_to(acc_value(s), ew);
+                if (L.live) ys[i + Q * p] = v;
+                top = imax(top, fx_abs_hi(v));
             }
         }
-        t = fx_block<Q * SP>(mag, E, L);
-        fx_store_out<DIM, Q, SP>(u + cell0 * NL, reinterpret_cast<const double *>(Y), ncl * NL, L.lane);
+        top >>= 20;
     } else {
-#pragma unroll 4
-        for (int i = L.sub; i < N; i += SP) {
-            const long long v = fx_from(ys[i], eu + FX_UNIT);
-            if (L.live) xs[i] = v;
-        }
-        __syncwarp();
+        top = fx_slab_top<DIM, Q, SP>(ys, L.sub);
     }
-    fx_all_traces<DIM, Q, SP, USER>(tab, cst, xc, t, L, active, cell, tr);
+    top = fx_cell_max<Q * SP>(top, L);
+    if (e0) fx_store_out<DIM, Q, SP>(u + cell0 * NL, reinterpret_cast<const double *>(Y), ncl * NL, L.lane);
+    const int eu = fx_unit(top);
+#pragma unroll 4
+    for (int i = L.sub; i < N; i += SP) {
+        const long long v = fx_from(ys[i], eu + FX_UNIT);
+        if (L.live) xs[i] = v;
+    }
+    __syncwarp();
+    const FxBlock t{eu, 0};
+    fx_all_traces<DIM, Q, SP, USER>(tab, cst, xc, t, L, active, cell, tr,
+                                    reinterpret_cast<const double *>(Y + L.c * G::C));
 }
 
 template <int DIM, int Q, int SP, bool USER>

@@ -93,3 +93,31 @@ def test_residual_keeps_the_bits_of_b(dgmg, n, p, basis):
     far = torch.ones(ctx.ndof // nl, dtype=torch.bool, device=DEV)
     far[[0, 1, n[0]] + ([n[0] * n[1]] if len(n) == 3 else [])] = False
     assert torch.equal(r.view(-1, nl)[far], b.view(-1, nl)[far])
+
+
+@pytest.mark.parametrize("n,p,basis", MESHES)
+def test_projection_keeps_the_bits_of_u(dgmg, n, p, basis):
+    """u + P e node by node: a correction that is zero leaves u as it is, one that is zero
+    at a node leaves that node; the value traces of the Lobatto basis are u's end nodes."""
+    rng = np.random.default_rng(p)
+    d, q = len(n), p + 1
+    ctx = dgmg.Context(n, p, _kappa(0, n, rng), basis=basis)
+    u = _t(_wide(rng, ctx.ndof))
+    tr, e = torch.empty(ctx.trace_size(), dtype=torch.float64, device=DEV), torch.zeros(int(ctx.info.nvert0), dtype=torch.float64, device=DEV)
+    v = u.clone()
+    ctx.project(v, e, tr)
+    assert torch.equal(v, u)
+    e[0] = 3.0                                       # the vertex (1, 1[, 1]): the cells around it
+    ctx.project(v, e, tr)
+    w, x = v.view(n[::-1] + (q,) * d), u.view(n[::-1] + (q,) * d)
+    near = torch.zeros(n[::-1], dtype=torch.bool, device=DEV)
+    near[(slice(0, 2),) * d] = True
+    assert torch.equal(w[~near], x[~near]) and not torch.equal(w[near], x[near])
+    if basis == 0:
+        assert torch.equal(w[(0,) * d][..., 0], x[(0,) * d][..., 0])     # the hat is zero on x = 0
+        faces = tr.view(ctx.ndof // q ** d, 2 * d, 2, -1)
+        vals = w.reshape(-1, *(q,) * d)
+        assert torch.equal(faces[:, 0, 0], vals[..., 0].reshape(len(faces), -1))
+        assert torch.equal(faces[:, 1, 0], vals[..., q - 1].reshape(len(faces), -1))
+        last = vals[:, 0].reshape(len(faces), -1)    # the first slab: the last axis' low face
+        assert torch.equal(faces[:, 2 * d - 2, 0], last)
