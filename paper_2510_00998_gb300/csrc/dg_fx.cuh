@@ -773,31 +773,38 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
             }
         }
     }
+    const bool traces = SMOOTH && !(flags & SM_NO_TRACES);
+    bool in_y = write_r;                                  // the result is in Y
     if constexpr (SMOOTH) {
         // the last pass ran along axis 0, in the lane's own slab
-        if (!zero) {                                     // u <- keep u + t
+        if (!zero) {
+            // u <- keep u + t node by node in FP64 (u keeps its bits, whatever its cell's
+            // largest value is); the block for the traces is read from the result
             fx_cp_wait();
             __syncwarp();
-            const int ev = fx_cell_max<Q * SP>(fx_slab_top<DIM, Q, SP>(ys, L.sub), L);
-            const int eu = fx_unit(ev) + cst.eKeep + 64, te = t.e - t.n, E = imax(eu, te) + 1;
-            FxMag mag;
+            int top = 0;
 #pragma unroll 4
             for (int i = L.sub; i < N; i += SP) {
-                Acc s;
-                acc_zero(s);
-                mac(s, cst.keep, limb_of(fx_from(ys[i], ev)));
-                const long long v = fx_shr(acc_value(s), E - eu) + fx_shr(xs[i] << t.n, E - te);
-                if (G::ALL || L.live) xs[i] = v;
-                mag.add(v);
+                const double v = fma(cst.keep, ys[i], fx_to(xs[i], t.e));
+                if (L.live) ys[i] = v;
+                top = imax(top, fx_abs_hi(v));
             }
-            t = fx_block<Q * SP>(mag, E, L);
+            in_y = true;
+            if (traces) {
+                t = FxBlock{fx_unit(fx_cell_max<Q * SP>(top >> 20, L)), 0};
+#pragma unroll 4
+                for (int i = L.sub; i < N; i += SP) {
+                    const long long v = fx_from(ys[i], t.e + FX_UNIT);
+                    if (G::ALL || L.live) xs[i] = v;
+                }
+            }
         }
     }
     // the result leaves through Y
     if (SMOOTH || (mode & RES_WRITE_R)) {
         // without b the block is A u: the residual b - A u is its negative
         const bool neg = !SMOOTH && !(mode & RES_NEGATE);
-        if (!write_r) {
+        if (!in_y) {
 #pragma unroll 4
             for (int i = L.sub; i < N; i += SP) {
                 const double v = fx_to(neg ? -xs[i] : xs[i], t.e);
@@ -808,7 +815,7 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
         fx_store_out<DIM, Q, SP>((SMOOTH ? u : r) + cell0 * NL, reinterpret_cast<const double *>(Y), ncl * NL, L.lane);
     }
     if constexpr (SMOOTH) {
-        if (!(flags & SM_NO_TRACES)) fx_all_traces<DIM, Q, SP>(tab, cst, xc, t, L, active, cell, tr_out);
+        if (traces) fx_all_traces<DIM, Q, SP>(tab, cst, xc, t, L, active, cell, tr_out);
     } else if (mode & RES_CORNERS) {
         // corner sums of b - A u: hat values along the slab's axes, then over the slabs
         constexpr int NS = DIM == 3 ? 4 : 2;             // sums per slab

@@ -217,8 +217,7 @@ struct FxConst {
     double sa[3];
     Limb cH[3][2][FXQ], dt[3][2][FXQ];  // neighbour's derivative trace; derivatives at the cell's ends
     int eH[3], eT[3];
-    Limb keep;                          // 1 - omega (exact blocks) or 1
-    int eKeep;
+    double keep;                        // 1 - omega (exact blocks) or 1
     const double *kfac;                 // [cell][2 axis + side], 0 on the boundary
 };
 

@@ -199,8 +199,7 @@ void fx_level(const RefElem1D &re, int penalty_p, int dim, const int *n, int64_t
                 cst.dt[a][s][i] = limb(d[s * q + i], cst.eT[a]);
             }
     }
-    cst.eKeep = unit_for(std::max(std::fabs((R)keep), (R)1e-300L), ONE_BITS);
-    cst.keep = limb((R)keep, cst.eKeep);
+    cst.keep = keep;
 }
 
 }  // namespace dgmg

@@ -121,3 +121,26 @@ def test_projection_keeps_the_bits_of_u(dgmg, n, p, basis):
         assert torch.equal(faces[:, 1, 0], vals[..., q - 1].reshape(len(faces), -1))
         last = vals[:, 0].reshape(len(faces), -1)    # the first slab: the last axis' low face
         assert torch.equal(faces[:, 2 * d - 2, 0], last)
+
+
+@pytest.mark.parametrize("n,p,basis", MESHES)
+@pytest.mark.parametrize("steps", [1, 3])
+def test_smoothing_keeps_the_bits_of_u(dgmg, n, p, basis, steps):
+    """u <- (1 - omega) u + omega D^-1 (b - N u) node by node: where b and the neighbours
+    are zero, every step multiplies, whatever range the cell's values have."""
+    rng = np.random.default_rng(p)
+    ctx, nl = dgmg.Context(n, p, _kappa(0, n, rng), basis=basis, omega_dg=0.75), (p + 1) ** len(n)
+    u = torch.zeros(ctx.ndof, dtype=torch.float64, device=DEV)
+    last = slice(ctx.ndof - nl, None)                # the last cell
+    u[last] = _t(_wide(rng, nl))
+    v = u.clone()
+    ctx.smooth(v, torch.zeros_like(u), 1)
+    assert torch.equal(v[last], 0.25 * u[last])
+    if steps > 1:
+        w = u.clone()
+        ctx.smooth(w, torch.zeros_like(u), steps)
+        x = v
+        for _ in range(steps - 1):
+            ctx.smooth(x, torch.zeros_like(u), 1)
+        # traces from the step and from the projection of its result: the same block
+        assert torch.equal(w, x)
