@@ -335,6 +335,56 @@ __device__ __forceinline__ int fx_slab_top(const double *y, int sub) {
     return mx >> 20;
 }
 
+// Unit of the block of the cell's FP64 values y (in the lanes' slabs), from the largest
+// biased exponent of this lane's values; a warp barrier. A cell that looks like zeros may
+// hold subnormal values: their own largest bit decides then.
+template <int DIM, int Q, int SP>
+__device__ __forceinline__ int fx_cell_unit(int mine, const double *y, FxLane &L) {
+    const int top = fx_cell_max<Q * SP>(mine, L);
+    int unit = fx_unit(top);
+    if (__any_sync(0xffffffffu, top == 0)) {
+        int bits = 0;                                    // of the largest subnormal value
+#pragma unroll 1
+        for (int i = L.sub; i < FxGeo<DIM, Q, SP>::N; i += SP) {
+            const int h = fx_abs_hi(y[i]), l = lo_word(y[i]);
+            bits = imax(bits, h != 0 ? 64 - clz32(h) : 32 - clz32(l));
+        }
+        bits = fx_cell_max<Q * SP>(bits, L);
+        if (top == 0 && bits > 0) unit = 1 - FX_UNIT - (53 - bits);
+    }
+    return unit;
+}
+
+// f(std::true_type) where the blocks of all the warp's cells hold normal numbers only, by
+// their exponent e, else f(std::false_type).
+template <typename F>
+__device__ __forceinline__ void fx_by_range(int e, F f) {
+    if (__any_sync(0xffffffffu, !fx_safe(e)))
+        f(std::false_type{});
+    else
+        f(std::true_type{});
+}
+
+// The lane's slab of FP64 values as block values of that unit.
+template <int DIM, int Q, int SP>
+__device__ __forceinline__ void fx_to_block(long long *xs, const double *ys, int unit, const FxLane &L) {
+    constexpr int N = FxGeo<DIM, Q, SP>::N;
+    const int ev = unit + FX_UNIT;
+    if (__any_sync(0xffffffffu, ev < FX_LOW)) {
+#pragma unroll 1
+        for (int i = L.sub; i < N; i += SP) {
+            const long long v = fx_from_any(ys[i], ev);
+            if (L.live) xs[i] = v;
+        }
+        return;
+    }
+#pragma unroll 4
+    for (int i = L.sub; i < N; i += SP) {
+        const long long v = fx_from(ys[i], ev);
+        if (L.live) xs[i] = v;
+    }
+}
+
 // Per cell after the traces {e, h[axis]}: values count 2^e (GL: 2^(e + eV + 64)),
 // derivatives along axis a 2^(e + eT[a] + 64); h packs the unused leading bits (of 60) of
 // the axis' traces, byte 2 side + (0 value, 1 derivative).
@@ -520,13 +570,17 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
             if constexpr (USER) {
                 const double *nb = face(a, f & 1, ((mask >> f) & 1) != 0);
                 int mg = 0, mh = 0;
+                bool sg = false, sh = false;              // some value is not 0 (it may be subnormal)
 #pragma unroll
                 for (int p = 0; p < NP; ++p) {
-                    mg = imax(mg, __ldg(reinterpret_cast<const int *>(nb + p) + 1) & 0x7fffffff);
-                    mh = imax(mh, __ldg(reinterpret_cast<const int *>(nb + G::NF + p) + 1) & 0x7fffffff);
+                    const double g = __ldg(nb + p), h = __ldg(nb + G::NF + p);
+                    mg = imax(mg, fx_abs_hi(g));
+                    mh = imax(mh, fx_abs_hi(h));
+                    sg = sg || fx_some(g);
+                    sh = sh || fx_some(h);
                 }
-                ug[f] = fx_unit(mg >> 20);
-                uh[f] = fx_unit(mh >> 20);
+                ug[f] = fx_unit(imax(mg >> 20, sg ? 1 : 0));
+                uh[f] = fx_unit(imax(mh >> 20, sh ? 1 : 0));
                 rg[f] = rh[f] = 0;
             } else {
                 const int64_t st = a == 0 ? 1 : (a == 1 ? s1 : s2);
@@ -604,15 +658,9 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
         // so the sum over the axes stays below 2^62
         int E = fx_cell_max<Q * SP>(top, L);
         if constexpr (FULL) {
-            const int ev = fx_cell_max<Q * SP>(fx_slab_top<DIM, Q, SP>(ys, L.sub), L);
-            E = imax(E, fx_unit(ev) + ed + 64);
+            E = imax(E, fx_cell_unit<DIM, Q, SP>(fx_slab_top<DIM, Q, SP>(ys, L.sub), ys, L) + ed + 64);
             // u as integers of the unit that makes D u come out in E
-            const int eu = E - ed - 64 + FX_UNIT;
-#pragma unroll 4
-            for (int i = L.sub; i < N; i += SP) {
-                const long long v = fx_from(ys[i], eu);
-                if (L.live) reinterpret_cast<long long *>(ys)[i] = v;
-            }
+            fx_to_block<DIM, Q, SP>(reinterpret_cast<long long *>(ys), ys, E - ed - 64, L);
             __syncwarp();
         }
         FxMag mag;
@@ -649,7 +697,7 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
 #pragma unroll
                     for (int c = 0; c < 2; ++c) {
                         const double w = __ldg(nb[s] + c * G::NF + p);
-                        const long long v = USER ? fx_from(w, ev[s][c])
+                        const long long v = USER ? fx_from_any(w, ev[s][c])
                                                  : (__double_as_longlong(w) << imax(-ev[s][c], 0)) >> imax(ev[s][c], 0);
                         g[s][c] = limb_of(in[s] ? v : 0ll);
                     }
@@ -704,25 +752,29 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
     // The residual on its way out keeps the bits of b: a subtraction in FP64 per node. (As
     // a block it has those of the cell's largest value, so that u = 0 did not give b back.)
     const bool write_r = !SMOOTH && has_b && (mode & RES_WRITE_R) != 0;
-    auto difference = [&](double bi, long long ti) {
-        const double w = fx_to(ti, t.e);
-        return mode & RES_NEGATE ? w - bi : bi - w;
-    };
+    auto difference = [&](double bi, double w) { return mode & RES_NEGATE ? w - bi : bi - w; };
     auto subtract_from_b = [&]() {                        // t = A u (or its neighbours' part); in the lane's slab
         fx_cp_wait();
         __syncwarp();
-        const int te = t.e - t.n, E = imax(fx_unit(fx_cell_max<Q * SP>(fx_slab_top<DIM, Q, SP>(ys, L.sub), L)), te) + 1;
+        const int tb = fx_cell_unit<DIM, Q, SP>(fx_slab_top<DIM, Q, SP>(ys, L.sub), ys, L);
+        const int te = t.e - t.n, E = imax(tb, te) + 1;
         const int ev = E + FX_UNIT;
         FxMag mag;
-#pragma unroll 4
-        for (int i = L.sub; i < N; i += SP) {
-            const double bi = ys[i];
-            const long long ti = xs[i], v = fx_from(bi, ev) - (zero ? 0 : fx_shr(ti << t.n, E - te));
+        auto at = [&](int i, long long v) {               // v: b as a block value
+            const long long ti = xs[i];
+            if (!zero) v -= fx_shr(ti << t.n, E - te);
             if (G::ALL || L.live) {
                 xs[i] = v;
-                if (write_r) ys[i] = difference(bi, ti);
+                if (write_r) ys[i] = difference(ys[i], fx_to(ti, te + t.n));
             }
             mag.add(v);
+        };
+        if (__any_sync(0xffffffffu, ev < FX_LOW)) {
+#pragma unroll 1
+            for (int i = L.sub; i < N; i += SP) at(i, fx_from_any(ys[i], ev));
+        } else {
+#pragma unroll 4
+            for (int i = L.sub; i < N; i += SP) at(i, fx_from(ys[i], ev));
         }
         t = fx_block<Q * SP>(mag, E, L);
     };
@@ -766,11 +818,13 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
         } else {
             fx_cp_wait();
             __syncwarp();
+            fx_by_range(t.e, [&](auto safe) {
 #pragma unroll 4
-            for (int i = L.sub; i < N; i += SP) {
-                const double v = difference(ys[i], xs[i]);
-                if (L.live) ys[i] = v;
-            }
+                for (int i = L.sub; i < N; i += SP) {
+                    const double v = difference(ys[i], fx_to<decltype(safe)::value>(xs[i], t.e));
+                    if (L.live) ys[i] = v;
+                }
+            });
         }
     }
     const bool traces = SMOOTH && !(flags & SM_NO_TRACES);
@@ -783,20 +837,18 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
             fx_cp_wait();
             __syncwarp();
             int top = 0;
-#pragma unroll 4
-            for (int i = L.sub; i < N; i += SP) {
-                const double v = fma(cst.keep, ys[i], fx_to(xs[i], t.e));
-                if (L.live) ys[i] = v;
-                top = imax(top, fx_abs_hi(v));
-            }
-            in_y = true;
-            if (traces) {
-                t = FxBlock{fx_unit(fx_cell_max<Q * SP>(top >> 20, L)), 0};
+            fx_by_range(t.e, [&](auto safe) {
 #pragma unroll 4
                 for (int i = L.sub; i < N; i += SP) {
-                    const long long v = fx_from(ys[i], t.e + FX_UNIT);
-                    if (G::ALL || L.live) xs[i] = v;
+                    const double v = fma(cst.keep, ys[i], fx_to<decltype(safe)::value>(xs[i], t.e));
+                    if (L.live) ys[i] = v;
+                    top = imax(top, fx_abs_hi(v));
                 }
+            });
+            in_y = true;
+            if (traces) {
+                t = FxBlock{fx_cell_unit<DIM, Q, SP>(top >> 20, ys, L), 0};
+                fx_to_block<DIM, Q, SP>(xs, ys, t.e, L);
             }
         }
     }
@@ -804,13 +856,14 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
     if (SMOOTH || (mode & RES_WRITE_R)) {
         // without b the block is A u: the residual b - A u is its negative
         const bool neg = !SMOOTH && !(mode & RES_NEGATE);
-        if (!in_y) {
+        if (!in_y)
+            fx_by_range(t.e, [&](auto safe) {
 #pragma unroll 4
-            for (int i = L.sub; i < N; i += SP) {
-                const double v = fx_to(neg ? -xs[i] : xs[i], t.e);
-                if (L.live) ys[i] = v;
-            }
-        }
+                for (int i = L.sub; i < N; i += SP) {
+                    const double v = fx_to<decltype(safe)::value>(neg ? -xs[i] : xs[i], t.e);
+                    if (L.live) ys[i] = v;
+                }
+            });
         __syncwarp();
         fx_store_out<DIM, Q, SP>((SMOOTH ? u : r) + cell0 * NL, reinterpret_cast<const double *>(Y), ncl * NL, L.lane);
     }
@@ -985,9 +1038,13 @@ __device__ __forceinline__ void fx_project_body(const FxTab &tab, const FxConst 
     int top = 0;                                          // of the new u, by its high words
     if (e0) {
         int mx = 0;
+        bool some = false;
 #pragma unroll
-        for (int c = 0; c < G::NC; ++c) mx = imax(mx, fx_abs_hi(ec[c]));
-        const int ev = mx >> 20;
+        for (int c = 0; c < G::NC; ++c) {
+            mx = imax(mx, fx_abs_hi(ec[c]));
+            some = some || fx_some(ec[c]);
+        }
+        const int ev = imax(mx >> 20, some ? 1 : 0);
         int ee = fx_unit(ev);
         constexpr int NH = G::NC / 2;
         long long z[NH];                                  // corners of the slab: the last axis interpolated at k
@@ -996,8 +1053,8 @@ __device__ __forceinline__ void fx_project_body(const FxTab &tab, const FxConst 
         for (int c = 0; c < NH; ++c) {
             Acc s;
             acc_zero(s);
-            mac(s, tab.hat[0][L.k], limb_of(fx_from(ec[c], ev)));
-            mac(s, tab.hat[1][L.k], limb_of(fx_from(ec[c + NH], ev)));
+            mac(s, tab.hat[0][L.k], limb_of(fx_from_any(ec[c], ev)));
+            mac(s, tab.hat[1][L.k], limb_of(fx_from_any(ec[c + NH], ev)));
             z[c] = acc_value(s);
             mag.add(z[c]);
         }
@@ -1035,16 +1092,10 @@ __device__ __forceinline__ void fx_project_body(const FxTab &tab, const FxConst 
     } else {
         top = fx_slab_top<DIM, Q, SP>(ys, L.sub);
     }
-    top = fx_cell_max<Q * SP>(top, L);
+    const FxBlock t{fx_cell_unit<DIM, Q, SP>(top, ys, L), 0};
     if (e0) fx_store_out<DIM, Q, SP>(u + cell0 * NL, reinterpret_cast<const double *>(Y), ncl * NL, L.lane);
-    const int eu = fx_unit(top);
-#pragma unroll 4
-    for (int i = L.sub; i < N; i += SP) {
-        const long long v = fx_from(ys[i], eu + FX_UNIT);
-        if (L.live) xs[i] = v;
-    }
+    fx_to_block<DIM, Q, SP>(xs, ys, t.e, L);
     __syncwarp();
-    const FxBlock t{eu, 0};
     fx_all_traces<DIM, Q, SP, USER>(tab, cst, xc, t, L, active, cell, tr,
                                     reinterpret_cast<const double *>(Y + L.c * G::C));
 }

@@ -17,8 +17,9 @@
 // (the reference's own rounding).
 //
 // An input that is not finite marks its block (e >= FX_BAD), and every value
-// computed from a marked block is output as NaN. Subnormal inputs count as 0,
-// results below the normal range are output as 0, above it as infinity.
+// computed from a marked block is output as NaN. Results above the normal range are
+// output as infinity, below it as subnormal numbers, and subnormal inputs count as what
+// they are.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -112,9 +113,11 @@ FX_HD int imin(int a, int b) { return a < b ? a : b; }
 
 // Largest biased exponent of a block of FP64 values: mx over fx_abs_hi, >> 20.
 FX_HD int fx_abs_hi(double v) { return hi_word(v) & 0x7fffffff; }
+FX_HD bool fx_some(double v) { return (fx_abs_hi(v) | lo_word(v)) != 0; }   // not 0
 
-// FP64 value as a block value of unit 2^(ev - FX_UNIT); ev >= its biased exponent.
-constexpr int FX_UNIT = 1023 + 59;
+// FP64 value as a block value of unit 2^(ev - FX_UNIT); ev >= its biased exponent, and at
+// least FX_LOW (subnormal values are below the unit then).
+constexpr int FX_UNIT = 1023 + 59, FX_LOW = 61;
 FX_HD long long fx_from(double v, int ev) {
     const int hi = hi_word(v), lo = lo_word(v);
     const int e = (hi >> 20) & 0x7ff, d = imin(ev - e, 63);      // the significand ends at bit 59: d >= 60 gives 0
@@ -123,10 +126,23 @@ FX_HD long long fx_from(double v, int ev) {
     const long long s = hi >> 31;
     return (m ^ s) - s;
 }
+// The same for every ev, below 1 (a block of subnormal values) too.
+FX_HD long long fx_from_any(double v, int ev) {
+    const int hi = hi_word(v), lo = lo_word(v), e = (hi >> 20) & 0x7ff, d = ev - imax(e, 1);
+    const unsigned top = (unsigned)(hi & 0xfffff) | (e ? 0x100000u : 0u);
+    const unsigned long long x = ((unsigned long long)top << 32 | (unsigned)lo) << 7;
+    const long long m = (long long)(d >= 0 ? x >> imin(d, 63) : x << imin(-d, 63)), s = hi >> 31;
+    return (m ^ s) - s;
+}
 // exponent (unit) of a block whose largest biased exponent is ev
 FX_HD int fx_unit(int ev) { return ev >= 2047 ? 2 * FX_BAD : (ev <= 0 ? FX_NONE : ev - FX_UNIT); }
 
-// Block value t 2^e as FP64, rounded to nearest (ties away from zero).
+// Block value t 2^e as FP64, rounded to nearest (ties away from zero). SAFE: every value of
+// the block is 0 or in the normal range (fx_safe), as nearly always: without the look at the
+// range, which costs more than its instructions (operator 64 x 60 x 57 p = 4 1142 us without
+// subnormal results, 1169 with their code behind every value, 1131 with the look by blocks).
+FX_HD bool fx_safe(int e) { return (unsigned)(e + 1022) <= 1900u; }
+template <bool SAFE = false>
 FX_HD double fx_to(long long t, int e) {
     const int s = (int)(t >> 63);
     unsigned long long a = (unsigned long long)((t ^ (long long)s) - (long long)s);
@@ -138,10 +154,17 @@ FX_HD double fx_to(long long t, int e) {
     a = (a << (n & 63)) + 512;
     const int be = e - n + 62 + 1023;            // biased exponent of bit 62
     int hi = ((int)(a >> 42) + ((be - 1) << 20)) | (s & (int)0x80000000), lo = (int)(unsigned)(a >> 10);
-    if ((unsigned)(be - 1) >= 2046u || t == 0) { // rare: outside the normal range
+    if (t == 0) hi = lo = 0;
+    if (!SAFE && ((unsigned)(be - 1) >= 2046u || (t == 0 && e >= FX_BAD - 64))) {
+        hi = 0x7ff00000 | (s & (int)0x80000000);
         lo = 0;
-        hi = (be < 1 || t == 0) ? 0 : (0x7ff00000 | (s & (int)0x80000000));
-        if (e >= FX_BAD) hi = 0x7ff80000;
+        if (t == 0 || be < 1) {                  // subnormal: fewer bits of the significand
+            const int d = imin(11 - be, 63);     // (63: half the least number)
+            a = t == 0 || be < -52 ? 0 : (a - 512 + (1ull << (d - 1))) >> d;
+            hi = (int)(a >> 32) | (s & (int)0x80000000);
+            lo = (int)(unsigned)a;
+        }
+        if (e >= FX_BAD - 64) hi = 0x7ff80000, lo = 0;
     }
     return from_words(hi, lo);
 }

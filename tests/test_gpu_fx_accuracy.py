@@ -144,3 +144,41 @@ def test_smoothing_keeps_the_bits_of_u(dgmg, n, p, basis, steps):
             ctx.smooth(x, torch.zeros_like(u), 1)
         # traces from the step and from the projection of its result: the same block
         assert torch.equal(w, x)
+
+
+@pytest.mark.parametrize("n,p,basis", MESHES)
+@pytest.mark.parametrize("scale", [-1015, -1020, -1030, -1050])
+def test_values_below_the_normal_range(dgmg, n, p, basis, scale):
+    """Residual, step and projection of values around and below 2^-1022: the relative bounds
+    of the normal range (the residual: sums of 4 d + 2 terms per pass, d + 1 passes of q
+    products) and the spacing of subnormal numbers, once per result and once per trace value
+    that the caller reads and hands on."""
+    rng = np.random.default_rng(p)
+    d, q = len(n), p + 1
+    kap = _kappa(0, n, rng)
+    ref, ctx = Reference(n, p, kap, basis), dgmg.Context(n, p, kap, basis=basis)
+    tiny = float(np.finfo(np.float64).smallest_subnormal)
+    u, b = rng.normal(size=(2, ctx.ndof)) * 2.0 ** scale
+    r = torch.empty(ctx.ndof, dtype=torch.float64, device=DEV)
+    ctx.residual(_t(u), _t(b), r)
+    exact = ref.residual(u, b)
+    size = float(np.abs(exact).max())
+
+    def err(x, y):
+        return float(np.abs(x.cpu().numpy().astype(L).reshape(y.shape) - y).max())
+
+    assert err(r, exact) <= 2 * (d + 1) * q * EPS * size + tiny
+    v = _t(u)
+    ctx.smooth(v, _t(b), 1)
+    exact = ref.step(u, b, 0.8)
+    assert err(v, exact) <= 2 * 3 * d * q * EPS * float(np.abs(exact).max()) + tiny
+    e = torch.zeros(int(ctx.info.nvert0), dtype=torch.float64, device=DEV)
+    e[0] = 2.0 ** scale
+    w, tr = _t(0 * u), torch.empty(ctx.trace_size(), dtype=torch.float64, device=DEV)
+    ctx.project(w, e, tr)
+    assert abs(float(w.max()) / tiny - 2.0 ** (scale + 1074)) <= (0 if basis == 0 else 2.0 ** (scale + 1074))
+    z = torch.zeros_like(w)
+    ctx.residual_restrict(z, z, tr, r, None)         # the traces alone: - A w without the cells' own blocks
+    full = -(ref.apply(w.cpu().numpy()) - ref.apply(w.cpu().numpy(), own=True))
+    gain = float(np.abs(ref.apply(np.ones(ctx.ndof))).max()) * 4 * d * q
+    assert err(r, full) <= 2 * (d + 1) * q * EPS * float(np.abs(full).max()) + (1 + gain) * tiny
