@@ -128,7 +128,8 @@ __global__ void __launch_bounds__(128) k_fd_factors(const __grid_constant__ FDIn
 
 // Largest exponent of an entry omega / (sum of eigenvalues) of a cell's table, from the
 // smallest eigenvalue of every axis (rounding can leave one that is not positive where kappa
-// jumps by 1e16: then from every sum); one thread per cell
+// jumps by 1e16: then from every sum); one thread per cell. A cell whose entries are not all
+// finite is marked: its steps give NaN.
 __global__ void k_fx_table_unit(int dim, int q, int64_t ncell, const double *__restrict__ fd, double omega,
                                 int *__restrict__ unit) {
     const int64_t cell = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -136,10 +137,13 @@ __global__ void k_fx_table_unit(int dim, int q, int64_t ncell, const double *__r
     const int fds = q * q + q;
     const double *f = fd + cell * dim * fds + q * q;
     double s = 0.0;
-    bool positive = true;
+    bool positive = true, finite = true;
     for (int a = 0; a < dim; ++a) {
         double m = f[a * fds];
-        for (int i = 1; i < q; ++i) m = fmin(m, f[a * fds + i]);
+        for (int i = 0; i < q; ++i) {
+            m = fmin(m, f[a * fds + i]);
+            finite = finite && isfinite(f[a * fds + i]);
+        }
         positive = positive && m > 0.0;
         s += m;
     }
@@ -150,7 +154,7 @@ __global__ void k_fx_table_unit(int dim, int q, int64_t ncell, const double *__r
             s = i == 0 || fabs(t) < fabs(s) ? t : s;
         }
     const double top = omega / fabs(s);
-    unit[cell] = isfinite(top) && top > 0.0 ? ilogb(top) : 0;
+    unit[cell] = finite && isfinite(top) && top > 0.0 ? ilogb(top) : 2 * FX_BAD;
 }
 
 // The inverse eigenvalue sums of every cell with the smoother's damping folded in
@@ -169,13 +173,14 @@ __global__ void k_fx_table(int dim, int q, int64_t ncell, const double *__restri
 
 // fd in place: S of every axis as limbs of one unit (every row and column sum of
 // the magnitudes below 2^63, an h below 2^31), the unit in the word after it, and in the word after
-// axis 0's the exponent of the table; one thread per cell and axis
+// axis 0's the exponent of the table; one thread per cell and axis. What is not finite marks
+// the unit.
 __global__ void k_fx_factors(int dim, int q, int64_t ncell, double *__restrict__ fd, const int *__restrict__ unit) {
     const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (id >= ncell * dim) return;
     double *S = fd + id * (q * q + q);
     Limb *out = reinterpret_cast<Limb *>(S);
-    double top = 0.0;
+    double top = 0.0, all = 0.0;
     for (int i = 0; i < q; ++i) {
         double rs = 0.0, cs = 0.0;
         for (int j = 0; j < q; ++j) {
@@ -183,8 +188,9 @@ __global__ void k_fx_factors(int dim, int q, int64_t ncell, double *__restrict__
             cs += fabs(S[j * q + i]);
         }
         top = fmax(top, fmax(rs, cs));
+        all += rs;
     }
-    const int ev = ilogb(top * (1.0 + 0x1p-30)) + 1023;
+    const int ev = isfinite(all) ? ilogb(top * (1.0 + 0x1p-30)) + 1023 : 2047;
     for (int i = 0; i < q * q; ++i) out[i] = limb_of(fx_from(S[i], ev) << 3);
     out[q * q] = Limb{fx_unit(ev) - 3, 0};
     if (id % dim == 0) out[q * q + 1] = Limb{unit[id / dim] + FX_SCALED, 0};

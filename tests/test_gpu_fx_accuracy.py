@@ -182,3 +182,16 @@ def test_values_below_the_normal_range(dgmg, n, p, basis, scale):
     full = -(ref.apply(w.cpu().numpy()) - ref.apply(w.cpu().numpy(), own=True))
     gain = float(np.abs(ref.apply(np.ones(ctx.ndof))).max()) * 4 * d * q
     assert err(r, full) <= 2 * (d + 1) * q * EPS * float(np.abs(full).max()) + (1 + gain) * tiny
+
+
+@pytest.mark.parametrize("n,p", [((4, 3), 2), ((4, 3, 2), 1), ((3, 3, 3), 4)])
+def test_factors_that_are_not_finite(dgmg, n, p):
+    """Coefficients whose blocks overflow leave no numbers that look like a result."""
+    ctx = dgmg.Context(n, p, np.full(int(np.prod(n)), 1e300))
+    b = torch.randn(ctx.ndof, dtype=torch.float64, device=DEV, generator=torch.Generator(DEV).manual_seed(1))
+    for u in (b.clone(), torch.zeros_like(b)):
+        ctx.smooth(u, b, 1)
+        assert torch.isnan(u).all()
+    e = torch.zeros_like(b)
+    ctx.vcycle(b, e)
+    assert torch.isnan(e).all()
