@@ -434,7 +434,7 @@ int finish_factors(dgmg_ctx &C, const DGSpace &S, DGDev<double> &D, cudaStream_t
 // input as at set-up; the residual's factors stay the set-up ones.
 template <typename T>
 int recompute_factors(dgmg_ctx &C, const DGSpace &S, DGDev<T> &D, cudaStream_t s) {
-    if (!D.fd || S.fdin.dim == 0) return DGMG_OK;   // no input kept for this level: the set-up factors stay
+    if (!D.fd || S.fdin.dim == 0) return fail(DGMG_EINVAL, "recompute_block: the level's factor input is missing");
     LC(launch_fd_factors<T>(S.fdin, C.d64.kappa, C.ncell, D.fd, s));
     if constexpr (std::is_same<T, double>::value) RC(finish_factors(C, S, D, s));
     return DGMG_OK;
@@ -491,10 +491,9 @@ int setup_dg(dgmg_ctx &C, const DGSpace &S, DGDev<T> &D, const std::vector<doubl
 // The lower DG levels of a gradual p-hierarchy (degrees p-1 .. 1, finest
 // penalty): fast-diagonalisation factors, constants, traces, the level's
 // vectors and the interpolation up to the next finer level, in FP64 and (mixed
-// precision) FP32; the finest residual scratch. dgs[0] (the finest space) is
-// always set.
+// precision) FP32; the finest residual scratch. dgs[0] (the finest space, with the
+// input of its factors) is set.
 int setup_dg_levels(dgmg_ctx &C, const std::vector<double> &kap) {
-    C.dgs.assign(1, finest_space(C));
     if (C.opts.p_coarsening == 0 || C.p < 2) return DGMG_OK;
     const bool mixed = C.opts.precision == DGMG_MIXED_FP32;
     for (int pc = C.p - 1; pc >= 1; --pc) {
@@ -1272,7 +1271,8 @@ int create_ctx(const dgmg_mesh *mesh, int p, const double *kappa, const dgmg_opt
     }
     trace.mark("coarse inverse");
 
-    const DGSpace S0 = finest_space(*C);
+    C->dgs.assign(1, finest_space(*C));
+    const DGSpace &S0 = C->dgs[0];                        // (until setup_dg_levels adds to them)
     RC(setup_dg<double>(*C, S0, C->d64, kap, !(flags & CREATE_NO_FP64_SMOOTHER)));
     trace.mark("dg fp64 (factors on the device)");
     if (!(flags & CREATE_NO_SOLVER)) {   // a batch member runs its Q1 levels in the batch's kernels
