@@ -421,7 +421,11 @@ template <typename T>
 int build_block_map(dgmg_batch &B, dgmg_batch::Group &grp, int stage) {
     auto &g = grp.prec<T>();
     const int nf = (int)(B.inst[grp.members[0]]->nloc / grp.q);
-    if (std::is_same<T, double>::value) g.tile[stage] = fx_cells_per_cta(B.dim, grp.q);
+    if (std::is_same<T, double>::value) {
+        int64_t cells = 0;
+        for (int i : grp.members) cells += B.inst[i]->ncell;
+        g.tile[stage] = fx_cells_per_cta(B.dim, grp.q, cells);
+    }
     int tile = g.tile[stage];
     if (tile <= 0) {
         // the one-thread-per-cell kernel where it applies, else ~128 threads

@@ -1244,7 +1244,7 @@ int create_ctx(const dgmg_mesh *mesh, int p, const double *kappa, const dgmg_opt
     const int nf = (int)(C->nloc / C->q);
     C->cpb = std::max(1, 256 / nf);   // per-pencil tile: as many cells as fit 256 threads
     for (int st = 0; st < 3; ++st) C->tile[1][st] = C->cpb;
-    for (int st = 0; st < 3; ++st) C->tile[0][st] = fx_cells_per_cta(C->dim, C->q);
+    for (int st = 0; st < 3; ++st) C->tile[0][st] = fx_cells_per_cta(C->dim, C->q, C->ncell);
     C->tile[1][TILE_PROJECT] = 0;   // the one-thread-per-cell kernels where they apply
     C->tile[1][TILE_SMOOTH] = 0;
     C->tile[1][TILE_RESIDUAL] = 0;

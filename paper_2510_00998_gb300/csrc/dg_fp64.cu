@@ -42,8 +42,8 @@ const FxTab &batch_tables(int q) {
 
 }  // namespace
 
-int fx_cells_per_cta(int dim, int q) {
-    return fx_dispatch(dim, q, [](auto run) { return decltype(run)::cells_per_cta(); });
+int fx_cells_per_cta(int dim, int q, int64_t ncell) {
+    return fx_dispatch(dim, q, [&](auto run) { return decltype(run)::cells_per_cta(ncell); });
 }
 
 template <>
@@ -85,27 +85,27 @@ cudaError_t launch_residual_user(int dim, int q, const DGConst<double> &c, int m
 
 template <>
 cudaError_t launch_project_batch<double>(int dim, int q, const BatchDG<double> *D, const BlockMap *map, int nblocks,
-                                         int, double *u, int with_e0, cudaStream_t s) {
+                                         int cpb, double *u, int with_e0, cudaStream_t s) {
     if (!fx_valid(dim, q)) return cudaErrorInvalidValue;
     return fx_dispatch(dim, q, [&](auto run) {
-        return decltype(run)::project_batch(batch_tables(q), D, map, nblocks, u, with_e0, s);
+        return decltype(run)::project_batch(batch_tables(q), cpb, D, map, nblocks, u, with_e0, s);
     });
 }
 template <>
-cudaError_t launch_smooth_batch<double>(int dim, int q, const BatchDG<double> *D, const BlockMap *map, int nblocks, int,
+cudaError_t launch_smooth_batch<double>(int dim, int q, const BatchDG<double> *D, const BlockMap *map, int nblocks, int cpb,
                                         int exact, int flags, double *u, const double *b, int cur, cudaStream_t s) {
     if (!fx_valid(dim, q)) return cudaErrorInvalidValue;
     return fx_dispatch(dim, q, [&](auto run) {
-        return decltype(run)::smooth_batch(batch_tables(q), exact != 0, D, map, nblocks, flags, u, b, cur, s);
+        return decltype(run)::smooth_batch(batch_tables(q), cpb, exact != 0, D, map, nblocks, flags, u, b, cur, s);
     });
 }
 template <>
 cudaError_t launch_residual_batch<double>(int dim, int q, const BatchDG<double> *D, const BlockMap *map, int nblocks,
-                                          int, int mode, const double *u, const double *b, double *r, int cur,
+                                          int cpb, int mode, const double *u, const double *b, double *r, int cur,
                                           cudaStream_t s) {
     if (!fx_valid(dim, q)) return cudaErrorInvalidValue;
     return fx_dispatch(dim, q, [&](auto run) {
-        return decltype(run)::residual_batch(batch_tables(q), D, map, nblocks, mode, u, b, r, cur, s);
+        return decltype(run)::residual_batch(batch_tables(q), cpb, D, map, nblocks, mode, u, b, r, cur, s);
     });
 }
 

@@ -1142,7 +1142,8 @@ inline void fx_allow_smem(K *kernel, size_t bytes) {      // beside the static d
 // steps, one lane / split: q = 5, 576 cells 37 and 154 / 20 and 70 us, 2197 cells 37 and
 // 154 / 35 and 109, 3375 cells 37 and 154 / 41 and 154; q = 6 576 cells 49 and 197 / 27 and
 // 103, 2744 cells 50 and 204 / 70 and 239 (its second round of pencils is nearly empty);
-// q = 7 512 cells 58 and 263 / 29 and 113, 2197 cells 62 and 271 / 58 and 251.
+// q = 7 512 cells 58 and 263 / 29 and 113, 2197 cells 62 and 271 / 58 and 251. In a batch the
+// cells of all problems of a degree count (they share the launch).
 template <int DIM, int Q>
 constexpr int fx_split() {
     return DIM == 3 && Q >= 5 ? (Q == 5 ? 5 : 32 / Q) : 1;
@@ -1176,18 +1177,30 @@ cudaError_t fx_run_cells(const FxLevel &l, int flags, int mode, double *u, const
     return fx_run_cells_of<DIM, Q, 1, MODE>(l, flags, mode, u, b, kappa, fd, linv, tri, tro, r, corners, s);
 }
 
+// f(lanes per slab) of the work items of cpb cells (those of one lane where there is no split)
+template <int DIM, int Q, typename F>
+cudaError_t fx_batch_split(int cpb, F f) {
+    constexpr int SP = fx_split<DIM, Q>();
+    if (SP > 1 && cpb == FxGeo<DIM, Q, SP>::CPB) return f(std::integral_constant<int, SP>{});
+    if (cpb == FxGeo<DIM, Q, 1>::CPB) return f(std::integral_constant<int, 1>{});
+    return cudaErrorInvalidValue;
+}
+
 template <int DIM, int Q, int MODE>
-cudaError_t fx_run_cells_batch(const FxTab &tab, const BatchDG<double> *D, const BlockMap *map, int nblocks, int flags,
-                               int mode, double *u, const double *b, double *r, int cur, cudaStream_t s) {
-    using G = FxGeo<DIM, Q>;
+cudaError_t fx_run_cells_batch(const FxTab &tab, int cpb, const BatchDG<double> *D, const BlockMap *map, int nblocks,
+                               int flags, int mode, double *u, const double *b, double *r, int cur, cudaStream_t s) {
     if (nblocks <= 0) return cudaSuccess;
-    const size_t sm = G::bytes(MODE);
-    fx_allow_smem(k_fx_cells_batch<DIM, Q, 1, MODE>, sm);
-    count_launches(1);
-    k_fx_cells_batch<DIM, Q, 1, MODE>
-        <<<persistent_grid((const void *)k_fx_cells_batch<DIM, Q, 1, MODE>, G::NW * 32, sm, nblocks), G::NW * 32, sm, s>>>(
-            tab, D, map, nblocks, flags, mode, u, b, r, cur);
-    return cudaGetLastError();
+    return fx_batch_split<DIM, Q>(cpb, [&](auto split) -> cudaError_t {
+        constexpr int SP = decltype(split)::value;
+        using G = FxGeo<DIM, Q, SP>;
+        const size_t sm = G::bytes(MODE);
+        const auto fn = k_fx_cells_batch<DIM, Q, SP, MODE>;
+        fx_allow_smem(fn, sm);
+        count_launches(1);
+        fn<<<persistent_grid((const void *)fn, G::NW * 32, sm, nblocks), G::NW * 32, sm, s>>>(tab, D, map, nblocks, flags,
+                                                                                           mode, u, b, r, cur);
+        return cudaGetLastError();
+    });
 }
 
 template <int DIM, int Q>
@@ -1224,35 +1237,39 @@ cudaError_t FxRun<DIM, Q>::residual(const FxLevel &l, bool user, int mode, const
                                               nullptr, r, corners, s);
 }
 template <int DIM, int Q>
-cudaError_t FxRun<DIM, Q>::project_batch(const FxTab &tab, const BatchDG<double> *D, const BlockMap *map, int nblocks,
-                                         double *u, int with_e0, cudaStream_t s) {
-    using G = FxGeo<DIM, Q>;
+cudaError_t FxRun<DIM, Q>::project_batch(const FxTab &tab, int cpb, const BatchDG<double> *D, const BlockMap *map,
+                                         int nblocks, double *u, int with_e0, cudaStream_t s) {
     if (nblocks <= 0) return cudaSuccess;
-    const size_t sm = G::bytes_project();
-    fx_allow_smem(k_fx_project_batch<DIM, Q, 1>, sm);
-    count_launches(1);
-    k_fx_project_batch<DIM, Q, 1>
-        <<<persistent_grid((const void *)k_fx_project_batch<DIM, Q, 1>, G::NW * 32, sm, nblocks), G::NW * 32, sm, s>>>(
-            tab, D, map, nblocks, u, with_e0);
-    return cudaGetLastError();
+    return fx_batch_split<DIM, Q>(cpb, [&](auto split) -> cudaError_t {
+        constexpr int SP = decltype(split)::value;
+        using G = FxGeo<DIM, Q, SP>;
+        const size_t sm = G::bytes_project();
+        const auto fn = k_fx_project_batch<DIM, Q, SP>;
+        fx_allow_smem(fn, sm);
+        count_launches(1);
+        fn<<<persistent_grid((const void *)fn, G::NW * 32, sm, nblocks), G::NW * 32, sm, s>>>(tab, D, map, nblocks, u,
+                                                                                           with_e0);
+        return cudaGetLastError();
+    });
 }
 template <int DIM, int Q>
-cudaError_t FxRun<DIM, Q>::smooth_batch(const FxTab &tab, bool exact, const BatchDG<double> *D, const BlockMap *map,
-                                        int nblocks, int flags, double *u, const double *b, int cur, cudaStream_t s) {
+cudaError_t FxRun<DIM, Q>::smooth_batch(const FxTab &tab, int cpb, bool exact, const BatchDG<double> *D,
+                                        const BlockMap *map, int nblocks, int flags, double *u, const double *b, int cur,
+                                        cudaStream_t s) {
     if (exact)
-        return fx_run_cells_batch<DIM, Q, FXM_SMOOTH>(tab, D, map, nblocks, flags, 0, u, b, nullptr, cur, s);
-    return fx_run_cells_batch<DIM, Q, FXM_SMOOTH_FULL>(tab, D, map, nblocks, flags, 0, u, b, nullptr, cur, s);
+        return fx_run_cells_batch<DIM, Q, FXM_SMOOTH>(tab, cpb, D, map, nblocks, flags, 0, u, b, nullptr, cur, s);
+    return fx_run_cells_batch<DIM, Q, FXM_SMOOTH_FULL>(tab, cpb, D, map, nblocks, flags, 0, u, b, nullptr, cur, s);
 }
 template <int DIM, int Q>
-cudaError_t FxRun<DIM, Q>::residual_batch(const FxTab &tab, const BatchDG<double> *D, const BlockMap *map, int nblocks,
-                                          int mode, const double *u, const double *b, double *r, int cur,
+cudaError_t FxRun<DIM, Q>::residual_batch(const FxTab &tab, int cpb, const BatchDG<double> *D, const BlockMap *map,
+                                          int nblocks, int mode, const double *u, const double *b, double *r, int cur,
                                           cudaStream_t s) {
-    return fx_run_cells_batch<DIM, Q, FXM_RESIDUAL>(tab, D, map, nblocks, 0, mode, const_cast<double *>(u), b, r, cur,
-                                                    s);
+    return fx_run_cells_batch<DIM, Q, FXM_RESIDUAL>(tab, cpb, D, map, nblocks, 0, mode, const_cast<double *>(u), b, r,
+                                                    cur, s);
 }
 template <int DIM, int Q>
-int FxRun<DIM, Q>::cells_per_cta() {
-    return FxGeo<DIM, Q>::CPB;
+int FxRun<DIM, Q>::cells_per_cta(int64_t ncell) {
+    return fx_small<DIM, Q>(ncell) ? FxGeo<DIM, Q, fx_split<DIM, Q>()>::CPB : FxGeo<DIM, Q>::CPB;
 }
 
 }  // namespace dgmg

@@ -167,8 +167,8 @@ struct DGConst<double> : FxLevel {};
 void fx_tables(const RefElem1D &re, int penalty_p, FxTab &tab);
 // mesh-dependent vectors; keep = 1 - omega (exact blocks) or 1
 void fx_level(const RefElem1D &re, int penalty_p, int dim, const int *n, int64_t ncell, double keep, FxConst &cst);
-// cells of one work item of the FP64 kernels
-int fx_cells_per_cta(int dim, int q);
+// cells of one work item of the FP64 kernels on ncell cells (of all problems of a launch)
+int fx_cells_per_cta(int dim, int q, int64_t ncell);
 template <typename T>
 struct BatchDG;
 struct BlockMap;
@@ -181,13 +181,14 @@ struct FxRun {
                               const double *fd, const double *linv, const double *tri, double *tro, cudaStream_t s);
     static cudaError_t residual(const FxLevel &l, bool user, int mode, const double *u, const double *b,
                                 const double *kappa, const double *tr, double *r, double *corners, cudaStream_t s);
-    static cudaError_t project_batch(const FxTab &tab, const BatchDG<double> *D, const BlockMap *map, int nblocks,
+    // cpb: cells of a work item of the map, as cells_per_cta gave them
+    static cudaError_t project_batch(const FxTab &tab, int cpb, const BatchDG<double> *D, const BlockMap *map, int nblocks,
                                      double *u, int with_e0, cudaStream_t s);
-    static cudaError_t smooth_batch(const FxTab &tab, bool exact, const BatchDG<double> *D, const BlockMap *map,
+    static cudaError_t smooth_batch(const FxTab &tab, int cpb, bool exact, const BatchDG<double> *D, const BlockMap *map,
                                     int nblocks, int flags, double *u, const double *b, int cur, cudaStream_t s);
-    static cudaError_t residual_batch(const FxTab &tab, const BatchDG<double> *D, const BlockMap *map, int nblocks,
+    static cudaError_t residual_batch(const FxTab &tab, int cpb, const BatchDG<double> *D, const BlockMap *map, int nblocks,
                                       int mode, const double *u, const double *b, double *r, int cur, cudaStream_t s);
-    static int cells_per_cta();
+    static int cells_per_cta(int64_t ncell);
 };
 // linv[cell][node] = omega / (sum of the cell's eigenvalues) as words of a table (fx.cuh),
 // from the FP64 factors [S | lambda]; then, in place, the factors as limbs: per axis S, its
