@@ -25,12 +25,15 @@
 // d q multiply-adds per node for M instead of two tangential masses per face and
 // field, and no mass at all in the first step from a zero iterate.
 //
-// What bounds it: the integer multiply-add pipe (59% busy at q = 4 with a last wave of
+// Numbers: a pass rounds to the block's unit, node-wise sums with the caller's vectors (b, u)
+// are FP64 (their pipe is idle otherwise: 5% busy).
+//
+// What bounds it: the integer multiply-add pipe (57% busy at q = 4 with a last wave of
 // CTAs that fills 68% of the chip; about 290 of its instructions per node of a smoothing
-// step) with the ALU at 39% and 12 to 16 warps per SM to cover the latencies. Measured
+// step) with the ALU at 28% and 12 to 16 warps per SM to cover the latencies. Measured
 // per launch, FP64 pipe kernels before / these: smoothing step 33 x 31 x 32 cells
-// p = 3 0.247 / 0.093 ms, 729^2 cells p = 4 1.11 / 0.50 ms; operator 64 x 60 x 57 cells
-// p = 4 3.04 / 0.96 ms; projection 32^3 cells p = 3 0.042 / 0.022 ms.
+// p = 3 0.261 / 0.093 ms, 729^2 cells p = 4 1.14 / 0.50 ms; operator (projection and
+// residual) 64 x 60 x 57 cells p = 4 3.37 / 1.13 ms.
 #pragma once
 
 #include <algorithm>
@@ -763,10 +766,7 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
         auto at = [&](int i, long long v) {               // v: b as a block value
             const long long ti = xs[i];
             if (!zero) v -= fx_shr(ti << t.n, E - te);
-            if (G::ALL || L.live) {
-                xs[i] = v;
-                if (write_r) ys[i] = difference(ys[i], fx_to(ti, te + t.n));
-            }
+            if (G::ALL || L.live) xs[i] = v;
             mag.add(v);
         };
         if (__any_sync(0xffffffffu, ev < FX_LOW)) {
@@ -814,6 +814,13 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
     }
     if (!SMOOTH && has_b) {
         if (mode & RES_CORNERS) {
+            if (write_r) {                               // (both are wanted by callers' calls only)
+                fx_cp_wait();
+                __syncwarp();
+#pragma unroll 1
+                for (int i = L.sub; i < N; i += SP)
+                    if (active) r[cell * NL + L.k * N + i] = difference(ys[i], fx_to(xs[i], t.e));
+            }
             subtract_from_b();
         } else {
             fx_cp_wait();
@@ -853,7 +860,7 @@ __device__ __forceinline__ void fx_cells_body(const FxTab &tab, const FxConst &c
         }
     }
     // the result leaves through Y
-    if (SMOOTH || (mode & RES_WRITE_R)) {
+    if (SMOOTH || ((mode & RES_WRITE_R) && !(write_r && (mode & RES_CORNERS)))) {
         // without b the block is A u: the residual b - A u is its negative
         const bool neg = !SMOOTH && !(mode & RES_NEGATE);
         if (!in_y)
