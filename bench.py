@@ -39,11 +39,12 @@ FP64_NOMINAL_TFLOPS = 1.25       # nominal GB300 dense FP64, context beside the 
 # DRAM bytes (read + write) of one launch of the FP64 smoothing kernel on this
 # workload from one ncu capture, valid only for the kernel sources it was taken
 # on (SHA-256 of the files below); once they change, `traffic` reads null
-SMOOTH_TRAFFIC = {"kernel": "k_fx_cells<3,4,0>", "bytes": 116_969_216 + 2_981_632,
-                  "sources_sha256": "fd894e1a3c43d8ad0ea3091e6a435c491da2f28dd828c7e830ee1822eec5361d",
+SMOOTH_TRAFFIC = {"kernel": "k_fx_cells<3,4,1,0>", "bytes": 116_991_744 + 3_138_816,
+                  "sources_sha256": "6c2630cf3b0925c6de12d9187e966c377ea8bb16b277fca438dcd910aced92b0",
                   "files": ("fx.cuh", "dg_fx.cuh", "dg_fp64.cu")}
-# 32 x 32 + 64 bit integer multiply-adds per SM and clock (a loop of independent
-# products); the FP64 kernels of the DG levels take three per multiply-add
+# 32 x 32 + 64 bit integer multiply-adds per SM and clock, a constant: what a loop of
+# independent products once reached on a GB300; no run of this program measures it. The
+# FP64 kernels of the DG levels take three per multiply-add
 INT_MAD_PER_SM_CLK = 30
 
 
@@ -584,7 +585,7 @@ def run_gb300(args):
     if rank == 0 and not args.no_mixed:
         mixed = mixed_section(flush, stream)
 
-    smooth_kernel = f"k_fx_cells<{d},{q},0>"
+    smooth_kernel = f"k_fx_cells<{d},{q},1,0>"   # one lane per slab (32^3 cells)
     props = torch.cuda.get_device_properties(local)
     int_peak = 2 * INT_MAD_PER_SM_CLK / 3 * props.multi_processor_count * (clk.get("sm_mhz") or 2070) * 1e-6
     traffic, traffic_note = smooth_traffic(smooth_kernel)
@@ -609,9 +610,9 @@ def run_gb300(args):
                          "flops_per_launch": flops,
                          "frac_at_10dq_flop_per_dof": survey_flops / (avg_ms * 1e-3) / 1e12 / int_peak,
                          "hbm_bytes_per_launch": smooth_bytes_per_cell(d, q) * ctx.info.ncell,
-                         "peak_note": ("64-bit fixed-point multiply-adds: a third of the measured integer "
-                                       f"multiply-add rate ({INT_MAD_PER_SM_CLK} per SM and clock) at the run's SM "
-                                       "clock; the FP64 pipe's FMA-loop peak (dgmg_fma_peak, this run) is under "
+                         "peak_note": ("64-bit fixed-point multiply-adds: a third of an assumed integer "
+                                       f"multiply-add rate (constant, {INT_MAD_PER_SM_CLK} per SM and clock, not "
+                                       "measured in this run) at the run's SM clock; the FP64 pipe's FMA-loop peak (dgmg_fma_peak, this run) is under "
                                        f"measured_peaks_tflops, its nominal {FP64_NOMINAL_TFLOPS}"),
                          "measured_peaks_tflops": {"fp64_fma": fp64_peak, "fp32_fma": fp32_peak,
                                                    "fp32x2_fma": fp32x2_peak, "clocks": peak_clk}},

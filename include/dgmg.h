@@ -27,6 +27,20 @@
  * without a host synchronisation unless stated. The library owns everything
  * inside a dgmg_ctx. A ctx may be used from one host thread at a time.
  *
+ * Accuracy of the FP64 DG stages (apply, residual, smooth, vcycle, solve, project,
+ * residual_restrict, FP64 batches): vectors are FP64, and b - A u, u + P e and
+ * (1 - omega) u + omega A_KK^{-1}(...) are taken element by element with all bits of
+ * b and u. Within a stage the values of a cell are 60-bit integers of one exponent:
+ * A u, the corrections and the corner sums of the restriction are accurate relative
+ * to the largest term in their cell and its face neighbours (about 2^-57 of it a
+ * stage), not relative to each element. An element far below its cell's largest (in
+ * the GL basis, say, whose mass is diagonal) therefore holds fewer digits than a sum
+ * of its own terms in FP64 would give it. A value that is not finite makes every
+ * value computed from its cell's block NaN, in its cell and the face neighbours.
+ * Subnormal inputs and results are kept; facet coefficients are not: the products of
+ * neighbouring kappa, and kappa times the cell's scale, have to lie in the normal
+ * range (kappa between about 1e-150 and 1e150).
+ *
  * Errors: every int-returning call returns DGMG_OK (0) or a negative code; the
  * thread-local message of the last failure is returned by dgmg_last_error().
  * Arguments are validated before any device work is queued.

@@ -9,12 +9,15 @@
 // A block of numbers (the tensor of a cell) shares one exponent: value = t 2^e with a
 // 64-bit integer t, |t| < 2^60. After every matrix the block is shifted left to use
 // all 60 bits, so a stage loses about 2^-58 of the block's largest value, where FP64
-// loses 2^-53 of every product. Inputs and outputs are FP64; rounding to 53 bits
-// happens once, on output. Measured against the FP64 kernels this replaces (largest
-// of the errors to a 64-bit reference, before / after): residual p = 4, 64 x 60 x 57
-// cells 1.7e-15 / 1.6e-15; p = 6, 243 x 241 cells 4.1e-15 / 3.9e-15; four smoothing
-// steps p = 3, 33 x 31 x 32 cells 2.5e-15 / 2.5e-15, p = 4, 729^2 cells 8.7e-16 / 9.1e-16
-// (the reference's own rounding).
+// loses 2^-53 of every product: norm by norm, cell by cell, the sums are at least as
+// exact, but a value far below its block's largest holds fewer bits than FP64 would keep.
+// So the vectors stay FP64 and are added to and subtracted from node by node (dg_fx.cuh),
+// and the table of the block inverses, whose entries span the cell's eigenvalues, keeps an
+// exponent per entry (fx_scaled). Largest errors against a 64-bit reference, FP64 pipe
+// kernels before / these: operator p = 4, 64 x 60 x 57 cells 2.4e-15 / 2.4e-15; residual p = 6
+// GL, 243 x 241 cells 4.3e-15 / 4.1e-15; four smoothing steps p = 3, 33 x 31 x 32 cells 2.5e-15
+// / 2.5e-15, p = 4, 729^2 cells 8.6e-16 / 8.3e-16 (near the reference's own rounding); V-cycles
+// 16^2 p = 2 7.1e-16 / 7.9e-16, 23 x 17 x 20 p = 2 9.9e-16 / 1.2e-15.
 //
 // An input that is not finite marks its block (e >= FX_BAD), and every value
 // computed from a marked block is output as NaN. Results above the normal range are

@@ -294,7 +294,10 @@ struct Q1Plan {
 // bytes. V-cycle (creation) with the level on the grid / as the dense one: 512
 // vertices 93 / 68 us (0.5 / 0.7 ms), 1089 64 / 50 us (0.55 / 0.8 ms), 1331 93 / 77 us
 // (0.9 / 1.9 ms), 2025 66 / 62 us (0.8 / 1.7 ms), 3025 66 / 76 us: the line lies where
-// the gain pays for the set-up within a solve or two. The server's contexts, admitted by
+// the gain pays for the set-up within a solve or two. dgmg_update_kappa forms it anew, beside
+// the cells' factors: it shows there only where it takes longer than they do (23 x 17 x 20
+// cells p = 2, 792 vertices: update and one cycle 4.5 ms, 4.3 with a launch per step; 33^2
+// p = 4 0.73 and 0.91). The server's contexts, admitted by
 // their bytes, stop at half a megabyte.
 constexpr int64_t Q1_DENSE_MAX = 1100, Q1_DENSE_MAX_SHARED = 256;
 constexpr size_t Q1_DENSE_SMEM = 160 * 1024;   // level vectors of the set-up kernel, at most
